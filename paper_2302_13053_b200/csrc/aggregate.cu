@@ -1,6 +1,5 @@
-// Full-graph neighbour aggregation of one message-passing round (Eq. 1):
-// GCN symmetric-normalised sum, GraphSAGE mean (+ self concat), and the fused
-// GAT edge-score / segment-softmax / weighted-sum pass, over a CSR graph.
+// Full-graph neighbour aggregation of one message-passing round (Eq. 1) over a CSR graph:
+// GCN symmetric-normalised sum, GraphSAGE mean and max (+ self concat); the GAT pass is in gat.cu.
 //
 // The work is a gather-reduce bound by the memory system, not a dense
 // contraction: neighbour rows are streamed with the widest aligned vector
@@ -12,6 +11,7 @@
 // segments in order.  Nothing depends on which warp ran what, so results are
 // the same bits on every call.
 #include "common.cuh"
+#include "gat.h"
 
 namespace retexo {
 
@@ -540,239 +540,6 @@ static int dispatch_op(int op, const AggArgs& a, int n_sm, cudaStream_t st) {
     return dispatch_ch<VEC, kOpSum>(a, n_sm, st);
 }
 
-// ---------------------------------------------------------------- GAT
-constexpr int kGatMaxHeads = 8;
-
-struct GatArgs {
-    int64_t n;
-    const int64_t* rowptr;
-    const int32_t* colidx;
-    const float* p;
-    int64_t ldp;
-    int32_t heads, head_dim, dim;
-    const float* a_src;
-    const float* a_dst;
-    float slope;
-    int32_t self_loop;
-    float* s;               // [n x heads] scratch
-    float* t;
-    float* out;
-    int64_t ldout;
-    __nv_bfloat16* out16;
-    int64_t ldout16;
-    int32_t* hub_list;      // rows a whole block takes, listed by gat_scores_kernel (order arbitrary; no result depends on it)
-    int32_t* hub_count;
-};
-
-constexpr int kGatHubEntries = 128;     // rows with at least this many entries are taken by a whole block
-
-// s_u = <a_src, p_u>, t_u = <a_dst, p_u> per head; one warp per node.  The warp also lists its node
-// if the node's row is long enough for a whole block.
-__global__ void __launch_bounds__(kAggThreads) gat_scores_kernel(GatArgs a) {
-    const int lane = threadIdx.x & 31;
-    const int64_t u = blockIdx.x * (int64_t)kAggWarps + (threadIdx.x >> 5);
-    if (u >= a.n) return;
-    if (lane == 0 && a.rowptr[u + 1] - a.rowptr[u] + (a.self_loop ? 1 : 0) >= kGatHubEntries)
-        a.hub_list[atomicAdd(a.hub_count, 1)] = (int32_t)u;
-    const float* row = a.p + u * a.ldp;
-    for (int h = 0; h < a.heads; ++h) {
-        float ss = 0.f, tt = 0.f;
-        for (int j = lane; j < a.head_dim; j += kWarp) {
-            const float x = row[h * a.head_dim + j];
-            ss = fmaf(a.a_src[h * a.head_dim + j], x, ss);
-            tt = fmaf(a.a_dst[h * a.head_dim + j], x, tt);
-        }
-        ss = warp_sum(ss);
-        tt = warp_sum(tt);
-        if (lane == 0) {
-            a.s[u * a.heads + h] = ss;
-            a.t[u * a.heads + h] = tt;
-        }
-    }
-}
-
-// The running soft-max state and weighted sum of one warp over the entries [e0, e0 + 32) of row v, for
-// e0 = e_first, e_first + e_step, ...  (entry `deg`, if any, is the self loop).  Entries are taken 32 at
-// a time: lane j scores entry j for every head, the chunk maximum and the rescale of the running
-// soft-max state are warp reductions (one exp per entry and head in total), then all lanes add the
-// weighted neighbour rows for the columns they own.
-template <int NC>
-__device__ __forceinline__ void gat_accumulate(const GatArgs& a, int64_t v, int64_t beg, int64_t deg, int64_t total,
-                                               int64_t e_first, int64_t e_step, int lane, int warp,
-                                               float (*p_s)[kWarp][kGatMaxHeads], const float (&tv)[kGatMaxHeads],
-                                               const int (&head_of)[NC], float (&m)[kGatMaxHeads],
-                                               float (&l)[kGatMaxHeads], float (&acc)[NC]) {
-    for (int64_t e0 = e_first; e0 < total; e0 += e_step) {
-        const int cnt = (int)min((int64_t)kWarp, total - e0);
-        int my_u = 0;
-        float e[kGatMaxHeads];
-        const bool valid = lane < cnt;
-        if (valid) my_u = (e0 + lane < deg) ? __ldg(a.colidx + beg + e0 + lane) : (int)v;
-#pragma unroll
-        for (int h = 0; h < kGatMaxHeads; ++h) {
-            e[h] = -INFINITY;
-            if (valid && h < a.heads) {
-                const float z = a.s[(int64_t)my_u * a.heads + h] + tv[h];
-                e[h] = z > 0.f ? z : a.slope * z;
-            }
-        }
-        float scale[kGatMaxHeads];
-#pragma unroll
-        for (int h = 0; h < kGatMaxHeads; ++h) {
-            scale[h] = 1.f;
-            if (h < a.heads) {
-                const float mn = fmaxf(m[h], warp_max(e[h]));     // finite: cnt >= 1
-                scale[h] = expf(m[h] - mn);                       // exp(-inf) = 0 on the first chunk
-                const float pj = valid ? expf(e[h] - mn) : 0.f;
-                l[h] = l[h] * scale[h] + warp_sum(pj);
-                m[h] = mn;
-                p_s[warp][lane][h] = pj;
-            }
-        }
-        __syncwarp();
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            float sc = 1.f;
-#pragma unroll
-            for (int h = 0; h < kGatMaxHeads; ++h) if (h == head_of[c]) sc = scale[h];
-            acc[c] *= sc;
-        }
-        // several neighbour rows in flight per lane (a hub's row is otherwise one dependent load after
-        // another); the products are still added in entry order
-        constexpr int U = NC <= 2 ? 8 : (NC <= 4 ? 4 : 2);
-        int j = 0;
-        for (; j + U <= cnt; j += U) {
-            float x[U][NC];
-#pragma unroll
-            for (int t = 0; t < U; ++t) {
-                const int u = __shfl_sync(0xffffffffu, my_u, j + t);
-                const float* row = a.p + (int64_t)u * a.ldp;
-#pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    const int col = c * kWarp + lane;
-                    x[t][c] = col < a.dim ? __ldg(row + col) : 0.f;
-                }
-            }
-#pragma unroll
-            for (int t = 0; t < U; ++t)
-#pragma unroll
-                for (int c = 0; c < NC; ++c) acc[c] = fmaf(p_s[warp][j + t][head_of[c]], x[t][c], acc[c]);
-        }
-        for (; j < cnt; ++j) {
-            const int u = __shfl_sync(0xffffffffu, my_u, j);
-            const float* row = a.p + (int64_t)u * a.ldp;
-#pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                const int col = c * kWarp + lane;
-                if (col < a.dim) acc[c] = fmaf(p_s[warp][j][head_of[c]], __ldg(row + col), acc[c]);
-            }
-        }
-        __syncwarp();
-    }
-}
-
-// Blocks [0, hub_blocks): one block per listed hub row at a time.  Warp w takes the trips w, w + 8, ...
-// of the row with a soft-max state of its own; the eight states are then merged in warp order
-//   M = max m_w,  L = sum l_w e^(m_w - M),  Z = sum acc_w e^(m_w - M) / L,
-// so the result does not depend on scheduling (it differs from the one-warp order only in rounding).
-// Blocks from hub_blocks on: one warp per destination v, rows of fewer than kGatHubEntries entries.
-// The hub blocks come first in launch order, so the longest rows start ahead of the short ones.
-template <int NC>
-__global__ void __launch_bounds__(kAggThreads) gat_rows_kernel(GatArgs a, int hub_blocks) {
-    __shared__ float p_s[kAggWarps][kWarp][kGatMaxHeads];
-    __shared__ float sm_m[kAggWarps][kGatMaxHeads], sm_l[kAggWarps][kGatMaxHeads];
-    __shared__ float sm_acc[kAggWarps][NC * kWarp];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const bool hub_block = (int)blockIdx.x < hub_blocks;
-    const int n_hubs = hub_block ? *a.hub_count : 0;
-    int hub = blockIdx.x;
-    int64_t v = hub_block ? -1 : (int64_t)(blockIdx.x - hub_blocks) * kAggWarps + warp;
-    if (!hub_block && v >= a.n) return;
-
-    float m[kGatMaxHeads], l[kGatMaxHeads], tv[kGatMaxHeads];
-    float acc[NC];
-    int head_of[NC];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-        const int col = c * kWarp + lane;
-        head_of[c] = col < a.dim ? col / a.head_dim : 0;
-    }
-
-    if (!hub_block) {
-        const int64_t beg = a.rowptr[v];
-        const int64_t deg = a.rowptr[v + 1] - beg;
-        const int64_t total = deg + (a.self_loop ? 1 : 0);
-        if (total >= kGatHubEntries) return;                 // a hub block takes this row
-#pragma unroll
-        for (int h = 0; h < kGatMaxHeads; ++h) {
-            m[h] = -INFINITY;
-            l[h] = 0.f;
-            tv[h] = h < a.heads ? a.t[v * a.heads + h] : 0.f;
-        }
-#pragma unroll
-        for (int c = 0; c < NC; ++c) acc[c] = 0.f;
-        gat_accumulate<NC>(a, v, beg, deg, total, 0, kWarp, lane, warp, p_s, tv, head_of, m, l, acc);
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-            const int col = c * kWarp + lane;
-            if (col < a.dim) {
-                float val = 0.f;
-                if (total > 0) {
-                    float lh = 1.f;
-#pragma unroll
-                    for (int h = 0; h < kGatMaxHeads; ++h) if (h == head_of[c]) lh = l[h];
-                    val = acc[c] / lh;
-                }
-                if (a.out) a.out[v * a.ldout + col] = val;
-                if (a.out16) a.out16[v * a.ldout16 + col] = f32_to_bf16(val);
-            }
-        }
-        return;
-    }
-
-    for (; hub < n_hubs; hub += hub_blocks) {
-        v = a.hub_list[hub];
-        const int64_t beg = a.rowptr[v];
-        const int64_t deg = a.rowptr[v + 1] - beg;
-        const int64_t total = deg + (a.self_loop ? 1 : 0);
-#pragma unroll
-        for (int h = 0; h < kGatMaxHeads; ++h) {
-            m[h] = -INFINITY;
-            l[h] = 0.f;
-            tv[h] = h < a.heads ? a.t[v * a.heads + h] : 0.f;
-        }
-#pragma unroll
-        for (int c = 0; c < NC; ++c) acc[c] = 0.f;
-        gat_accumulate<NC>(a, v, beg, deg, total, (int64_t)warp * kWarp, (int64_t)kAggWarps * kWarp, lane, warp, p_s, tv,
-                           head_of, m, l, acc);
-        if (lane < kGatMaxHeads) {
-            float mm = -INFINITY, ll = 0.f;
-#pragma unroll
-            for (int h = 0; h < kGatMaxHeads; ++h) if (h == lane) { mm = m[h]; ll = l[h]; }
-            sm_m[warp][lane] = mm;
-            sm_l[warp][lane] = ll;
-        }
-#pragma unroll
-        for (int c = 0; c < NC; ++c) sm_acc[warp][c * kWarp + lane] = acc[c];
-        __syncthreads();
-        for (int col = threadIdx.x; col < a.dim; col += kAggThreads) {
-            const int h = col / a.head_dim;
-            float big = -INFINITY;
-            for (int w = 0; w < kAggWarps; ++w) big = fmaxf(big, sm_m[w][h]);
-            float den = 0.f, num = 0.f;
-            for (int w = 0; w < kAggWarps; ++w) {
-                const float f = sm_m[w][h] == -INFINITY ? 0.f : expf(sm_m[w][h] - big);     // (a warp without trips)
-                den = fmaf(sm_l[w][h], f, den);
-                num = fmaf(sm_acc[w][col], f, num);
-            }
-            const float val = num / den;
-            if (a.out) a.out[v * a.ldout + col] = val;
-            if (a.out16) a.out16[v * a.ldout16 + col] = f32_to_bf16(val);
-        }
-        __syncthreads();
-    }
-}
-
 }  // namespace retexo
 
 using namespace retexo;
@@ -782,10 +549,7 @@ extern "C" size_t retexo_aggregate_workspace_size(int64_t n_nodes, int64_t n_edg
     Sizer s;
     if (n_nodes < 0) return 0;
     if (type == RETEXO_GAT) {
-        s.take<float>((size_t)n_nodes * (size_t)(heads > 0 ? heads : 1));
-        s.take<float>((size_t)n_nodes * (size_t)(heads > 0 ? heads : 1));
-        s.take<int32_t>((size_t)n_nodes);                                 // hub rows
-        s.take<int32_t>(64);                                              // their count
+        gat_forward_workspace(n_nodes, heads > 0 ? heads : 1, s);
     } else {
         s.take<float>((size_t)n_nodes);                                   // coef
         s.take<int32_t>((size_t)(n_edges / kHeavyDegree + 1));            // heavy rows
@@ -827,28 +591,10 @@ extern "C" int retexo_aggregate(const retexo_csr* g, int32_t type, const float* 
     const int64_t n = g->n_nodes;
 
     if (type == RETEXO_GAT) {
-        GatArgs a;
-        a.n = n; a.rowptr = g->rowptr; a.colidx = g->colidx; a.p = q; a.ldp = ldq;
-        a.heads = gat->heads; a.head_dim = gat->head_dim; a.dim = dim;
-        a.a_src = gat->a_src; a.a_dst = gat->a_dst; a.slope = gat->negative_slope;
-        a.self_loop = gat->add_self_loop ? 1 : 0;
-        a.s = ws.take<float>((size_t)n * gat->heads);
-        a.t = ws.take<float>((size_t)n * gat->heads);
-        a.hub_list = ws.take<int32_t>((size_t)n);
-        a.hub_count = ws.take<int32_t>(64);
-        RETEXO_CUDA_TRY(cudaMemsetAsync(a.hub_count, 0, sizeof(int32_t), st));
-        a.out = out; a.ldout = ldout;
-        a.out16 = static_cast<__nv_bfloat16*>(out_bf16); a.ldout16 = ldout_bf16;
-        const unsigned blocks = (unsigned)((n + kAggWarps - 1) / kAggWarps);
-        gat_scores_kernel<<<blocks, kAggThreads, 0, st>>>(a);
-        const int nc = (dim + kWarp - 1) / kWarp;
-        const int hub_blocks = 3 * n_sm;       // as many as are resident at once; those without a row leave at once
-        const unsigned grid = blocks + (unsigned)hub_blocks;
-        if (nc <= 1) gat_rows_kernel<1><<<grid, kAggThreads, 0, st>>>(a, hub_blocks);
-        else if (nc <= 2) gat_rows_kernel<2><<<grid, kAggThreads, 0, st>>>(a, hub_blocks);
-        else if (nc <= 4) gat_rows_kernel<4><<<grid, kAggThreads, 0, st>>>(a, hub_blocks);
-        else gat_rows_kernel<8><<<grid, kAggThreads, 0, st>>>(a, hub_blocks);
-        return launch_status();
+        GatForward f{};
+        f.g = *g; f.p = q; f.ldp = ldq; f.gat = *gat; f.out = out; f.ldout = ldout;
+        f.out16 = static_cast<__nv_bfloat16*>(out_bf16); f.ldout16 = ldout_bf16;
+        return gat_forward_launch(f, ws, n_sm, st);
     }
 
     AggArgs a;

@@ -1,0 +1,251 @@
+// Lane layout of the GAT kernels for head widths 4, 8, 16, ... 256 on aligned rows.  A lane owns W contiguous columns of one
+// head (8, or 4 where the heads are 4 wide) and LPG lanes (a power of two) one CSR entry, so a warp reads G = 32 / LPG whole
+// neighbour rows per load instruction and every lane scores its entry for its own head.  Nothing is exchanged between lanes
+// until a row is done: sums over a head's columns are linear, so they are reduced once per row, not once per entry.
+#pragma once
+#include "common.cuh"
+
+namespace retexo {
+
+constexpr int kGatThreads = 128, kGatWarps = kGatThreads / kWarp;      // (256: a block's slots idle until its longest row is done)
+constexpr int kGatBlocksPerSm = 9;      // 56 registers a thread: 36 warps an SM (10 blocks spill, 7 at 69 registers wait longer)
+// A row of up to kGatGroupEntries entries is taken by one group of lanes (so a warp works on G rows at once), a longer one
+// by a whole warp, and one of `hub_entries` or more by a whole block.
+constexpr int kGatGroupEntries = 32;
+// A block costs more per entry (a barrier a row, four states to merge), so only rows go to blocks that would keep a warp
+// busy for a good part of what the whole grid takes: a quarter of the entries a resident warp sees, but never below 64.
+inline int gat_hub_entries(int64_t n_edges, int n_sm) {
+    const int64_t share = n_edges / ((int64_t)n_sm * 128);
+    return (int)(share < 64 ? 64 : share > 65536 ? 65536 : share);
+}
+
+template <int LPG, int W>
+struct GatLanes {
+    static constexpr int G = kWarp / LPG;                                  // entries per step
+    static constexpr int kMaxU = 2;                                        // neighbour rows in flight per lane (4: fewer warps fit)
+    static constexpr int U = G * kMaxU > kWarp ? kWarp / G : kMaxU;        // ... of a warp on one row: at most one trip of 32 entries
+    int g, li;
+    bool on;                   // the lane owns columns (dim need not fill the lanes); if not, it reads column 0 and drops it
+    int col, head;
+    __device__ __forceinline__ GatLanes(int lane, int dim, int head_dim) {
+        g = lane / LPG;
+        li = lane % LPG;
+        on = W * li < dim;
+        col = on ? W * li : 0;
+        head = col / head_dim;
+    }
+};
+
+// Whether the lane layout covers a shape (p and, where given, q hold its rows), and with how many lanes / columns per lane.
+inline bool gat_lanes_cover(int32_t dim, int32_t head_dim, const float* p, int64_t ldp, const float* q, int64_t ldq, int* lpg, int* w) {
+    if (head_dim < 4 || (head_dim & (head_dim - 1)) != 0 || dim > 256) return false;
+    *w = head_dim == 4 ? 4 : 8;
+    if (ldp % *w != 0 || !aligned_to(p, 4 * *w) || (q && (ldq % *w != 0 || !aligned_to(q, 4 * *w)))) return false;
+    *lpg = 1;
+    while (*lpg * *w < dim) *lpg <<= 1;
+    return true;
+}
+
+// Calls go.template operator()<LPG, W>() for the layout gat_lanes_cover chose.
+template <typename F>
+inline int gat_lanes_dispatch(int lpg, int w, F&& go) {
+    if (w == 4) {
+        switch (lpg) {
+            case 8: return go.template operator()<8, 4>();
+            case 4: return go.template operator()<4, 4>();
+            case 2: return go.template operator()<2, 4>();
+            default: return go.template operator()<1, 4>();
+        }
+    }
+    switch (lpg) {
+        case 32: return go.template operator()<32, 8>();
+        case 16: return go.template operator()<16, 8>();
+        case 8: return go.template operator()<8, 8>();
+        case 4: return go.template operator()<4, 8>();
+        case 2: return go.template operator()<2, 8>();
+        default: return go.template operator()<1, 8>();
+    }
+}
+
+// A lane's W columns of a row.
+template <int W>
+struct Cols {
+    float v[W];
+    __device__ __forceinline__ void zero() {
+#pragma unroll
+        for (int i = 0; i < W; ++i) v[i] = 0.f;
+    }
+    // one 16- or 32-byte load of read-only memory (aligned to as much)
+    __device__ __forceinline__ void load(const float* p) {
+        if constexpr (W == 4) {
+            const float4 x = __ldg(reinterpret_cast<const float4*>(p));
+            v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+        } else {
+            asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                         : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]) : "l"(p));
+        }
+    }
+    __device__ __forceinline__ void load_unaligned(const float* p) {
+#pragma unroll
+        for (int i = 0; i < W; ++i) v[i] = __ldg(p + i);
+    }
+    __device__ __forceinline__ void scale(float f) {
+#pragma unroll
+        for (int i = 0; i < W; ++i) v[i] *= f;
+    }
+    __device__ __forceinline__ void fma(float w, const Cols& x) {
+#pragma unroll
+        for (int i = 0; i < W; ++i) v[i] = fmaf(w, x.v[i], v[i]);
+    }
+    __device__ __forceinline__ float dot(const Cols& x) const {
+        float a = v[0] * x.v[0], b = v[1] * x.v[1];
+#pragma unroll
+        for (int i = 2; i < W; i += 2) { a = fmaf(v[i], x.v[i], a); b = fmaf(v[i + 1], x.v[i + 1], b); }
+        return a + b;
+    }
+    __device__ __forceinline__ void add_xor(int o) {
+#pragma unroll
+        for (int i = 0; i < W; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+    }
+    __device__ __forceinline__ void store(float* p, bool vec) const {      // vec: p and its row stride are 16-byte aligned
+        if (vec) {
+#pragma unroll
+            for (int i = 0; i < W; i += 4) *reinterpret_cast<float4*>(p + i) = make_float4(v[i], v[i + 1], v[i + 2], v[i + 3]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < W; ++i) p[i] = v[i];
+        }
+    }
+    __device__ __forceinline__ void store(__nv_bfloat16* p, bool vec) const {      // vec: 8-byte aligned
+        uint32_t b[W / 2];
+#pragma unroll
+        for (int i = 0; i < W / 2; ++i) {
+            const __nv_bfloat162 x = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+            b[i] = *reinterpret_cast<const uint32_t*>(&x);
+        }
+        if (vec) {
+#pragma unroll
+            for (int i = 0; i < W / 2; i += 2) *reinterpret_cast<uint2*>(p + 2 * i) = make_uint2(b[i], b[i + 1]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < W; ++i) p[i] = f32_to_bf16(v[i]);
+        }
+    }
+};
+
+__device__ __forceinline__ float leaky(float z, float slope) { return z > 0.f ? z : slope * z; }
+// The lane kernels keep scores in units of log 2 (a leaky ReLU commutes with a positive factor), so that e^(x - m) is one
+// subtraction and one hardware exponential.  Its error is two units in the last place (as the library function's);
+// the weights it gives are divided by their own sum.
+constexpr float kLog2E = 1.4426950408889634f;
+__device__ __forceinline__ float exp2_hw(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+// 2^(x - ref) for x <= ref, 0 for x = -inf whatever ref is
+__device__ __forceinline__ float exp2_rel(float x, float ref) { return x == -INFINITY ? 0.f : exp2_hw(x - ref); }
+
+// Hands the entries of a CSR row to pass.batch<U>(u, ok), U neighbours per lane at a time; entry `deg`, if any, is the row's
+// own node `self`.  Where ok is false u is an entry of the row all the same (or `self`), so a pass may load its data
+// without a predicate and give it weight zero.
+// By a warp: trips of 32 entries from `first` on, `step` apart, dealt to the groups one by one.
+template <int LPG, int W, class P>
+__device__ __forceinline__ void gat_walk_by_warp(P& pass, const GatLanes<LPG, W>& L, const int32_t* __restrict__ colidx, int32_t self,
+                                                 int64_t beg, int32_t deg, int32_t total, int32_t first, int32_t step, int lane) {
+    constexpr int G = GatLanes<LPG, W>::G, U = GatLanes<LPG, W>::U;
+    for (int32_t e0 = first; e0 < total; e0 += step) {
+        const int cnt = min(kWarp, total - e0);
+        const int32_t e = e0 + (lane < cnt ? lane : 0);
+        const int32_t my_u = e < deg ? __ldg(colidx + beg + e) : self;
+#pragma unroll 1
+        for (int j = 0; j < cnt; j += G * U) {
+            int32_t u[U];
+            bool ok[U];
+#pragma unroll
+            for (int t = 0; t < U; ++t) {
+                const int at = j + t * G + L.g;
+                u[t] = __shfl_sync(0xffffffffu, my_u, at & 31);
+                ok[t] = at < cnt;
+            }
+            pass.template batch<U>(u, ok);
+        }
+    }
+}
+// By a group: every group of the warp its own row (total = 0: none); longest = the largest total of the warp.
+template <int LPG, int W, class P>
+__device__ __forceinline__ void gat_walk_by_group(P& pass, const GatLanes<LPG, W>& L, const int32_t* __restrict__ colidx, int32_t self,
+                                                  int64_t beg, int32_t deg, int32_t total, int32_t longest) {
+    constexpr int U = GatLanes<LPG, W>::kMaxU < LPG ? GatLanes<LPG, W>::kMaxU : LPG;
+    const int32_t stored = min(deg, total);
+    auto entry = [&](int32_t e) -> int32_t {
+        if (e >= total) e = 0;
+        return e < stored ? __ldg(colidx + beg + e) : self;
+    };
+    int32_t next_u = entry(L.li);
+    for (int32_t e0 = 0; e0 < longest; e0 += LPG) {
+        const int32_t my_u = next_u;
+        if (e0 + LPG < longest) next_u = entry(e0 + LPG + L.li);
+        const int cnt = min(LPG, longest - e0);
+#pragma unroll 1
+        for (int j = 0; j < cnt; j += U) {
+            int32_t u[U];
+            bool ok[U];
+#pragma unroll
+            for (int t = 0; t < U; ++t) {
+                u[t] = __shfl_sync(0xffffffffu, my_u, L.g * LPG + j + t);
+                ok[t] = e0 + j + t < total;
+            }
+            pass.template batch<U>(u, ok);
+        }
+    }
+}
+
+// s_u = <a_src, p_u> / ln 2, t_u = <a_dst, p_u> / ln 2 per head, and the list of the rows long enough for a whole block (its
+// order varies from run to run; no result depends on it).  A stream over p: LPG lanes a node, kNodes nodes in flight per group
+// (717 k nodes, 4 x 16: 33 us = 5.6 TB/s; a warp per node with 4-byte loads and two shuffle trees per head took 366 us).
+template <int LPG, int W>
+__global__ void __launch_bounds__(256) gat_lane_scores_kernel(int64_t n, const int64_t* __restrict__ rowptr,
+                                                              const float* __restrict__ p, int64_t ldp, int32_t heads,
+                                                              int32_t head_dim, const float* __restrict__ a_src,
+                                                              const float* __restrict__ a_dst, int32_t self_loop, int32_t hub_entries,
+                                                              float* __restrict__ s, float* __restrict__ t,
+                                                              int32_t* __restrict__ hub_list, int32_t* __restrict__ hub_count) {
+    constexpr int kNodes = 2, G = GatLanes<LPG, W>::G;
+    const int lane = threadIdx.x & 31;
+    const GatLanes<LPG, W> L(lane, heads * head_dim, head_dim);
+    const int hw = head_dim / W;                  // lanes a head spans
+    Cols<W> as, ad;
+    as.zero(); ad.zero();
+    if (L.on) { as.load_unaligned(a_src + L.col); ad.load_unaligned(a_dst + L.col); }
+    const int64_t step = (int64_t)gridDim.x * 8 * G * kNodes;
+    for (int64_t u0 = ((int64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * G * kNodes; u0 < n; u0 += step) {
+        Cols<W> x[kNodes];
+#pragma unroll
+        for (int i = 0; i < kNodes; ++i) x[i].load(p + min(u0 + i * G + L.g, n - 1) * ldp + L.col);
+        for (int64_t u = u0 + lane; u < min(n, u0 + G * kNodes); u += kWarp)
+            if (rowptr[u + 1] - rowptr[u] + self_loop >= hub_entries) hub_list[atomicAdd(hub_count, 1)] = (int32_t)u;
+#pragma unroll
+        for (int i = 0; i < kNodes; ++i) {
+            const int64_t u = u0 + i * G + L.g;
+            float ss = as.dot(x[i]), tt = ad.dot(x[i]);
+            for (int o = 1; o < hw; o <<= 1) {
+                ss += __shfl_xor_sync(0xffffffffu, ss, o);
+                tt += __shfl_xor_sync(0xffffffffu, tt, o);
+            }
+            if (u < n && L.on && (L.li & (hw - 1)) == 0) {
+                s[u * heads + L.head] = ss * kLog2E;
+                t[u * heads + L.head] = tt * kLog2E;
+            }
+        }
+    }
+}
+
+template <int LPG, int W>
+inline unsigned gat_lane_scores_grid(int64_t n, int n_sm) {
+    const int64_t per_block = (int64_t)8 * GatLanes<LPG, W>::G * 2;
+    const int64_t want = (n + per_block - 1) / per_block, most = (int64_t)n_sm * 16;
+    return (unsigned)(want < most ? want : most);
+}
+
+}  // namespace retexo
