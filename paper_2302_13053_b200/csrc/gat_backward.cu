@@ -7,10 +7,14 @@
 //   dp_u = sum_v alpha_uv dz_v + ds_u a_src + dt_u a_dst
 //   da_src = sum_u ds_u p_u             da_dst = sum_v dt_v p_v
 // Two passes over the same CSR (the graph is symmetric, so the rows that attend over u are u's own row):
-// one warp per destination v computes the soft-max statistics, c_v and dt_v; one warp per source u then walks
-// the destinations v that attend over it and accumulates ds_u and dp_u in CSR order.  No floating-point
-// atomics: the parameter gradients are summed per block and the block sums in block order.
+// the destinations first (soft-max statistics, c_v and dt_v), then the sources u, which walk the destinations v that attend
+// over them and accumulate ds_u and dp_u.  No floating-point atomics: the parameter gradients are summed per block and the
+// block sums in block order.  Shapes the lane layout of gat_lanes.cuh covers take its kernels, every other shape the general
+// ones (one warp per row, shuffles per entry).
+#include <algorithm>
+
 #include "common.cuh"
+#include "gat_lanes.cuh"
 
 namespace retexo {
 
@@ -26,18 +30,14 @@ struct GatBwdArgs {
     float slope; int32_t self_loop;
     const float* dz; int64_t lddz;
     float* s; float* t;              // [n x heads]
-    float4* stats;                   // [n x heads]: (row maximum, 1 / soft-max sum (0 = dz_v is zero), c_v, dt_v)
+    float4* stats;                   // [n x heads]: (row maximum, 1 / soft-max sum (0 = dz_v is zero), c_v, dt_v; lane layout: t_v)
     float* dp; int64_t lddp;
     __nv_bfloat16* dp16; int64_t lddp16;
     float* partial;                  // [blocks x 2 x dim]: per-block sums of ds_u p_u and dt_u p_u
-    // rows of kGbHubEntries entries or more ("hub rows") are listed by the score kernel and taken by whole blocks
-    int32_t* hub_count; int32_t* hub_list;      // how many, which (in the order the score kernel met them)
-    int32_t* hub_pos;                           // [n]: position in the list, -1 for every other row
-    float* hub_sum;                             // [hubs x 72]: per hub row the 64 column sums of its source pass, then ds per head
+    // lane layout only
+    float* ds; float* dt;                       // [n x heads]
+    int32_t* hub_count; int32_t* hub_list;      // rows a whole block takes: how many ([1]: blocks that are done), which
 };
-
-constexpr int kGbHubEntries = 128;   // a warp takes 32 entries per trip: rows this long keep one warp busy while the grid drains
-constexpr int kGbHubBlocks = 296;    // blocks of the hub kernels (they loop over the list)
 
 __global__ void __launch_bounds__(kGbThreads) gat_bwd_scores_kernel(GatBwdArgs a) {
     const int lane = threadIdx.x & 31;
@@ -54,15 +54,6 @@ __global__ void __launch_bounds__(kGbThreads) gat_bwd_scores_kernel(GatBwdArgs a
         ss = warp_sum(ss);
         tt = warp_sum(tt);
         if (lane == 0) { a.s[u * a.heads + h] = ss; a.t[u * a.heads + h] = tt; }
-    }
-    if (a.hub_pos && lane == 0) {
-        const int64_t total = a.rowptr[u + 1] - a.rowptr[u] + (a.self_loop ? 1 : 0);
-        int32_t pos = -1;
-        if (total >= kGbHubEntries) {      // (the list's order varies from run to run; no result depends on it)
-            pos = atomicAdd(a.hub_count, 1);
-            a.hub_list[pos] = (int32_t)u;
-        }
-        a.hub_pos[u] = pos;
     }
 }
 
@@ -255,403 +246,332 @@ __global__ void __launch_bounds__(256) gat_bwd_reduce_kernel(const float* partia
     }
 }
 
-// ---- rows of up to 64 columns, head width a power of two (the shapes of the paper's RetexoGAT): one lane per
-// entry.  A lane fetches its entry's whole row (16-byte loads, all independent) and takes the per-head dot
-// products by itself against the warp's own row, which sits in shared memory; nothing is exchanged between
-// lanes until the row is done, so a row of several hundred entries is a few dozen trips of 32.
-constexpr int kGb64Warps = 4, kGb64Threads = kGb64Warps * kWarp;
-
-template <int HD>
-__global__ void __launch_bounds__(kGb64Threads) gat_bwd_dst64_kernel(GatBwdArgs a) {
-    __shared__ __align__(16) float g_s[kGb64Warps][64];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t v = blockIdx.x * (int64_t)kGb64Warps + warp;
-    if (v >= a.n) return;
-    const int nv = a.dim >> 2;                      // float4 pieces per row
-    bool any = false;
-    for (int c = lane; c < 64; c += kWarp) {
-        const float x = c < a.dim ? a.dz[v * a.lddz + c] : 0.f;
-        g_s[warp][c] = x;
-        any = any || x != 0.f;
+// ---------------------------------------------------------------- lane layout (gat_lanes.cuh)
+// Destinations: for row v, with its own gradient dz_v in registers, the soft-max statistics and the sums
+//   c_v = sum alpha dalpha,   dt_v = sum alpha g' dalpha - c_v sum alpha g'      (g' = 1 or the slope)
+// in one pass over the entries with a running maximum.  dalpha = <dz_v, p_u> over the head's columns enters linearly, so a lane
+// keeps the share of its own columns and the head's lanes are added once per row.
+template <int LPG, int W>
+struct GatDstPass {
+    const GatBwdArgs& a;
+    const float* p;
+    const float* s;
+    int head, col;
+    bool on;
+    float tv, m, den, c, b1, b2;
+    Cols<W> g;
+    __device__ __forceinline__ GatDstPass(const GatBwdArgs& a_, const GatLanes<LPG, W>& L)
+        : a(a_), p(a_.p + L.col), s(a_.s + L.head), head(L.head), col(L.col), on(L.on) {}
+    // Returns whether this lane's part of the gradient has a non-zero entry.
+    __device__ __forceinline__ bool begin(int64_t v) {
+        tv = __ldg(a.t + v * a.heads + head);
+        m = -INFINITY; den = c = b1 = b2 = 0.f;
+        g.load(a.dz + v * a.lddz + col);
+        bool any = false;
+#pragma unroll
+        for (int i = 0; i < W; ++i) any = any || g.v[i] != 0.f;
+        return on && any;
     }
-    const int64_t beg = a.rowptr[v];
-    const int64_t deg = a.rowptr[v + 1] - beg;
-    const int64_t total = deg + (a.self_loop ? 1 : 0);
-    if (total >= kGbHubEntries) return;             // a hub row: gat_bwd_dst64_hub_kernel's
-    if (!__any_sync(0xffffffffu, any) || total == 0) {
-        if (lane < a.heads) a.stats[v * a.heads + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+    template <int U>
+    __device__ __forceinline__ void batch(const int32_t (&u)[U], const bool (&ok)[U]) {
+        Cols<W> x[U];
+        float z[U];
+#pragma unroll
+        for (int t = 0; t < U; ++t) {
+            z[t] = __ldg(s + (int64_t)u[t] * a.heads);
+            x[t].load(p + (int64_t)u[t] * a.ldp);
+        }
+        float big = m, e[U];
+#pragma unroll
+        for (int t = 0; t < U; ++t) {
+            z[t] += tv;
+            e[t] = ok[t] ? leaky(z[t], a.slope) : -INFINITY;
+            big = fmaxf(big, e[t]);
+        }
+        const float f = exp2_rel(m, big), ref = big == -INFINITY ? 0.f : big;
+        m = big;
+        den *= f; c *= f; b1 *= f; b2 *= f;
+#pragma unroll
+        for (int t = 0; t < U; ++t) {
+            const float w = exp2_hw(e[t] - ref), wg = z[t] > 0.f ? w : w * a.slope, d = g.dot(x[t]);
+            den += w;
+            b2 += wg;
+            c = fmaf(w, d, c);
+            b1 = fmaf(wg, d, b1);
+        }
+    }
+    __device__ __forceinline__ void merge(float m2, float den2, float c2, float b12, float b22) {
+        const float big = fmaxf(m, m2), f = exp2_rel(m, big), f2 = exp2_rel(m2, big);
+        den = den * f + den2 * f2; c = c * f + c2 * f2; b1 = b1 * f + b12 * f2; b2 = b2 * f + b22 * f2;
+        m = big;
+    }
+    // Adds the states of the warp's groups (for a row of the whole warp) in a fixed tree.
+    __device__ __forceinline__ void merge_groups() {
+#pragma unroll
+        for (int o = LPG; o < kWarp; o <<= 1) {
+            const float m2 = __shfl_xor_sync(0xffffffffu, m, o), den2 = __shfl_xor_sync(0xffffffffu, den, o);
+            const float c2 = __shfl_xor_sync(0xffffffffu, c, o), b12 = __shfl_xor_sync(0xffffffffu, b1, o);
+            const float b22 = __shfl_xor_sync(0xffffffffu, b2, o);
+            merge(m2, den2, c2, b12, b22);
+        }
+    }
+    // The lanes of a head add their columns' shares and its first lane writes the row's statistics; warp-uniform call.
+    __device__ __forceinline__ void finish(int64_t v, bool live, bool write, int hw) {
+        for (int o = 1; o < hw; o <<= 1) {
+            c += __shfl_xor_sync(0xffffffffu, c, o);
+            b1 += __shfl_xor_sync(0xffffffffu, b1, o);
+        }
+        if (!write || !on || col % a.head_dim != 0) return;
+        const float inv = live ? 1.f / den : 0.f, cn = live ? c * inv : 0.f;
+        a.stats[v * a.heads + head] = make_float4(live ? m : 0.f, inv, cn, tv);
+        a.dt[v * a.heads + head] = live ? b1 * inv - cn * (b2 * inv) : 0.f;
+    }
+};
+
+// Bound like the forward pass by the gather of p_u (4 dim + 4 heads bytes an entry); rows whose gradient is zero gather nothing.
+// Measured, whole backward pass (a lane per entry reading its own row in 16-byte pieces before; heads of other shapes a warp
+// per entry): 717 k nodes, 14 M entries, 4 x 16: 5319 -> 1850 us; 60 k nodes, 12 M entries: 2960 -> 684 us; 100 k nodes, 3 M
+// entries, 8 x 32: 26.6 -> 0.87 ms; 200 k nodes, 4 M entries, 1 x 8: 834 -> 163 us.
+template <int LPG, int W>
+__global__ void __launch_bounds__(kGatThreads, kGatBlocksPerSm) gat_lane_dst_kernel(GatBwdArgs a, int hub_entries, int hub_blocks) {
+    constexpr int G = GatLanes<LPG, W>::G;
+    __shared__ float sm[2][kGatWarps][5][LPG];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const GatLanes<LPG, W> L(lane, a.dim, a.head_dim);
+    GatDstPass<LPG, W> pass(a, L);
+    const int hw = a.head_dim / W;
+    if ((int)blockIdx.x >= hub_blocks) {
+        const int64_t v0 = ((int64_t)(blockIdx.x - hub_blocks) * kGatWarps + warp) * G;
+        if (v0 >= a.n) return;
+        const int64_t v = min(v0 + L.g, a.n - 1);
+        const int64_t beg = __ldg(a.rowptr + v);
+        const int32_t deg = (int32_t)(__ldg(a.rowptr + v + 1) - beg);
+        const int32_t total = v0 + L.g < a.n ? deg + a.self_loop : INT32_MAX;
+        const bool mine = total <= kGatGroupEntries;
+        const unsigned lanes = __ballot_sync(0xffffffffu, pass.begin(v));
+        const unsigned group = LPG == 32 ? 0xffffffffu : ((1u << (LPG & 31)) - 1u) << (L.g * LPG);
+        const bool live = (lanes & group) != 0 && total > 0;      // else nothing flows back through this row
+        const int32_t take = mine && live ? total : 0;
+        gat_walk_by_group<LPG, W>(pass, L, a.colidx, (int32_t)v, beg, deg, take, __reduce_max_sync(0xffffffffu, take));
+        pass.finish(v, live, mine, hw);
+        unsigned longer = __ballot_sync(0xffffffffu, L.li == 0 && !mine && total < hub_entries);
+        while (longer) {
+            const int src = __ffs(longer) - 1;
+            longer &= longer - 1;
+            const int64_t w = __shfl_sync(0xffffffffu, v, src), w_beg = __shfl_sync(0xffffffffu, beg, src);
+            const int32_t w_deg = __shfl_sync(0xffffffffu, deg, src);
+            const bool w_live = __any_sync(0xffffffffu, pass.begin(w));
+            if (w_live) {
+                gat_walk_by_warp<LPG, W>(pass, L, a.colidx, (int32_t)w, w_beg, w_deg, w_deg + a.self_loop, 0, kWarp, lane);
+                pass.merge_groups();
+            }
+            pass.finish(w, w_live, L.g == 0, hw);
+        }
         return;
     }
-    __syncwarp();
-    constexpr int NH = 64 / HD;                     // heads at most
-    float tv[NH], m[NH], den[NH], csum[NH], a1[NH], a2[NH];
-#pragma unroll
-    for (int h = 0; h < NH; ++h) {
-        tv[h] = h < a.heads ? a.t[v * a.heads + h] : 0.f;
-        m[h] = -INFINITY; den[h] = 0.f; csum[h] = 0.f; a1[h] = 0.f; a2[h] = 0.f;
-    }
-    for (int64_t e0 = 0; e0 < total; e0 += kWarp) {
-        const bool valid = e0 + lane < total;
-        const int64_t u = !valid ? v : (e0 + lane < deg ? (int64_t)__ldg(a.colidx + beg + e0 + lane) : v);
-#pragma unroll
-        for (int h = 0; h < NH; ++h) {
-            if (h < a.heads) {
-                const float z = a.s[u * a.heads + h] + tv[h];
-                const float e = valid ? (z > 0.f ? z : a.slope * z) : -INFINITY;
-                const float mn = fmaxf(m[h], warp_max(e));
-                den[h] = den[h] * expf(m[h] - mn) + warp_sum(valid ? expf(e - mn) : 0.f);
-                m[h] = mn;
+    const int n_hubs = *a.hub_count;
+    int turn = 0;      // (of the rows that meet a barrier)
+    for (int hub = blockIdx.x; hub < n_hubs; hub += hub_blocks) {
+        const int64_t v = a.hub_list[hub];
+        const int64_t beg = a.rowptr[v];
+        const int32_t deg = (int32_t)(a.rowptr[v + 1] - beg);
+        const bool live = __any_sync(0xffffffffu, pass.begin(v));      // (the same in every warp)
+        if (live) {
+            gat_walk_by_warp<LPG, W>(pass, L, a.colidx, (int32_t)v, beg, deg, deg + a.self_loop, warp * kWarp, kGatWarps * kWarp, lane);
+            pass.merge_groups();
+            if (L.g == 0) {
+                sm[turn][warp][0][L.li] = pass.m; sm[turn][warp][1][L.li] = pass.den; sm[turn][warp][2][L.li] = pass.c;
+                sm[turn][warp][3][L.li] = pass.b1; sm[turn][warp][4][L.li] = pass.b2;
             }
+            __syncthreads();
+        }
+        if (warp == 0) {      // the warps' states in warp order
+            if (live) {
+                for (int w = 1; w < kGatWarps; ++w)
+                    pass.merge(sm[turn][w][0][L.li], sm[turn][w][1][L.li], sm[turn][w][2][L.li], sm[turn][w][3][L.li], sm[turn][w][4][L.li]);
+            }
+            pass.finish(v, live, L.g == 0, hw);
+        }
+        turn ^= live ? 1 : 0;
+    }
+}
+
+// Sources: the rows v that attend over u are u's own row (the graph is symmetric) and u itself; with p_u in registers
+//   acc_u = sum alpha_uv dz_v,   ds_u = sum alpha g' (<dz_v, p_u> - c_v),   dp_u = acc_u + ds_u a_src + dt_u a_dst.
+// A destination whose gradient is zero (1 / den = 0 in its statistics) is not read.
+template <int LPG, int W>
+struct GatSrcPass {
+    const GatBwdArgs& a;
+    const float* dz;
+    const float4* stats;
+    int head, col;
+    float su, ds, dc;            // ds: sum alpha g' <dz_v, p_u> over this lane's columns; dc: sum alpha g' c_v
+    Cols<W> px, acc;
+    __device__ __forceinline__ GatSrcPass(const GatBwdArgs& a_, const GatLanes<LPG, W>& L)
+        : a(a_), dz(a_.dz + L.col), stats(a_.stats + L.head), head(L.head), col(L.col) {}
+    __device__ __forceinline__ void begin(int64_t u) {
+        su = __ldg(a.s + u * a.heads + head);
+        px.load(a.p + u * a.ldp + col);
+        ds = dc = 0.f;
+        acc.zero();
+    }
+    template <int U>
+    __device__ __forceinline__ void batch(const int32_t (&v)[U], const bool (&ok)[U]) {
+        Cols<W> g[U];
+        float4 st[U];
+#pragma unroll
+        for (int t = 0; t < U; ++t) {
+            st[t] = __ldg(stats + (int64_t)v[t] * a.heads);
+            if (!ok[t]) st[t].y = 0.f;
+        }
+#pragma unroll
+        for (int t = 0; t < U; ++t) {
+            g[t].zero();
+            if (st[t].y != 0.f) g[t].load(dz + (int64_t)v[t] * a.lddz);
+        }
+#pragma unroll
+        for (int t = 0; t < U; ++t) {
+            const float z = su + st[t].w;
+            const float alpha = st[t].y != 0.f ? exp2_hw(leaky(z, a.slope) - st[t].x) * st[t].y : 0.f;
+            const float ag = z > 0.f ? alpha : alpha * a.slope;
+            ds = fmaf(ag, px.dot(g[t]), ds);
+            dc = fmaf(ag, st[t].z, dc);
+            acc.fma(alpha, g[t]);
         }
     }
-    for (int64_t e0 = 0; e0 < total; e0 += kWarp) {
-        const bool valid = e0 + lane < total;
-        const int64_t u = !valid ? v : (e0 + lane < deg ? (int64_t)__ldg(a.colidx + beg + e0 + lane) : v);
-        float dalpha[NH];
+    __device__ __forceinline__ void merge_groups() {
 #pragma unroll
-        for (int h = 0; h < NH; ++h) dalpha[h] = 0.f;
-        const float4* row = reinterpret_cast<const float4*>(a.p + u * a.ldp);
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            if (i < nv) {
-                const float4 x = valid ? __ldg(row + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-                const float4 gg = *reinterpret_cast<const float4*>(&g_s[warp][4 * i]);
-                dalpha[(4 * i) / HD] += (x.x * gg.x + x.y * gg.y) + (x.z * gg.z + x.w * gg.w);
-            }
-        }
-#pragma unroll
-        for (int h = 0; h < NH; ++h) {
-            if (h < a.heads && valid) {
-                const float z = a.s[u * a.heads + h] + tv[h];
-                const float alpha = expf((z > 0.f ? z : a.slope * z) - m[h]) / den[h];
-                const float gp = z > 0.f ? 1.f : a.slope;
-                csum[h] = fmaf(alpha, dalpha[h], csum[h]);
-                a1[h] = fmaf(alpha * gp, dalpha[h], a1[h]);
-                a2[h] = fmaf(alpha, gp, a2[h]);
-            }
+        for (int o = LPG; o < kWarp; o <<= 1) {
+            ds += __shfl_xor_sync(0xffffffffu, ds, o);
+            dc += __shfl_xor_sync(0xffffffffu, dc, o);
+            acc.add_xor(o);
         }
     }
-#pragma unroll
-    for (int h = 0; h < NH; ++h) {
-        if (h < a.heads) {
-            const float c = warp_sum(csum[h]), s1 = warp_sum(a1[h]), s2 = warp_sum(a2[h]);
-            if (lane == 0) a.stats[v * a.heads + h] = make_float4(m[h], 1.f / den[h], c, s1 - c * s2);
+    // Warp-uniform call; as, ad: this lane's columns of the attention vectors.
+    __device__ __forceinline__ void finish(int64_t u, bool write, int hw, const Cols<W>& as, const Cols<W>& ad, bool vec, bool vec16) {
+        for (int o = 1; o < hw; o <<= 1) ds += __shfl_xor_sync(0xffffffffu, ds, o);
+        if (!write) return;
+        const float d = ds - dc, dt = __ldg(a.dt + u * a.heads + head);
+        acc.fma(d, as);
+        acc.fma(dt, ad);
+        if (a.dp) acc.store(a.dp + u * a.lddp + col, vec);
+        if (a.dp16) acc.store(a.dp16 + u * a.lddp16 + col, vec16);
+        if (col % a.head_dim == 0) a.ds[u * a.heads + head] = d;
+    }
+};
+
+// Bound by the gather of dz_v and the statistics (4 dim + 16 heads bytes an entry).
+template <int LPG, int W>
+__global__ void __launch_bounds__(kGatThreads, kGatBlocksPerSm) gat_lane_src_kernel(GatBwdArgs a, int hub_entries, int hub_blocks,
+                                                                                    int vec, int vec16) {
+    constexpr int G = GatLanes<LPG, W>::G;
+    __shared__ Cols<W> sm_acc[2][kGatWarps][LPG];
+    __shared__ float2 sm_ds[2][kGatWarps][LPG];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const GatLanes<LPG, W> L(lane, a.dim, a.head_dim);
+    GatSrcPass<LPG, W> pass(a, L);
+    const int hw = a.head_dim / W;
+    Cols<W> as, ad;
+    as.zero(); ad.zero();
+    if (L.on) { as.load_unaligned(a.a_src + L.col); ad.load_unaligned(a.a_dst + L.col); }
+    if ((int)blockIdx.x >= hub_blocks) {
+        const int64_t u0 = ((int64_t)(blockIdx.x - hub_blocks) * kGatWarps + warp) * G;
+        if (u0 >= a.n) return;
+        const int64_t u = min(u0 + L.g, a.n - 1);
+        const int64_t beg = __ldg(a.rowptr + u);
+        const int32_t deg = (int32_t)(__ldg(a.rowptr + u + 1) - beg);
+        const int32_t total = u0 + L.g < a.n ? deg + a.self_loop : INT32_MAX;
+        const bool mine = total <= kGatGroupEntries;
+        pass.begin(u);
+        gat_walk_by_group<LPG, W>(pass, L, a.colidx, (int32_t)u, beg, deg, mine ? total : 0, __reduce_max_sync(0xffffffffu, mine ? total : 0));
+        pass.finish(u, mine && L.on, hw, as, ad, vec != 0, vec16 != 0);
+        unsigned longer = __ballot_sync(0xffffffffu, L.li == 0 && !mine && total < hub_entries);
+        while (longer) {
+            const int src = __ffs(longer) - 1;
+            longer &= longer - 1;
+            const int64_t w = __shfl_sync(0xffffffffu, u, src), w_beg = __shfl_sync(0xffffffffu, beg, src);
+            const int32_t w_deg = __shfl_sync(0xffffffffu, deg, src);
+            pass.begin(w);
+            gat_walk_by_warp<LPG, W>(pass, L, a.colidx, (int32_t)w, w_beg, w_deg, w_deg + a.self_loop, 0, kWarp, lane);
+            pass.merge_groups();
+            pass.finish(w, L.g == 0 && L.on, hw, as, ad, vec != 0, vec16 != 0);
+        }
+        return;
+    }
+    const int n_hubs = *a.hub_count;
+    int turn = 0;
+    for (int hub = blockIdx.x; hub < n_hubs; hub += hub_blocks, turn ^= 1) {
+        const int64_t u = a.hub_list[hub];
+        const int64_t beg = a.rowptr[u];
+        const int32_t deg = (int32_t)(a.rowptr[u + 1] - beg);
+        pass.begin(u);
+        gat_walk_by_warp<LPG, W>(pass, L, a.colidx, (int32_t)u, beg, deg, deg + a.self_loop, warp * kWarp, kGatWarps * kWarp, lane);
+        pass.merge_groups();
+        if (L.g == 0) {
+            sm_acc[turn][warp][L.li] = pass.acc;
+            sm_ds[turn][warp][L.li] = make_float2(pass.ds, pass.dc);
+        }
+        __syncthreads();
+        if (warp == 0) {      // the warps' sums in warp order
+            for (int w = 1; w < kGatWarps; ++w) {
+                pass.acc.fma(1.f, sm_acc[turn][w][L.li]);
+                pass.ds += sm_ds[turn][w][L.li].x;
+                pass.dc += sm_ds[turn][w][L.li].y;
+            }
+            pass.finish(u, L.g == 0 && L.on, hw, as, ad, vec != 0, vec16 != 0);
         }
     }
 }
 
-template <int HD>
-__global__ void __launch_bounds__(kGb64Threads, 5) gat_bwd_src64_kernel(GatBwdArgs a) {
-    __shared__ __align__(16) float p_s[kGb64Warps][64];
-    __shared__ float red[kGb64Warps][kWarp][65];
-    __shared__ float sm_part[kGb64Warps][2][64];
+// da_src = sum_u ds_u p_u, da_dst = sum_u dt_u p_u: one stream over p (the sums of a hub row come from whichever block took it, so
+// they are added here, where every node has a fixed place), per block, and by the last block to finish in block order.
+template <int LPG, int W>
+__global__ void __launch_bounds__(256) gat_lane_params_kernel(GatBwdArgs a, float* __restrict__ da_src, float* __restrict__ da_dst) {
+    constexpr int G = GatLanes<LPG, W>::G, kParts = 256 / LPG;
+    __shared__ Cols<W> sm[2][kParts][LPG];
+    __shared__ bool last;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t u = blockIdx.x * (int64_t)kGb64Warps + warp;
-    const int nv = a.dim >> 2;
-    constexpr int NH = 64 / HD;
-    // A lane's 64 column sums live in its own row of `red` (stride 65: no two lanes of a warp meet in a bank), not
-    // in registers: the registers go to the sixteen loads in flight, and more warps fit on an SM.
-    float* mine = red[warp][lane];
-    float ds[NH], su[NH];
-#pragma unroll
-    for (int h = 0; h < NH; ++h) { ds[h] = 0.f; su[h] = 0.f; }
-    for (int c = lane; c < 64; c += kWarp) p_s[warp][c] = (u < a.n && c < a.dim) ? a.p[u * a.ldp + c] : 0.f;
-    __syncwarp();
-    bool first = true;                              // nothing stored in `mine` yet
-    if (u < a.n) {
-#pragma unroll
-        for (int h = 0; h < NH; ++h) if (h < a.heads) su[h] = a.s[u * a.heads + h];
-        const int64_t beg = a.rowptr[u];
-        const int64_t deg = a.rowptr[u + 1] - beg;
-        int64_t total = deg + (a.self_loop ? 1 : 0);
-        if (total >= kGbHubEntries) {               // a hub row: its sums come from gat_bwd_src64_hub_kernel
-            const float* hs = a.hub_sum + (int64_t)a.hub_pos[u] * 72;
-#pragma unroll 8
-            for (int c = 0; c < 64; ++c) mine[c] = lane == 0 ? hs[c] : 0.f;
-            if (lane == 0) {
-#pragma unroll
-                for (int h = 0; h < NH; ++h) ds[h] = hs[64 + h];
-            }
-            first = false;
-            total = 0;
-        }
-        for (int64_t e0 = 0; e0 < total; e0 += kWarp) {
-            const bool valid = e0 + lane < total;
-            const int64_t v = !valid ? u : (e0 + lane < deg ? (int64_t)__ldg(a.colidx + beg + e0 + lane) : u);
-            const bool live = valid && a.stats[v * a.heads].y != 0.f;      // dz_v is zero otherwise
-            float4 g[16];
-            float dalpha[NH], alpha[NH];
-#pragma unroll
-            for (int h = 0; h < NH; ++h) { dalpha[h] = 0.f; alpha[h] = 0.f; }
-            const float4* row = reinterpret_cast<const float4*>(a.dz + v * a.lddz);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                g[i] = (live && i < nv) ? __ldg(row + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-                const float4 pp = *reinterpret_cast<const float4*>(&p_s[warp][4 * i]);
-                dalpha[(4 * i) / HD] += (g[i].x * pp.x + g[i].y * pp.y) + (g[i].z * pp.z + g[i].w * pp.w);
-            }
-#pragma unroll
-            for (int h = 0; h < NH; ++h) {
-                if (h < a.heads && live) {
-                    const float4 st = a.stats[v * a.heads + h];
-                    const float z = su[h] + a.t[v * a.heads + h];
-                    alpha[h] = expf((z > 0.f ? z : a.slope * z) - st.x) * st.y;
-                    ds[h] = fmaf(alpha[h] * (z > 0.f ? 1.f : a.slope), dalpha[h] - st.z, ds[h]);
-                }
-            }
-            if (first) {
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const float al = alpha[(4 * i) / HD];
-                    mine[4 * i] = al * g[i].x; mine[4 * i + 1] = al * g[i].y;
-                    mine[4 * i + 2] = al * g[i].z; mine[4 * i + 3] = al * g[i].w;
-                }
-                first = false;
-            } else {
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const float al = alpha[(4 * i) / HD];
-                    mine[4 * i] = fmaf(al, g[i].x, mine[4 * i]); mine[4 * i + 1] = fmaf(al, g[i].y, mine[4 * i + 1]);
-                    mine[4 * i + 2] = fmaf(al, g[i].z, mine[4 * i + 2]); mine[4 * i + 3] = fmaf(al, g[i].w, mine[4 * i + 3]);
-                }
-            }
-        }
+    const GatLanes<LPG, W> L(lane, a.dim, a.head_dim);
+    Cols<W> s0, s1;
+    s0.zero(); s1.zero();
+#pragma unroll 2
+    for (int64_t u = ((int64_t)blockIdx.x * 8 + warp) * G + L.g; u < a.n; u += (int64_t)gridDim.x * 8 * G) {
+        Cols<W> x;
+        x.load(a.p + u * a.ldp + L.col);
+        s0.fma(__ldg(a.ds + u * a.heads + L.head), x);
+        s1.fma(__ldg(a.dt + u * a.heads + L.head), x);
     }
-    if (first) {
-#pragma unroll 8
-        for (int c = 0; c < 64; ++c) mine[c] = 0.f;
-    }
-    // the lanes' partial rows are added in lane order; the lanes' ds in a shuffle tree
-#pragma unroll
-    for (int h = 0; h < NH; ++h) ds[h] = warp_sum(ds[h]);
-    __syncwarp();
-    for (int c = lane; c < 64; c += kWarp) {
-        float sum = 0.f;
-        for (int l = 0; l < kWarp; ++l) sum += red[warp][l][c];
-        float dsc = 0.f, dtc = 0.f;
-#pragma unroll
-        for (int h = 0; h < NH; ++h) if (h == c / HD) dsc = ds[h];
-        if (u < a.n && c < a.dim) {
-            dtc = a.stats[u * a.heads + c / HD].w;
-            const float val = sum + dsc * a.a_src[c] + dtc * a.a_dst[c];
-            if (a.dp) a.dp[u * a.lddp + c] = val;
-            if (a.dp16) a.dp16[u * a.lddp16 + c] = f32_to_bf16(val);
-        } else {
-            dsc = 0.f;
-        }
-        sm_part[warp][0][c] = dsc * p_s[warp][c];
-        sm_part[warp][1][c] = dtc * p_s[warp][c];
-    }
+    sm[0][warp * G + L.g][L.li] = s0;
+    sm[1][warp * G + L.g][L.li] = s1;
     __syncthreads();
-    for (int i = threadIdx.x; i < 2 * a.dim; i += kGb64Threads) {
+    for (int i = threadIdx.x; i < 2 * a.dim; i += 256) {
         const int which = i / a.dim, col = i % a.dim;
         float sum = 0.f;
-        for (int w = 0; w < kGb64Warps; ++w) sum += sm_part[w][which][col];
-        a.partial[((int64_t)blockIdx.x * 2 + which) * a.dim + col] = sum;
+        for (int k = 0; k < kParts; ++k) sum += sm[which][k][col / W].v[col % W];
+        a.partial[(int64_t)blockIdx.x * 2 * a.dim + i] = sum;
     }
-}
-
-// ---- hub rows: one block per listed row, its warps taking the trips w, w + W, ...; per-warp results are merged in
-// warp order, so the bits depend neither on timing nor on the list's order.
-constexpr int kGbHubWarps = 8, kGbHubThreads = kGbHubWarps * kWarp;
-
-template <int HD>
-__global__ void __launch_bounds__(kGbHubThreads) gat_bwd_dst64_hub_kernel(GatBwdArgs a) {
-    constexpr int NH = 64 / HD;
-    __shared__ __align__(16) float g_s[64];
-    __shared__ float st_m[kGbHubWarps][NH], st_den[kGbHubWarps][NH], part[kGbHubWarps][NH][3];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int nv = a.dim >> 2;
-    const int32_t count = *a.hub_count;
-    for (int32_t item = blockIdx.x; item < count; item += gridDim.x) {
-        const int64_t v = a.hub_list[item];
-        __syncthreads();                                 // the previous row's shared values are done with
-        bool any = false;
-        if (threadIdx.x < 64) {
-            const float x = (int)threadIdx.x < a.dim ? a.dz[v * a.lddz + threadIdx.x] : 0.f;
-            g_s[threadIdx.x] = x;
-            any = x != 0.f;
-        }
-        if (!__syncthreads_or(any)) {
-            if ((int)threadIdx.x < a.heads) a.stats[v * a.heads + threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
-            continue;
-        }
-        const int64_t beg = a.rowptr[v];
-        const int64_t deg = a.rowptr[v + 1] - beg;
-        const int64_t total = deg + (a.self_loop ? 1 : 0);
-        float tv[NH], m[NH], den[NH], csum[NH], a1[NH], a2[NH];
-#pragma unroll
-        for (int h = 0; h < NH; ++h) {
-            tv[h] = h < a.heads ? a.t[v * a.heads + h] : 0.f;
-            m[h] = -INFINITY; den[h] = 0.f; csum[h] = 0.f; a1[h] = 0.f; a2[h] = 0.f;
-        }
-        for (int64_t e0 = (int64_t)warp * kWarp; e0 < total; e0 += kGbHubThreads) {
-            const bool valid = e0 + lane < total;
-            const int64_t u = !valid ? v : (e0 + lane < deg ? (int64_t)__ldg(a.colidx + beg + e0 + lane) : v);
-#pragma unroll
-            for (int h = 0; h < NH; ++h) {
-                if (h < a.heads) {
-                    const float z = a.s[u * a.heads + h] + tv[h];
-                    const float e = valid ? (z > 0.f ? z : a.slope * z) : -INFINITY;
-                    const float mn = fmaxf(m[h], warp_max(e));
-                    den[h] = den[h] * expf(m[h] - mn) + warp_sum(valid ? expf(e - mn) : 0.f);
-                    m[h] = mn;
-                }
-            }
-        }
-        if (lane == 0) {
-#pragma unroll
-            for (int h = 0; h < NH; ++h) { st_m[warp][h] = m[h]; st_den[warp][h] = den[h]; }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int h = 0; h < NH; ++h) {                   // every thread merges the warps' states in warp order
-            float mm = -INFINITY, dd = 0.f;
-            for (int w = 0; w < kGbHubWarps; ++w) mm = fmaxf(mm, st_m[w][h]);
-            for (int w = 0; w < kGbHubWarps; ++w)
-                if (st_den[w][h] > 0.f) dd += st_den[w][h] * expf(st_m[w][h] - mm);
-            m[h] = mm; den[h] = dd;
-        }
-        for (int64_t e0 = (int64_t)warp * kWarp; e0 < total; e0 += kGbHubThreads) {
-            const bool valid = e0 + lane < total;
-            const int64_t u = !valid ? v : (e0 + lane < deg ? (int64_t)__ldg(a.colidx + beg + e0 + lane) : v);
-            float dalpha[NH];
-#pragma unroll
-            for (int h = 0; h < NH; ++h) dalpha[h] = 0.f;
-            const float4* row = reinterpret_cast<const float4*>(a.p + u * a.ldp);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                if (i < nv) {
-                    const float4 x = valid ? __ldg(row + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-                    const float4 gg = *reinterpret_cast<const float4*>(&g_s[4 * i]);
-                    dalpha[(4 * i) / HD] += (x.x * gg.x + x.y * gg.y) + (x.z * gg.z + x.w * gg.w);
-                }
-            }
-#pragma unroll
-            for (int h = 0; h < NH; ++h) {
-                if (h < a.heads && valid) {
-                    const float z = a.s[u * a.heads + h] + tv[h];
-                    const float alpha = expf((z > 0.f ? z : a.slope * z) - m[h]) / den[h];
-                    const float gp = z > 0.f ? 1.f : a.slope;
-                    csum[h] = fmaf(alpha, dalpha[h], csum[h]);
-                    a1[h] = fmaf(alpha * gp, dalpha[h], a1[h]);
-                    a2[h] = fmaf(alpha, gp, a2[h]);
-                }
-            }
-        }
-#pragma unroll
-        for (int h = 0; h < NH; ++h) {
-            const float c = warp_sum(csum[h]), s1 = warp_sum(a1[h]), s2 = warp_sum(a2[h]);
-            if (lane == 0) { part[warp][h][0] = c; part[warp][h][1] = s1; part[warp][h][2] = s2; }
-        }
-        __syncthreads();
-        if ((int)threadIdx.x < a.heads && (int)threadIdx.x < NH) {
-            const int h = threadIdx.x;
-            float c = 0.f, s1 = 0.f, s2 = 0.f, mm = -INFINITY, dd = 0.f;
-            for (int w = 0; w < kGbHubWarps; ++w) { c += part[w][h][0]; s1 += part[w][h][1]; s2 += part[w][h][2]; }
-            for (int w = 0; w < kGbHubWarps; ++w) mm = fmaxf(mm, st_m[w][h]);
-            for (int w = 0; w < kGbHubWarps; ++w)
-                if (st_den[w][h] > 0.f) dd += st_den[w][h] * expf(st_m[w][h] - mm);
-            a.stats[v * a.heads + h] = make_float4(mm, 1.f / dd, c, s1 - c * s2);
-        }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(a.hub_count + 1, 1) == (int)gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    // every column by 256 / (2 dim) threads (one where the columns are more), each its share of the blocks in order
+    const int cols = 2 * a.dim, shares = cols < 256 ? 256 / cols : 1;
+    float* share_sum = &sm[0][0][0].v[0];
+    for (int i = threadIdx.x; i < shares * cols; i += 256) {
+        const int col = i % cols, share = i / cols;
+        float sum = 0.f;
+#pragma unroll 8
+        for (int b = share; b < (int)gridDim.x; b += shares) sum += __ldcg(a.partial + (int64_t)b * cols + col);
+        share_sum[i] = sum;
     }
-}
-
-// The source pass of a hub row u: the entry sums only (sum_v alpha_uv dz_v per column and ds_u per head); the row's
-// own epilogue (dp_u, the parameter-gradient partials) stays with gat_bwd_src64_kernel, which picks the sums up.
-template <int HD>
-__global__ void __launch_bounds__(kGb64Threads) gat_bwd_src64_hub_kernel(GatBwdArgs a) {
-    constexpr int NH = 64 / HD;
-    __shared__ __align__(16) float p_s[64];
-    __shared__ float red[kGb64Warps][kWarp][65];
-    __shared__ float rows[kGb64Warps][64], dsw[kGb64Warps][NH];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int nv = a.dim >> 2;
-    const int32_t count = *a.hub_count;
-    for (int32_t item = blockIdx.x; item < count; item += gridDim.x) {
-        const int64_t u = a.hub_list[item];
-        __syncthreads();
-        if (threadIdx.x < 64) p_s[threadIdx.x] = (int)threadIdx.x < a.dim ? a.p[u * a.ldp + threadIdx.x] : 0.f;
-        __syncthreads();
-        float acc[64], ds[NH], su[NH];
-#pragma unroll
-        for (int c = 0; c < 64; ++c) acc[c] = 0.f;
-#pragma unroll
-        for (int h = 0; h < NH; ++h) { ds[h] = 0.f; su[h] = h < a.heads ? a.s[u * a.heads + h] : 0.f; }
-        const int64_t beg = a.rowptr[u];
-        const int64_t deg = a.rowptr[u + 1] - beg;
-        const int64_t total = deg + (a.self_loop ? 1 : 0);
-        for (int64_t e0 = (int64_t)warp * kWarp; e0 < total; e0 += kGb64Threads) {
-            const bool valid = e0 + lane < total;
-            const int64_t v = !valid ? u : (e0 + lane < deg ? (int64_t)__ldg(a.colidx + beg + e0 + lane) : u);
-            const bool live = valid && a.stats[v * a.heads].y != 0.f;      // dz_v is zero otherwise
-            float4 g[16];
-            float dalpha[NH], alpha[NH];
-#pragma unroll
-            for (int h = 0; h < NH; ++h) { dalpha[h] = 0.f; alpha[h] = 0.f; }
-            const float4* row = reinterpret_cast<const float4*>(a.dz + v * a.lddz);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                g[i] = (live && i < nv) ? __ldg(row + i) : make_float4(0.f, 0.f, 0.f, 0.f);
-                const float4 pp = *reinterpret_cast<const float4*>(&p_s[4 * i]);
-                dalpha[(4 * i) / HD] += (g[i].x * pp.x + g[i].y * pp.y) + (g[i].z * pp.z + g[i].w * pp.w);
-            }
-#pragma unroll
-            for (int h = 0; h < NH; ++h) {
-                if (h < a.heads && live) {
-                    const float4 st = a.stats[v * a.heads + h];
-                    const float z = su[h] + a.t[v * a.heads + h];
-                    alpha[h] = expf((z > 0.f ? z : a.slope * z) - st.x) * st.y;
-                    ds[h] = fmaf(alpha[h] * (z > 0.f ? 1.f : a.slope), dalpha[h] - st.z, ds[h]);
-                }
-            }
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const float al = alpha[(4 * i) / HD];
-                acc[4 * i] = fmaf(al, g[i].x, acc[4 * i]);
-                acc[4 * i + 1] = fmaf(al, g[i].y, acc[4 * i + 1]);
-                acc[4 * i + 2] = fmaf(al, g[i].z, acc[4 * i + 2]);
-                acc[4 * i + 3] = fmaf(al, g[i].w, acc[4 * i + 3]);
-            }
-        }
-        // lanes in lane order, then warps in warp order
-#pragma unroll
-        for (int c = 0; c < 64; ++c) red[warp][lane][c] = acc[c];
-#pragma unroll
-        for (int h = 0; h < NH; ++h) {
-            const float d = warp_sum(ds[h]);
-            if (lane == 0) dsw[warp][h] = d;
-        }
-        __syncwarp();
-        for (int c = lane; c < 64; c += kWarp) {
-            float sum = 0.f;
-            for (int l = 0; l < kWarp; ++l) sum += red[warp][l][c];
-            rows[warp][c] = sum;
-        }
-        __syncthreads();
-        float* hs = a.hub_sum + (int64_t)item * 72;
-        if (threadIdx.x < 64) {
-            float sum = 0.f;
-            for (int w = 0; w < kGb64Warps; ++w) sum += rows[w][threadIdx.x];
-            hs[threadIdx.x] = sum;
-        } else if ((int)threadIdx.x - 64 < NH) {
-            const int h = threadIdx.x - 64;
-            float sum = 0.f;
-            for (int w = 0; w < kGb64Warps; ++w) sum += dsw[w][h];
-            hs[64 + h] = sum;
-        }
+    __syncthreads();
+    for (int col = threadIdx.x; col < cols; col += 256) {
+        float sum = 0.f;
+        for (int share = 0; share < shares; ++share) sum += share_sum[share * cols + col];
+        (col < a.dim ? da_src : da_dst)[col % a.dim] = sum;
     }
-}
-
-template <int HD>
-static int launch_bwd64(const GatBwdArgs& a, float* da_src, float* da_dst, cudaStream_t st) {
-    const unsigned blocks = (unsigned)((a.n + kGb64Warps - 1) / kGb64Warps);
-    gat_bwd_dst64_kernel<HD><<<blocks, kGb64Threads, 0, st>>>(a);
-    gat_bwd_dst64_hub_kernel<HD><<<kGbHubBlocks, kGbHubThreads, 0, st>>>(a);
-    gat_bwd_src64_hub_kernel<HD><<<kGbHubBlocks, kGb64Threads, 0, st>>>(a);
-    gat_bwd_src64_kernel<HD><<<blocks, kGb64Threads, 0, st>>>(a);
-    gat_bwd_reduce_kernel<<<(unsigned)(2 * a.dim), 256, 0, st>>>(a.partial, blocks, a.dim, da_src, da_dst);
-    return launch_status();
 }
 
 template <int NC>
@@ -666,8 +586,7 @@ static int launch_bwd(const GatBwdArgs& a, unsigned blocks, float* da_src, float
 
 using namespace retexo;
 
-// rows of kGbHubEntries entries or more a graph can hold at most (with the self loop counted as an entry)
-static inline int64_t max_hub_rows(int64_t n_nodes, int64_t n_edges) { return (n_edges + n_nodes) / kGbHubEntries + 1; }
+constexpr int64_t kGatParamBlocks = 296;      // blocks of gat_lane_params_kernel at most (the last one adds their sums)
 
 extern "C" size_t retexo_gat_backward_workspace_size(int64_t n_nodes, int64_t n_edges, int32_t heads, int32_t dim) {
     if (n_nodes < 0 || n_edges < 0 || heads <= 0 || dim <= 0) return 0;
@@ -675,11 +594,11 @@ extern "C" size_t retexo_gat_backward_workspace_size(int64_t n_nodes, int64_t n_
     s.take<float>((size_t)n_nodes * heads);
     s.take<float>((size_t)n_nodes * heads);
     s.take<float4>((size_t)n_nodes * heads);
-    s.take<float>((size_t)((n_nodes + kGb64Warps - 1) / kGb64Warps + 1) * 2 * (size_t)dim);
+    s.take<float>((size_t)std::max<int64_t>((n_nodes + kGbWarps - 1) / kGbWarps, kGatParamBlocks) * 2 * (size_t)dim);
+    s.take<float>((size_t)n_nodes * heads);
+    s.take<float>((size_t)n_nodes * heads);
     s.take<int32_t>(64);
-    s.take<int32_t>((size_t)max_hub_rows(n_nodes, n_edges));
     s.take<int32_t>((size_t)n_nodes);
-    s.take<float>((size_t)max_hub_rows(n_nodes, n_edges) * 72);
     return s.off + kAlign;
 }
 
@@ -713,28 +632,32 @@ extern "C" int retexo_gat_backward(const retexo_csr* g, const float* p, int64_t 
     a.t = ws.take<float>((size_t)n * gat->heads);
     a.stats = ws.take<float4>((size_t)n * gat->heads);
     const unsigned blocks = (unsigned)((n + kGbWarps - 1) / kGbWarps);
-    a.partial = ws.take<float>((size_t)((n + kGb64Warps - 1) / kGb64Warps + 1) * 2 * (size_t)dim);
+    a.partial = ws.take<float>((size_t)std::max<int64_t>(blocks, kGatParamBlocks) * 2 * (size_t)dim);
     a.dp = dp; a.lddp = lddp; a.dp16 = static_cast<__nv_bfloat16*>(dp_bf16); a.lddp16 = lddp_bf16;
-    int32_t* hub_count = ws.take<int32_t>(64);
-    int32_t* hub_list = ws.take<int32_t>((size_t)max_hub_rows(n, g->n_edges));
-    int32_t* hub_pos = ws.take<int32_t>((size_t)n);
-    float* hub_sum = ws.take<float>((size_t)max_hub_rows(n, g->n_edges) * 72);
-    // rows of up to 64 columns in whole 16-byte pieces, head width 8 / 16 / 32 / 64: one lane per entry, hub rows by blocks
-    const int hdw = gat->head_dim;
-    const bool lane_per_entry = dim <= 64 && dim % 4 == 0 && ldp % 4 == 0 && lddz % 4 == 0 && aligned_to(p, 16) && aligned_to(dz, 16) &&
-                                (hdw == 8 || hdw == 16 || hdw == 32 || hdw == 64);
-    a.hub_count = nullptr; a.hub_list = nullptr; a.hub_pos = nullptr; a.hub_sum = nullptr;
-    if (lane_per_entry) {
-        a.hub_count = hub_count; a.hub_list = hub_list; a.hub_pos = hub_pos; a.hub_sum = hub_sum;
-        RETEXO_CUDA_TRY(cudaMemsetAsync(hub_count, 0, sizeof(int32_t), st));
+    a.ds = ws.take<float>((size_t)n * gat->heads);
+    a.dt = ws.take<float>((size_t)n * gat->heads);
+    a.hub_count = ws.take<int32_t>(64);
+    a.hub_list = ws.take<int32_t>((size_t)n);
+    int lpg, w;
+    if (gat_lanes_cover(dim, gat->head_dim, p, ldp, dz, lddz, &lpg, &w)) {
+        const int n_sm = sm_count();
+        if (n_sm <= 0) return RETEXO_ERR_CUDA;
+        RETEXO_CUDA_TRY(cudaMemsetAsync(a.hub_count, 0, 2 * sizeof(int32_t), st));
+        const int vec = dp && lddp % 4 == 0 && aligned_to(dp, 16), vec16 = dp_bf16 && lddp_bf16 % 4 == 0 && aligned_to(dp_bf16, 8);
+        const int hub_entries = gat_hub_entries(g->n_edges, n_sm), hub_blocks = 6 * n_sm;
+        return gat_lanes_dispatch(lpg, w, [&]<int LPG, int W>() {
+            constexpr int64_t rows = kGatWarps * GatLanes<LPG, W>::G;
+            const unsigned grid = (unsigned)((n + rows - 1) / rows + hub_blocks);
+            gat_lane_scores_kernel<LPG, W><<<gat_lane_scores_grid<LPG, W>(n, n_sm), 256, 0, st>>>(
+                n, a.rowptr, a.p, a.ldp, a.heads, a.head_dim, a.a_src, a.a_dst, a.self_loop, hub_entries, a.s, a.t, a.hub_list, a.hub_count);
+            gat_lane_dst_kernel<LPG, W><<<grid, kGatThreads, 0, st>>>(a, hub_entries, hub_blocks);
+            gat_lane_src_kernel<LPG, W><<<grid, kGatThreads, 0, st>>>(a, hub_entries, hub_blocks, vec, vec16);
+            const int64_t want = (n + 64 * GatLanes<LPG, W>::G - 1) / (64 * GatLanes<LPG, W>::G);      // 8 nodes per group
+            gat_lane_params_kernel<LPG, W><<<(unsigned)std::min(want, kGatParamBlocks), 256, 0, st>>>(a, da_src, da_dst);
+            return launch_status();
+        });
     }
     gat_bwd_scores_kernel<<<blocks, kGbThreads, 0, st>>>(a);
-    if (lane_per_entry) {
-        if (hdw == 8) return launch_bwd64<8>(a, da_src, da_dst, st);
-        if (hdw == 16) return launch_bwd64<16>(a, da_src, da_dst, st);
-        if (hdw == 32) return launch_bwd64<32>(a, da_src, da_dst, st);
-        return launch_bwd64<64>(a, da_src, da_dst, st);
-    }
     const int nc = (dim + kWarp - 1) / kWarp;
     if (nc <= 1) return launch_bwd<1>(a, blocks, da_src, da_dst, st);
     if (nc <= 2) return launch_bwd<2>(a, blocks, da_src, da_dst, st);

@@ -1,0 +1,45 @@
+"""The GAT kernels' lane layout at its edges: every number of lanes per entry (1 .. 32, 4 or 8 columns each), lanes without
+columns, rows around the lengths at which a group, a warp or a block takes them, and rows the layout does not cover."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from gpu_util import assert_rows_close, dev
+from paper_2302_13053_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("heads,dh,pad", [(1, 4, 0), (3, 4, 0), (8, 4, 0), (1, 8, 0), (3, 16, 0), (7, 8, 0), (1, 256, 0), (2, 128, 0), (5, 32, 8),
+                                          (4, 16, 4)])
+def test_gat_forward_and_backward(heads, dh, pad):
+    """pad > 0: the rows have a stride of heads * dh + pad floats (4: not in 32-byte pieces, the general kernels)."""
+    from paper_2302_13053_b200 import binding as B
+    n, rowptr, colidx, _ = wl.degree_ladder_graph([0, 1, 2, 3, 7, 8, 9, 30, 31, 32, 33, 61, 62, 63, 64, 65, 127, 129, 300], seed=heads)
+    rng = np.random.default_rng(dh)
+    d = heads * dh
+    buf = rng.standard_normal((n, d + pad)).astype(np.float32)
+    p = np.ascontiguousarray(buf[:, :d])
+    dz = rng.standard_normal((n, d)).astype(np.float32)
+    dz[rng.random(n) < 0.4] = 0.0
+    scale = 1.0 / np.sqrt(dh)
+    gat = dict(heads=heads, head_dim=dh, negative_slope=0.2, add_self_loop=1,
+               a_src=(rng.standard_normal((heads, dh)) * scale).astype(np.float32),
+               a_dst=(rng.standard_normal((heads, dh)) * scale).astype(np.float32))
+    g = dict(gat, a_src=torch.from_numpy(gat["a_src"]), a_dst=torch.from_numpy(gat["a_dst"]))
+    rp, ci = dev(rowptr.astype(np.int64)), dev(colidx.astype(np.int32))
+    q = dev(buf)[:, :d]
+    out, out16 = B.retexo_aggregate(B.GAT, rp, ci, q, gat=g, want_bf16=True)
+    assert_rows_close(out.cpu().numpy(), oracle.aggregate(oracle.GAT, rowptr, colidx, p, gat=gat), what="%d x %d" % (heads, dh))
+    assert torch.equal(out16[:, :d], out.to(torch.bfloat16))
+    dp, dp16, da_src, da_dst = B.retexo_gat_backward(rp, ci, q, g, dev(dz), want_bf16=True)
+    again = B.retexo_gat_backward(rp, ci, q, g, dev(dz))
+    assert torch.equal(dp, again[0]) and torch.equal(da_src, again[2]) and torch.equal(da_dst, again[3])
+    assert torch.equal(dp16[:, :d], dp.to(torch.bfloat16))
+    ref_dp, ref_as, ref_ad = oracle.gat_backward(rowptr, colidx, p, gat, dz.astype(np.float64))
+    # a row of up to 300 fp32 terms: 2e-5 of its norm, or of the largest gradient where its terms cancel
+    err = np.abs(dp.cpu().numpy() - ref_dp).max(axis=1)
+    assert np.all(err <= 2e-5 * np.linalg.norm(ref_dp, axis=1) + 1e-5 * np.abs(ref_dp).max()), float(err.max())
+    for got, ref in ((da_src, ref_as), (da_dst, ref_ad)):      # sums over the n nodes, as in the other backward tests
+        np.testing.assert_allclose(got.cpu().numpy(), ref, rtol=0, atol=2e-6 * max(1.0, np.abs(ref).max()) * np.sqrt(n))
