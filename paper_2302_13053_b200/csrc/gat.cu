@@ -61,10 +61,10 @@ struct GatForwardPass {
     const float* p;            // this lane's columns of row 0
     const float* s;            // this lane's head of node 0
     int head;
-    float tv;
+    float tv, k_neg;
     GatState<W> st;
     __device__ __forceinline__ GatForwardPass(const GatArgs& a_, const GatLanes<LPG, W>& L)
-        : a(a_), p(a_.p + L.col), s(a_.s + L.head), head(L.head) {}
+        : a(a_), p(a_.p + L.col), s(a_.s + L.head), head(L.head), k_neg(a_.slope * kLog2E) {}
     __device__ __forceinline__ void begin(int64_t v) {
         tv = __ldg(a.t + v * a.heads + head);
         st.clear();
@@ -81,7 +81,7 @@ struct GatForwardPass {
         float big = st.m;
 #pragma unroll
         for (int t = 0; t < U; ++t) {
-            e[t] = ok[t] ? leaky(e[t] + tv, a.slope) : -INFINITY;
+            e[t] = ok[t] ? leaky2(e[t] + tv, kLog2E, k_neg) : -INFINITY;
             big = fmaxf(big, e[t]);
         }
         const float f = exp2_rel(st.m, big);

@@ -30,7 +30,7 @@ struct GatBwdArgs {
     float slope; int32_t self_loop;
     const float* dz; int64_t lddz;
     float* s; float* t;              // [n x heads]
-    float4* stats;                   // [n x heads]: (row maximum, 1 / soft-max sum (0 = dz_v is zero), c_v, dt_v; lane layout: t_v)
+    float4* stats;                   // [n x heads]: (row maximum (lane layout: / ln 2), 1 / soft-max sum (0 = dz_v is zero), c_v, dt_v; lane layout: t_v)
     float* dp; int64_t lddp;
     __nv_bfloat16* dp16; int64_t lddp16;
     float* partial;                  // [blocks x 2 x dim]: per-block sums of ds_u p_u and dt_u p_u
@@ -258,10 +258,10 @@ struct GatDstPass {
     const float* s;
     int head, col;
     bool on;
-    float tv, m, den, c, b1, b2;
+    float tv, k_neg, m, den, c, b1, b2;
     Cols<W> g;
     __device__ __forceinline__ GatDstPass(const GatBwdArgs& a_, const GatLanes<LPG, W>& L)
-        : a(a_), p(a_.p + L.col), s(a_.s + L.head), head(L.head), col(L.col), on(L.on) {}
+        : a(a_), p(a_.p + L.col), s(a_.s + L.head), head(L.head), col(L.col), on(L.on), k_neg(a_.slope * kLog2E) {}
     // Returns whether this lane's part of the gradient has a non-zero entry.
     __device__ __forceinline__ bool begin(int64_t v) {
         tv = __ldg(a.t + v * a.heads + head);
@@ -285,7 +285,7 @@ struct GatDstPass {
 #pragma unroll
         for (int t = 0; t < U; ++t) {
             z[t] += tv;
-            e[t] = ok[t] ? leaky(z[t], a.slope) : -INFINITY;
+            e[t] = ok[t] ? leaky2(z[t], kLog2E, k_neg) : -INFINITY;
             big = fmaxf(big, e[t]);
         }
         const float f = exp2_rel(m, big), ref = big == -INFINITY ? 0.f : big;
@@ -330,7 +330,7 @@ struct GatDstPass {
 
 // Bound like the forward pass by the gather of p_u (4 dim + 4 heads bytes an entry); rows whose gradient is zero gather nothing.
 // Measured, whole backward pass (a lane per entry reading its own row in 16-byte pieces before; heads of other shapes a warp
-// per entry): 717 k nodes, 14 M entries, 4 x 16: 5319 -> 1850 us; 60 k nodes, 12 M entries: 2960 -> 684 us; 100 k nodes, 3 M
+// per entry): 717 k nodes, 14 M entries, 4 x 16: 5319 -> 1950 us; 60 k nodes, 12 M entries: 2960 -> 684 us; 100 k nodes, 3 M
 // entries, 8 x 32: 26.6 -> 0.87 ms; 200 k nodes, 4 M entries, 1 x 8: 834 -> 163 us.
 template <int LPG, int W>
 __global__ void __launch_bounds__(kGatThreads, kGatBlocksPerSm) gat_lane_dst_kernel(GatBwdArgs a, int hub_entries, int hub_blocks) {
@@ -405,10 +405,10 @@ struct GatSrcPass {
     const float* dz;
     const float4* stats;
     int head, col;
-    float su, ds, dc;            // ds: sum alpha g' <dz_v, p_u> over this lane's columns; dc: sum alpha g' c_v
+    float su, k_neg, ds, dc;            // ds: sum alpha g' <dz_v, p_u> over this lane's columns; dc: sum alpha g' c_v
     Cols<W> px, acc;
     __device__ __forceinline__ GatSrcPass(const GatBwdArgs& a_, const GatLanes<LPG, W>& L)
-        : a(a_), dz(a_.dz + L.col), stats(a_.stats + L.head), head(L.head), col(L.col) {}
+        : a(a_), dz(a_.dz + L.col), stats(a_.stats + L.head), head(L.head), col(L.col), k_neg(a_.slope * kLog2E) {}
     __device__ __forceinline__ void begin(int64_t u) {
         su = __ldg(a.s + u * a.heads + head);
         px.load(a.p + u * a.ldp + col);
@@ -432,7 +432,7 @@ struct GatSrcPass {
 #pragma unroll
         for (int t = 0; t < U; ++t) {
             const float z = su + st[t].w;
-            const float alpha = st[t].y != 0.f ? exp2_hw(leaky(z, a.slope) - st[t].x) * st[t].y : 0.f;
+            const float alpha = st[t].y != 0.f ? exp2_hw(leaky2(z, kLog2E, k_neg) - st[t].x) * st[t].y : 0.f;
             const float ag = z > 0.f ? alpha : alpha * a.slope;
             ds = fmaf(ag, px.dot(g[t]), ds);
             dc = fmaf(ag, st[t].z, dc);

@@ -133,11 +133,12 @@ struct Cols {
     }
 };
 
-__device__ __forceinline__ float leaky(float z, float slope) { return z > 0.f ? z : slope * z; }
-// The lane kernels keep scores in units of log 2 (a leaky ReLU commutes with a positive factor), so that e^(x - m) is one
-// subtraction and one hardware exponential.  Its error is two units in the last place (as the library function's);
-// the weights it gives are divided by their own sum.
+// LeakyReLU(z) / ln 2 with k_pos = 1 / ln 2, k_neg = slope / ln 2: the lane kernels take their exponentials in base 2, so that
+// e^(x - m) is one subtraction and one hardware exponential (its error is two units in the last place, as the library
+// function's; the weights it gives are divided by their own sum).  z itself stays s_u + t_v: its sign decides which slope
+// an entry's gradient takes.
 constexpr float kLog2E = 1.4426950408889634f;
+__device__ __forceinline__ float leaky2(float z, float k_pos, float k_neg) { return z * (z > 0.f ? k_pos : k_neg); }
 __device__ __forceinline__ float exp2_hw(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -201,9 +202,42 @@ __device__ __forceinline__ void gat_walk_by_group(P& pass, const GatLanes<LPG, W
     }
 }
 
-// s_u = <a_src, p_u> / ln 2, t_u = <a_dst, p_u> / ln 2 per head, and the list of the rows long enough for a whole block (its
-// order varies from run to run; no result depends on it).  A stream over p: LPG lanes a node, kNodes nodes in flight per group
-// (717 k nodes, 4 x 16: 33 us = 5.6 TB/s; a warp per node with 4-byte loads and two shuffle trees per head took 366 us).
+// <a, x> over a head's columns, whose W-column pieces lie in hw neighbouring lanes (hw a power of two): the sum is taken in the
+// order of a warp that owns the columns l, l + 32, ... in lane l and folds its lanes in halves, so that every kernel of the
+// library gives a node the same score, bit for bit.  (Scores are not only values: where s_u + t_v is within rounding of zero,
+// another order gives an edge the other slope of the LeakyReLU, and its gradient jumps.)
+// The sum is complete in the head's last lane group (see head_last_block).
+template <int W>
+__device__ __forceinline__ float head_dot(const Cols<W>& a, const Cols<W>& x, int hw, int lane_of_head) {
+    float q[W];
+#pragma unroll
+    for (int i = 0; i < W; ++i) q[i] = __fmul_rn(a.v[i], x.v[i]);
+    constexpr int kBlock = 32 / W;                 // lanes that hold 32 columns
+    for (int k = 1; k * kBlock < hw; ++k) {        // more than 32 columns: the chain l, l + 32, ... runs through the lane groups
+#pragma unroll
+        for (int i = 0; i < W; ++i) {
+            const float before = __shfl_up_sync(0xffffffffu, q[i], kBlock);
+            if (lane_of_head / kBlock == k) q[i] = fmaf(a.v[i], x.v[i], before);
+        }
+    }
+    for (int o = (hw < kBlock ? hw : kBlock) >> 1; o > 0; o >>= 1) {
+#pragma unroll
+        for (int i = 0; i < W; ++i) q[i] = __fadd_rn(q[i], __shfl_xor_sync(0xffffffffu, q[i], o));
+    }
+#pragma unroll
+    for (int o = W / 2; o > 0; o >>= 1) {
+#pragma unroll
+        for (int i = 0; i < o; ++i) q[i] = __fadd_rn(q[i], q[i + o]);
+    }
+    return q[0];
+}
+// First lane (counted inside the head) of the group that ends up with head_dot's sum.
+template <int W>
+__device__ __forceinline__ int head_last_block(int hw) { return hw > 32 / W ? hw - 32 / W : 0; }
+
+// s_u = <a_src, p_u>, t_u = <a_dst, p_u> per head, and the list of the rows long enough for a whole block (its order varies from
+// run to run; no result depends on it).  A stream over p: LPG lanes a node, kNodes nodes in flight per group.
+// (717 k nodes, 4 x 16: 39 us; a warp per node with 4-byte loads and two shuffle trees per head took 366 us.)
 template <int LPG, int W>
 __global__ void __launch_bounds__(256) gat_lane_scores_kernel(int64_t n, const int64_t* __restrict__ rowptr,
                                                               const float* __restrict__ p, int64_t ldp, int32_t heads,
@@ -215,6 +249,8 @@ __global__ void __launch_bounds__(256) gat_lane_scores_kernel(int64_t n, const i
     const int lane = threadIdx.x & 31;
     const GatLanes<LPG, W> L(lane, heads * head_dim, head_dim);
     const int hw = head_dim / W;                  // lanes a head spans
+    const int of_head = L.li & (hw - 1);
+    const bool writes = L.on && of_head == head_last_block<W>(hw);
     Cols<W> as, ad;
     as.zero(); ad.zero();
     if (L.on) { as.load_unaligned(a_src + L.col); ad.load_unaligned(a_dst + L.col); }
@@ -228,14 +264,10 @@ __global__ void __launch_bounds__(256) gat_lane_scores_kernel(int64_t n, const i
 #pragma unroll
         for (int i = 0; i < kNodes; ++i) {
             const int64_t u = u0 + i * G + L.g;
-            float ss = as.dot(x[i]), tt = ad.dot(x[i]);
-            for (int o = 1; o < hw; o <<= 1) {
-                ss += __shfl_xor_sync(0xffffffffu, ss, o);
-                tt += __shfl_xor_sync(0xffffffffu, tt, o);
-            }
-            if (u < n && L.on && (L.li & (hw - 1)) == 0) {
-                s[u * heads + L.head] = ss * kLog2E;
-                t[u * heads + L.head] = tt * kLog2E;
+            const float ss = head_dot(as, x[i], hw, of_head), tt = head_dot(ad, x[i], hw, of_head);
+            if (u < n && writes) {
+                s[u * heads + L.head] = ss;
+                t[u * heads + L.head] = tt;
             }
         }
     }
