@@ -94,6 +94,24 @@ __global__ void merge_status_kernel(int32_t* run, const int32_t* a, const int32_
     if (*run == 0 && a && *a != 0) *run = *a;
     if (*run == 0 && b && *b != 0) *run = *b;
 }
+// dst[i] = [src[i] | zeros], rows of ld_dst (a multiple of 4) floats from densely packed or strided rows of dim floats: the re-lay
+// of features whose rows do not start on 16-byte boundaries.  A warp a row, whole 16-byte stores; a stream (561 MB in, 566 MB
+// out: 193 us; a pitched device-to-device copy and the clearing of its padding took 420 us).
+__global__ void __launch_bounds__(256) relay_rows_kernel(const float* __restrict__ src, int64_t ld_src, int32_t dim, int64_t n,
+                                                         float* __restrict__ dst, int64_t ld_dst) {
+    const int lane = threadIdx.x & 31;
+    const int64_t i = blockIdx.x * 8ll + (threadIdx.x >> 5);
+    if (i >= n) return;
+    const float* s = src + i * ld_src;
+    float4* d = reinterpret_cast<float4*>(dst + i * ld_dst);
+#pragma unroll 4
+    for (int p = lane; p < (int)(ld_dst >> 2); p += 32) {
+        float v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = 4 * p + k < dim ? __ldcs(s + 4 * p + k) : 0.f;
+        d[p] = make_float4(v[0], v[1], v[2], v[3]);
+    }
+}
 __global__ void fill_u64_kernel(unsigned long long* p, int64_t n, unsigned long long v) {
     const int64_t i = blockIdx.x * 256ll + threadIdx.x;
     if (i < n) p[i] = v;
@@ -169,7 +187,7 @@ static RoundDims round_dims(const retexo_lmp_config& c, int m /*1-based*/) {
 
 struct LmpBuffers {
     // staged inputs (host mode only)
-    int64_t* rowptr; int32_t* colidx; float* features; int32_t* labels;
+    int64_t* rowptr; int32_t* colidx; float* features; float* features_in; int32_t* labels;
     int32_t *train_idx, *val_idx, *test_idx, *part;
     // representations
     float* q[2];
@@ -214,6 +232,8 @@ static void lmp_layout(const retexo_lmp_config& c, int64_t n, int64_t e, int64_t
     const int64_t ld16 = round_up(max_din, 64);      // bf16 rows start on 128-byte lines
     l.features = t.template take<float>((size_t)n * round_up(c.d0, 32));   // 128-byte-row copy of the features
     if (host) {
+        // rows as the caller packs them, where they have to be re-laid on the device
+        l.features_in = t.template take<float>(c.d0 % 4 != 0 ? (size_t)n * c.d0 : 1);
         l.rowptr = t.template take<int64_t>((size_t)n + 1);
         l.colidx = t.template take<int32_t>((size_t)e);
         l.labels = t.template take<int32_t>((size_t)n);
@@ -359,10 +379,19 @@ extern "C" int retexo_lmp_train(const retexo_lmp_config* cfg, const retexo_lmp_i
     if (host) {
         RETEXO_CUDA_TRY(cudaMemcpyAsync(b.rowptr, g.rowptr, sizeof(int64_t) * (size_t)(n + 1), in_kind, st));
         if (e > 0) RETEXO_CUDA_TRY(cudaMemcpyAsync(b.colidx, g.colidx, sizeof(int32_t) * (size_t)e, in_kind, st));
-        const int64_t ldp = round_up(c.d0, 32);
-        if (ldp != c.d0) RETEXO_CUDA_TRY(cudaMemsetAsync(b.features, 0, sizeof(float) * (size_t)n * ldp, st));
-        RETEXO_CUDA_TRY(cudaMemcpy2DAsync(b.features, sizeof(float) * ldp, feat, sizeof(float) * ld_feat,
-                                          sizeof(float) * c.d0, (size_t)n, in_kind, st));
+        // Densely packed rows come over in one flat copy (51 GB/s; a pitched one moved rows of 2 KB at 16 GB/s) and stay as they
+        // are where they start on 16-byte boundaries; otherwise a kernel re-lays them.
+        const bool dense = ld_feat == c.d0, keep = dense && c.d0 % 4 == 0;
+        const int64_t ldp = keep ? c.d0 : round_up(c.d0, 32);
+        if (dense) {
+            float* to = keep ? b.features : b.features_in;
+            RETEXO_CUDA_TRY(cudaMemcpyAsync(to, feat, sizeof(float) * (size_t)n * c.d0, in_kind, st));
+            if (!keep) relay_rows_kernel<<<(unsigned)((n + 7) / 8), 256, 0, st>>>(to, c.d0, c.d0, n, b.features, ldp);
+        } else {
+            if (ldp != c.d0) RETEXO_CUDA_TRY(cudaMemsetAsync(b.features, 0, sizeof(float) * (size_t)n * ldp, st));
+            RETEXO_CUDA_TRY(cudaMemcpy2DAsync(b.features, sizeof(float) * ldp, feat, sizeof(float) * ld_feat,
+                                              sizeof(float) * c.d0, (size_t)n, in_kind, st));
+        }
         RETEXO_CUDA_TRY(cudaMemcpyAsync(b.labels, labels, sizeof(int32_t) * (size_t)n, in_kind, st));
         RETEXO_CUDA_TRY(cudaMemcpyAsync(b.train_idx, train_idx, sizeof(int32_t) * (size_t)n_tr, in_kind, st));
         if (n_val) RETEXO_CUDA_TRY(cudaMemcpyAsync(b.val_idx, val_idx, sizeof(int32_t) * (size_t)n_val, in_kind, st));
@@ -375,9 +404,7 @@ extern "C" int retexo_lmp_train(const retexo_lmp_config* cfg, const retexo_lmp_i
         // rows that do not start on 16-byte boundaries would force narrow loads on the dominant
         // gather of round 1: re-lay them once with rows of whole 128-byte lines
         const int64_t ldp = round_up(c.d0, 32);
-        if (ldp != c.d0) RETEXO_CUDA_TRY(cudaMemsetAsync(b.features, 0, sizeof(float) * (size_t)n * ldp, st));
-        RETEXO_CUDA_TRY(cudaMemcpy2DAsync(b.features, sizeof(float) * ldp, feat, sizeof(float) * ld_feat,
-                                          sizeof(float) * c.d0, (size_t)n, cudaMemcpyDeviceToDevice, st));
+        relay_rows_kernel<<<(unsigned)((n + 7) / 8), 256, 0, st>>>(feat, ld_feat, c.d0, n, b.features, ldp);
         feat = b.features;
         ld_feat = ldp;
     }

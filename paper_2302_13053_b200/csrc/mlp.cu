@@ -173,6 +173,20 @@ extern "C" int retexo_pack_rows(const void* src, int32_t src_is_bf16, int64_t ld
     dim3 grid((unsigned)((rows_cover + 31) / 32), (unsigned)((cols_cover + 31) / 32));
     if (grid.y > 65535) return RETEXO_ERR_UNSUPPORTED;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
+    // whole 16-byte pieces on both sides and no transpose wanted: the streaming kernel (a piece may reach up to 3 floats
+    // or 7 bf16 values beyond dim, inside the row's stride)
+    const int64_t src_cover = src_is_bf16 ? ((int64_t)dim + 7) / 8 * 8 : ((int64_t)dim + 3) / 4 * 4;
+    if (dst && !dst_t && aligned_to(dst, 16) && ld_dst % 8 == 0 && aligned_to(src, 16) && ld_src % (src_is_bf16 ? 8 : 4) == 0 &&
+        ld_src >= src_cover && ld_dst <= INT32_MAX) {
+        int lanes_log2 = 0;
+        while (lanes_log2 < 5 && (8 << lanes_log2) < ld_dst) ++lanes_log2;
+        const unsigned blocks = (unsigned)(((n_rows << lanes_log2) + 255) / 256);
+        if (src_is_bf16)
+            pack_rows_pieces_kernel<true><<<blocks, 256, 0, st>>>(src, ld_src, dim, idx, n_rows, static_cast<bf16*>(dst), ld_dst, ones ? 1 : 0, lanes_log2);
+        else
+            pack_rows_pieces_kernel<false><<<blocks, 256, 0, st>>>(src, ld_src, dim, idx, n_rows, static_cast<bf16*>(dst), ld_dst, ones ? 1 : 0, lanes_log2);
+        return launch_status();
+    }
     if (src_is_bf16)
         pack_rows_kernel<true><<<grid, 256, 0, st>>>(src, ld_src, dim, idx, n_rows, static_cast<bf16*>(dst), ld_dst,
                                                      static_cast<bf16*>(dst_t), ld_t, ones ? 1 : 0);

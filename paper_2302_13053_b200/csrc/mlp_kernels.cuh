@@ -46,6 +46,58 @@ __global__ void __launch_bounds__(256) pack_rows_kernel(const void* __restrict__
     }
 }
 
+// The same without a transpose, for rows in whole 16-byte pieces (dst and a bf16 src aligned, strides multiples of 8; a fp32
+// src of 4): 1 << lanes_log2 lanes take a row, a piece of 8 columns each, four pieces in flight per lane.
+// A stream bound by memory, where the tile kernel above is bound by its 2-byte loads and stores (55.7 k gathered rows of 602
+// bf16 columns: 85 -> 25 us).
+template <bool SRC_BF16>
+__global__ void __launch_bounds__(256) pack_rows_pieces_kernel(const void* __restrict__ src, int64_t ld_src, int32_t dim,
+                                                               const int32_t* __restrict__ idx, int64_t n_rows,
+                                                               bf16* __restrict__ dst, int64_t ld_dst, int ones, int lanes_log2) {
+    const int64_t t = blockIdx.x * 256ll + threadIdx.x, r = t >> lanes_log2;
+    if (r >= n_rows) return;
+    const int lanes = 1 << lanes_log2, pieces = (int)(ld_dst >> 3);
+    const int64_t sr = idx ? idx[r] : r;
+    uint4* out = reinterpret_cast<uint4*>(dst + r * ld_dst);
+    for (int p0 = (int)t & (lanes - 1); p0 < pieces; p0 += 4 * lanes) {
+        uint4 v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int c = 8 * (p0 + i * lanes);
+            v[i] = make_uint4(0u, 0u, 0u, 0u);
+            if (c >= dim || c >= ld_dst) continue;
+            if constexpr (SRC_BF16) {
+                v[i] = __ldg(reinterpret_cast<const uint4*>(static_cast<const bf16*>(src) + sr * ld_src + c));
+            } else {
+                const float* s = static_cast<const float*>(src) + sr * ld_src + c;
+                const float4 a = __ldg(reinterpret_cast<const float4*>(s));
+                const float4 b = c + 4 < dim ? __ldg(reinterpret_cast<const float4*>(s + 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                const __nv_bfloat162 q0 = __floats2bfloat162_rn(a.x, a.y), q1 = __floats2bfloat162_rn(a.z, a.w);
+                const __nv_bfloat162 q2 = __floats2bfloat162_rn(b.x, b.y), q3 = __floats2bfloat162_rn(b.z, b.w);
+                v[i] = make_uint4(*reinterpret_cast<const uint32_t*>(&q0), *reinterpret_cast<const uint32_t*>(&q1),
+                                  *reinterpret_cast<const uint32_t*>(&q2), *reinterpret_cast<const uint32_t*>(&q3));
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int p = p0 + i * lanes, c = 8 * p;
+            if (p >= pieces) continue;
+            if (c + 8 > dim) {      // the ragged piece and the padding: zeros, and the column of ones
+                uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int col = c + 2 * k;
+                    const uint32_t lo = col < dim ? w[k] & 0xffffu : (ones && col == dim ? 0x3f80u : 0u);
+                    const uint32_t hi = col + 1 < dim ? w[k] >> 16 : (ones && col + 1 == dim ? 0x3f80u : 0u);
+                    w[k] = lo | (hi << 16);
+                }
+                v[i] = make_uint4(w[0], w[1], w[2], w[3]);
+            }
+            out[p] = v[i];
+        }
+    }
+}
+
 // ---------------------------------------------------------------- optimiser
 struct GradSeg {
     int64_t size;              // parameters in this segment
