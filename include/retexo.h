@@ -115,11 +115,14 @@ size_t retexo_aggregate_workspace_size(int64_t n_nodes, int64_t n_edges, int32_t
  * out      fp32 [n x ldout], may be NULL if out_bf16 is given.
  * out_bf16 optional bf16 (round-to-nearest-even) copy of the same matrix,
  *          row stride ldout_bf16 elements; NULL if not wanted.
- * Sums are taken in CSR order per row in fp32; rows of at least 4096 entries
- * are cut into segments of 2048 entries whose sums are added in segment order.
- * 128-bit loads are used when q is 16-byte aligned, ldq % 4 == 0 and
- * ldq >= round_up(dim, 4); 64-bit loads under the analogous rule; otherwise
- * scalar loads.  Nothing is an error for being unaligned.
+ * Sums are taken in fp32 in an order that depends on the row's length and the
+ * layout only (short rows in CSR order, longer ones in a few interleaved or
+ * consecutive parts that are added in a fixed order); GCN may scale q by n_u
+ * into the workspace first.  256-bit loads are used when q is 32-byte aligned,
+ * ldq % 8 == 0 and ldq >= round_up(dim, 8), 128-bit loads when it is 16-byte
+ * aligned, ldq % 4 == 0 and ldq >= round_up(dim, 4), 64-bit loads under the
+ * analogous rule, otherwise scalar loads.  Nothing is an error for being
+ * unaligned.
  * dim <= 4096.  Errors: INVALID_ARG, WORKSPACE, UNSUPPORTED. */
 int retexo_aggregate(const retexo_csr* g, int32_t type,
                      const float* q, int64_t ldq, int32_t dim,

@@ -1,129 +1,439 @@
 // Full-graph neighbour aggregation of one message-passing round (Eq. 1) over a CSR graph:
 // GCN symmetric-normalised sum, GraphSAGE mean and max (+ self concat); the GAT pass is in gat.cu.
 //
-// The work is a gather-reduce bound by the memory system, not a dense
-// contraction: neighbour rows are streamed with the widest aligned vector
-// loads, several rows in flight per lane, sums kept in registers.  Work is
-// handed out warp by warp from one counter (a persistent grid), so a power-law
-// degree distribution does not leave SMs idle: rows of kHeavyDegree entries or
-// more are cut into segments of kSegLen entries that are handed out first,
-// each segment's partial sum goes to scratch, and a second kernel adds a row's
-// segments in order.  Nothing depends on which warp ran what, so results are
-// the same bits on every call.
+//
+// The work is a gather-reduce bound by the memory system, not a dense contraction: neighbour rows are streamed with the
+// widest aligned vector loads, several rows in flight per lane, sums kept in registers.  Rows go to lanes by a fixed
+// rule (no work counter: a draw per row from one address is 2 ns each, more than a row of ten entries takes the chip),
+// rows of heavy_degree() entries or more are cut into segments that are taken first, each segment's partial sum goes to
+// scratch, and a second kernel adds a row's segments in order.  Nothing depends on which warp ran what when, so results
+// are the same bits on every call.
 #include "common.cuh"
+#include "aggregate.h"
 #include "gat.h"
 
 namespace retexo {
 
-constexpr int kHeavyDegree = 4096;     // rows at least this long are cut into segments
-constexpr int kSegLen = 2048;          // entries per segment
-constexpr int kAggThreads = 256;
+constexpr int kAggThreads = 128, kAggBlocksPerSm = 9;      // (56 registers a thread)
 constexpr int kAggWarps = kAggThreads / kWarp;
-constexpr int kUnroll = 4;             // neighbour rows in flight per lane and column chunk
 
-// Upper bound on the number of segments of a graph with n_edges entries.
-static inline int64_t max_segments(int64_t n_edges) { return n_edges / kSegLen + n_edges / kHeavyDegree + 1; }
+// Rows of heavy_degree entries or more are cut into segments of half as many: 2048 entries, fewer on graphs so small that
+// one warp on a long row would keep the grid waiting.
+static inline int32_t seg_len(int64_t n_edges) {
+    int32_t len = 64;
+    while (len < 2048 && (int64_t)len * 148 * 128 < n_edges) len *= 2;
+    return len;
+}
+static inline int32_t heavy_degree(int64_t n_edges) { return 2 * seg_len(n_edges); }
+
+// Upper bounds on the number of heavy rows and of segments of a graph with n_edges entries.
+static inline int64_t max_heavy(int64_t n_edges) { return n_edges / heavy_degree(n_edges) + 1; }
+static inline int64_t max_segments(int64_t n_edges) { return n_edges / seg_len(n_edges) + max_heavy(n_edges); }
 
 // ---------------------------------------------------------------- pre-pass
-// coef[v]: GCN (deg+1)^-1/2, SAGE 1/deg (0 for isolated nodes).  Also lists
-// the heavy rows and their segments (list order is arbitrary; no result
-// depends on it).
-__global__ void prep_rows_kernel(int64_t n, const int64_t* __restrict__ rowptr, int mode,
-                                 float* __restrict__ coef, int32_t* __restrict__ heavy_list,
-                                 int32_t* __restrict__ heavy_seg_base, int32_t* __restrict__ seg_slot,
-                                 int32_t* __restrict__ counters /* [0] heavy rows, [1] segments, [2] work */) {
-    int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+struct HeavyRows {
+    int32_t seg_entries;             // entries per segment; rows of twice as many are heavy
+    int32_t* list;                   // [heavy rows] node id
+    int32_t* seg_base;               // [heavy rows] first segment of the row
+    int32_t* seg_slot;               // [segments] index into list
+    int32_t* counters;               // [0] heavy rows, [1] segments
+};
+
+// Lists row v and its segments if it is heavy (list order is arbitrary; no result depends on it).
+__device__ __forceinline__ void list_if_heavy(const HeavyRows& h, int64_t v, int64_t deg) {
+    if (deg < 2 * h.seg_entries) return;
+    const int32_t slot = atomicAdd(h.counters + 0, 1);
+    const int32_t nseg = (int32_t)((deg + h.seg_entries - 1) / h.seg_entries);
+    const int32_t base = atomicAdd(h.counters + 1, nseg);
+    h.list[slot] = (int32_t)v;
+    h.seg_base[slot] = base;
+    for (int32_t i = 0; i < nseg; ++i) h.seg_slot[base + i] = slot;
+}
+
+__device__ __forceinline__ float gcn_coef(int64_t deg) { return 1.0f / sqrtf((float)deg + 1.0f); }
+
+// Heavy rows, and (GCN, coef != nullptr) the normalisation (deg + 1)^-1/2.
+__global__ void prep_rows_kernel(int64_t n, const int64_t* __restrict__ rowptr, HeavyRows h, float* __restrict__ coef) {
+    const int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (v >= n) return;
-    int64_t deg = rowptr[v + 1] - rowptr[v];
-    float c;
-    if (mode == RETEXO_GCN) c = 1.0f / sqrtf((float)deg + 1.0f);
-    else c = deg > 0 ? 1.0f / (float)deg : 0.0f;
-    coef[v] = c;
-    if (deg >= kHeavyDegree) {
-        const int32_t slot = atomicAdd(counters + 0, 1);
-        const int32_t nseg = (int32_t)((deg + kSegLen - 1) / kSegLen);
-        const int32_t base = atomicAdd(counters + 1, nseg);
-        heavy_list[slot] = (int32_t)v;
-        heavy_seg_base[slot] = base;
-        for (int32_t i = 0; i < nseg; ++i) seg_slot[base + i] = slot;
+    const int64_t deg = rowptr[v + 1] - rowptr[v];
+    if (coef) coef[v] = gcn_coef(deg);
+    list_if_heavy(h, v, deg);
+}
+
+// The same for a GCN round whose rows are scaled ahead: qs[u] = n_u q[u] in rows of ld_qs = round_up(dim, 8) floats, so that the
+// gather needs no coefficient per entry (one more random access each, a quarter of the gather's time) and always finds
+// rows in whole 32-byte pieces.  1 << lanes_log2 lanes a row, 8 columns each; a stream over q.
+__global__ void __launch_bounds__(256) gcn_scale_rows_kernel(int64_t n, const int64_t* __restrict__ rowptr, HeavyRows h,
+                                                             const float* __restrict__ q, int64_t ldq, int32_t dim, int vec4,
+                                                             float* __restrict__ qs, int64_t ld_qs, int lanes_log2) {
+    const int64_t t = blockIdx.x * 256ll + threadIdx.x, v = t >> lanes_log2;
+    if (v >= n) return;
+    const int lanes = 1 << lanes_log2, lane = (int)t & (lanes - 1);
+    const int64_t deg = rowptr[v + 1] - rowptr[v];
+    if (lane == 0) list_if_heavy(h, v, deg);
+    const float c = gcn_coef(deg);
+    const float* src = q + v * ldq;
+    float* dst = qs + v * ld_qs;
+    for (int col = 8 * lane; col < ld_qs; col += 8 * lanes) {
+        float x[8];
+        if (vec4 && col + 8 <= dim) {
+            const float4 a = __ldg(reinterpret_cast<const float4*>(src + col)), b = __ldg(reinterpret_cast<const float4*>(src + col + 4));
+            x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) x[i] = col + i < dim ? __ldg(src + col + i) : 0.f;
+        }
+        *reinterpret_cast<float4*>(dst + col) = make_float4(c * x[0], c * x[1], c * x[2], c * x[3]);
+        *reinterpret_cast<float4*>(dst + col + 4) = make_float4(c * x[4], c * x[5], c * x[6], c * x[7]);
     }
 }
 
-// ---------------------------------------------------------------- vectors
-template <int VEC> struct VecT;
-template <> struct VecT<4> { using type = float4; };
-template <> struct VecT<2> { using type = float2; };
-template <> struct VecT<1> { using type = float; };
-
-template <int VEC>
-__device__ __forceinline__ void vec_zero(typename VecT<VEC>::type& a);
-template <> __device__ __forceinline__ void vec_zero<4>(float4& a) { a = make_float4(0.f, 0.f, 0.f, 0.f); }
-template <> __device__ __forceinline__ void vec_zero<2>(float2& a) { a = make_float2(0.f, 0.f); }
-template <> __device__ __forceinline__ void vec_zero<1>(float& a) { a = 0.f; }
-
-__device__ __forceinline__ void vec_fma(float4& a, float w, const float4& x) {
-    a.x = fmaf(w, x.x, a.x); a.y = fmaf(w, x.y, a.y); a.z = fmaf(w, x.z, a.z); a.w = fmaf(w, x.w, a.w);
-}
-__device__ __forceinline__ void vec_fma(float2& a, float w, const float2& x) {
-    a.x = fmaf(w, x.x, a.x); a.y = fmaf(w, x.y, a.y);
-}
-__device__ __forceinline__ void vec_fma(float& a, float w, const float& x) { a = fmaf(w, x, a); }
-__device__ __forceinline__ void vec_add(float4& a, const float4& x) { a.x += x.x; a.y += x.y; a.z += x.z; a.w += x.w; }
-__device__ __forceinline__ void vec_add(float2& a, const float2& x) { a.x += x.x; a.y += x.y; }
-__device__ __forceinline__ void vec_add(float& a, const float& x) { a += x; }
-
-__device__ __forceinline__ void vec_max(float4& a, const float4& x) {
-    a.x = fmaxf(a.x, x.x); a.y = fmaxf(a.y, x.y); a.z = fmaxf(a.z, x.z); a.w = fmaxf(a.w, x.w);
-}
-__device__ __forceinline__ void vec_max(float2& a, const float2& x) { a.x = fmaxf(a.x, x.x); a.y = fmaxf(a.y, x.y); }
-__device__ __forceinline__ void vec_max(float& a, const float& x) { a = fmaxf(a, x); }
-
-// What a row's accumulator does with a neighbour row: plain sum (SAGE mean),
-// sum weighted by coef[u] (GCN), or element-wise maximum (SAGE max-pooling).
+// What a row's accumulator does with a neighbour row: plain sum (SAGE mean; GCN: of rows scaled ahead, or weighted by coef[u]
+// as they come), or element-wise maximum (SAGE max-pooling).
 constexpr int kOpSum = 0, kOpGcn = 1, kOpMax = 2;
-
-template <int VEC, int OP>
-__device__ __forceinline__ void vec_init(typename VecT<VEC>::type& a) {
-    if constexpr (OP != kOpMax) vec_zero<VEC>(a);
-    else if constexpr (VEC == 4) a = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-    else if constexpr (VEC == 2) a = make_float2(-INFINITY, -INFINITY);
-    else a = -INFINITY;
-}
-
-template <int VEC>
-__device__ __forceinline__ float vec_get(const typename VecT<VEC>::type& a, int i);
-template <> __device__ __forceinline__ float vec_get<4>(const float4& a, int i) {
-    return i == 0 ? a.x : i == 1 ? a.y : i == 2 ? a.z : a.w;
-}
-template <> __device__ __forceinline__ float vec_get<2>(const float2& a, int i) { return i == 0 ? a.x : a.y; }
-template <> __device__ __forceinline__ float vec_get<1>(const float& a, int) { return a; }
 
 struct AggArgs {
     int64_t n;
     const int64_t* rowptr;
     const int32_t* colidx;
-    const float* q;
+    const float* q;         // the rows that are gathered (GCN through agg_lanes_kernel: scaled by n_u)
     int64_t ldq;
     int32_t dim;
-    const float* coef;
+    const float* coef;      // agg_rows_kernel only
     float* out;             // may be null
     int64_t ldout;
     __nv_bfloat16* out16;   // may be null
     int64_t ldout16;
     int32_t concat_self;    // SAGE
-    const int32_t* heavy_list;       // [heavy rows] node id
-    const int32_t* heavy_seg_base;   // [heavy rows] first segment of the row
-    const int32_t* seg_slot;         // [segments] index into heavy_list
-    int32_t* counters;               // [0] heavy rows, [1] segments, [2] next work item
+    int32_t vec_out, vec_out16;      // 16-byte stores of 4 floats / 8-byte stores of 4 bf16 values are aligned
+    HeavyRows heavy;
     float* seg_partial;              // [segments x round_up(dim, 4)] raw sums
     int64_t ld_partial;
-    float hub_coef;                  // GCN, matrix larger than L2: rows of nodes with coef <= hub_coef (hubs) are
-                                     // loaded "evict last", all others "evict first"; 0 = no hints
+    int32_t* next_item;              // agg_rows_kernel: work counter
+    float hub_coef;                  // agg_rows_kernel: rows of nodes with coef <= hub_coef (hubs) are loaded "evict last", all
+                                     // others "evict first"
 };
 
-// L2 eviction priorities for the gathers of a matrix that does not fit the cache: a power-law graph
-// reads its hubs' rows again and again, every other row a few times; left to itself the cache keeps
-// neither.  The hints change nothing but which lines stay resident.
+__device__ __forceinline__ void store_elem(const AggArgs& a, int64_t v, int col, float val) {
+    if (a.out) a.out[v * a.ldout + col] = val;
+    if (a.out16) a.out16[v * a.ldout16 + col] = f32_to_bf16(val);
+}
+
+// E floats from read-only memory, aligned to as much.
+template <int E>
+__device__ __forceinline__ void load_vec(const float* p, float (&v)[E]) {
+    if constexpr (E == 8) {
+        asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]) : "l"(p));
+    } else if constexpr (E == 4) {
+        const float4 x = __ldg(reinterpret_cast<const float4*>(p));
+        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+    } else if constexpr (E == 2) {
+        const float2 x = __ldg(reinterpret_cast<const float2*>(p));
+        v[0] = x.x; v[1] = x.y;
+    } else {
+        v[0] = __ldg(p);
+    }
+}
+// ---------------------------------------------------------------- rows to lanes
+// A slab of LPG x E x NV columns is aggregated at a time.  LPG lanes (a power of two) take one CSR entry: lane `li` of group
+// `g` owns the NV vectors of E columns at E (li + LPG k) of the slab, so a warp reads G = 32 / LPG neighbour rows per load
+// instruction in whole runs.  A row of up to kGroupEntries entries is summed by one group in CSR order (a warp works on G rows
+// at once), a longer one by the whole warp: group g adds the entries g, g + G, ... and the groups' sums are added in a fixed tree.
+constexpr int kGroupEntries = 32;
+
+template <int LPG, int E, int NV, int OP>
+struct AggLanes {
+    static constexpr int G = kWarp / LPG, kCols = LPG * E * NV;
+    static constexpr int U = E >= 4 ? 4 : 8;      // entries in flight per lane
+    const AggArgs& a;
+    int g, li;
+    bool on[NV];                        // the vector exists; if not, vector 0 of the slab is read and dropped
+    int off[NV];
+    float acc[NV][E], self[NV][E];
+
+    __device__ __forceinline__ AggLanes(const AggArgs& a_, int lane, int slab) : a(a_) {
+        g = lane / LPG;
+        li = lane % LPG;
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            const int c = slab * kCols + E * (li + LPG * k);
+            on[k] = c < a.dim;
+            off[k] = on[k] ? c : slab * kCols;
+        }
+    }
+    __device__ __forceinline__ void clear() {
+#pragma unroll
+        for (int k = 0; k < NV; ++k)
+#pragma unroll
+            for (int i = 0; i < E; ++i) acc[k][i] = OP == kOpMax ? -INFINITY : 0.f;
+    }
+    // Asks for what the end of row v needs, ahead of time.
+    __device__ __forceinline__ void begin(int64_t v) {
+        clear();
+        if (OP == kOpGcn || a.concat_self) {
+#pragma unroll
+            for (int k = 0; k < NV; ++k) load_vec<E>(a.q + v * a.ldq + off[k], self[k]);
+        }
+    }
+    // Adds the rows u[t] where ok[t]; where it is not, u[t] is some node whose row is loaded and dropped.
+    template <int N>
+    __device__ __forceinline__ void batch(const int32_t (&u)[N], const bool (&ok)[N]) {
+        float x[N][NV][E];
+#pragma unroll
+        for (int t = 0; t < N; ++t)
+#pragma unroll
+            for (int k = 0; k < NV; ++k) load_vec<E>(a.q + (int64_t)u[t] * a.ldq + off[k], x[t][k]);
+#pragma unroll
+        for (int t = 0; t < N; ++t) {
+            if (!ok[t]) continue;
+#pragma unroll
+            for (int k = 0; k < NV; ++k)
+#pragma unroll
+                for (int i = 0; i < E; ++i) acc[k][i] = OP == kOpMax ? fmaxf(acc[k][i], x[t][k][i]) : acc[k][i] + x[t][k][i];
+        }
+    }
+    // Entries [first, last) of the CSR by the whole warp, 32 columns at a time, fetched two trips ahead.
+    __device__ __forceinline__ void walk_by_warp(int64_t first, int64_t last, int lane) {
+        auto column = [&](int64_t e0) -> int32_t { return __ldcs(a.colidx + (e0 + lane < last ? e0 + lane : first)); };
+        if (first >= last) return;
+        int32_t next_u = column(first), after_u = first + kWarp < last ? column(first + kWarp) : 0;
+        for (int64_t e0 = first; e0 < last; e0 += kWarp) {
+            const int cnt = (int)min((int64_t)kWarp, last - e0);
+            const int32_t my_u = next_u;
+            next_u = after_u;
+            if (e0 + 2 * kWarp < last) after_u = column(e0 + 2 * kWarp);
+            constexpr int N = G * U > kWarp ? kWarp / G : U;
+#pragma unroll 1
+            for (int j = 0; j < cnt; j += G * N) {
+                int32_t u[N];
+                bool ok[N];
+#pragma unroll
+                for (int t = 0; t < N; ++t) {
+                    const int at = j + t * G + g;
+                    u[t] = __shfl_sync(0xffffffffu, my_u, at & 31);
+                    ok[t] = at < cnt;
+                }
+                batch<N>(u, ok);
+            }
+        }
+#pragma unroll
+        for (int o = LPG; o < kWarp; o <<= 1) {
+#pragma unroll
+            for (int k = 0; k < NV; ++k)
+#pragma unroll
+                for (int i = 0; i < E; ++i) {
+                    const float y = __shfl_xor_sync(0xffffffffu, acc[k][i], o);
+                    acc[k][i] = OP == kOpMax ? fmaxf(acc[k][i], y) : acc[k][i] + y;
+                }
+        }
+    }
+    // Every group its own row of `total` entries from beg on (0: none); longest = the largest total of the warp.
+    __device__ __forceinline__ void walk_by_group(int64_t beg, int total, int longest, int32_t some_node) {
+        constexpr int N = U < LPG ? U : LPG;
+        auto column = [&](int e) -> int32_t { return total > 0 ? __ldg(a.colidx + beg + (e < total ? e : 0)) : some_node; };
+        int32_t next_u = column(li);
+        for (int e0 = 0; e0 < longest; e0 += LPG) {
+            const int32_t my_u = next_u;
+            if (e0 + LPG < longest) next_u = column(e0 + LPG + li);
+            const int cnt = min(LPG, longest - e0);
+#pragma unroll 1
+            for (int j = 0; j < cnt; j += N) {
+                int32_t u[N];
+                bool ok[N];
+#pragma unroll
+                for (int t = 0; t < N; ++t) {
+                    u[t] = __shfl_sync(0xffffffffu, my_u, g * LPG + j + t);
+                    ok[t] = e0 + j + t < total;
+                }
+                batch<N>(u, ok);
+            }
+        }
+    }
+    __device__ __forceinline__ void store(int64_t v, int col, const float (&x)[E]) {
+        if (a.out) {
+            float* o = a.out + v * a.ldout + col;
+            if (E >= 4 && a.vec_out) {
+#pragma unroll
+                for (int i = 0; i < E; i += 4) *reinterpret_cast<float4*>(o + i) = make_float4(x[i], x[(i + 1) % E], x[(i + 2) % E], x[(i + 3) % E]);
+            } else {
+#pragma unroll
+                for (int i = 0; i < E; ++i) o[i] = x[i];
+            }
+        }
+        if (a.out16) {
+            __nv_bfloat16* o = a.out16 + v * a.ldout16 + col;
+            if (E >= 4 && a.vec_out16) {
+#pragma unroll
+                for (int i = 0; i < E; i += 4) {
+                    const __nv_bfloat162 lo = __floats2bfloat162_rn(x[i], x[(i + 1) % E]), hi = __floats2bfloat162_rn(x[(i + 2) % E], x[(i + 3) % E]);
+                    *reinterpret_cast<uint2*>(o + i) = make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+                }
+            } else {
+#pragma unroll
+                for (int i = 0; i < E; ++i) o[i] = f32_to_bf16(x[i]);
+            }
+        }
+    }
+    // GCN adds the (scaled) self row and scales, SAGE divides by the degree and (optionally) copies the self row.
+    __device__ __forceinline__ void finish(int64_t v, int64_t deg) {
+        const float cv = OP == kOpGcn ? gcn_coef(deg) : 0.f;
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            if (!on[k]) continue;
+#pragma unroll
+            for (int i = 0; i < E; ++i) {
+                if (OP == kOpGcn) acc[k][i] = cv * (self[k][i] + acc[k][i]);
+                else acc[k][i] = deg <= 0 ? 0.f : OP == kOpMax ? acc[k][i] : acc[k][i] / (float)deg;
+            }
+            const bool concat = OP != kOpGcn && a.concat_self;
+            const int n_cols = a.dim - off[k];
+            if (E == 1 || n_cols >= E) {
+                if (concat) store(v, off[k], self[k]);
+                store(v, off[k] + (concat ? a.dim : 0), acc[k]);
+            } else {                    // the ragged last vector
+#pragma unroll
+                for (int i = 0; i < E; ++i) {
+                    if (i >= n_cols) break;
+                    if (concat) store_elem(a, v, off[k] + i, self[k][i]);
+                    store_elem(a, v, off[k] + (concat ? a.dim : 0) + i, acc[k][i]);
+                }
+            }
+        }
+    }
+};
+
+// Blocks are ordered slab by slab, so that at any time the whole grid gathers from the same few columns of the matrix: a slab of
+// 64 columns stays in L2 where the whole matrix does not.  A slab's first seg_blocks blocks take the segments of the heavy rows
+// (their raw sums go to scratch), the others a fixed set of rows each, G per warp.
+// Bound by the L2 -> SM path (64 bytes a cycle and SM) on dense graphs, by row pointer -> column -> row latencies on sparse ones;
+// measured against a persistent kernel that drew its rows from one counter, a warp each (SAGE, bf16 out, with concatenation):
+//   233 k nodes, 115 M entries, 256 columns: 6.95 -> 6.4 ms (18.4 TB/s of neighbour rows); GCN 9.5 -> 7.8 ms
+//   58 k nodes, 7 M entries, 256 columns: 820 -> 467 us (15.8 TB/s); GCN 1036 -> 520 us
+//   600 k nodes, 30 M entries, 256 columns: 4.05 -> 3.4 ms;  20 k nodes, 88 k entries, 500 columns: 142 -> 66 us
+// Slabs of 32 or 128 columns instead of 64 take 1.4 and 1.2 times as long on the first of these; 4 entries in flight, since
+// with 56 registers 36 warps fit an SM (64: 32 warps, level; 48: spills, 5 % slower; 80 and more: 1.4 times as long).
+template <int LPG, int E, int NV, int OP>
+__global__ void __launch_bounds__(kAggThreads, kAggBlocksPerSm) agg_lanes_kernel(AggArgs a, unsigned blocks_per_slab, unsigned seg_blocks) {
+    const unsigned slab = blockIdx.x / blocks_per_slab, b = blockIdx.x % blocks_per_slab;
+    constexpr int G = kWarp / LPG;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    AggLanes<LPG, E, NV, OP> L(a, lane, (int)slab);
+    const int32_t seg_entries = a.heavy.seg_entries;
+    if (b < seg_blocks) {
+        const int n_seg = a.heavy.counters[1];
+        for (int item = (int)b * kAggWarps + warp; item < n_seg; item += (int)seg_blocks * kAggWarps) {
+            const int32_t slot = a.heavy.seg_slot[item];
+            const int64_t v = a.heavy.list[slot];
+            const int64_t beg = a.rowptr[v] + (int64_t)(item - a.heavy.seg_base[slot]) * seg_entries;
+            L.clear();
+            L.walk_by_warp(beg, min(a.rowptr[v + 1], beg + seg_entries), lane);
+            float* dst = a.seg_partial + (int64_t)item * a.ld_partial;
+            if (L.g == 0) {
+#pragma unroll
+                for (int k = 0; k < NV; ++k)
+#pragma unroll
+                    for (int i = 0; i < E; ++i) if (L.on[k] && L.off[k] + i < a.dim) dst[L.off[k] + i] = L.acc[k][i];
+            }
+        }
+        return;
+    }
+    const int64_t v0 = ((int64_t)(b - seg_blocks) * kAggWarps + warp) * G;
+    if (v0 >= a.n) return;
+    const int64_t v = min(v0 + L.g, a.n - 1);
+    const int64_t beg = __ldg(a.rowptr + v);
+    const int32_t total = v0 + L.g < a.n ? (int32_t)(__ldg(a.rowptr + v + 1) - beg) : INT32_MAX;      // (beyond the last row: nobody's)
+    const bool mine = G > 1 && total <= kGroupEntries;
+    if constexpr (G > 1) {
+        if (__any_sync(0xffffffffu, mine)) {
+            const int longest = __reduce_max_sync(0xffffffffu, mine ? total : 0);
+            L.begin(v);
+            L.walk_by_group(beg, mine ? total : 0, longest, (int32_t)v);
+            if (mine) L.finish(v, total);
+        }
+    }
+    unsigned longer = __ballot_sync(0xffffffffu, L.li == 0 && !mine && total < 2 * seg_entries);
+    while (longer) {
+        const int src = __ffs(longer) - 1;
+        longer &= longer - 1;
+        const int64_t w = __shfl_sync(0xffffffffu, v, src), w_beg = __shfl_sync(0xffffffffu, beg, src);
+        const int32_t w_total = __shfl_sync(0xffffffffu, total, src);
+        L.begin(w);
+        L.walk_by_warp(w_beg, w_beg + w_total, lane);
+        if (L.g == 0) L.finish(w, w_total);
+    }
+}
+
+// Adds the heavy rows' segment sums in segment order and finishes the rows; a block per row, a thread per column.  self_scaled: q
+// holds rows scaled by n_u (GCN).
+template <int OP>
+__global__ void __launch_bounds__(kAggThreads) agg_combine_kernel(AggArgs a, int self_scaled) {
+    const int n_heavy = a.heavy.counters[0];
+    for (int h = blockIdx.x; h < n_heavy; h += gridDim.x) {
+        const int64_t v = a.heavy.list[h];
+        const int64_t deg = a.rowptr[v + 1] - a.rowptr[v];
+        const int nseg = (int)((deg + a.heavy.seg_entries - 1) / a.heavy.seg_entries);
+        const float* src = a.seg_partial + (int64_t)a.heavy.seg_base[h] * a.ld_partial;
+        const float cv = OP == kOpGcn ? gcn_coef(deg) : 0.f;
+        for (int col = threadIdx.x; col < a.dim; col += kAggThreads) {
+            float acc = OP == kOpMax ? -INFINITY : 0.f;
+#pragma unroll 4
+            for (int i = 0; i < nseg; ++i) {
+                const float x = src[(int64_t)i * a.ld_partial + col];
+                acc = OP == kOpMax ? fmaxf(acc, x) : acc + x;
+            }
+            const float self = a.q[v * a.ldq + col];
+            if (OP == kOpGcn) {
+                store_elem(a, v, col, cv * (self_scaled ? self + acc : fmaf(cv, self, acc)));
+            } else {
+                const float mean = OP == kOpMax ? acc : acc / (float)deg;
+                if (a.concat_self) store_elem(a, v, col, self);
+                store_elem(a, v, col + (a.concat_self ? a.dim : 0), mean);
+            }
+        }
+    }
+}
+
+static int launch_combine(int op, const AggArgs& a, int64_t n_edges, int self_scaled, int n_sm, cudaStream_t st) {
+    if (n_edges < heavy_degree(n_edges)) return launch_status();      // no row can be heavy
+    if (op == kOpGcn) agg_combine_kernel<kOpGcn><<<n_sm, kAggThreads, 0, st>>>(a, self_scaled);
+    else if (op == kOpMax) agg_combine_kernel<kOpMax><<<n_sm, kAggThreads, 0, st>>>(a, 0);
+    else agg_combine_kernel<kOpSum><<<n_sm, kAggThreads, 0, st>>>(a, 0);
+    return launch_status();
+}
+
+template <int LPG, int E, int NV>
+static int launch_lanes(int op, const AggArgs& a, int64_t n_edges, int n_sm, cudaStream_t st) {
+    constexpr int64_t kRows = (int64_t)kAggWarps * (kWarp / LPG);
+    const int64_t n_slabs = (a.dim + LPG * E * NV - 1) / (LPG * E * NV);
+    const int64_t segs = n_edges >= heavy_degree(n_edges) ? (max_segments(n_edges) + kAggWarps - 1) / kAggWarps : 0;
+    const unsigned seg_blocks = (unsigned)(segs < 4ll * n_sm ? segs : 4ll * n_sm);
+    const int64_t per_slab = (a.n + kRows - 1) / kRows + seg_blocks;
+    if (per_slab * n_slabs > INT32_MAX) return RETEXO_ERR_UNSUPPORTED;
+    const unsigned grid = (unsigned)(per_slab * n_slabs);
+    if constexpr (E == 8) {
+        if (op == kOpGcn) agg_lanes_kernel<LPG, E, NV, kOpGcn><<<grid, kAggThreads, 0, st>>>(a, (unsigned)per_slab, seg_blocks);
+    }
+    if (op == kOpMax) agg_lanes_kernel<LPG, E, NV, kOpMax><<<grid, kAggThreads, 0, st>>>(a, (unsigned)per_slab, seg_blocks);
+    else if (op == kOpSum) agg_lanes_kernel<LPG, E, NV, kOpSum><<<grid, kAggThreads, 0, st>>>(a, (unsigned)per_slab, seg_blocks);
+    return launch_combine(op, a, n_edges, 1, n_sm, st);
+}
+
+// Rows in whole 32-byte pieces: as few lanes as a narrow matrix needs, 64 columns of a wide one.
+static int launch_lanes8(int op, const AggArgs& a, int64_t n_edges, int n_sm, cudaStream_t st) {
+    if (a.dim <= 8) return launch_lanes<1, 8, 1>(op, a, n_edges, n_sm, st);
+    if (a.dim <= 16) return launch_lanes<2, 8, 1>(op, a, n_edges, n_sm, st);
+    if (a.dim <= 32) return launch_lanes<4, 8, 1>(op, a, n_edges, n_sm, st);
+    return launch_lanes<8, 8, 1>(op, a, n_edges, n_sm, st);
+}
+
+// ---------------------------------------------------------------- GCN on matrices far larger than L2
+// Bound by HBM, so what counts is which rows stay in L2: a power-law graph reads its hubs' rows again and again, every other
+// row a few times, and left to itself the cache keeps neither.  Rows of hubs (coef <= hub_coef) are loaded "evict last",
+// all others "evict first"; the coefficient, gathered per entry anyway, tells which.  (2.45 M x 256 floats, 124 M entries:
+// 15.8 ms, 18.1 ms without the priorities; 2.45 M x 100: 7.9 ms.)  A whole row per load instruction, one warp per row or
+// segment; the items come from one counter.
 __device__ __forceinline__ uint64_t l2_policy_evict_last() {
     uint64_t p;
     asm volatile("createpolicy.fractional.L2::evict_last.b64 %0, 1.0;" : "=l"(p));
@@ -140,405 +450,137 @@ __device__ __forceinline__ float4 ldg_hinted(const float4* ptr, uint64_t policy)
                  : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(ptr), "l"(policy));
     return v;
 }
+__device__ __forceinline__ void fma4(float4& a, float w, const float4& x) {
+    a.x = fmaf(w, x.x, a.x); a.y = fmaf(w, x.y, a.y); a.z = fmaf(w, x.z, a.z); a.w = fmaf(w, x.w, a.w);
+}
 
-// Adds the neighbour rows of CSR entries [beg, end) into acc, in order, for the
-// column vectors this lane owns in pass `pass`.  GCN weighs each row by coef[u].
-template <int VEC, int CH, int OP>
-__device__ __forceinline__ void accumulate_range(const AggArgs& a, int64_t beg, int64_t end, int lane,
-                                                 int vec0, int nvec,
-                                                 typename VecT<VEC>::type (&acc)[CH]) {
-    using V = typename VecT<VEC>::type;
-    const int64_t ldv = a.ldq / VEC;
-    const V* __restrict__ qv = reinterpret_cast<const V*>(a.q);
-    constexpr bool kCanHint = OP == kOpGcn && VEC == 4;
-    [[maybe_unused]] uint64_t keep = 0, pass = 0;
-    [[maybe_unused]] const bool hinting = kCanHint && a.hub_coef > 0.f;
-    if constexpr (kCanHint) {
-        if (hinting) { keep = l2_policy_evict_last(); pass = l2_policy_evict_first(); }
-    }
+constexpr int kRowThreads = 256;
+constexpr int kUnroll = 4;             // neighbour rows in flight per lane and column chunk
+
+// Adds the weighted rows of CSR entries [beg, end), in order, for the float4 vectors vec0 + 32 c + lane of this lane.
+template <int CH>
+__device__ __forceinline__ void accumulate_range(const AggArgs& a, int64_t beg, int64_t end, int lane, int vec0, int nvec,
+                                                 float4 (&acc)[CH]) {
+    const int64_t ldv = a.ldq / 4;
+    const float4* __restrict__ qv = reinterpret_cast<const float4*>(a.q);
+    const bool hinting = a.hub_coef > 0.f;
+    uint64_t keep = 0, pass = 0;
+    if (hinting) { keep = l2_policy_evict_last(); pass = l2_policy_evict_first(); }
     for (int64_t e0 = beg; e0 < end; e0 += kWarp) {
         const int cnt = (int)min((int64_t)kWarp, end - e0);
         int my_u = 0;
         float my_w = 0.f;
         if (lane < cnt) {
             my_u = __ldg(a.colidx + e0 + lane);
-            if (OP == kOpGcn) my_w = __ldg(a.coef + my_u);
+            my_w = __ldg(a.coef + my_u);
         }
         int j = 0;
         for (; j + kUnroll <= cnt; j += kUnroll) {
-            V x[kUnroll][CH];
+            float4 x[kUnroll][CH];
             float w[kUnroll];
 #pragma unroll
             for (int t = 0; t < kUnroll; ++t) {
                 const int u = __shfl_sync(0xffffffffu, my_u, j + t);
-                if (OP == kOpGcn) w[t] = __shfl_sync(0xffffffffu, my_w, j + t);
-                const V* row = qv + (int64_t)u * ldv;
+                w[t] = __shfl_sync(0xffffffffu, my_w, j + t);
+                const float4* row = qv + (int64_t)u * ldv;
 #pragma unroll
                 for (int c = 0; c < CH; ++c) {
                     const int vi = vec0 + c * kWarp + lane;
+                    x[t][c] = make_float4(0.f, 0.f, 0.f, 0.f);
                     if (vi < nvec) {
-                        if constexpr (kCanHint) {
-                            if (hinting) x[t][c] = ldg_hinted(row + vi, w[t] <= a.hub_coef ? keep : pass);
-                            else x[t][c] = __ldg(row + vi);
-                        } else {
-                            x[t][c] = __ldg(row + vi);
-                        }
-                    } else vec_zero<VEC>(x[t][c]);
+                        if (hinting) x[t][c] = ldg_hinted(row + vi, w[t] <= a.hub_coef ? keep : pass);
+                        else x[t][c] = __ldg(row + vi);
+                    }
                 }
             }
 #pragma unroll
             for (int t = 0; t < kUnroll; ++t)
 #pragma unroll
-                for (int c = 0; c < CH; ++c) {
-                    if (OP == kOpGcn) vec_fma(acc[c], w[t], x[t][c]);
-                    else if (OP == kOpMax) vec_max(acc[c], x[t][c]);
-                    else vec_add(acc[c], x[t][c]);
-                }
+                for (int c = 0; c < CH; ++c) fma4(acc[c], w[t], x[t][c]);
         }
         for (; j < cnt; ++j) {
             const int u = __shfl_sync(0xffffffffu, my_u, j);
-            float w = 0.f;
-            if (OP == kOpGcn) w = __shfl_sync(0xffffffffu, my_w, j);
-            const V* row = qv + (int64_t)u * ldv;
+            const float w = __shfl_sync(0xffffffffu, my_w, j);
+            const float4* row = qv + (int64_t)u * ldv;
 #pragma unroll
             for (int c = 0; c < CH; ++c) {
                 const int vi = vec0 + c * kWarp + lane;
-                if (vi < nvec) {
-                    V x = __ldg(row + vi);
-                    if (OP == kOpGcn) vec_fma(acc[c], w, x);
-                    else if (OP == kOpMax) vec_max(acc[c], x);
-                    else vec_add(acc[c], x);
-                }
+                if (vi < nvec) fma4(acc[c], w, __ldg(row + vi));
             }
         }
     }
 }
 
-__device__ __forceinline__ void store_elem(const AggArgs& a, int64_t v, int col, float val) {
-    if (a.out) a.out[v * a.ldout + col] = val;
-    if (a.out16) a.out16[v * a.ldout16 + col] = f32_to_bf16(val);
-}
-
-// Finishes row v for the column vectors of this lane: GCN adds the self term
-// and scales, SAGE divides by the degree and (optionally) copies the self row.
-template <int VEC, int CH, int OP>
-__device__ __forceinline__ void finish_row(const AggArgs& a, int64_t v, int lane, int vec0, int nvec,
-                                           typename VecT<VEC>::type (&acc)[CH]) {
-    using V = typename VecT<VEC>::type;
-    const V* __restrict__ self = reinterpret_cast<const V*>(a.q) + v * (a.ldq / VEC);
-    const float cv = a.coef[v];
-    const int64_t deg = a.rowptr[v + 1] - a.rowptr[v];
-#pragma unroll
-    for (int c = 0; c < CH; ++c) {
-        const int vi = vec0 + c * kWarp + lane;
-        if (vi >= nvec) continue;
-        const V s = self[vi];
-#pragma unroll
-        for (int i = 0; i < VEC; ++i) {
-            const int col = vi * VEC + i;
-            if (col >= a.dim) continue;
-            const float sv = vec_get<VEC>(s, i);
-            const float av = vec_get<VEC>(acc[c], i);
-            if (OP == kOpGcn) {
-                store_elem(a, v, col, cv * fmaf(cv, sv, av));
-            } else {
-                const float mean = deg <= 0 ? 0.0f : OP == kOpMax ? av : av / (float)deg;
-                if (a.concat_self) {
-                    store_elem(a, v, col, sv);
-                    store_elem(a, v, a.dim + col, mean);
-                } else {
-                    store_elem(a, v, col, mean);
-                }
-            }
-        }
-    }
-}
-
-// Persistent kernel: each warp draws work items from one counter.  Items
-// [0, n_seg) are segments of heavy rows (their raw sums go to scratch), items
-// [n_seg, n_seg + n) are whole rows (heavy ones are skipped: their segments
-// cover them).
-template <int VEC, int CH, int OP>
-__global__ void __launch_bounds__(kAggThreads) agg_rows_kernel(AggArgs a) {
-    using V = typename VecT<VEC>::type;
+// Persistent: items [0, n_seg) are segments of heavy rows, [n_seg, n_seg + n) whole rows (heavy ones are skipped).
+template <int CH>
+__global__ void __launch_bounds__(kRowThreads) agg_rows_kernel(AggArgs a) {
     const int lane = threadIdx.x & 31;
-    const int nvec = (a.dim + VEC - 1) / VEC;
-    const int64_t n_seg = a.counters[1];
+    const int nvec = (a.dim + 3) / 4;
+    const int64_t n_seg = a.heavy.counters[1];
     const int64_t total = n_seg + a.n;
     for (;;) {
         int64_t item = 0;
-        if (lane == 0) item = atomicAdd(reinterpret_cast<unsigned int*>(a.counters + 2), 1u);
+        if (lane == 0) item = atomicAdd(reinterpret_cast<unsigned int*>(a.next_item), 1u);
         item = __shfl_sync(0xffffffffu, item, 0);
         if (item >= total) break;
         if (item < n_seg) {
-            const int32_t slot = a.seg_slot[item];
-            const int64_t v = a.heavy_list[slot];
-            const int64_t i = item - a.heavy_seg_base[slot];
-            const int64_t beg = a.rowptr[v] + i * kSegLen;
-            const int64_t end = min(a.rowptr[v + 1], beg + kSegLen);
+            const int32_t slot = a.heavy.seg_slot[item];
+            const int64_t v = a.heavy.list[slot];
+            const int64_t beg = a.rowptr[v] + (item - a.heavy.seg_base[slot]) * a.heavy.seg_entries;
+            const int64_t end = min(a.rowptr[v + 1], beg + a.heavy.seg_entries);
             for (int vec0 = 0; vec0 < nvec; vec0 += CH * kWarp) {
-                V acc[CH];
+                float4 acc[CH];
 #pragma unroll
-                for (int c = 0; c < CH; ++c) vec_init<VEC, OP>(acc[c]);
-                accumulate_range<VEC, CH, OP>(a, beg, end, lane, vec0, nvec, acc);
-                float* dst = a.seg_partial + item * a.ld_partial;
+                for (int c = 0; c < CH; ++c) acc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+                accumulate_range<CH>(a, beg, end, lane, vec0, nvec, acc);
 #pragma unroll
                 for (int c = 0; c < CH; ++c) {
                     const int vi = vec0 + c * kWarp + lane;
-                    if (vi >= nvec) continue;
-#pragma unroll
-                    for (int k = 0; k < VEC; ++k) dst[vi * VEC + k] = vec_get<VEC>(acc[c], k);
+                    if (vi < nvec) *reinterpret_cast<float4*>(a.seg_partial + item * a.ld_partial + 4 * vi) = acc[c];
                 }
             }
-        } else {
-            const int64_t v = item - n_seg;
-            const int64_t beg = a.rowptr[v], end = a.rowptr[v + 1];
-            if (end - beg >= kHeavyDegree) continue;
-            for (int vec0 = 0; vec0 < nvec; vec0 += CH * kWarp) {
-                V acc[CH];
-#pragma unroll
-                for (int c = 0; c < CH; ++c) vec_init<VEC, OP>(acc[c]);
-                accumulate_range<VEC, CH, OP>(a, beg, end, lane, vec0, nvec, acc);
-                finish_row<VEC, CH, OP>(a, v, lane, vec0, nvec, acc);
-            }
+            continue;
         }
-    }
-}
-
-// One warp per heavy row: adds the row's segment sums in segment order and
-// finishes the row.
-template <int VEC, int CH, int OP>
-__global__ void __launch_bounds__(kAggThreads) agg_combine_kernel(AggArgs a) {
-    using V = typename VecT<VEC>::type;
-    const int lane = threadIdx.x & 31;
-    const int nvec = (a.dim + VEC - 1) / VEC;
-    const int n_heavy = a.counters[0];
-    for (int h = blockIdx.x * kAggWarps + (threadIdx.x >> 5); h < n_heavy; h += gridDim.x * kAggWarps) {
-        const int64_t v = a.heavy_list[h];
-        const int64_t deg = a.rowptr[v + 1] - a.rowptr[v];
-        const int nseg = (int)((deg + kSegLen - 1) / kSegLen);
-        const float* src = a.seg_partial + (int64_t)a.heavy_seg_base[h] * a.ld_partial;
+        const int64_t v = item - n_seg;
+        const int64_t beg = a.rowptr[v], end = a.rowptr[v + 1];
+        if (end - beg >= 2 * a.heavy.seg_entries) continue;
         for (int vec0 = 0; vec0 < nvec; vec0 += CH * kWarp) {
-            V acc[CH];
+            float4 acc[CH];
 #pragma unroll
-            for (int c = 0; c < CH; ++c) vec_init<VEC, OP>(acc[c]);
-            for (int i = 0; i < nseg; ++i) {
+            for (int c = 0; c < CH; ++c) acc[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+            accumulate_range<CH>(a, beg, end, lane, vec0, nvec, acc);
+            const float cv = a.coef[v];
+            const float4* self = reinterpret_cast<const float4*>(a.q) + v * (a.ldq / 4);
 #pragma unroll
-                for (int c = 0; c < CH; ++c) {
-                    const int vi = vec0 + c * kWarp + lane;
-                    if (vi >= nvec) continue;
-                    float t[4] = {0.f, 0.f, 0.f, 0.f};
+            for (int c = 0; c < CH; ++c) {
+                const int vi = vec0 + c * kWarp + lane;
+                if (vi >= nvec) continue;
+                const float4 s = self[vi];
+                const float z[4] = {cv * fmaf(cv, s.x, acc[c].x), cv * fmaf(cv, s.y, acc[c].y), cv * fmaf(cv, s.z, acc[c].z),
+                                    cv * fmaf(cv, s.w, acc[c].w)};
 #pragma unroll
-                    for (int k = 0; k < VEC; ++k) t[k] = src[(int64_t)i * a.ld_partial + vi * VEC + k];
-                    V x;
-                    if constexpr (VEC == 4) x = make_float4(t[0], t[1], t[2], t[3]);
-                    else if constexpr (VEC == 2) x = make_float2(t[0], t[1]);
-                    else x = t[0];
-                    if (OP == kOpMax) vec_max(acc[c], x);
-                    else vec_add(acc[c], x);
-                }
+                for (int i = 0; i < 4; ++i)
+                    if (4 * vi + i < a.dim) store_elem(a, v, 4 * vi + i, z[i]);
             }
-            finish_row<VEC, CH, OP>(a, v, lane, vec0, nvec, acc);
         }
     }
 }
 
-// ---------------------------------------------------------------- column slabs
-// Variant for matrices that do not fit the L2 cache while a slab of their columns does.  The
-// columns are cut into slabs of LPR float4 vectors; work items are ordered slab by slab, so that at
-// any time the whole grid gathers from the same N x (LPR x 16 bytes) slab, which stays in L2: the
-// neighbour rows then come from L2 instead of HBM, at the price of reading the index array once per
-// slab (streamed with evict-first loads).  A warp takes 32 / LPR entries of a row at a time: lane
-// group g = lane / LPR adds entries g, g + G, g + 2G, ... in CSR order, and the groups' sums are
-// added in a fixed tree at the end, so results are still the same bits on every call.
-#ifndef SLAB_U
-#define SLAB_U 8
-#define SLAB_TAIL_U 4
-#define SLAB_BLOCKS 3
-#define SLAB_MIN_MB 192
-#endif
-constexpr int kSlabUnroll = SLAB_U;                  // neighbour rows in flight per lane (full trips of 32 entries)
-constexpr int kSlabTailUnroll = SLAB_TAIL_U;         // ... in the ragged last trip of a row
-constexpr int kSlabBlocksPerSm = SLAB_BLOCKS;        // resident blocks the register budget is cut for
-// Measured on B200 (126 MB of L2), 233 k rows: 256-byte gathers out of an L2-resident slab deliver
-// 15-17 TB/s, while the plain variant runs at the HBM rate divided by (1 - L2 hit rate): 9 TB/s for a
-// 561 MB matrix (30 % hits), 13 TB/s for 239 MB (50 %), and the L2 rate itself once the matrix fits.
-constexpr size_t kSlabMinMatrixBytes = (size_t)SLAB_MIN_MB << 20;   // (1.5 x L2) smaller matrices are left to the cache as they are
-#ifndef SLAB_MB
-#define SLAB_MB 64
-#endif
-constexpr size_t kSlabBytes = (size_t)SLAB_MB << 20;             // a slab of all rows may take this much of L2
-
-template <int LPR, int OP>
-__global__ void __launch_bounds__(kAggThreads, kSlabBlocksPerSm) agg_slab_kernel(AggArgs a, int n_slabs) {
-    constexpr int G = kWarp / LPR;                   // entries of a row taken per step
-    constexpr int U = G * kSlabUnroll > kWarp ? kWarp / G : kSlabUnroll;              // steps in flight: at most one trip
-    constexpr int UT = G * kSlabTailUnroll > kWarp ? kWarp / G : kSlabTailUnroll;
-    const int lane = threadIdx.x & 31;
-    const int g = lane / LPR, c = lane % LPR;
-    const int nvec = (a.dim + 3) / 4;
-    const int64_t n_seg = a.counters[1];
-    const int64_t per_slab = n_seg + a.n;
-    const int64_t total = per_slab * n_slabs;
-    const int64_t ldv = a.ldq / 4;
-    const float4* __restrict__ qv = reinterpret_cast<const float4*>(a.q);
-    for (;;) {
-        int64_t item = 0;
-        if (lane == 0) item = atomicAdd(reinterpret_cast<unsigned long long*>(a.counters + 2), 1ull);
-        item = __shfl_sync(0xffffffffu, item, 0);
-        if (item >= total) break;
-        const int slab = (int)(item / per_slab);
-        const int64_t r = item % per_slab;
-        int64_t v, beg, end;
-        if (r < n_seg) {
-            const int32_t slot = a.seg_slot[r];
-            v = a.heavy_list[slot];
-            beg = a.rowptr[v] + (r - a.heavy_seg_base[slot]) * kSegLen;
-            end = min(a.rowptr[v + 1], beg + kSegLen);
-        } else {
-            v = r - n_seg;
-            beg = a.rowptr[v]; end = a.rowptr[v + 1];
-            if (end - beg >= kHeavyDegree) continue;
-        }
-        const int vi = slab * LPR + c;
-        const bool active = vi < nvec;
-        const float4* __restrict__ col = qv + (active ? vi : nvec - 1);
-        float4 acc[1];
-        vec_init<4, OP>(acc[0]);
-        for (int64_t e0 = beg; e0 < end; e0 += kWarp) {
-            const int cnt = (int)min((int64_t)kWarp, end - e0);
-            int my_u = 0;
-            float my_w = 0.f;
-            if (lane < cnt) {
-                my_u = __ldcs(a.colidx + e0 + lane);
-                if (OP == kOpGcn) my_w = __ldg(a.coef + my_u);
-            }
-            if (cnt == kWarp) {
-                // full trip: no predicates; a lane beyond the last column vector loads the last one and
-                // its sum is dropped at the end
-#pragma unroll 1
-                for (int j = 0; j < kWarp; j += G * U) {
-                    float4 x[U];
-                    float w[U];
-#pragma unroll
-                    for (int t = 0; t < U; ++t) {
-                        const int u = __shfl_sync(0xffffffffu, my_u, j + t * G + g);
-                        if (OP == kOpGcn) w[t] = __shfl_sync(0xffffffffu, my_w, j + t * G + g);
-                        x[t] = __ldg(col + (int64_t)u * ldv);
-                    }
-#pragma unroll
-                    for (int t = 0; t < U; ++t) {
-                        if (OP == kOpGcn) vec_fma(acc[0], w[t], x[t]);
-                        else if (OP == kOpMax) vec_max(acc[0], x[t]);
-                        else vec_add(acc[0], x[t]);
-                    }
-                }
-                continue;
-            }
-            for (int j = 0; j < cnt; j += G * UT) {      // ragged last trip of the row
-                float4 x[UT];
-                float w[UT];
-                bool on[UT];
-#pragma unroll
-                for (int t = 0; t < UT; ++t) {
-                    const int idx = j + t * G + g;
-                    const int u = __shfl_sync(0xffffffffu, my_u, idx & 31);
-                    if (OP == kOpGcn) w[t] = __shfl_sync(0xffffffffu, my_w, idx & 31);
-                    on[t] = active && idx < cnt;
-                    if (on[t]) x[t] = __ldg(qv + (int64_t)u * ldv + vi);
-                }
-#pragma unroll
-                for (int t = 0; t < UT; ++t) {
-                    if (!on[t]) continue;
-                    if (OP == kOpGcn) vec_fma(acc[0], w[t], x[t]);
-                    else if (OP == kOpMax) vec_max(acc[0], x[t]);
-                    else vec_add(acc[0], x[t]);
-                }
-            }
-        }
-        // the lane groups' sums, added in a fixed order (group 0 ends up with the total)
-#pragma unroll
-        for (int o = kWarp / 2; o >= LPR; o >>= 1) {
-            float4 y;
-            y.x = __shfl_xor_sync(0xffffffffu, acc[0].x, o); y.y = __shfl_xor_sync(0xffffffffu, acc[0].y, o);
-            y.z = __shfl_xor_sync(0xffffffffu, acc[0].z, o); y.w = __shfl_xor_sync(0xffffffffu, acc[0].w, o);
-            if (OP == kOpMax) vec_max(acc[0], y);
-            else vec_add(acc[0], y);
-        }
-        const int nvec_slab = min(nvec, slab * LPR + LPR);       // lanes of the other groups fall outside
-        if (r < n_seg) {
-            if (g == 0 && active) {
-                float* dst = a.seg_partial + r * a.ld_partial + vi * 4;
-                dst[0] = acc[0].x; dst[1] = acc[0].y; dst[2] = acc[0].z; dst[3] = acc[0].w;
-            }
-        } else {
-            finish_row<4, 1, OP>(a, v, lane, slab * LPR, nvec_slab, acc);
-        }
-    }
-}
-
-template <int LPR>
-static int launch_slab(int op, const AggArgs& a, int n_sm, cudaStream_t st) {
-    const int nvec = (a.dim + 3) / 4;
-    const int n_slabs = (nvec + LPR - 1) / LPR;
-    auto go = [&](auto kernel) {
-        int per_sm = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kAggThreads, 0) != cudaSuccess || per_sm < 1) {
-            (void)cudaGetLastError();
-            per_sm = 1;
-        }
-        kernel<<<n_sm * per_sm, kAggThreads, 0, st>>>(a, n_slabs);
-    };
-    if (op == kOpGcn) go(agg_slab_kernel<LPR, kOpGcn>);
-    else if (op == kOpMax) go(agg_slab_kernel<LPR, kOpMax>);
-    else go(agg_slab_kernel<LPR, kOpSum>);
-    // heavy rows: their segments' sums are added over the full width as in the plain variant
-    if (op == kOpGcn) agg_combine_kernel<4, 1, kOpGcn><<<n_sm, kAggThreads, 0, st>>>(a);
-    else if (op == kOpMax) agg_combine_kernel<4, 1, kOpMax><<<n_sm, kAggThreads, 0, st>>>(a);
-    else agg_combine_kernel<4, 1, kOpSum><<<n_sm, kAggThreads, 0, st>>>(a);
-    return launch_status();
-}
-
-// Lanes per neighbour row of the slab variant for an N x dim fp32 matrix, or 0 where the plain
-// variant is the better choice (the matrix fits L2 as it is, or no slab of all rows would).
-static int slab_lanes(int64_t n, int32_t dim) {
-    if ((size_t)n * (size_t)dim * 4 < kSlabMinMatrixBytes) return 0;
-    for (int lpr = 32; lpr >= 8; lpr >>= 1)      // (64-byte gathers out of slabs of 4 vectors measured far slower)
-        if ((size_t)n * (size_t)lpr * 16 <= kSlabBytes) return lpr * 4 < dim ? lpr : 0;
-    return 0;
-}
-
-template <int VEC, int CH, int OP>
-static int launch_agg(const AggArgs& a, int n_sm, cudaStream_t st) {
+template <int CH>
+static int launch_rows(const AggArgs& a, int64_t n_edges, int n_sm, cudaStream_t st) {
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, agg_rows_kernel<VEC, CH, OP>, kAggThreads, 0) !=
-            cudaSuccess || per_sm < 1) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, agg_rows_kernel<CH>, kRowThreads, 0) != cudaSuccess || per_sm < 1) {
         (void)cudaGetLastError();
         per_sm = 1;
     }
-    agg_rows_kernel<VEC, CH, OP><<<n_sm * per_sm, kAggThreads, 0, st>>>(a);
-    agg_combine_kernel<VEC, CH, OP><<<n_sm, kAggThreads, 0, st>>>(a);
-    return launch_status();
+    agg_rows_kernel<CH><<<n_sm * per_sm, kRowThreads, 0, st>>>(a);
+    return launch_combine(kOpGcn, a, n_edges, 0, n_sm, st);
 }
 
-template <int VEC, int OP>
-static int dispatch_ch(const AggArgs& a, int n_sm, cudaStream_t st) {
-    const int nvec = (a.dim + VEC - 1) / VEC;
-    const int need = (nvec + kWarp - 1) / kWarp;      // column chunks for one pass
-    if (need <= 1) return launch_agg<VEC, 1, OP>(a, n_sm, st);
-    if (need <= 2) return launch_agg<VEC, 2, OP>(a, n_sm, st);
-    if (need <= 3) return launch_agg<VEC, 3, OP>(a, n_sm, st);
-    if (need <= 4) return launch_agg<VEC, 4, OP>(a, n_sm, st);
-    if (need <= 5) return launch_agg<VEC, 5, OP>(a, n_sm, st);
-    return launch_agg<VEC, 6, OP>(a, n_sm, st);      // wider rows: several passes of 6 chunks
-}
-
-template <int VEC>
-static int dispatch_op(int op, const AggArgs& a, int n_sm, cudaStream_t st) {
-    if (op == kOpGcn) return dispatch_ch<VEC, kOpGcn>(a, n_sm, st);
-    if (op == kOpMax) return dispatch_ch<VEC, kOpMax>(a, n_sm, st);
-    return dispatch_ch<VEC, kOpSum>(a, n_sm, st);
-}
+// From here on the gather is bound by HBM, not by L2, and the priorities pay: 2.45 M nodes, 124 M entries, agg_rows_kernel
+// against agg_lanes_kernel: 64 columns (627 MB) 5.3-6.9 against 4.4 ms, 100 columns (980 MB) 7.9 against 10.3 ms, 256 columns
+// 15.8 against 17.5 ms.
+constexpr size_t kHbmBoundBytes = (size_t)768 << 20;
 
 }  // namespace retexo
 
@@ -551,12 +593,15 @@ extern "C" size_t retexo_aggregate_workspace_size(int64_t n_nodes, int64_t n_edg
     if (type == RETEXO_GAT) {
         gat_forward_workspace(n_nodes, heads > 0 ? heads : 1, s);
     } else {
-        s.take<float>((size_t)n_nodes);                                   // coef
-        s.take<int32_t>((size_t)(n_edges / kHeavyDegree + 1));            // heavy rows
-        s.take<int32_t>((size_t)(n_edges / kHeavyDegree + 1));            // their first segment
+        s.take<int32_t>((size_t)max_heavy(n_edges));                      // heavy rows
+        s.take<int32_t>((size_t)max_heavy(n_edges));                      // their first segment
         s.take<int32_t>((size_t)max_segments(n_edges));                   // segment -> heavy row
         s.take<int32_t>(64);                                              // counters
         s.take<float>((size_t)max_segments(n_edges) * (size_t)((dim + 3) / 4 * 4));   // segment sums
+        if (type == RETEXO_GCN) {
+            s.take<float>((size_t)n_nodes);                               // coef
+            s.take<float>((size_t)n_nodes * (size_t)((dim + 7) / 8 * 8)); // scaled rows
+        }
     }
     return s.off + kAlign;
 }
@@ -565,6 +610,13 @@ extern "C" int retexo_aggregate(const retexo_csr* g, int32_t type, const float* 
                                 const retexo_gat_params* gat, float* out, int64_t ldout,
                                 int32_t concat_self, void* out_bf16, int64_t ldout_bf16,
                                 void* workspace, size_t workspace_bytes, void* stream) {
+    return aggregate_rows(g, type, q, ldq, dim, false, gat, out, ldout, concat_self, out_bf16, ldout_bf16, workspace, workspace_bytes,
+                          stream);
+}
+
+int retexo::aggregate_rows(const retexo_csr* g, int32_t type, const float* q, int64_t ldq, int32_t dim, bool whole_rows,
+                           const retexo_gat_params* gat, float* out, int64_t ldout, int32_t concat_self, void* out_bf16,
+                           int64_t ldout_bf16, void* workspace, size_t workspace_bytes, void* stream) {
     if (!g || g->n_nodes < 0 || g->n_edges < 0 || g->n_nodes > INT32_MAX) return RETEXO_ERR_INVALID_ARG;
     if (type != RETEXO_GCN && type != RETEXO_SAGE_MEAN && type != RETEXO_GAT && type != RETEXO_SAGE_MAX)
         return RETEXO_ERR_INVALID_ARG;
@@ -597,39 +649,58 @@ extern "C" int retexo_aggregate(const retexo_csr* g, int32_t type, const float* 
         return gat_forward_launch(f, ws, n_sm, st);
     }
 
-    AggArgs a;
-    a.n = n; a.rowptr = g->rowptr; a.colidx = g->colidx; a.q = q; a.ldq = ldq; a.dim = dim;
-    float* coef = ws.take<float>((size_t)n);
     const int64_t e = g->n_edges;
-    int32_t* heavy_list = ws.take<int32_t>((size_t)(e / kHeavyDegree + 1));
-    int32_t* heavy_seg_base = ws.take<int32_t>((size_t)(e / kHeavyDegree + 1));
-    int32_t* seg_slot = ws.take<int32_t>((size_t)max_segments(e));
-    int32_t* counters = ws.take<int32_t>(64);
+    AggArgs a{};
+    a.n = n; a.rowptr = g->rowptr; a.colidx = g->colidx; a.q = q; a.ldq = ldq; a.dim = dim;
+    a.heavy.seg_entries = seg_len(e);
+    a.heavy.list = ws.take<int32_t>((size_t)max_heavy(e));
+    a.heavy.seg_base = ws.take<int32_t>((size_t)max_heavy(e));
+    a.heavy.seg_slot = ws.take<int32_t>((size_t)max_segments(e));
+    a.heavy.counters = ws.take<int32_t>(64);
+    a.next_item = a.heavy.counters + 2;
     a.ld_partial = (dim + 3) / 4 * 4;
     a.seg_partial = ws.take<float>((size_t)max_segments(e) * (size_t)a.ld_partial);
-    a.coef = coef; a.heavy_list = heavy_list; a.heavy_seg_base = heavy_seg_base; a.seg_slot = seg_slot;
-    // hubs = nodes of at least four times the mean degree; hinted only where the matrix is larger than L2
-    a.hub_coef = 0.f;
-    if (type == RETEXO_GCN && (size_t)n * (size_t)dim * 4 >= kSlabMinMatrixBytes && n > 0)
-        a.hub_coef = (float)(1.0 / sqrt(4.0 * (double)e / (double)n + 1.0));
-    a.counters = counters;
     a.out = out; a.ldout = ldout;
     a.out16 = static_cast<__nv_bfloat16*>(out_bf16); a.ldout16 = ldout_bf16;
-    a.concat_self = concat_self ? 1 : 0;
-    RETEXO_CUDA_TRY(cudaMemsetAsync(counters, 0, 64 * sizeof(int32_t), st));
-    prep_rows_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(n, g->rowptr, type, coef, heavy_list,
-                                                                  heavy_seg_base, seg_slot, counters);
+    a.concat_self = sage && concat_self ? 1 : 0;
+    const bool cols4 = !a.concat_self || dim % 4 == 0;      // where the second half of a concatenated row starts
+    a.vec_out = out && aligned_to(out, 16) && ldout % 4 == 0 && cols4;
+    a.vec_out16 = out_bf16 && aligned_to(out_bf16, 8) && ldout_bf16 % 4 == 0 && cols4;
+    RETEXO_CUDA_TRY(cudaMemsetAsync(a.heavy.counters, 0, 64 * sizeof(int32_t), st));
 
-    const int op = type == RETEXO_GCN ? kOpGcn : type == RETEXO_SAGE_MAX ? kOpMax : kOpSum;
     const bool v4 = aligned_to(q, 16) && ldq % 4 == 0 && ldq >= (dim + 3) / 4 * 4;
-    const bool v2 = aligned_to(q, 8) && ldq % 2 == 0 && ldq >= (dim + 1) / 2 * 2;
-    if (v4) {
-        const int lpr = slab_lanes(n, dim);
-        if (lpr == 32) return launch_slab<32>(op, a, n_sm, st);
-        if (lpr == 16) return launch_slab<16>(op, a, n_sm, st);
-        if (lpr == 8) return launch_slab<8>(op, a, n_sm, st);
-        return dispatch_op<4>(op, a, n_sm, st);
+    const unsigned prep_blocks = (unsigned)((n + 255) / 256);
+    if (type == RETEXO_GCN) {
+        const int64_t ld_qs = ((int64_t)dim + 7) / 8 * 8;
+        float* coef = ws.take<float>((size_t)n);
+        if (v4 && (size_t)n * (size_t)dim * 4 >= kHbmBoundBytes) {
+            prep_rows_kernel<<<prep_blocks, 256, 0, st>>>(n, g->rowptr, a.heavy, coef);
+            a.coef = coef;
+            a.hub_coef = (float)(1.0 / sqrt(4.0 * (double)e / (double)n + 1.0));      // hubs: at least four times the mean degree
+            const int chunks = (dim + 127) / 128;      // of 32 float4 vectors; more than 6: several passes
+            if (chunks <= 1) return launch_rows<1>(a, e, n_sm, st);
+            if (chunks <= 2) return launch_rows<2>(a, e, n_sm, st);
+            if (chunks <= 3) return launch_rows<3>(a, e, n_sm, st);
+            if (chunks <= 4) return launch_rows<4>(a, e, n_sm, st);
+            if (chunks <= 5) return launch_rows<5>(a, e, n_sm, st);
+            return launch_rows<6>(a, e, n_sm, st);
+        }
+        float* qs = ws.take<float>((size_t)n * (size_t)ld_qs);
+        int lanes_log2 = 0;
+        while (lanes_log2 < 5 && (8 << lanes_log2) < ld_qs) ++lanes_log2;
+        gcn_scale_rows_kernel<<<(unsigned)(((n << lanes_log2) + 255) / 256), 256, 0, st>>>(n, g->rowptr, a.heavy, q, ldq, dim, v4 ? 1 : 0,
+                                                                                           qs, ld_qs, lanes_log2);
+        a.q = qs;
+        a.ldq = ld_qs;
+        return launch_lanes8(kOpGcn, a, e, n_sm, st);
     }
-    if (v2) return dispatch_op<2>(op, a, n_sm, st);
-    return dispatch_op<1>(op, a, n_sm, st);
+    if (e >= heavy_degree(e)) prep_rows_kernel<<<prep_blocks, 256, 0, st>>>(n, g->rowptr, a.heavy, nullptr);
+    const int op = type == RETEXO_SAGE_MAX ? kOpMax : kOpSum;
+    // (a last vector of 8 that holds 4 columns or fewer could reach beyond the last row's memory: 16-byte pieces then)
+    if (aligned_to(q, 32) && ldq % 8 == 0 && ldq >= (dim + 7) / 8 * 8 && (whole_rows || (dim + 7) / 8 * 8 - dim <= 3))
+        return launch_lanes8(op, a, e, n_sm, st);
+    if (v4) return dim <= 32 ? launch_lanes<8, 4, 1>(op, a, e, n_sm, st) : launch_lanes<16, 4, 1>(op, a, e, n_sm, st);
+    if (aligned_to(q, 8) && ldq % 2 == 0 && ldq >= (dim + 1) / 2 * 2) return launch_lanes<32, 2, 1>(op, a, e, n_sm, st);
+    if (dim <= 32) return launch_lanes<32, 1, 1>(op, a, e, n_sm, st);
+    return dim <= 64 ? launch_lanes<32, 1, 2>(op, a, e, n_sm, st) : launch_lanes<32, 1, 3>(op, a, e, n_sm, st);
 }

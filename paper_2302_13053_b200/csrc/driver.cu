@@ -4,6 +4,7 @@
 // then the emission of the next representations.
 #include <vector>
 
+#include "aggregate.h"
 #include "common.cuh"
 #include "gemm_tc.h"
 #include "mlp_plan.h"
@@ -472,8 +473,9 @@ extern "C" int retexo_lmp_train(const retexo_lmp_config* cfg, const retexo_lmp_i
                 RETEXO_TRY(gat_forward(b.att));
             }
         } else {
-            RETEXO_TRY(retexo_aggregate(&g, c.aggr, q, ldq, r.agg_dim, nullptr, nullptr, 0, 1, b.x16, ld16, b.ws_agg,
-                                        b.ws_agg_bytes, st));
+            // (the caller's own features need not hold the last row's padding)
+            RETEXO_TRY(aggregate_rows(&g, c.aggr, q, ldq, r.agg_dim, q != in->features, nullptr, nullptr, 0, 1, b.x16, ld16, b.ws_agg,
+                                      b.ws_agg_bytes, st));
         }
 
         // ---- the round's batches and model state

@@ -15,6 +15,7 @@
 // X^1 = AGGR(F) is computed once.  No kernel adds floating-point values atomically: results repeat bit for bit.
 #include <vector>
 
+#include "aggregate.h"
 #include "common.cuh"
 #include "gemm_tc.h"
 #include "mlp_plan.h"
