@@ -39,38 +39,68 @@ static __global__ void std_ones_column_kernel(bf16* __restrict__ x, int64_t ld, 
     const int64_t i = blockIdx.x * 256ll + threadIdx.x;
     if (i < n) x[i * ld + col] = f32_to_bf16(1.f);
 }
-// g[idx[i]][0 .. dim) = dx[i][0 .. dim): the batch-ordered input gradient goes to node order (g cleared before).
-static __global__ void std_scatter_rows_kernel(const float* __restrict__ dx, int64_t ld_dx, const int32_t* __restrict__ idx,
-                                               int64_t n_rows, int32_t dim, float* __restrict__ g, int64_t ld_g) {
-    const int64_t t = blockIdx.x * 256ll + threadIdx.x;
-    const int64_t i = t / dim;
-    const int32_t c = (int32_t)(t % dim);
-    if (i < n_rows) g[(int64_t)idx[i] * ld_g + c] = dx[i * ld_dx + c];
+// The row kernels below give a row to a warp and 32 neighbouring columns to its lanes, eight loads in flight per lane; they are
+// streams (58 k rows of 256 floats: 60 MB a matrix).  One thread per element, which found its row by a 64-bit division, took
+// 65 to 76 us each.
+constexpr int kStdRowWarps = 8;
+__device__ __forceinline__ int64_t std_row() { return blockIdx.x * (int64_t)kStdRowWarps + (threadIdx.x >> 5); }
+static unsigned std_row_blocks(int64_t n) { return (unsigned)((n + kStdRowWarps - 1) / kStdRowWarps); }
+
+// dst[i] = [src[i][0 .. dim) | zeros]: features whose rows do not start on 16-byte boundaries, laid out for wide loads.
+static __global__ void __launch_bounds__(32 * kStdRowWarps) std_relay_kernel(const float* __restrict__ src, int64_t ld_src, int32_t dim, int64_t n,
+                                                                             float* __restrict__ dst, int64_t ld_dst) {
+    const int64_t v = std_row();
+    if (v >= n) return;
+#pragma unroll 8
+    for (int c = threadIdx.x & 31; c < ld_dst; c += 32) dst[v * ld_dst + c] = c < dim ? __ldcs(src + v * ld_src + c) : 0.f;
+}
+// The batch-ordered gradient dx[i][0 .. dim) goes to node order (the destinations are cleared before).  GCN (s == nullptr): all of
+// it to g.  SAGE: the self half to g, the mean half, divided by the degree for the transposed mean, to s.
+static __global__ void __launch_bounds__(32 * kStdRowWarps) std_scatter_rows_kernel(const float* __restrict__ dx, int64_t ld_dx,
+                                                                                    const int32_t* __restrict__ idx, int64_t n_rows, int32_t dim,
+                                                                                    const int64_t* __restrict__ rowptr, float* __restrict__ g,
+                                                                                    int64_t ld_g, float* __restrict__ s, int64_t ld_s) {
+    const int64_t i = std_row();
+    if (i >= n_rows) return;
+    const int64_t v = idx[i];
+    const int32_t self = s ? dim / 2 : dim;
+    const float* src = dx + i * ld_dx;
+#pragma unroll 8
+    for (int c = threadIdx.x & 31; c < self; c += 32) g[v * ld_g + c] = __ldcs(src + c);
+    if (!s) return;
+    const int64_t deg = rowptr[v + 1] - rowptr[v];
+#pragma unroll 8
+    for (int c = threadIdx.x & 31; c < self; c += 32) s[v * ld_s + c] = deg > 0 ? __ldcs(src + self + c) / (float)deg : 0.f;
 }
 // s[v][j] = g[v][off + j] / deg v (0 where deg v = 0): the mean half of a SAGE gradient, scaled for the transposed mean.
-static __global__ void std_prescale_kernel(const float* __restrict__ g, int64_t ld_g, int32_t off, int32_t dim,
-                                           const int64_t* __restrict__ rowptr, int64_t n, float* __restrict__ s, int64_t ld_s) {
-    const int64_t t = blockIdx.x * 256ll + threadIdx.x;
-    const int64_t v = t / dim;
-    const int32_t j = (int32_t)(t % dim);
+static __global__ void __launch_bounds__(32 * kStdRowWarps) std_prescale_kernel(const float* __restrict__ g, int64_t ld_g, int32_t off, int32_t dim,
+                                                                                const int64_t* __restrict__ rowptr, int64_t n,
+                                                                                float* __restrict__ s, int64_t ld_s) {
+    const int64_t v = std_row();
     if (v >= n) return;
     const int64_t deg = rowptr[v + 1] - rowptr[v];
-    s[v * ld_s + j] = deg > 0 ? g[v * ld_g + off + j] / (float)deg : 0.f;
+#pragma unroll 8
+    for (int j = threadIdx.x & 31; j < dim; j += 32) s[v * ld_s + j] = deg > 0 ? __ldcs(g + v * ld_g + off + j) / (float)deg : 0.f;
 }
 // dz[v][j] = bf16(dH[v][j]) where unit j of row v passed the ReLU, else 0, with
 //   dH = a[v][j]                         (self == nullptr: GCN, a = AGGR(G))
 //   dH = self[v][j] + deg v * a[v][j]    (SAGE: a = mean over N(v) of the scaled gradient rows)
-static __global__ void std_gate_kernel(const float* __restrict__ a, int64_t ld_a, const float* __restrict__ self, int64_t ld_self,
-                                       const int64_t* __restrict__ rowptr, const uint32_t* __restrict__ bits, int64_t ld_bits,
-                                       int64_t n, int32_t dim, bf16* __restrict__ dz, int64_t ld_dz) {
-    const int64_t t = blockIdx.x * 256ll + threadIdx.x;
-    const int64_t v = t / dim;
-    const int32_t j = (int32_t)(t % dim);
+static __global__ void __launch_bounds__(32 * kStdRowWarps) std_gate_kernel(const float* __restrict__ a, int64_t ld_a, const float* __restrict__ self,
+                                                                            int64_t ld_self, const int64_t* __restrict__ rowptr,
+                                                                            const uint32_t* __restrict__ bits, int64_t ld_bits, int64_t n,
+                                                                            int32_t dim, bf16* __restrict__ dz, int64_t ld_dz) {
+    const int64_t v = std_row();
     if (v >= n) return;
-    float d = a[v * ld_a + j];
-    if (self) d = self[v * ld_self + j] + (float)(rowptr[v + 1] - rowptr[v]) * d;
-    const bool open = (bits[v * ld_bits + (j >> 5)] >> (j & 31)) & 1u;
-    dz[v * ld_dz + j] = f32_to_bf16(open ? d : 0.f);
+    const int lane = threadIdx.x & 31;
+    const float deg = (float)(rowptr[v + 1] - rowptr[v]);
+#pragma unroll 8
+    for (int k = 0; 32 * k < dim; ++k) {
+        const int j = 32 * k + lane;
+        if (j >= dim) break;
+        float d = __ldcs(a + v * ld_a + j);
+        if (self) d = __ldcs(self + v * ld_self + j) + deg * d;
+        dz[v * ld_dz + j] = f32_to_bf16((__ldg(bits + v * ld_bits + k) >> lane) & 1u ? d : 0.f);
+    }
 }
 static __global__ void std_copy_if_kernel(const int32_t* decision, const float* src, float* dst, int64_t n) {
     if (!*decision) return;
@@ -110,6 +140,7 @@ struct StdLayer {
 
 struct StdBuffers {
     StdLayer L[kStdMaxLayers];
+    float* feat; int64_t ld_feat;   // features in rows of whole 128-byte lines (copied only if the caller's rows are not 16-byte aligned)
     float* g; int64_t ld_g;     // gradient at an aggregated matrix X^m, node order [n x ld_g]
     float* a; int64_t ld_a;     // result of a transposed aggregation [n x ld_a]
     float* s;                   // SAGE: scaled mean half [n x ld_a]
@@ -173,6 +204,8 @@ static void std_layout(const retexo_standard_config& c, int64_t n, int64_t e, in
         if (l.rep > max_rep && m > 0) max_rep = l.rep;
     }
     const StdLayer& last = b.L[c.K - 1];
+    b.ld_feat = std_round_up(c.d0, 32);
+    b.feat = t.template take<float>((size_t)n * b.ld_feat);
     b.ld_g = std_round_up(max_d, 32);
     b.ld_a = std_round_up(c.K > 1 ? c.hidden : 1, 32);
     b.ld_dz = std_round_up(c.K > 1 ? c.hidden : 1, 64);
@@ -269,8 +302,16 @@ extern "C" int retexo_standard_train(const retexo_standard_config* cfg, const re
     RETEXO_CUDA_TRY(cudaMemsetAsync(b.counters, 0, 8 * sizeof(unsigned long long), st));
     RETEXO_CUDA_TRY(cudaMemsetAsync(b.have_best, 0, 8 * sizeof(int32_t), st));
     RETEXO_TRY(launch_status());
-    RETEXO_TRY(retexo_aggregate(&g, c.aggr, in->features, in->ld_features, c.d0, nullptr, nullptr, 0, sage ? 1 : 0,
-                                b.L[0].x, b.L[0].ldx, b.ws_agg, b.ws_agg_bytes, st));
+    const float* feat = in->features;
+    int64_t ld_feat = in->ld_features;
+    const bool relaid = ld_feat % 4 != 0 || !aligned_to(feat, 16);
+    if (relaid) {
+        std_relay_kernel<<<std_row_blocks(n), 32 * kStdRowWarps, 0, st>>>(feat, ld_feat, c.d0, n, b.feat, b.ld_feat);
+        feat = b.feat;
+        ld_feat = b.ld_feat;
+    }
+    RETEXO_TRY(aggregate_rows(&g, c.aggr, feat, ld_feat, c.d0, relaid, nullptr, nullptr, 0, sage ? 1 : 0, b.L[0].x, b.L[0].ldx, b.ws_agg,
+                              b.ws_agg_bytes, st));
 
     const MlpPlan plan = make_plan(last.d, 0, c.n_classes, n_tr, n_val);
     MlpBuffers sb{};
@@ -293,7 +334,7 @@ extern "C" int retexo_standard_train(const retexo_standard_config* cfg, const re
             f.relu_bits = l.bits; f.ld_bits = l.ld_bits; f.status = sb.status;
             RETEXO_TRY(tc_gemm_launch(f, st));
             StdLayer& nx = b.L[m + 1];
-            RETEXO_TRY(retexo_aggregate(&g, c.aggr, l.h, l.ld_h32, c.hidden, nullptr, nullptr, 0, sage ? 1 : 0, nx.x, nx.ldx,
+            RETEXO_TRY(aggregate_rows(&g, c.aggr, l.h, l.ld_h32, c.hidden, true, nullptr, nullptr, 0, sage ? 1 : 0, nx.x, nx.ldx,
                                         b.ws_agg, b.ws_agg_bytes, st));
         }
         return RETEXO_OK;
@@ -319,9 +360,11 @@ extern "C" int retexo_standard_train(const retexo_standard_config* cfg, const re
                                          K > 1 ? b.dx : nullptr, b.ld_dx));
         model.step += 1;
         if (K > 1) {
-            RETEXO_CUDA_TRY(cudaMemsetAsync(b.g, 0, sizeof(float) * (size_t)n * b.ld_g, st));
-            std_scatter_rows_kernel<<<(unsigned)((n_tr * last.d + 255) / 256), 256, 0, st>>>(b.dx, b.ld_dx, in->train_idx, n_tr,
-                                                                                              last.d, b.g, b.ld_g);
+            // rows outside the batch have no gradient; the columns beyond the scattered ones are not read
+            RETEXO_CUDA_TRY(cudaMemset2DAsync(b.g, sizeof(float) * b.ld_g, 0, sizeof(float) * c.hidden, (size_t)n, st));
+            if (sage) RETEXO_CUDA_TRY(cudaMemsetAsync(b.s, 0, sizeof(float) * (size_t)n * b.ld_a, st));
+            std_scatter_rows_kernel<<<std_row_blocks(n_tr), 32 * kStdRowWarps, 0, st>>>(b.dx, b.ld_dx, in->train_idx, n_tr, last.d, g.rowptr,
+                                                                                        b.g, b.ld_g, sage ? b.s : nullptr, b.ld_a);
         }
         for (int m = K - 2; m >= 0; --m) {
             StdLayer& l = b.L[m];
@@ -329,16 +372,16 @@ extern "C" int retexo_standard_train(const retexo_standard_config* cfg, const re
             // the hidden layers' kept copies follow the last layer's decision (their weights are still iteration it - 1's)
             std_copy_if_kernel<<<(unsigned)((l.nt + 255) / 256), 256, 0, st>>>(b.decision, l.theta, l.best, l.nt);
             // dH^m = AGGR^T(G^{m+1})
-            const unsigned eb = (unsigned)((n * H + 255) / 256);
+            const unsigned eb = std_row_blocks(n), et = 32 * kStdRowWarps;
             if (sage) {
-                std_prescale_kernel<<<eb, 256, 0, st>>>(b.g, b.ld_g, H, H, g.rowptr, n, b.s, b.ld_a);
-                RETEXO_TRY(retexo_aggregate(&g, RETEXO_SAGE_MEAN, b.s, b.ld_a, H, nullptr, b.a, b.ld_a, 0, nullptr, 0, b.ws_agg,
+                if (m < K - 2) std_prescale_kernel<<<eb, et, 0, st>>>(b.g, b.ld_g, H, H, g.rowptr, n, b.s, b.ld_a);
+                RETEXO_TRY(aggregate_rows(&g, RETEXO_SAGE_MEAN, b.s, b.ld_a, H, true, nullptr, b.a, b.ld_a, 0, nullptr, 0, b.ws_agg,
                                             b.ws_agg_bytes, st));
-                std_gate_kernel<<<eb, 256, 0, st>>>(b.a, b.ld_a, b.g, b.ld_g, g.rowptr, l.bits, l.ld_bits, n, H, b.dz, b.ld_dz);
+                std_gate_kernel<<<eb, et, 0, st>>>(b.a, b.ld_a, b.g, b.ld_g, g.rowptr, l.bits, l.ld_bits, n, H, b.dz, b.ld_dz);
             } else {
                 RETEXO_TRY(retexo_aggregate(&g, RETEXO_GCN, b.g, b.ld_g, H, nullptr, b.a, b.ld_a, 0, nullptr, 0, b.ws_agg,
                                             b.ws_agg_bytes, st));
-                std_gate_kernel<<<eb, 256, 0, st>>>(b.a, b.ld_a, nullptr, 0, g.rowptr, l.bits, l.ld_bits, n, H, b.dz, b.ld_dz);
+                std_gate_kernel<<<eb, et, 0, st>>>(b.a, b.ld_a, nullptr, 0, g.rowptr, l.bits, l.ld_bits, n, H, b.dz, b.ld_dz);
             }
             // [dW_m ; db_m] = [X^m | 1]^T dZ^m, reduced over the nodes
             TcGemm gw{};
