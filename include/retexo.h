@@ -236,10 +236,8 @@ size_t retexo_mlp_train_step_workspace_size_norm(int32_t d_in, int32_t hidden, i
  *       16-byte aligned.  The weight-gradient products read it as it lies,
  *       reducing over the rows.
  * x_has_ones  1: column d_in of x holds 1 in every row (ldx > d_in;
- *       retexo_pack_rows with ones = 1 writes it).  That column makes the bias
- *       gradient one more output row of the weight-gradient product.  0: the
- *       call first copies x into its workspace with that column added, at the
- *       price of one more pass over x per call.
+ *       retexo_pack_rows with ones = 1 writes it).  The bias gradients do not
+ *       need that column: both values give the same result at the same cost.
  * y     int32 [n_rows] labels in [0, n_classes).
  * loss_out  device float, the loss before the update (may be NULL).
  * grad_out  optional device fp32 array shaped like theta: the gradient.

@@ -133,9 +133,9 @@ __global__ void __launch_bounds__(kBnThreads) bn_forward_kernel(BnForward a) {
             if (a.out_f32) a.out_f32[row * a.ld_f32 + j] = y;
         }
     }
-    if (a.out_bf16)      // the rest of the row: the column of ones behind the hidden units (or a zero), then zeros
+    if (a.out_bf16)      // the padding behind the hidden units
         for (int64_t j = a.H + lane; j < a.ld_bf16; j += 32)
-            a.out_bf16[row * a.ld_bf16 + j] = f32_to_bf16((a.ones && j == a.H) ? 1.f : 0.f);
+            a.out_bf16[row * a.ld_bf16 + j] = f32_to_bf16(0.f);
     if (a.bits && lane == 0)
         for (int64_t w = (a.H + 31) / 32; w < a.ld_bits; ++w) a.bits[row * a.ld_bits + w] = 0u;
 }

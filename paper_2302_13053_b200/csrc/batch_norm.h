@@ -36,8 +36,7 @@ struct BnForward {
     int64_t n_batch;                        // rows [0, n_batch) are normalised with `batch` (mean | var | rstd),
     const float* batch;                     //   rows [n_batch, n_rows) with the running statistics
     const float* r_mean; const float* r_var; float eps;
-    __nv_bfloat16* out_bf16; int64_t ld_bf16;   // (optional) ReLU(gamma zhat + beta); columns [H, ld_bf16) zero-filled,
-    int32_t ones;                               //   column H with 1 if `ones` (needs ld_bf16 > H)
+    __nv_bfloat16* out_bf16; int64_t ld_bf16;   // (optional) ReLU(gamma zhat + beta); columns [H, ld_bf16) zero-filled
     float* out_f32; int64_t ld_f32;             // (optional) the same in fp32
     uint32_t* bits; int64_t ld_bits;            // (optional) bit j & 31 of word [row][j / 32] = [output j > 0]
 };

@@ -268,9 +268,8 @@ static void lmp_layout(const retexo_lmp_config& c, int64_t n, int64_t e, int64_t
         l.ws_gatbwd_bytes = retexo_gat_backward_workspace_size(n, e, c.gat_heads, hd);
         l.ws_gatbwd = t.template take<char>(l.ws_gatbwd_bytes);
     }
-    // training rows, then validation rows, each followed by a column of ones (it carries the bias gradient
-    // through the weight-gradient product); after the round's last iteration the test rows take their place
-    l.xtr16 = t.template take<bf16>((size_t)(n_tr + n_val > n_te ? n_tr + n_val : n_te) * (size_t)round_up(max_din + 1, 64));
+    // training rows, then validation rows; after the round's last iteration the test rows take their place
+    l.xtr16 = t.template take<bf16>((size_t)(n_tr + n_val > n_te ? n_tr + n_val : n_te) * (size_t)ld16);
     l.xval16 = nullptr;
     l.y_tr = t.template take<int32_t>((size_t)n_tr);
     l.y_val = t.template take<int32_t>((size_t)(n_val > 0 ? n_val : 1));
@@ -479,13 +478,12 @@ extern "C" int retexo_lmp_train(const retexo_lmp_config* cfg, const retexo_lmp_i
         }
 
         // ---- the round's batches and model state
-        const int64_t ld_tr = round_up(r.d_in + 1, 64);
-        bf16* xval16 = b.xtr16 + (size_t)n_tr * ld_tr;
-        // the training rows (followed by their column of ones), then the validation rows; a round that trains
+        bf16* xval16 = b.xtr16 + (size_t)n_tr * ld16;
+        // the training rows, then the validation rows; a round that trains
         // its aggregator packs them anew after every local aggregation
         auto pack_batches = [&]() -> int {
-            RETEXO_TRY(retexo_pack_rows(b.x16, 1, ld16, r.d_in, train_idx, n_tr, b.xtr16, ld_tr, nullptr, 0, 1, st));
-            if (n_val) RETEXO_TRY(retexo_pack_rows(b.x16, 1, ld16, r.d_in, val_idx, n_val, xval16, ld_tr, nullptr, 0, 0, st));
+            RETEXO_TRY(retexo_pack_rows(b.x16, 1, ld16, r.d_in, train_idx, n_tr, b.xtr16, ld16, nullptr, 0, 0, st));
+            if (n_val) RETEXO_TRY(retexo_pack_rows(b.x16, 1, ld16, r.d_in, val_idx, n_val, xval16, ld16, nullptr, 0, 0, st));
             return RETEXO_OK;
         };
         if (!gat_train) RETEXO_TRY(pack_batches());
@@ -573,12 +571,12 @@ extern "C" int retexo_lmp_train(const retexo_lmp_config* cfg, const retexo_lmp_i
             // per-node model's step, the attention's backward pass and update after it)
             auto enqueue = [&](bool shadows_ready) -> int {
                 if (!gat_train)
-                    return mlp_train_step_launch(plan, sb, &model, b.xtr16, ld_tr, true, b.y_tr, loss_slot, nullptr,
+                    return mlp_train_step_launch(plan, sb, &model, b.xtr16, ld16, b.y_tr, loss_slot, nullptr,
                                                  shadows_ready, riding, st, &dev);
                 RETEXO_TRY(gat_forward(b.att));
                 RETEXO_TRY(pack_batches());
                 if (!riding) RETEXO_CUDA_TRY(cudaMemsetAsync(b.decision, 0, sizeof(int32_t), st));
-                RETEXO_TRY(mlp_train_step_launch(plan, sb, &model, b.xtr16, ld_tr, true, b.y_tr, loss_slot, nullptr,
+                RETEXO_TRY(mlp_train_step_launch(plan, sb, &model, b.xtr16, ld16, b.y_tr, loss_slot, nullptr,
                                                  shadows_ready, riding, st, &dev, b.dx, ld_dx));
                 return gat_backward_and_update();
             };
@@ -626,7 +624,7 @@ extern "C" int retexo_lmp_train(const retexo_lmp_config* cfg, const retexo_lmp_i
                     RETEXO_TRY(gat_forward(b.att));
                     RETEXO_TRY(pack_batches());
                 }
-                RETEXO_TRY(mlp_count_hits_launch(plan, sb, &model, xval16, ld_tr, n_val, val_hd, b.y_val,
+                RETEXO_TRY(mlp_count_hits_launch(plan, sb, &model, xval16, ld16, n_val, val_hd, b.y_val,
                                                  b.cur_correct, st, val_z));
                 snapshot_if_better_kernel<<<(unsigned)((nt + 255) / 256), 256, 0, st>>>(
                     b.cur_correct, b.best_correct, b.have_best, b.theta, b.theta_best, nt);

@@ -56,7 +56,6 @@ struct TcKernelArgs {
     const float* bias;
     float* out_f32; int64_t ld_f32;
     __nv_bfloat16* out_bf16; int64_t ld_bf16;
-    int ones_col;
     uint32_t* relu_bits; int64_t ld_bits;
     const __nv_bfloat16* mask; int64_t ld_mask;
     float gate_scale;
@@ -665,10 +664,6 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                         }
                         if (row0 < g.M && g.out_bf16)
                             store_block(v, stage, lane, col0, g.N, row0, g.M, g.out_bf16, g.ld_bf16, rows_map);
-                        // the column of ones behind the last output column (it makes the bias gradient one more
-                        // row of the weight-gradient product that reads this matrix)
-                        if (g.out_bf16 && g.ones_col && col0 == 0 && row < g.M)
-                            g.out_bf16[row * g.ld_bf16 + g.N] = __float2bfloat16_rn(1.0f);
                     }
                 }
             }
@@ -758,7 +753,6 @@ static int launch_tc_mode(const TcGemm& t, const CUtensorMap& ma, const CUtensor
     g.splits = splits;
     g.mode = t.mode; g.relu = t.relu; g.bias = t.bias;
     g.out_f32 = t.out_f32; g.ld_f32 = t.ld_f32; g.out_bf16 = t.out_bf16; g.ld_bf16 = t.ld_bf16;
-    g.ones_col = (t.ones_col && t.out_bf16 && t.ld_bf16 > t.N) ? 1 : 0;
     g.relu_bits = t.relu_bits; g.ld_bits = t.ld_bits;
     g.mask = t.mask; g.ld_mask = t.ld_mask;
     g.gate_scale = t.gate_scale != 0.f ? t.gate_scale : 1.f;
@@ -773,9 +767,7 @@ static int launch_tc_mode(const TcGemm& t, const CUtensorMap& ma, const CUtensor
     memset(&m_rows, 0, sizeof(m_rows));
     const bool ce = t.mode == TC_EPI_SOFTMAX_CE;
     const bool bias_like = t.mode == TC_EPI_BIAS || t.mode == TC_EPI_BIAS_DROP;
-    // (with a column of ones behind an output whose width is not a whole number of 16-byte pieces, the store of
-    //  the last piece and the plain store of the ones would meet in one piece: such shapes take plain stores)
-    if (t.out_bf16 && (bias_like || t.mode == TC_EPI_MASK || ce) && !(g.ones_col && t.N % 8 != 0))
+    if (t.out_bf16 && (bias_like || t.mode == TC_EPI_MASK || ce))
         g.tma_rows = make_store_map(&m_rows, t.out_bf16, ce ? g.n_train : t.M, ce ? t.ld_bf16 : t.N, t.ld_bf16) ? 1 : 0;
     const int64_t n_tiles = ((t.M + kTcBM - 1) / kTcBM) * ((t.N + BN - 1) / BN) * splits;
     const int n_sm = sm_count();
@@ -812,12 +804,11 @@ static int launch_tc_pair(const TcGemm& t, cudaStream_t st) {
     g.splits = 1;
     g.mode = t.mode; g.relu = t.relu; g.bias = t.bias;
     g.out_f32 = t.out_f32; g.ld_f32 = t.ld_f32; g.out_bf16 = t.out_bf16; g.ld_bf16 = t.ld_bf16;
-    g.ones_col = (t.ones_col && t.out_bf16 && t.ld_bf16 > t.N) ? 1 : 0;
     g.relu_bits = t.relu_bits; g.ld_bits = t.ld_bits;
     g.drop_thresh = t.drop_thresh; g.drop_step = t.drop_step; g.drop_key0 = t.drop_key[0]; g.drop_key1 = t.drop_key[1];
     g.drop_scale = t.drop_scale; g.drop_rows = t.drop_rows; g.drop_step_dev = t.drop_step_dev;
     g.status = t.status; g.n_train = t.M;
-    if (t.out_bf16 && !(g.ones_col && t.N % 8 != 0)) g.tma_rows = make_store_map(&m_rows, t.out_bf16, t.M, t.N, t.ld_bf16) ? 1 : 0;
+    if (t.out_bf16) g.tma_rows = make_store_map(&m_rows, t.out_bf16, t.M, t.N, t.ld_bf16) ? 1 : 0;
     const int64_t n_tiles = ((t.M + 2 * kTcBM - 1) / (2 * kTcBM)) * ((t.N + BN - 1) / BN);
     OverlapLaunch ol(dim3(2), dim3(64 + 32 * EW), smem, st, 2);
     cudaLaunchConfig_t& cfg = ol.cfg;

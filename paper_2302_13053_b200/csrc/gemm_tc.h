@@ -13,10 +13,7 @@ enum TcEpilogue { TC_EPI_BIAS = 0, TC_EPI_PARTIAL = 1, TC_EPI_SOFTMAX_CE = 3, TC
 // C[M x N] = A[M x K] * B[N x K]^T with A and B bf16, K contiguous (row strides
 // lda / ldb elements, multiples of 8; bases 16-byte aligned).
 //   TC_EPI_BIAS   : out = acc + bias[n] (bias optional), optional ReLU, written as
-//                   fp32 (out_f32, ld_f32) and/or bf16 (out_bf16, ld_bf16).  With ones_col
-//                   (needs ld_bf16 > N) column N of out_bf16 is set to 1 in every row: the
-//                   all-ones column that turns a bias gradient into one more output row of
-//                   the weight-gradient product that reads this matrix.  relu_bits (optional)
+//                   fp32 (out_f32, ld_f32) and/or bf16 (out_bf16, ld_bf16).  relu_bits (optional)
 //                   receives one bit per element, set where the value written is positive.
 //   TC_EPI_PARTIAL: C = A^T B with the operands as they lie in memory, A [K x lda] holding M
 //                   columns and B [K x ldb] holding N columns (the reduction runs over the rows,
@@ -41,7 +38,6 @@ struct TcGemm {
     const float* bias;
     float* out_f32; int64_t ld_f32;
     __nv_bfloat16* out_bf16; int64_t ld_bf16;
-    int ones_col;
     // TC_EPI_BIAS / TC_EPI_BIAS_DROP (optional): one bit per output element, bit n & 31 of word [m][n / 32] = [out > 0]
     uint32_t* relu_bits; int64_t ld_bits;
     const __nv_bfloat16* mask; int64_t ld_mask;
@@ -70,8 +66,10 @@ int tc_gemm_launch(const TcGemm& t, cudaStream_t st);
 bool tc_make_map_2d(CUtensorMap* map, const void* base, int64_t rows, int64_t cols, int64_t ld, int box_rows, int box_cols,
                     int swizzle_bytes, bool l2_promote);
 
+constexpr int32_t kHeadMaxHidden = 256;
+
 // The class product, the soft-max cross-entropy and the gated back-propagation of one training iteration in
-// one kernel (hidden <= 256, n_classes <= 64); see mlp_fused.cu.
+// one kernel (hidden <= kHeadMaxHidden, n_classes <= 64); see mlp_fused.cu.
 struct HeadBackward {
     const __nv_bfloat16* hd; int64_t ld_hd;         // Hd [n_all x ld_hd], hidden columns
     const uint32_t* gate_bits; int64_t ld_bits;     // [n_train x ld_bits] words: bit j & 31 of word j / 32 = [Hd[row][j] > 0]

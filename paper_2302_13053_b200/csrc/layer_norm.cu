@@ -59,9 +59,9 @@ __global__ void __launch_bounds__(kLnThreads) ln_forward_kernel(LnForward a) {
         }
     }
     if (a.out_bf16) {
-        // the rest of the row: the column of ones behind the hidden units (or a zero), then zeros
+        // the padding behind the hidden units
         for (int64_t j = a.H + lane; j < a.ld_bf16; j += 32)
-            a.out_bf16[row * a.ld_bf16 + j] = f32_to_bf16((a.ones && j == a.H) ? 1.f : 0.f);
+            a.out_bf16[row * a.ld_bf16 + j] = f32_to_bf16(0.f);
     }
     if (a.bits && lane == 0)
         for (int64_t w = (a.H + 31) / 32; w < a.ld_bits; ++w) a.bits[row * a.ld_bits + w] = 0u;

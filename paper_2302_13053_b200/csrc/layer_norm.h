@@ -17,8 +17,7 @@ struct LnForward {
     float eps;
     int32_t H;
     int64_t n_rows;
-    __nv_bfloat16* out_bf16; int64_t ld_bf16;   // (optional) ReLU(gamma zhat + beta); columns [H, ld_bf16) are zero-filled,
-    int32_t ones;                               //   column H with 1 if `ones` (needs ld_bf16 > H)
+    __nv_bfloat16* out_bf16; int64_t ld_bf16;   // (optional) ReLU(gamma zhat + beta); columns [H, ld_bf16) are zero-filled
     float* out_f32; int64_t ld_f32;             // (optional) the same in fp32
     uint32_t* bits; int64_t ld_bits;            // (optional) bit j & 31 of word [row][j / 32] = [output j > 0]
     float2* stats;                              // (optional) [n_rows] (mean, 1 / sqrt(var + eps)), for the backward pass

@@ -5,15 +5,15 @@
 // gradients are kept row-major only (one batch row per line): the forward products
 // read them with the reduction dimension contiguous, the weight-gradient products,
 // whose reduction runs over the batch, read the same arrays with M / N contiguous.
-//   forward   [Hd | 1] = ReLU(X W1 + b1)                 gemm_tc.cu, A = X, B = W1^T
+//   forward   Hd = ReLU(X W1 + b1)                       gemm_tc.cu, A = X, B = W1^T
 //   middle    L = Hd W2 + b2, loss, dL,                  mlp_fused.cu: one kernel, Hd read once,
 //             dHd = (dL W2^T) .* [Hd > 0]                the logits never leave the SM
-//   backward  [dW2 ; db2] = [Hd | 1]^T dL                gemm_tc.cu, split over the batch
-//             [dW1 ; db1] = [X | 1]^T dHd                gemm_tc.cu, split over the batch
+//   backward  [dW2 ; db2] = [Hd | 1]^T dL                grad_tc.cu, both in one launch, split over the batch;
+//             [dW1 ; db1] = [X | 1]^T dHd
 // (hidden > 256: the middle runs as two products of gemm_tc.cu instead.)
-// The column of ones behind X and Hd turns each bias gradient into one more output
-// row, so the partial sums come out laid out exactly like theta = [W1 | b1 | W2 | b2].
+// The bias gradients are one more row of each product, kept in partial sums of their own.
 #include "gemm_tc.h"
+#include "grad_tc.h"
 #include "batch_norm.h"
 #include "layer_norm.h"
 #include "mlp_kernels.cuh"
@@ -55,14 +55,11 @@ MlpPlan make_plan(int32_t d_in, int32_t hidden, int32_t n_classes, int64_t n_row
     p.nt = retexo_theta_size_norm(d_in, hidden, n_classes, p.norm);
     p.ld_dl = pad_ld(n_classes);                           // 64: classes padded with zero columns
     p.ld_h = pad_ld(hidden > 0 ? hidden : 1);
-    p.ld_h1 = pad_ld(hidden > 0 ? hidden + 1 : 1);
     p.ld_bits = hidden > 0 ? 2 * (((int64_t)hidden + 63) / 64) : 2;
     p.ld_k = pad_ld(d_in);
     p.ld_o1 = pad_ld(p.out1);
-    p.ld_x1 = pad_ld((int64_t)d_in + 1);
     p.sm_blocks = 4 * ((n_rows + n_eval + 127) / 128);     // up to four loss partials per 128-row tile
-    p.split_w1 = tc_split((int64_t)d_in + 1, p.out1, n_rows);
-    p.split_w2 = hidden > 0 ? tc_split((int64_t)hidden + 1, n_classes, n_rows) : 0;
+    grad_splits(d_in, p.out1, hidden, hidden > 0 ? n_classes : 0, n_rows, &p.split_w1, &p.split_w2);
     return p;
 }
 
@@ -76,14 +73,15 @@ static void layout(const MlpPlan& p, Taker& t, MlpBuffers* out) {
     b.w1r16 = t.template take<bf16>((size_t)p.d_in * p.ld_o1);
     b.w2t16 = t.template take<bf16>(h ? (size_t)p.n_classes * p.ld_h : 1);
     b.w2p16 = t.template take<bf16>(h ? (size_t)p.hidden * p.ld_dl : 1);
-    b.x1 = t.template take<bf16>(n_all * p.ld_x1);
-    b.hd16 = t.template take<bf16>(h ? n_all * p.ld_h1 : 1);
+    b.hd16 = t.template take<bf16>(h ? n_all * p.ld_h : 1);
     b.dl16 = t.template take<bf16>(n * p.ld_dl);
     b.dhd16 = t.template take<bf16>(h ? n * p.ld_h : 1);
     b.gate_bits = t.template take<uint32_t>(h ? n_all * (size_t)p.ld_bits : 1);
     b.loss_partial = t.template take<float>((size_t)p.sm_blocks);
-    b.pw1 = t.template take<float>((size_t)p.split_w1 * (p.d_in + 1) * p.out1);
-    b.pw2 = t.template take<float>(h ? (size_t)p.split_w2 * (p.hidden + 1) * p.n_classes : 1);
+    b.pw1 = t.template take<float>((size_t)p.split_w1 * p.d_in * p.out1);
+    b.pb1 = t.template take<float>((size_t)p.split_w1 * grad_bias_shares(p.d_in) * p.out1);
+    b.pw2 = t.template take<float>(h ? (size_t)p.split_w2 * p.hidden * p.n_classes : 1);
+    b.pb2 = t.template take<float>(h ? (size_t)p.split_w2 * grad_bias_shares(p.hidden) * p.n_classes : 1);
     b.status = t.template take<int32_t>(64);
     if (p.norm) {
         b.z1 = t.template take<float>(n_all * (size_t)p.hidden);
@@ -130,15 +128,21 @@ static int check_model(const retexo_mlp* m) {
 
 static int32_t norm_of(const retexo_mlp* m) { return m->hidden > 0 ? m->norm : RETEXO_NORM_NONE; }
 
-// bf16 shadows of the weights in the orientations the products need.
-static int build_weight_shadows(const MlpPlan& p, const MlpBuffers& b, const float* theta, cudaStream_t st) {
-    const int32_t d_in = p.d_in, H = p.hidden, O = p.n_classes, out1 = p.out1;
-    RETEXO_TRY(retexo_pack_rows(theta, 0, out1, out1, nullptr, d_in, b.w1r16, b.w1r16 ? p.ld_o1 : 0, b.w1t16, p.ld_k, 0, st));
-    if (H > 0) {
-        const float* w2 = theta + (int64_t)d_in * out1 + out1;
-        RETEXO_TRY(retexo_pack_rows(w2, 0, O, O, nullptr, H, b.w2p16, p.ld_dl, b.w2t16, p.ld_h, 0, st));
+// bf16 shadows of the weights in the orientations the products need (row-major ones where asked for); clears the status word.
+static int build_weight_shadows(const MlpPlan& p, const MlpBuffers& b, const float* theta, bool w1_rows, bool w2_rows, cudaStream_t st) {
+    WeightShadows w{};
+    w.w[0] = theta; w.rows[0] = p.d_in; w.cols[0] = p.out1; w.wt[0] = b.w1t16; w.ld_wt[0] = p.ld_k;
+    w.wr[0] = w1_rows ? b.w1r16 : nullptr; w.ld_wr[0] = p.ld_o1;
+    w.status = b.status;
+    const int64_t tiles0 = (((int64_t)p.d_in + 31) / 32) * ((p.out1 + 31) / 32);
+    int64_t tiles1 = 0;
+    if (p.hidden > 0) {
+        w.w[1] = theta + (int64_t)p.d_in * p.out1 + p.out1; w.rows[1] = p.hidden; w.cols[1] = p.n_classes;
+        w.wt[1] = b.w2t16; w.ld_wt[1] = p.ld_h; w.wr[1] = w2_rows ? b.w2p16 : nullptr; w.ld_wr[1] = p.ld_dl;
+        tiles1 = (((int64_t)p.hidden + 31) / 32) * ((p.n_classes + 31) / 32);
     }
-    return RETEXO_OK;
+    weight_shadows_kernel<<<(unsigned)(tiles0 + tiles1), 256, 0, st>>>(w, (int)tiles0);
+    return launch_status();
 }
 
 static TcGemm tc_base(const bf16* A, int64_t lda, const bf16* B, int64_t ldb, int64_t M, int64_t N, int64_t K,
@@ -227,8 +231,8 @@ extern "C" int retexo_mlp_train_step(retexo_mlp* model, const void* x, int64_t l
     Arena ws(workspace, workspace_bytes);
     MlpBuffers b{};
     layout(p, ws, &b);
-    RETEXO_TRY(mlp_train_step_launch(p, b, model, static_cast<const bf16*>(x), ldx, x_has_ones != 0, y, loss_out, grad_out,
-                                     false, nullptr, st, nullptr, dx_out, ld_dx));
+    RETEXO_TRY(mlp_train_step_launch(p, b, model, static_cast<const bf16*>(x), ldx, y, loss_out, grad_out, false, nullptr, st, nullptr,
+                                     dx_out, ld_dx, false));
     model->step += 1;
     return RETEXO_OK;
 }
@@ -238,9 +242,9 @@ namespace retexo {
 // The launch sequence of one iteration; `model->step` is the count of updates
 // already applied.
 int mlp_train_step_launch(const MlpPlan& p, const MlpBuffers& b, const retexo_mlp* model,
-                          const bf16* x, int64_t ldx, bool x_has_ones, const int32_t* y,
+                          const bf16* x, int64_t ldx, const int32_t* y,
                           float* loss_out, float* grad_out, bool shadows_ready, const EvalTail* tail,
-                          cudaStream_t st, const DeviceIter* dev, float* dx_out, int64_t ld_dx) {
+                          cudaStream_t st, const DeviceIter* dev, float* dx_out, int64_t ld_dx, bool keep_shadows) {
     const int64_t n = p.n_rows;
     const int64_t n_all = n + (tail ? p.n_eval : 0);          // evaluation rows ride along in the forward pass
     const int32_t d_in = p.d_in, H = p.hidden, O = p.n_classes, out1 = p.out1;
@@ -248,15 +252,8 @@ int mlp_train_step_launch(const MlpPlan& p, const MlpBuffers& b, const retexo_ml
     const float* b1 = theta + (int64_t)d_in * out1;
     const float* b2 = b1 + out1 + (int64_t)H * O;
     // (a caller that chains iterations clears the status word once: a give-up then marks every later loss)
-    if (!shadows_ready) {
-        RETEXO_CUDA_TRY(cudaMemsetAsync(b.status, 0, sizeof(int32_t), st));
-        RETEXO_TRY(build_weight_shadows(p, b, theta, st));
-    }
-    if (!x_has_ones) {      // no column of ones behind the caller's batch: copy it with one (one more pass over X per call)
-        RETEXO_TRY(retexo_pack_rows(x, 1, ldx, d_in, nullptr, n_all, b.x1, p.ld_x1, nullptr, 0, 1, st));
-        x = b.x1;
-        ldx = p.ld_x1;
-    }
+    const bool w1_rows = dx_out != nullptr, w2_rows = H > kHeadMaxHidden;      // who reads the row-major copies
+    if (!shadows_ready) RETEXO_TRY(build_weight_shadows(p, b, theta, w1_rows, w2_rows, st));
 
     // ---- forward
     if (tail && !tail->done) RETEXO_CUDA_TRY(cudaMemsetAsync(tail->correct, 0, sizeof(unsigned long long), st));
@@ -274,10 +271,10 @@ int mlp_train_step_launch(const MlpPlan& p, const MlpBuffers& b, const retexo_ml
     if (H > 0) {
         if (ln || bn) {
             // the product leaves z = X W1 + b1 in fp32; the normalisation's kernel applies the ReLU and
-            // writes [Hd | 1] and the gate bits as the plain forward epilogue would
+            // writes Hd and the gate bits as the plain forward epilogue would
             fwd.out_f32 = b.z1; fwd.ld_f32 = H;
         } else {
-            fwd.relu = 1; fwd.out_bf16 = b.hd16; fwd.ld_bf16 = p.ld_h1; fwd.ones_col = 1;
+            fwd.relu = 1; fwd.out_bf16 = b.hd16; fwd.ld_bf16 = p.ld_h;
             fwd.relu_bits = b.gate_bits; fwd.ld_bits = p.ld_bits;
         }
         if (dropping) {
@@ -294,7 +291,7 @@ int mlp_train_step_launch(const MlpPlan& p, const MlpBuffers& b, const retexo_ml
         if (ln) {
             LnForward lf{};
             lf.z = b.z1; lf.ld_z = H; lf.gamma = ln_gamma; lf.beta = ln_gamma + H; lf.eps = model->norm_eps; lf.H = H;
-            lf.n_rows = n_all; lf.out_bf16 = b.hd16; lf.ld_bf16 = p.ld_h1; lf.ones = 1;
+            lf.n_rows = n_all; lf.out_bf16 = b.hd16; lf.ld_bf16 = p.ld_h;
             lf.bits = b.gate_bits; lf.ld_bits = p.ld_bits; lf.stats = b.ln_stats;
             RETEXO_TRY(ln_forward_launch(lf, st));
         }
@@ -303,12 +300,12 @@ int mlp_train_step_launch(const MlpPlan& p, const MlpBuffers& b, const retexo_ml
             BnForward bf{};
             bf.z = b.z1; bf.ld_z = H; bf.gamma = ln_gamma; bf.beta = ln_gamma + H; bf.H = H; bf.n_rows = n_all; bf.n_batch = n;
             bf.batch = b.bn_batch; bf.r_mean = ln_gamma + 2 * H; bf.r_var = ln_gamma + 3 * H; bf.eps = model->norm_eps;
-            bf.out_bf16 = b.hd16; bf.ld_bf16 = p.ld_h1; bf.ones = 1; bf.bits = b.gate_bits; bf.ld_bits = p.ld_bits;
+            bf.out_bf16 = b.hd16; bf.ld_bf16 = p.ld_h; bf.bits = b.gate_bits; bf.ld_bits = p.ld_bits;
             RETEXO_TRY(bn_forward_launch(bf, st));
         }
         // ---- class product, loss and gated back-propagation
         HeadBackward hb{};
-        hb.hd = b.hd16; hb.ld_hd = p.ld_h1; hb.gate_bits = b.gate_bits; hb.ld_bits = p.ld_bits; hb.w2t = b.w2t16; hb.ld_w2t = p.ld_h; hb.b2 = b2;
+        hb.hd = b.hd16; hb.ld_hd = p.ld_h; hb.gate_bits = b.gate_bits; hb.ld_bits = p.ld_bits; hb.w2t = b.w2t16; hb.ld_w2t = p.ld_h; hb.b2 = b2;
         hb.hidden = H; hb.n_classes = O; hb.n_train = n; hb.n_all = n_all;
         hb.y = y; hb.y_eval = tail ? tail->y_eval : nullptr;
         hb.inv_rows = 1.0f / (float)n; hb.gate_scale = keep_scale;      // a dropped unit has Hd = 0: the gate holds the mask
@@ -318,21 +315,18 @@ int mlp_train_step_launch(const MlpPlan& p, const MlpBuffers& b, const retexo_ml
             RETEXO_TRY(head_backward_launch(hb, st));
             n_loss *= 4;
         } else {      // wide hidden layers: the same three steps as two products
-            TcGemm head = tc_base(b.hd16, p.ld_h1, b.w2t16, p.ld_h, n_all, O, H, b.status);
+            if (!w2_rows) return RETEXO_ERR_UNSUPPORTED;
+            TcGemm head = tc_base(b.hd16, p.ld_h, b.w2t16, p.ld_h, n_all, O, H, b.status);
             head.bias = b2;
             head.mode = TC_EPI_SOFTMAX_CE; head.y = y; head.inv_rows = 1.0f / (float)n; head.loss_partial = b.loss_partial;
             head.out_bf16 = b.dl16; head.ld_bf16 = p.ld_dl;
             if (tail) { head.eval_from = n; head.y_eval = tail->y_eval; head.correct = tail->correct; }
             RETEXO_TRY(tc_gemm_launch(head, st));
             TcGemm bk = tc_base(b.dl16, p.ld_dl, b.w2p16, p.ld_dl, n, H, O, b.status);
-            bk.mode = TC_EPI_MASK; bk.mask = b.hd16; bk.ld_mask = p.ld_h1; bk.out_bf16 = b.dhd16; bk.ld_bf16 = p.ld_h;
+            bk.mode = TC_EPI_MASK; bk.mask = b.hd16; bk.ld_mask = p.ld_h; bk.out_bf16 = b.dhd16; bk.ld_bf16 = p.ld_h;
             bk.gate_scale = keep_scale;
             RETEXO_TRY(tc_gemm_launch(bk, st));
         }
-        // ---- [dW2 ; db2] = [Hd | 1]^T dL
-        TcGemm g2 = tc_base(b.hd16, p.ld_h1, b.dl16, p.ld_dl, (int64_t)H + 1, O, n, b.status);
-        g2.mode = TC_EPI_PARTIAL; g2.splits = (int)p.split_w2; g2.partial = b.pw2;
-        RETEXO_TRY(tc_gemm_launch(g2, st));
         if (ln) {      // through the normalisation: dHd (in place) becomes the gradient at z; partials of d gamma, d beta
             LnBackward lb{};
             lb.z = b.z1; lb.ld_z = H; lb.stats = b.ln_stats; lb.gamma = ln_gamma; lb.H = H; lb.n_rows = n;
@@ -355,19 +349,19 @@ int mlp_train_step_launch(const MlpPlan& p, const MlpBuffers& b, const retexo_ml
         dxg.out_f32 = dx_out; dxg.ld_f32 = ld_dx;
         RETEXO_TRY(tc_gemm_launch(dxg, st));
     }
-    // ---- [dW1 ; db1] = [X | 1]^T grad1
-    TcGemm g1 = tc_base(x, ldx, grad1, ld_grad1, (int64_t)d_in + 1, out1, n, b.status);
-    g1.mode = TC_EPI_PARTIAL; g1.splits = (int)p.split_w1; g1.partial = b.pw1;
-    RETEXO_TRY(tc_gemm_launch(g1, st));
+    // ---- [dW1 ; db1] = [X | 1]^T grad1,  [dW2 ; db2] = [Hd | 1]^T dL
+    GradProduct prod[2] = {{x, ldx, grad1, ld_grad1, d_in, out1, (int32_t)p.split_w1, b.pw1, b.pb1},
+                           {b.hd16, p.ld_h, b.dl16, p.ld_dl, H, O, (int32_t)p.split_w2, b.pw2, b.pb2}};
+    RETEXO_TRY(grad_launch(prod, H > 0 ? 2 : 1, n, b.status, st));
 
     // ---- reduce the partials and update
     UpdateArgs u{};
     u.n_seg = H > 0 ? 2 : 1;
-    u.seg[0] = {((int64_t)d_in + 1) * out1, b.pw1, p.split_w1};
-    if (H > 0) u.seg[1] = {((int64_t)H + 1) * O, b.pw2, p.split_w2};
-    if (ln) { u.n_seg = 3; u.seg[2] = {2 * (int64_t)H, b.pln, p.ln_blocks}; }
+    u.seg[0] = {((int64_t)d_in + 1) * out1, b.pw1, p.split_w1, b.pb1, p.split_w1 * grad_bias_shares(d_in)};
+    if (H > 0) u.seg[1] = {((int64_t)H + 1) * O, b.pw2, p.split_w2, b.pb2, p.split_w2 * grad_bias_shares(H)};
+    if (ln) { u.n_seg = 3; u.seg[2] = {2 * (int64_t)H, b.pln, p.ln_blocks, nullptr, 0}; }
     if (bn) {      // [d gamma | d beta] arrive summed; the running statistics behind them move towards the batch's
-        u.n_seg = 3; u.seg[2] = {2 * (int64_t)H, b.bn_sums, 1};
+        u.n_seg = 3; u.seg[2] = {2 * (int64_t)H, b.bn_sums, 1, nullptr, 0};
         u.bn_batch = b.bn_batch; u.bn_momentum = model->bn_momentum; u.bn_unbias = (float)((double)n / (double)(n - 1));
     }
     u.theta = model->theta; u.m = model->adam_m; u.v = model->adam_v; u.grad_out = grad_out;
@@ -379,8 +373,11 @@ int mlp_train_step_launch(const MlpPlan& p, const MlpBuffers& b, const retexo_ml
     u.loss_partial = b.loss_partial; u.n_loss = n_loss;      // the partials this launch's loss kernel wrote
     u.inv_rows = 1.0f / (float)n; u.loss_out = loss_out;
     u.status = b.status;
-    u.w1t16 = b.w1t16; u.ld_k = p.ld_k; u.w1r16 = b.w1r16; u.ld_o1 = p.ld_o1; u.w2t16 = H > 0 ? b.w2t16 : nullptr; u.ld_h = p.ld_h;
-    u.w2p16 = H > 0 ? b.w2p16 : nullptr; u.ld_dl = p.ld_dl;
+    u.ld_k = p.ld_k; u.ld_o1 = p.ld_o1; u.ld_h = p.ld_h; u.ld_dl = p.ld_dl;
+    if (keep_shadows) {
+        u.w1t16 = b.w1t16; u.w1r16 = w1_rows ? b.w1r16 : nullptr;
+        u.w2t16 = H > 0 ? b.w2t16 : nullptr; u.w2p16 = w2_rows ? b.w2p16 : nullptr;
+    }
     u.d_in = d_in; u.out1 = out1; u.hidden = H; u.n_classes = O;
     if (tail) {
         u.snap_decision = tail->decision;
@@ -408,7 +405,7 @@ int linear_update_launch(int32_t d_in, int32_t out, float* theta, float* adam_m,
                          bf16* wt16, int64_t ld_k, bf16* wr16, int64_t ld_o1, float* grad_out, cudaStream_t st) {
     UpdateArgs u{};
     u.n_seg = 1;
-    u.seg[0] = {((int64_t)d_in + 1) * out, partial, splits};
+    u.seg[0] = {((int64_t)d_in + 1) * out, partial, splits, nullptr, 0};
     u.theta = theta; u.m = adam_m; u.v = adam_v; u.grad_out = grad_out;
     u.optimizer = optimizer; u.lr = lr; u.beta1 = beta1; u.beta2 = beta2; u.eps = eps;
     u.corr1 = (float)(1.0 - pow((double)beta1, (double)step));
@@ -532,13 +529,12 @@ extern "C" int retexo_embed(const retexo_mlp* model, const void* x, int64_t ldx,
 
     if (correct) RETEXO_CUDA_TRY(cudaMemsetAsync(correct, 0, sizeof(unsigned long long), st));
     if (n_rows == 0) return RETEXO_OK;
-    RETEXO_CUDA_TRY(cudaMemsetAsync(b.status, 0, sizeof(int32_t), st));
     const float* theta = model->theta;
     const float* b1 = theta + (int64_t)d_in * out1;
     const float* b2 = b1 + out1 + (int64_t)H * O;
     const bool want_logits = logits_out || pred_out || correct;
 
-    RETEXO_TRY(build_weight_shadows(p, b, theta, st));
+    RETEXO_TRY(build_weight_shadows(p, b, theta, false, false, st));
     // One pass of the tensor-core path over `rows` dense rows xd; `off` is their position in the outputs.
     auto dense = [&](const bf16* xd, int64_t ldxd, int64_t rows, int64_t off) -> int {
         float* hid = hidden_out ? hidden_out + off * ld_hidden : nullptr;

@@ -390,7 +390,7 @@ head_backward_kernel(const __grid_constant__ CUtensorMap map_hd, const __grid_co
 }
 
 bool head_backward_supported(const HeadBackward& h) {
-    if (h.hidden < 1 || h.hidden > 256 || h.n_classes < 1 || h.n_classes > 64) return false;
+    if (h.hidden < 1 || h.hidden > kHeadMaxHidden || h.n_classes < 1 || h.n_classes > 64) return false;
     if (h.n_train < 1 || h.n_all < h.n_train || h.n_all > INT32_MAX - 256) return false;
     if (!h.hd || !h.w2t || !h.dl || !h.dhd || !h.y || h.ld_dl != 64) return false;
     if (!h.gate_bits || h.ld_bits < 2 * ((h.hidden + 63) / 64) || h.ld_bits % 2 != 0 || !aligned_to(h.gate_bits, 8)) return false;

@@ -98,11 +98,43 @@ __global__ void __launch_bounds__(256) pack_rows_pieces_kernel(const void* __res
     }
 }
 
+// bf16 copies of both layers' weights, transposed (and row-major where wanted), and the status word cleared: everything an iteration
+// needs before its first product, in one launch.  A block turns a 32 x 32 tile; the first tiles0 tiles are W1's.
+struct WeightShadows {
+    const float* w[2]; int32_t rows[2], cols[2];      // [rows x cols] fp32; rows[1] = 0: one layer
+    bf16* wt[2]; int64_t ld_wt[2];                    // [cols x ld_wt]
+    bf16* wr[2]; int64_t ld_wr[2];                    // [rows x ld_wr], may be null
+    int32_t* status;
+};
+static __global__ void __launch_bounds__(256) weight_shadows_kernel(WeightShadows w, int tiles0) {
+    __shared__ float tile[32][33];
+    if (blockIdx.x == 0 && threadIdx.x == 0 && w.status) *w.status = 0;
+    const int l = (int)blockIdx.x >= tiles0 ? 1 : 0, t = (int)blockIdx.x - (l ? tiles0 : 0), tc = (w.cols[l] + 31) >> 5;
+    const int r0 = (t / tc) * 32, c0 = (t % tc) * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+#pragma unroll
+    for (int i = ty; i < 32; i += 8) {
+        const int r = r0 + i, c = c0 + tx;
+        const bool in = r < w.rows[l] && c < w.cols[l];
+        const float v = in ? w.w[l][(int64_t)r * w.cols[l] + c] : 0.f;
+        tile[i][tx] = v;
+        if (in && w.wr[l]) w.wr[l][(int64_t)r * w.ld_wr[l] + c] = f32_to_bf16(v);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = ty; i < 32; i += 8) {
+        const int c = c0 + i, r = r0 + tx;
+        if (c < w.cols[l] && r < w.rows[l]) w.wt[l][(int64_t)c * w.ld_wt[l] + r] = f32_to_bf16(tile[tx][i]);
+    }
+}
+
 // ---------------------------------------------------------------- optimiser
 struct GradSeg {
     int64_t size;              // parameters in this segment
     const float* partial;      // [count x size], summed in index order
     int64_t count;
+    // (optional) the segment's last row, the bias, comes in partials of its own, [bias_count x columns], and partial holds the
+    // other rows only
+    const float* bias_partial; int64_t bias_count;
 };
 struct UpdateArgs {
     GradSeg seg[3];            // [W1 | b1], (hidden > 0) [W2 | b2] and (normalisation) [gamma | beta], each laid out like theta
@@ -148,6 +180,41 @@ __host__ __device__ __forceinline__ double pow_whole(double base, unsigned long 
         e >>= 1;
     }
     return r;
+}
+
+// Books the validation count that rode along and moves the iteration state on.  Called by one thread of every block once the whole
+// block has read that state (before the block's own stores, so the fence has nothing to wait for); the last block to arrive
+// does the work while the others are already updating their parameters.
+__device__ __forceinline__ void update_bookkeeping(const UpdateArgs& u, unsigned long long step_now, unsigned long long snap_cur,
+                                                   unsigned long long snap_best, int32_t snap_have, bool snapshot) {
+    __threadfence();
+    if (atomicAdd(u.done, 1ull) != (unsigned long long)gridDim.x - 1ull) return;
+    __threadfence();
+    if (u.snap_decision) *u.snap_decision = snapshot ? 1 : 0;
+    if (u.snap_cur) {
+        unsigned long long* slot = u.step_dev ? (u.history_base && step_now > 0 ? u.history_base + (step_now - 1) : nullptr) : u.rec_history_slot;
+        if (slot) *slot = snap_cur;
+        if (!snap_have || snap_cur > snap_best) {
+            *u.snap_best = snap_cur;
+            if (u.rec_best_iter) *u.rec_best_iter = u.step_dev ? (int32_t)step_now : u.rec_iter;
+            *u.snap_have = 1;
+        }
+        *u.snap_cur = 0ull;
+    }
+    if (u.step_dev) *u.step_dev = step_now + 1;
+    *u.done = 0ull;
+}
+
+// The step's loss and status, by one warp of the grid (fixed order: per-lane strided sums, then a shuffle tree).
+__device__ __forceinline__ void update_loss(const UpdateArgs& u, unsigned long long step_now, int lane) {
+    float* loss_out = u.step_dev ? (u.loss_base ? u.loss_base + step_now : nullptr) : u.loss_out;
+    if (loss_out) {
+        float s = 0.f;
+        for (int64_t i = lane; i < u.n_loss; i += 32) s += u.loss_partial[i];
+        s = warp_sum(s);
+        if (lane == 0) *loss_out = (u.status && *u.status) ? __int_as_float(0x7fc00000) : s * u.inv_rows;
+    }
+    if (lane == 0 && u.status_out && u.status) *u.status_out = *u.status;
 }
 
 // Sum of one parameter's split-K partials in index order.  BATCH loads are in flight before the first addition
@@ -215,56 +282,28 @@ __global__ void __launch_bounds__(256, BATCH == 16 ? 4 : 2) reduce_update_kernel
             g = u.bn_batch[q - 2 * (int64_t)cols] * (row == 3 ? u.bn_unbias : 1.f);      // the statistic it moves towards
         } else {
             if (adam) { m = u.m[p]; v = u.v[p]; }
-            g = sum_partials<BATCH>(u.seg[sidx].partial + q, (int32_t)u.seg[sidx].count, sidx == 2 ? 2 * (int64_t)cols : size);      // (a partial of the third segment holds its two trained rows)
+            const GradSeg& seg = u.seg[sidx];
+            if (seg.bias_partial && row == rows - 1) g = sum_partials<BATCH>(seg.bias_partial + col, (int32_t)seg.bias_count, cols);
+            else      // (a partial of the third segment holds its two trained rows)
+                g = sum_partials<BATCH>(seg.partial + q, (int32_t)seg.count, sidx == 2 ? 2 * (int64_t)cols : seg.bias_partial ? size - cols : size);
         }
     }
 
     float corr1 = u.corr1, corr2 = u.corr2;
-    float* loss_out = u.loss_out;
-    if (u.step_dev) {      // the iteration number lives on the device: bias corrections and slots follow from it
+    if (u.step_dev) {      // the iteration number lives on the device: bias corrections follow from it
         __shared__ float corr_s[2];
         if (threadIdx.x == 0) corr_s[0] = (float)(1.0 - pow_whole((double)u.beta1, step_now + 1));
         if (threadIdx.x == 32) corr_s[1] = (float)(1.0 - pow_whole((double)u.beta2, step_now + 1));
         __syncthreads();
         corr1 = corr_s[0]; corr2 = corr_s[1];
-        loss_out = u.loss_base ? u.loss_base + step_now : nullptr;
     }
     // keep-the-best: are the weights as they stand (validated in this iteration's forward pass) the best so far?
     const bool snapshot = u.theta_best && (!snap_have || snap_cur > snap_best);
     if (u.done) {
-        // Once every block has read the validation state and the iteration number (signalled here, before
-        // the block's own stores, so the fence has nothing to wait for), the last block to arrive books
-        // the count and moves the state on, while the others are already updating their parameters.
         __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            if (atomicAdd(u.done, 1ull) == (unsigned long long)gridDim.x - 1ull) {
-                __threadfence();
-                if (u.snap_decision) *u.snap_decision = snapshot ? 1 : 0;
-                if (u.snap_cur) {
-                    unsigned long long* slot = u.step_dev ? (u.history_base && step_now > 0 ? u.history_base + (step_now - 1) : nullptr)
-                                                          : u.rec_history_slot;
-                    if (slot) *slot = snap_cur;
-                    if (!snap_have || snap_cur > snap_best) {
-                        *u.snap_best = snap_cur;
-                        if (u.rec_best_iter) *u.rec_best_iter = u.step_dev ? (int32_t)step_now : u.rec_iter;
-                        *u.snap_have = 1;
-                    }
-                    *u.snap_cur = 0ull;
-                }
-                if (u.step_dev) *u.step_dev = step_now + 1;
-                *u.done = 0ull;
-            }
-        }
+        if (threadIdx.x == 0) update_bookkeeping(u, step_now, snap_cur, snap_best, snap_have, snapshot);
     }
-    if (blockIdx.x == 0 && threadIdx.x >= 224 && loss_out) {      // the block's last warp: not the one that signals
-        const int lane = threadIdx.x - 224;
-        float s = 0.f;
-        for (int64_t i = lane; i < u.n_loss; i += 32) s += u.loss_partial[i];
-        s = warp_sum(s);
-        if (lane == 0) *loss_out = (u.status && *u.status) ? __int_as_float(0x7fc00000) : s * u.inv_rows;
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 64 && u.status_out && u.status) *u.status_out = *u.status;
+    if (blockIdx.x == 0 && threadIdx.x >= 224) update_loss(u, step_now, threadIdx.x - 224);      // the block's last warp: not the one that signals
 
     bf16 t16 = f32_to_bf16(0.f);
     if (live) {

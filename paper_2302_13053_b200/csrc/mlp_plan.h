@@ -17,12 +17,10 @@ struct MlpPlan {
     int64_t n_rows, nt;                     // training rows; nt = parameters in theta
     int64_t n_eval;                         // rows after the training rows that are only evaluated (validation)
     int64_t ld_dl;                          // row stride of bf16 dL and of the padded W2 (classes rounded up to 64)
-    int64_t ld_h;                           // row stride of bf16 dHd and of W2^T (hidden rounded up to 64)
-    int64_t ld_h1;                          // row stride of [Hd | 1] (hidden + 1 rounded up to 64)
+    int64_t ld_h;                           // row stride of bf16 Hd, dHd and of W2^T (hidden rounded up to 64)
     int64_t ld_bits;                        // words per row of the ReLU bits (two per 64 hidden units)
     int64_t ld_k;                           // row stride of W1^T (d_in rounded up to 64)
     int64_t ld_o1;                          // row stride of the bf16 copy of W1 (out1 rounded up to 64)
-    int64_t ld_x1;                          // row stride of the workspace copy [X | 1] (d_in + 1 rounded up to 64)
     int64_t sm_blocks;                      // loss partials the workspace has room for
     int64_t split_w1, split_w2;             // split-K factors of the two weight-gradient products
     int32_t norm;                           // retexo_norm (0 where hidden == 0): f_theta = Linear -> norm -> ReLU; theta ends in
@@ -36,15 +34,16 @@ struct MlpBuffers {
     __nv_bfloat16* w1r16;                   // W1              [d_in x ld_o1]  (may be null: retexo_embed does not need it)
     __nv_bfloat16* w2t16;                   // W2^T            [n_classes x ld_h]
     __nv_bfloat16* w2p16;                   // W2, padded rows [hidden x ld_dl]
-    __nv_bfloat16* x1;                      // [X | 1]         [n x ld_x1]  (only when the caller's batch has no column of ones)
-    __nv_bfloat16* hd16;                    // [Hd | 1]        [n x ld_h1]
+    __nv_bfloat16* hd16;                    // Hd              [n x ld_h]
     float* logits;                          //                 [n x n_classes]  (retexo_embed only)
     __nv_bfloat16* dl16;                    // dL              [n x ld_dl]
     __nv_bfloat16* dhd16;                   // dHd             [n x ld_h]
     uint32_t* gate_bits;                    // [Hd > 0], a bit per unit   [n x ld_bits]
     float* loss_partial;
-    float* pw1;                             // [split_w1 x (d_in+1) x out1]   partials of [dW1 ; db1]
-    float* pw2;                             // [split_w2 x (hidden+1) x n_classes]   partials of [dW2 ; db2]
+    float* pw1;                             // [split_w1 x d_in x out1]   partials of dW1
+    float* pb1;                             // [split_w1 x shares x out1] partials of db1 (grad_bias_shares)
+    float* pw2;                             // [split_w2 x hidden x n_classes]   partials of dW2
+    float* pb2;                             // [split_w2 x shares x n_classes]   partials of db2
     int32_t* status;                        // raised by a tensor-core kernel whose bounded wait gave up
     float* z1;                              // layer / batch norm: x W1 + b1 in fp32   [n x hidden]
     float2* ln_stats;                       // layer norm: (mean, 1 / sqrt(var + eps)) per row   [n]
@@ -103,14 +102,12 @@ void mlp_step_buffers(const MlpPlan& p, void* workspace, size_t bytes, MlpBuffer
 
 // One training iteration.  shadows_ready: the bf16 weight copies in `b` already hold the
 // current theta (the previous iteration's update refreshed them), so they are not rebuilt.
-// On return they hold the updated theta.
-// x_has_ones: column d_in of x holds 1 in every row (ldx > d_in); otherwise the batch is first copied into
-// the workspace with that column added.
+// On return they hold the updated theta (keep_shadows; a caller that rebuilds them anyway spares the stores).
 int mlp_train_step_launch(const MlpPlan& p, const MlpBuffers& b, const retexo_mlp* model,
-                          const __nv_bfloat16* x, int64_t ldx, bool x_has_ones,
-                          const int32_t* y, float* loss_out, float* grad_out, bool shadows_ready,
+                          const __nv_bfloat16* x, int64_t ldx, const int32_t* y, float* loss_out, float* grad_out, bool shadows_ready,
                           const EvalTail* tail, cudaStream_t st, const DeviceIter* dev = nullptr,
-                          float* dx_out = nullptr, int64_t ld_dx = 0);      // dx_out: fp32 [n_rows x ld_dx], dLoss / dX
+                          float* dx_out = nullptr, int64_t ld_dx = 0,      // dx_out: fp32 [n_rows x ld_dx], dLoss / dX
+                          bool keep_shadows = true);
 
 // Forward + arg-max + hit count over a dense batch with the weight copies in `b` (which must
 // hold model->theta): what validation needs after every iteration.  hd_ws: bf16 [n_rows x p.ld_h];

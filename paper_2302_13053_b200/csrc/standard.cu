@@ -355,7 +355,7 @@ extern "C" int retexo_standard_train(const retexo_standard_config* cfg, const re
         const EvalTail* riding = pending_it ? &tail : nullptr;
         if (!riding) RETEXO_CUDA_TRY(cudaMemsetAsync(b.decision, 0, sizeof(int32_t), st));
         const bool want_grad = out->grad_last && it == c.R;
-        RETEXO_TRY(mlp_train_step_launch(plan, sb, &model, b.xb, b.ld_xb, true, b.y_tr, out->loss_history + (it - 1),
+        RETEXO_TRY(mlp_train_step_launch(plan, sb, &model, b.xb, b.ld_xb, b.y_tr, out->loss_history + (it - 1),
                                          want_grad ? out->grad_last[K - 1] : nullptr, it > 1, riding, st, nullptr,
                                          K > 1 ? b.dx : nullptr, b.ld_dx));
         model.step += 1;
