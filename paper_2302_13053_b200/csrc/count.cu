@@ -11,13 +11,15 @@ namespace retexo {
 constexpr int kCntThreads = 256;
 constexpr int kCntWarps = kCntThreads / kWarp;
 constexpr int kBitmapParts = 8192;                  // per-warp shared bitmap covers this many partitions
-constexpr int kBitmapWords = kBitmapParts / 32;
 constexpr int kHashSlots = 1024;                    // per-warp shared hash set
 constexpr int kHashMaxDeg = 512;                    // rows up to this length use it
 constexpr int kHashWarps = 4;
 constexpr int kBigRowBlocks = 148;                  // blocks (and global bitmaps) of the long-row pass
 constexpr int kBlockRowDeg = 4096;                  // rows longer than this go to the long-row pass at once
 constexpr int32_t kCrossCounted = INT32_MIN;        // list flag: the row's cross edges are already tallied
+constexpr int64_t kRowCost = 32;                    // what a row costs beside its edges, in edges
+constexpr int kWideRowDeg = 1024;                   // bitmap kernel: longer rows are spread over the block's warps
+constexpr int kWideRows = 64;                       //   as many of them as its list holds
 
 struct CountArgs {
     int64_t n;
@@ -47,6 +49,40 @@ __device__ __forceinline__ int64_t next_rows(const CountArgs& a, int lane) {
     return (int64_t)__shfl_sync(0xffffffffu, u, 0);
 }
 
+// A block takes the rows whose start, rowptr[u] + kRowCost u, lies in its equal share of the total: about the same number of edges
+// and rows for every block, without a counter that all warps draw from (about 2 ns a draw wherever it comes from, and draws of one or two
+// rows is what balance takes).  First row at or above `target`, found by one warp, 32 probes at a time.
+__device__ __forceinline__ int64_t first_row_from(const CountArgs& a, int64_t target, int lane) {
+    int64_t lo = 0, hi = a.n;                     // the answer is in [lo, hi]
+    while (lo < hi) {
+        const int64_t step = (hi - lo + kWarp - 1) / kWarp, u = lo + step * lane;
+        const bool below = u < hi && __ldg(a.rowptr + u) + kRowCost * u < target;
+        const int k = __popc(__ballot_sync(0xffffffffu, below));      // probes 0 .. k-1 are below
+        if (k == 0) return lo;
+        const int64_t last = lo + step * (k - 1);
+        hi = min(hi, last + step);
+        lo = last + 1;
+    }
+    return lo;
+}
+
+// The block's rows: *next counts through them (all threads of the block call this; ends with a barrier).
+__device__ __forceinline__ void block_rows(const CountArgs& a, long long* next, long long* end) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp < 2) {
+        const int64_t total = __ldg(a.rowptr + a.n) + kRowCost * a.n, share = (total + gridDim.x - 1) / gridDim.x;
+        const int64_t u = first_row_from(a, share * ((int64_t)blockIdx.x + warp), lane);
+        if (lane == 0) *(warp ? end : next) = u;
+    }
+    __syncthreads();
+}
+
+__device__ __forceinline__ int64_t next_in_block(long long* next, int lane) {
+    unsigned long long u = 0;
+    if (lane == 0) u = atomicAdd(reinterpret_cast<unsigned long long*>(next), 1ull);
+    return (int64_t)__shfl_sync(0xffffffffu, u, 0);
+}
+
 // Partition id of node x; an id outside [0, n_parts) raises the flag and is
 // replaced by 0 so that every table access stays in bounds.
 __device__ __forceinline__ int32_t part_of(const CountArgs& a, int64_t x) {
@@ -64,79 +100,125 @@ __device__ __forceinline__ unsigned long long warp_sum_u64(unsigned long long v)
     return v;
 }
 
-// Partition count <= kBitmapParts: one warp per row, the set of destination
-// partitions already seen is a bitmap in shared memory.
+// The block's totals, added up by lane 0 of its warps in shared memory first: an atomic to one address costs about 2 ns wherever it
+// comes from.  All threads of the block call this.
+__device__ __forceinline__ void add_block_sums(const CountArgs& a, unsigned long long cross, unsigned long long pairs) {
+    __shared__ unsigned long long sums[2];
+    if (threadIdx.x < 2) sums[threadIdx.x] = 0ull;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) {
+        if (cross) atomicAdd(&sums[0], cross);
+        if (pairs) atomicAdd(&sums[1], pairs);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (sums[0]) atomicAdd(a.cross_edges, sums[0]);
+        if (sums[1]) atomicAdd(a.pairs, sums[1]);
+    }
+}
+
+// Marks the partitions other than pu of entries [beg, end) in a bitmap, each `step` entries from e0 = beg + first; returns this lane's
+// number of such entries.  Four chunks of 32 entries per trip: the index loads, then the partition-id gathers, are issued together,
+// so a trip costs two memory latencies instead of eight.
+__device__ __forceinline__ unsigned mark_parts(const CountArgs& a, int64_t beg, int64_t end, int64_t step, int32_t pu, uint32_t* bm, int lane) {
+    unsigned n_cross = 0;
+    for (int64_t e0 = beg; e0 < end; e0 += step) {
+        int32_t nb[4], pv[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const int64_t e = e0 + t * kWarp + lane;
+            nb[t] = e < end ? __ldg(a.colidx + e) : -1;
+        }
+#pragma unroll
+        for (int t = 0; t < 4; ++t) pv[t] = nb[t] >= 0 ? part_of(a, nb[t]) : pu;
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+            if (pv[t] != pu) {
+                atomicOr(bm + (pv[t] >> 5), 1u << (pv[t] & 31));
+                ++n_cross;
+            }
+    }
+    return n_cross;
+}
+
+// Partition count <= 1024 W: one warp per row, the set of destination partitions is a bitmap in shared memory, W words a lane,
+// that is read and cleared once at the end of the row (with one width for all counts, clearing a row meant reading its ids again).
+// Bound by the gathers of partition ids, one 32-byte sector each, at the rate an SM's first-level cache asks the second for
+// (about one a clock): a graph of 233 k nodes and 114 M directed edges with 1000 partitions 672 -> 429 us; ids kept in shared memory instead (packed, as many as fit) measured 448 us there and twice the time on 2.4 M nodes.
+// Rows above kWideRowDeg entries are put off until the block's others are done and then shared by its warps, eight rows at a time:
+// one warp alone is the block's tail (100 k nodes, hubs of 60 k entries: 861 -> 134 us), and one row at a time leaves the block
+// waiting at barriers.  Limits of 1024, 2048 and 4096 entries: 438, 438 and 458 us on the first graph, 27, 31 and 44 us on one of 20 k nodes.
+// The grid is what the device holds at once: shares are equal, so a second wave would double the time.
+template <int W>
 __global__ void __launch_bounds__(kCntThreads) count_bitmap_kernel(CountArgs a) {
-    __shared__ uint32_t bm[kCntWarps][kBitmapWords];
+    __shared__ uint32_t bm[kCntWarps][W * kWarp];
+    __shared__ long long row_next, row_end;
+    __shared__ int32_t wide[kWideRows];
+    __shared__ int n_wide;
     // per-partition receive tally of this block (only when asked for: n_parts words of dynamic shared
     // memory), added to the global one once at the end: one global atomic per message would serialise
     // on the few hundred addresses
     extern __shared__ uint32_t recv_block[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int i = lane; i < kBitmapWords; i += kWarp) bm[warp][i] = 0u;
-    if (a.recv) {
+#pragma unroll
+    for (int i = 0; i < W; ++i) bm[warp][i * kWarp + lane] = 0u;
+    if (a.recv)
         for (int i = threadIdx.x; i < a.n_parts; i += kCntThreads) recv_block[i] = 0u;
-        __syncthreads();
-    }
-    __syncwarp();
+    if (threadIdx.x == 0) n_wide = 0;
+    block_rows(a, &row_next, &row_end);
     unsigned long long my_cross = 0, my_pairs = 0;
-    for (int64_t u0 = next_rows(a, lane); u0 < a.n; u0 = next_rows(a, lane))
-    for (int64_t u = u0; u < min(a.n, u0 + a.row_batch); ++u) {
+    // the bitmap of a finished row: counted, tallied and cleared
+    auto finish_row = [&](int32_t pu) {
+        unsigned row_new = 0;
+#pragma unroll
+        for (int i = 0; i < W; ++i) {
+            const uint32_t w = bm[warp][i * kWarp + lane];
+            bm[warp][i * kWarp + lane] = 0u;
+            row_new += __popc(w);
+            if (a.recv)
+                for (uint32_t b = w; b; b &= b - 1) atomicAdd(recv_block + ((i * kWarp + lane) * 32 + __ffs(b) - 1), 1u);
+        }
+        row_new = __reduce_add_sync(0xffffffffu, row_new);
+        if (lane == 0 && row_new) {
+            my_pairs += row_new;
+            if (a.send) atomicAdd(a.send + pu, (unsigned long long)row_new);
+        }
+    };
+    const int64_t end_row = row_end;
+    for (int64_t u = next_in_block(&row_next, lane); u < end_row; u = next_in_block(&row_next, lane)) {
         const int64_t beg = a.rowptr[u], end = a.rowptr[u + 1];
         if (beg == end) continue;
+        if (end - beg > kWideRowDeg) {
+            int slot = 0;
+            if (lane == 0) slot = atomicAdd(&n_wide, 1);
+            slot = __shfl_sync(0xffffffffu, slot, 0);
+            if (slot < kWideRows) {
+                if (lane == 0) wide[slot] = (int32_t)u;
+                continue;
+            }
+        }
         const int32_t pu = part_of(a, u);
-        unsigned row_new = 0;
-        // four chunks of 32 entries per trip: the index loads, then the partition-id gathers, are
-        // issued together, so a trip costs two memory latencies instead of eight
-        for (int64_t e0 = beg; e0 < end; e0 += 4 * kWarp) {
-            int32_t nb[4], pv[4];
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                const int64_t e = e0 + t * kWarp + lane;
-                nb[t] = e < end ? __ldg(a.colidx + e) : -1;
-            }
-#pragma unroll
-            for (int t = 0; t < 4; ++t) pv[t] = nb[t] >= 0 ? part_of(a, nb[t]) : pu;
-#pragma unroll
-            for (int t = 0; t < 4; ++t) {
-                const bool cross = pv[t] != pu;
-                bool is_new = false;
-                if (cross) {
-                    const uint32_t bit = 1u << (pv[t] & 31);
-                    const uint32_t old = atomicOr(&bm[warp][pv[t] >> 5], bit);
-                    is_new = !(old & bit);
-                    if (is_new && a.recv) atomicAdd(&recv_block[pv[t]], 1u);
-                }
-                my_cross += cross ? 1ull : 0ull;
-                row_new += __popc(__ballot_sync(0xffffffffu, is_new));
-            }
-        }
+        my_cross += mark_parts(a, beg, end, 4 * kWarp, pu, bm[warp], lane);
         __syncwarp();
-        // clear the touched words again
-        if (end - beg >= kBitmapWords) {
-            for (int i = lane; i < kBitmapWords; i += kWarp) bm[warp][i] = 0u;
-        } else {
-            for (int64_t e = beg + lane; e < end; e += kWarp) {
-                const int32_t pv = part_of(a, __ldg(a.colidx + e));
-                bm[warp][pv >> 5] = 0u;
-            }
-        }
+        finish_row(pu);
         __syncwarp();
-        if (lane == 0) {
-            my_pairs += row_new;
-            if (a.send && row_new) atomicAdd(a.send + pu, (unsigned long long)row_new);
+    }
+    __syncthreads();
+    // long rows, kCntWarps at a time: every warp marks its part of each, then each warp finishes one
+    for (int r0 = 0; r0 < min(n_wide, kWideRows); r0 += kCntWarps) {
+        const int rows = min(min(n_wide, kWideRows) - r0, kCntWarps);
+        for (int k = 0; k < rows; ++k) {
+            const int64_t u = wide[r0 + k], beg = a.rowptr[u], end = a.rowptr[u + 1];
+            my_cross += mark_parts(a, beg + (warp + k) % kCntWarps * 4 * kWarp, end, 4 * kCntThreads, part_of(a, u), bm[k], lane);
         }
-    }
-    my_cross = warp_sum_u64(my_cross);
-    if (lane == 0) {
-        if (my_cross) atomicAdd(a.cross_edges, my_cross);
-        if (my_pairs) atomicAdd(a.pairs, my_pairs);
-    }
-    if (a.recv) {
         __syncthreads();
+        if (warp < rows) finish_row(part_of(a, wide[r0 + warp]));
+        __syncthreads();
+    }
+    add_block_sums(a, warp_sum_u64(my_cross), my_pairs);
+    if (a.recv)
         for (int i = threadIdx.x; i < a.n_parts; i += kCntThreads)
             if (recv_block[i]) atomicAdd(a.recv + i, (unsigned long long)recv_block[i]);
-    }
 }
 
 __device__ __forceinline__ uint32_t hash32(uint32_t x) {
@@ -245,10 +327,7 @@ __global__ void __launch_bounds__(kHashWarps * kWarp) count_general_kernel(Count
             if (a.send && n_new) atomicAdd(a.send + pu, (unsigned long long)n_new);
         }
     }
-    if (lane == 0) {
-        if (my_cross) atomicAdd(a.cross_edges, my_cross);
-        if (my_pairs) atomicAdd(a.pairs, my_pairs);
-    }
+    add_block_sums(a, my_cross, my_pairs);
 }
 
 // Long unordered rows with many partitions: one block per row, the seen-set is
@@ -456,12 +535,12 @@ extern "C" int retexo_cross_partition_bytes(const retexo_csr* g, const int32_t* 
     if (a.n > 0) {
         if (n_parts <= kBitmapParts) {
             const int64_t want = (a.n + kCntWarps - 1) / kCntWarps;
-            const unsigned blocks = (unsigned)(want < (int64_t)n_sm * 8 ? want : (int64_t)n_sm * 8);
-            // ~16 draws per warp: fine enough to balance hub rows, coarse enough for the counter
-            const int64_t batch = a.n / ((int64_t)blocks * kCntWarps * 16);
-            a.row_batch = (int32_t)(batch < 1 ? 1 : batch > 64 ? 64 : batch);
             const size_t tally = a.recv ? sizeof(uint32_t) * (size_t)n_parts : 0;      // <= 32 KB
-            count_bitmap_kernel<<<blocks, kCntThreads, tally, st>>>(a);
+            const auto kernel = n_parts <= 1024 ? count_bitmap_kernel<1> : n_parts <= 2048 ? count_bitmap_kernel<2>
+                              : n_parts <= 4096 ? count_bitmap_kernel<4> : count_bitmap_kernel<8>;
+            int resident = 0;
+            RETEXO_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, kernel, kCntThreads, tally));
+            kernel<<<(unsigned)(want < (int64_t)n_sm * resident ? want : (int64_t)n_sm * resident), kCntThreads, tally, st>>>(a);
         } else {
             a.big_list = ws.take<int32_t>((size_t)a.n);
             a.big_count = ws.take<int32_t>(64);

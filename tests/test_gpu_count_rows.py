@@ -1,0 +1,18 @@
+"""The bitmap kernel of the cross-partition count at the edges of its dispatch: bitmap widths (1024, 2048, 4096 and 8192
+partitions), rows around the 128-entry trip and the 1024-entry limit above which a block shares a row, rows without entries."""
+import numpy as np
+import pytest
+
+from paper_2302_13053_b200 import workloads as wl
+from test_gpu_counts import compare
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("n_parts", [1024, 1025, 2049, 4096, 4097])
+def test_row_lengths_around_the_limits(n_parts):
+    rng = np.random.default_rng(n_parts)
+    for degrees in ([1], [0, 1, 31, 127, 128, 129, 1023], [1024, 1025, 2047, 2048, 5000] + [1100] * 20):
+        n, rowptr, colidx, _ = wl.degree_ladder_graph(degrees, seed=n_parts)
+        compare(rowptr, colidx, rng.integers(0, n_parts, n).astype(np.int32), n_parts)
+        compare(rowptr, colidx, np.full(n, n_parts - 1, dtype=np.int32), n_parts)
