@@ -320,8 +320,8 @@ def retexo_mlp_train_step(model: Mlp, x: torch.Tensor, y: torch.Tensor, x_has_on
     assert x.dtype == torch.bfloat16 and y.dtype == torch.int32 and x.stride(1) == 1
     n_rows = x.shape[0]
     dev = x.device
-    loss = torch.zeros((), dtype=torch.float32, device=dev)
-    grad = torch.zeros_like(model.theta) if return_grad else None
+    loss = torch.empty((), dtype=torch.float32, device=dev)
+    grad = torch.empty_like(model.theta) if return_grad else None      # (the call writes every entry)
     dx = torch.empty((n_rows, model.d_in), dtype=torch.float32, device=dev) if return_dx else None
     need = lib().retexo_mlp_train_step_workspace_size_norm(C.c_int32(model.d_in), C.c_int32(model.hidden),
                                                          C.c_int32(model.n_classes), C.c_int64(n_rows),
@@ -370,23 +370,24 @@ def retexo_cross_partition_bytes(rowptr: torch.Tensor, colidx: torch.Tensor, par
     n = rowptr.numel() - 1
     K = len(dims)
     g = _csr(rowptr, colidx)
-    scal = torch.zeros(3 + max(K, 1), dtype=torch.int64, device=dev)   # cross, pairs, total, per round...
-    send = torch.zeros(n_parts, dtype=torch.int64, device=dev) if per_part else None
-    recv = torch.zeros(n_parts, dtype=torch.int64, device=dev) if per_part else None
+    # cross, pairs, total, per round..., then sent and received per part: all written by the call, and read back in one copy
+    out = torch.empty(3 + K + (2 * n_parts if per_part else 0), dtype=torch.int64, device=dev)
+    send = C.c_void_p(out.data_ptr() + 8 * (3 + K)) if per_part else None
+    recv = C.c_void_p(out.data_ptr() + 8 * (3 + K + n_parts)) if per_part else None
     dims_a = (C.c_int32 * max(K, 1))(*[int(d) for d in dims])
     need = lib().retexo_cross_partition_workspace_size(C.c_int64(n), C.c_int64(colidx.numel()), C.c_int32(n_parts))
     ws = _workspace(need, dev)
-    base = scal.data_ptr()
+    base = out.data_ptr()
     rc = lib().retexo_cross_partition_bytes(C.byref(g), _ptr(part), C.c_int32(n_parts), C.c_int32(K), dims_a,
                                             C.c_int32(elem_bytes), C.c_void_p(base), C.c_void_p(base + 8),
-                                            C.c_void_p(base + 24), C.c_void_p(base + 16), _ptr(send), _ptr(recv),
+                                            C.c_void_p(base + 24) if K else None, C.c_void_p(base + 16), send, recv,
                                             _ptr(ws), C.c_size_t(ws.numel()), _stream())
     _check(rc, "retexo_cross_partition_bytes")
-    s = scal.cpu().numpy().view(np.uint64)
+    s = out.cpu().numpy().view(np.uint64)
     return dict(cross_edges=int(s[0]), boundary_pairs=int(s[1]), bytes_total=int(s[2]),
                 bytes_per_round=s[3:3 + K].copy(), dv_lazy_lt=2 * int(s[2]),
-                send_per_part=None if send is None else send.cpu().numpy().view(np.uint64),
-                recv_per_part=None if recv is None else recv.cpu().numpy().view(np.uint64))
+                send_per_part=s[3 + K:3 + K + n_parts] if per_part else None,
+                recv_per_part=s[3 + K + n_parts:] if per_part else None)
 
 
 def retexo_cross_partition_bytes_static(rowptr: torch.Tensor, colidx: torch.Tensor, part: torch.Tensor, n_parts: int,
