@@ -197,8 +197,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     constexpr int kTileRows = PAIR ? 2 * kTcBM : kTcBM;
     static_assert(!PAIR || (MODE != TC_EPI_PARTIAL && BN == 256 && TG == 1), "pairs: K-major 256-column tiles");
     const uint32_t pair_rank = PAIR ? cluster_rank() : 0u;
-    const int64_t tile_first = PAIR ? (int64_t)(blockIdx.x >> 1) : (int64_t)blockIdx.x;
-    const int64_t tile_stride = PAIR ? (int64_t)(gridDim.x >> 1) : (int64_t)gridDim.x;
+    // (tiles are counted in 32 bits: rows are, and a 64-bit division costs a tenth of a microsecond before the first load)
+    const int32_t tile_first = (int32_t)(PAIR ? blockIdx.x >> 1 : blockIdx.x), tile_stride = (int32_t)(PAIR ? gridDim.x >> 1 : gridDim.x);
     // The split-K products reduce over the batch, and their operands (activations and gradients, one batch row
     // per line) are read as they lie in memory: M and N are the contiguous dimensions ("MN-major" operands).
     constexpr bool kMnMajor = MODE == TC_EPI_PARTIAL;
@@ -216,9 +216,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     float (*xch_all)[2][128] = reinterpret_cast<float (*)[2][128]>(stage_base + EW * kStageBytesPerWarp);   // [TG][4][2][128]
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t n_m = (g.M + kTileRows - 1) / kTileRows, n_n = (g.N + BN - 1) / BN;
-    const int64_t per_split = n_m * n_n;
-    const int64_t n_tiles = per_split * g.splits;
+    const int32_t n_m = (int32_t)((g.M + kTileRows - 1) / kTileRows), n_n = (int32_t)((g.N + BN - 1) / BN);
+    const int32_t per_split = n_m * n_n;
+    const int32_t n_tiles = per_split * g.splits;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { mbar_init(full + s, 1); mbar_init(empty + s, 1); }
@@ -229,6 +229,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (threadIdx.x == 32) { prefetch_map(&map_a); prefetch_map(&map_b); }
     if (warp == 1) {      // tensor memory: NACC accumulators of BN fp32 columns x 128 lanes
         if constexpr (PAIR) {
             asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(NACC * BN));
@@ -250,10 +251,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         if (lane == 0) {
             int64_t it = 0;                       // k-blocks issued so far, over all tiles
             bool ok = true;
-            for (int64_t t = tile_first; t < n_tiles && ok; t += tile_stride) {
-                const int64_t z = t / per_split, rem = t % per_split;
+            for (int32_t t = tile_first; t < n_tiles && ok; t += tile_stride) {
+                const int32_t z = t / per_split, rem = t % per_split;
                 const int32_t m0 = (int32_t)((rem % n_m) * kTileRows + pair_rank * kTcBM), n0 = (int32_t)((rem / n_m) * BN);
-                const int32_t kb0 = (int32_t)z * g.k_blocks_per_split;
+                const int32_t kb0 = z * g.k_blocks_per_split;
                 const int32_t kb1 = min(g.k_blocks_total, kb0 + g.k_blocks_per_split);
                 for (int32_t kb = kb0; kb < kb1; ++kb, ++it) {
                     const int s = (int)(it % STAGES);
@@ -295,9 +296,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             constexpr uint32_t idesc = make_idesc(BN, kMnMajor, kMnMajor, kTileRows);
             int64_t it = 0, lt = 0;               // k-blocks consumed, tiles done by this block
             bool ok = true;
-            for (int64_t t = tile_first; t < n_tiles && ok; t += tile_stride, ++lt) {
-                const int64_t z = t / per_split;
-                const int32_t kb0 = (int32_t)z * g.k_blocks_per_split;
+            for (int32_t t = tile_first; t < n_tiles && ok; t += tile_stride, ++lt) {
+                const int32_t z = t / per_split;
+                const int32_t kb0 = z * g.k_blocks_per_split;
                 const int32_t kb1 = min(g.k_blocks_total, kb0 + g.k_blocks_per_split);
                 const int b = (int)(lt % NACC);
                 const uint32_t pb = (uint32_t)(lt / NACC) & 1;
@@ -359,11 +360,11 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         // gated epilogue: the gate block of the next chunk is fetched while the current chunk is processed
         uint4 gate_next[4];
         bool gate_have = false;
-        [[maybe_unused]] auto gate_prefetch = [&](int64_t tile, int c0) {
+        [[maybe_unused]] auto gate_prefetch = [&](int32_t tile, int c0) {
             gate_have = false;
             if (tile >= n_tiles) return;
-            const int64_t rem = tile % per_split;
-            const int64_t r0 = (rem % n_m) * kTcBM + q * 32, cc0 = (rem / n_m) * BN + c0;
+            const int32_t rem = tile % per_split;
+            const int64_t r0 = (int64_t)(rem % n_m) * kTcBM + q * 32, cc0 = (int64_t)(rem / n_m) * BN + c0;
             if (!rows_map || r0 >= g.M || cc0 + 32 > g.N || (g.ld_mask & 7) != 0 || !aligned16(g.mask)) return;
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -374,14 +375,14 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
             }
             gate_have = true;
         };
-        if constexpr (kGated) gate_prefetch(tile_first + (int64_t)gi * tile_stride, half * kPartCols);
+        if constexpr (kGated) gate_prefetch(tile_first + gi * tile_stride, half * kPartCols);
         int64_t lt = gi;
-        for (int64_t t = tile_first + (int64_t)gi * tile_stride; t < n_tiles && !(row_owner && half == 1);
-             t += (int64_t)TG * tile_stride, lt += TG) {
-            const int64_t z = t / per_split, rem = t % per_split;
-            const int64_t mt = rem % n_m;
-            const int64_t m0 = mt * kTileRows + (int64_t)pair_rank * kTcBM, n0 = (rem / n_m) * BN;
-            const int32_t kb0 = (int32_t)z * g.k_blocks_per_split;
+        for (int32_t t = tile_first + gi * tile_stride; t < n_tiles && !(row_owner && half == 1);
+             t += TG * tile_stride, lt += TG) {
+            const int32_t z = t / per_split, rem = t % per_split;
+            const int32_t mt = rem % n_m;
+            const int64_t m0 = (int64_t)mt * kTileRows + (int64_t)pair_rank * kTcBM, n0 = (int64_t)(rem / n_m) * BN;
+            const int32_t kb0 = z * g.k_blocks_per_split;
             const int32_t n_kb = min(g.k_blocks_total, kb0 + g.k_blocks_per_split) - kb0;
             const int b = (int)(lt % NACC);
             const uint32_t pb = (uint32_t)(lt / NACC) & 1;
@@ -567,7 +568,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 #pragma unroll
                         for (int i = 0; i < 4; ++i) gate_cur[i] = gate_next[i];
                         if (c0 + 32 < c_end) gate_prefetch(t, c0 + 32);
-                        else gate_prefetch(t + (int64_t)TG * tile_stride, c_begin);
+                        else gate_prefetch(t + TG * tile_stride, c_begin);
                         if (gate_runs && out_map) {
                             // the two staging blocks take turns: the bulk store issued two chunks ago has read this one
                             flip ^= 1;

@@ -69,6 +69,7 @@ grad_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant__ 
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (threadIdx.x == 32) { prefetch_map(&map_a0); prefetch_map(&map_b0); if (g.p[1].tiles) { prefetch_map(&map_a1); prefetch_map(&map_b1); } }
     if (warp == 1) {      // tensor memory: the tile's accumulator and the bias row's, BN columns each
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(2 * BN));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");

@@ -85,16 +85,22 @@ head_backward_kernel(const __grid_constant__ CUtensorMap map_hd, const __grid_co
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (threadIdx.x == 32) { prefetch_map(&map_hd); prefetch_map(&map_dl); prefetch_map(&map_dhd); }
     if (warp == 1) {      // all of tensor memory: two logit accumulators of 64 columns, one gradient accumulator of 256
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
-    grid_dependency_wait();          // everything from here on may read what the previous kernel wrote
-    grid_dependency_release();
+    // the weights are older than the kernel that this one overlaps (it wrote Hd): they need not wait for it
+    if (threadIdx.x == 0 && nt > 0) {
+        mbar_expect_tx(bars + HB_W2_FULL, (uint32_t)np * kHbW2PanelBytes);
+        for (int p = 0; p < np; ++p) tma_load_2d(w2_s + p * kHbW2PanelBytes, &map_w2, 64 * p, 0, bars + HB_W2_FULL);
+    }
     if (threadIdx.x >= 64 && threadIdx.x < 128) {
         const int c = threadIdx.x - 64;
         bias_s[c] = (g.b2 && c < g.O) ? g.b2[c] : 0.f;
     }
+    grid_dependency_wait();          // everything from here on may read what the previous kernel wrote
+    grid_dependency_release();
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -102,8 +108,6 @@ head_backward_kernel(const __grid_constant__ CUtensorMap map_hd, const __grid_co
 
     if (warp == 0) {
         if (lane == 0 && nt > 0) {
-            mbar_expect_tx(bars + HB_W2_FULL, (uint32_t)np * kHbW2PanelBytes);
-            for (int p = 0; p < np; ++p) tma_load_2d(w2_s + p * kHbW2PanelBytes, &map_w2, 64 * p, 0, bars + HB_W2_FULL);
             int64_t issued = 0;
             for (int64_t i = 0; i < nt; ++i) {
                 const int b = (int)(i & 1);

@@ -268,9 +268,8 @@ __global__ void __launch_bounds__(256, BATCH == 16 ? 4 : 2) reduce_update_kernel
     const bool adam = u.optimizer != RETEXO_SGD;
     const bool state = sidx == 2 && row >= 2;      // a running statistic of batch normalisation
 
-    grid_dependency_wait();
-    grid_dependency_release();
-    // ---- loads with no dependence
+    // ---- what is older than the kernel before this one (it wrote the partials): the parameters, their moments and the iteration
+    // state, left by the previous update, and the validation count of this iteration's forward pass
     unsigned long long step_now = 0, snap_cur = 0, snap_best = 0;
     int32_t snap_have = 1;
     if (u.step_dev) step_now = *u.step_dev;
@@ -278,17 +277,8 @@ __global__ void __launch_bounds__(256, BATCH == 16 ? 4 : 2) reduce_update_kernel
     float theta = 0.f, m = 0.f, v = 0.f, g = 0.f;
     if (live) {
         theta = u.theta[p];
-        if (state) {
-            g = u.bn_batch[q - 2 * (int64_t)cols] * (row == 3 ? u.bn_unbias : 1.f);      // the statistic it moves towards
-        } else {
-            if (adam) { m = u.m[p]; v = u.v[p]; }
-            const GradSeg& seg = u.seg[sidx];
-            if (seg.bias_partial && row == rows - 1) g = sum_partials<BATCH>(seg.bias_partial + col, (int32_t)seg.bias_count, cols);
-            else      // (a partial of the third segment holds its two trained rows)
-                g = sum_partials<BATCH>(seg.partial + q, (int32_t)seg.count, sidx == 2 ? 2 * (int64_t)cols : seg.bias_partial ? size - cols : size);
-        }
+        if (!state && adam) { m = u.m[p]; v = u.v[p]; }
     }
-
     float corr1 = u.corr1, corr2 = u.corr2;
     if (u.step_dev) {      // the iteration number lives on the device: bias corrections follow from it
         __shared__ float corr_s[2];
@@ -297,6 +287,19 @@ __global__ void __launch_bounds__(256, BATCH == 16 ? 4 : 2) reduce_update_kernel
         __syncthreads();
         corr1 = corr_s[0]; corr2 = corr_s[1];
     }
+    grid_dependency_wait();
+    grid_dependency_release();
+    if (live) {
+        if (state) {
+            g = u.bn_batch[q - 2 * (int64_t)cols] * (row == 3 ? u.bn_unbias : 1.f);      // the statistic it moves towards
+        } else {
+            const GradSeg& seg = u.seg[sidx];
+            if (seg.bias_partial && row == rows - 1) g = sum_partials<BATCH>(seg.bias_partial + col, (int32_t)seg.bias_count, cols);
+            else      // (a partial of the third segment holds its two trained rows)
+                g = sum_partials<BATCH>(seg.partial + q, (int32_t)seg.count, sidx == 2 ? 2 * (int64_t)cols : seg.bias_partial ? size - cols : size);
+        }
+    }
+
     // keep-the-best: are the weights as they stand (validated in this iteration's forward pass) the best so far?
     const bool snapshot = u.theta_best && (!snap_have || snap_cur > snap_best);
     if (u.done) {
