@@ -503,11 +503,23 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 float bv = v[0];
 #pragma unroll
                 for (int c = 1; c < 64; ++c) if (v[c] > bv) { bv = v[c]; best = c; }   // strict: lowest index wins ties
-                if (live) {
-                    if (g.pred) g.pred[row] = best;
-                    if (g.out_f32) {
+                if (live && g.pred) g.pred[row] = best;
+                if (g.out_f32) {
+                    // Rows leave whole, 32 columns at a time, over the warp's staging block (column j of row r in word j ^ r: no bank
+                    // twice either way).  A thread storing its own row touches 32 lines per store: the logits and classes of 55703
+                    // rows and 41 classes, in two launches, 37.6 -> 33.5 us.
+                    float* st = reinterpret_cast<float*>(stage);
 #pragma unroll
-                        for (int c = 0; c < 64; ++c) if (c < g.N) g.out_f32[row * g.ld_f32 + c] = v[c];
+                    for (int h = 0; h < 64; h += 32) {
+                        if (h >= g.N) break;
+                        __syncwarp();
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) st[lane * 32 + (j ^ lane)] = v[h + j];
+                        __syncwarp();
+                        float* dst = g.out_f32 + row0 * g.ld_f32 + h + lane;
+                        const int n_lines = (int)min((int64_t)32, g.M - row0);
+                        if (h + lane < g.N)
+                            for (int r = 0; r < n_lines; ++r) dst[r * g.ld_f32] = st[r * 32 + (lane ^ r)];
                     }
                 }
                 if (g.correct) {
