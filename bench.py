@@ -212,10 +212,12 @@ def launches_per_step(w, R: int) -> int:
 
 
 def shared_launches(w, R: int) -> int:
-    """Of launches_per_step's kernels, those that share a launch: an iteration's two weight-gradient products and, wherever
-    the weight copies are built, both layers'."""
+    """Of launches_per_step's kernels, those that share a launch: an iteration's two weight-gradient products, wherever the
+    weight copies are built both layers', and a trained aggregator's scatter and kept copy."""
+    from paper_2302_13053_b200 import workloads as wl
     per_round = R + 1 + 2 + 1                        # iterations, the round's first copies, two test passes, the emission
-    return per_round * sum(1 for rd in w.round_dims() if rd["hidden"] > 0)
+    total = per_round * sum(1 for rd in w.round_dims() if rd["hidden"] > 0)
+    return total + (R * w.K if w.aggr == wl.GAT and not FREEZE_ATTENTION else 0)
 
 
 def time_calls(fn, reps: int, warm: int = 3):

@@ -44,18 +44,24 @@ __global__ void record_validation_kernel(const unsigned long long* cur, unsigned
     }
 }
 // dz[idx[i]][0 .. dim) = dx[i][0 .. dim): the batch-ordered input gradient goes back to node order.
+// Blocks from scatter_blocks on: att_best = att if *decision is set (the trained aggregator's parameters follow theta into the
+// kept copy).  One launch for both: each is a few hundred kilobytes, so a launch of its own is what it costs (a run of 100 trained
+// iterations 15.18 ms with two, 15.00 with one).  vec: four columns a thread.
 __global__ void scatter_rows_kernel(const float* __restrict__ dx, int64_t ld_dx, const int32_t* __restrict__ idx,
-                                    int64_t n_rows, int32_t dim, float* __restrict__ dz, int64_t ld_dz) {
+                                    int64_t n_rows, int32_t dim, int vec, float* __restrict__ dz, int64_t ld_dz, unsigned scatter_blocks,
+                                    const int32_t* __restrict__ decision, const float* __restrict__ att, float* __restrict__ att_best, int64_t n_att) {
+    if (blockIdx.x >= scatter_blocks) {
+        const int64_t p = (blockIdx.x - scatter_blocks) * 256ll + threadIdx.x;
+        if (p < n_att && *decision) att_best[p] = att[p];
+        return;
+    }
     const int64_t t = blockIdx.x * 256ll + threadIdx.x;
-    const int64_t i = t / dim;
-    const int32_t c = (int32_t)(t % dim);
-    if (i < n_rows) dz[(int64_t)idx[i] * ld_dz + c] = dx[i * ld_dx + c];
-}
-// dst = src if *decision is set (the trained aggregator's parameters follow theta into the kept copy).
-__global__ void copy_if_kernel(const int32_t* decision, const float* src, float* dst, int64_t n) {
-    if (!*decision) return;
-    const int64_t p = blockIdx.x * 256ll + threadIdx.x;
-    if (p < n) dst[p] = src[p];
+    const int32_t per_row = vec ? dim >> 2 : dim;
+    const int64_t i = t / per_row;
+    const int32_t c = (int32_t)(t % per_row);
+    if (i >= n_rows) return;
+    if (vec) reinterpret_cast<float4*>(dz + (int64_t)idx[i] * ld_dz)[c] = reinterpret_cast<const float4*>(dx + i * ld_dx)[c];
+    else dz[(int64_t)idx[i] * ld_dz + c] = dx[i * ld_dx + c];
 }
 // One optimiser update of the aggregator's parameters [W_att | a_src | a_dst]: the gradient of W_att is the
 // sum of split-K partials (added in index order), those of the attention vectors come ready-made.
@@ -534,8 +540,10 @@ extern "C" int retexo_lmp_train(const retexo_lmp_config* cfg, const retexo_lmp_i
         // before the step, projection + aggregation + batches; after it, the kept copy follows theta's, the
         // input gradient goes back through the attention, and [W_att | a_src | a_dst] take their update.
         auto gat_backward_and_update = [&]() -> int {
-            copy_if_kernel<<<(unsigned)((n_att + 255) / 256), 256, 0, st>>>(b.decision, b.att, b.att_best, n_att);
-            scatter_rows_kernel<<<(unsigned)((n_tr * hd + 255) / 256), 256, 0, st>>>(b.dx, ld_dx, train_idx, n_tr, hd, b.dz, ldp);
+            const int vec = hd % 4 == 0 && ld_dx % 4 == 0 && ldp % 4 == 0;      // (the buffers start on 256-byte boundaries)
+            const unsigned scatter_blocks = (unsigned)((n_tr * (vec ? hd / 4 : hd) + 255) / 256);
+            scatter_rows_kernel<<<scatter_blocks + (unsigned)((n_att + 255) / 256), 256, 0, st>>>(
+                b.dx, ld_dx, train_idx, n_tr, hd, vec, b.dz, ldp, scatter_blocks, b.decision, b.att, b.att_best, n_att);
             retexo_gat_params gp;
             gp.heads = c.gat_heads; gp.head_dim = c.gat_head_dim; gp.a_src = b.att + (int64_t)r.rep_dim * hd;
             gp.a_dst = gp.a_src + hd; gp.negative_slope = c.gat_negative_slope; gp.add_self_loop = 1;
