@@ -43,7 +43,7 @@ struct GatState {
 #pragma unroll
         for (int o = LPG; o < kWarp; o <<= 1) {
             const float big = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-            const float f = exp2_rel(m, big);
+            const float f = exp_rel(m, big);
             l *= f;
             acc.scale(f);
             l += __shfl_xor_sync(0xffffffffu, l, o);
@@ -61,10 +61,10 @@ struct GatForwardPass {
     const float* p;            // this lane's columns of row 0
     const float* s;            // this lane's head of node 0
     int head;
-    float tv, k_neg;
+    float tv;
     GatState<W> st;
     __device__ __forceinline__ GatForwardPass(const GatArgs& a_, const GatLanes<LPG, W>& L)
-        : a(a_), p(a_.p + L.col), s(a_.s + L.head), head(L.head), k_neg(a_.slope * kLog2E) {}
+        : a(a_), p(a_.p + L.col), s(a_.s + L.head), head(L.head) {}
     __device__ __forceinline__ void begin(int64_t v) {
         tv = __ldg(a.t + v * a.heads + head);
         st.clear();
@@ -81,17 +81,17 @@ struct GatForwardPass {
         float big = st.m;
 #pragma unroll
         for (int t = 0; t < U; ++t) {
-            e[t] = ok[t] ? leaky2(e[t] + tv, kLog2E, k_neg) : -INFINITY;
+            e[t] = ok[t] ? leaky(e[t] + tv, a.slope) : -INFINITY;
             big = fmaxf(big, e[t]);
         }
-        const float f = exp2_rel(st.m, big);
+        const float f = exp_rel(st.m, big);
         const float ref = big == -INFINITY ? 0.f : big;         // (a group without entries yet)
         st.m = big;
         st.l *= f;
         st.acc.scale(f);
 #pragma unroll
         for (int t = 0; t < U; ++t) {
-            const float w = exp2_hw(e[t] - ref);
+            const float w = exp_below(e[t], ref);
             st.l += w;
             st.acc.fma(w, x[t]);
         }
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(kGatThreads, kGatBlocksPerSm) gat_lane_rows_ke
             Cols<W> z;
             z.zero();
             for (int w = 0; w < kGatWarps; ++w) {
-                const float f = exp2_rel(sm_ml[turn][w][L.li].x, big);                 // (0 for a warp without trips)
+                const float f = exp_rel(sm_ml[turn][w][L.li].x, big);                 // (0 for a warp without trips)
                 den = fmaf(sm_ml[turn][w][L.li].y, f, den);
                 z.fma(f, sm_acc[turn][w][L.li]);
             }

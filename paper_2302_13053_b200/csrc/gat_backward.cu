@@ -30,7 +30,7 @@ struct GatBwdArgs {
     float slope; int32_t self_loop;
     const float* dz; int64_t lddz;
     float* s; float* t;              // [n x heads]
-    float4* stats;                   // [n x heads]: (row maximum (lane layout: / ln 2), 1 / soft-max sum (0 = dz_v is zero), c_v, dt_v; lane layout: t_v)
+    float4* stats;                   // [n x heads]: (row maximum, 1 / soft-max sum (0 = dz_v is zero), c_v, dt_v; lane layout: t_v)
     float* dp; int64_t lddp;
     __nv_bfloat16* dp16; int64_t lddp16;
     float* partial;                  // [blocks x 2 x dim]: per-block sums of ds_u p_u and dt_u p_u
@@ -258,10 +258,10 @@ struct GatDstPass {
     const float* s;
     int head, col;
     bool on;
-    float tv, k_neg, m, den, c, b1, b2;
+    float tv, m, den, c, b1, b2;
     Cols<W> g;
     __device__ __forceinline__ GatDstPass(const GatBwdArgs& a_, const GatLanes<LPG, W>& L)
-        : a(a_), p(a_.p + L.col), s(a_.s + L.head), head(L.head), col(L.col), on(L.on), k_neg(a_.slope * kLog2E) {}
+        : a(a_), p(a_.p + L.col), s(a_.s + L.head), head(L.head), col(L.col), on(L.on) {}
     // Returns whether this lane's part of the gradient has a non-zero entry.
     __device__ __forceinline__ bool begin(int64_t v) {
         tv = __ldg(a.t + v * a.heads + head);
@@ -285,15 +285,15 @@ struct GatDstPass {
 #pragma unroll
         for (int t = 0; t < U; ++t) {
             z[t] += tv;
-            e[t] = ok[t] ? leaky2(z[t], kLog2E, k_neg) : -INFINITY;
+            e[t] = ok[t] ? leaky(z[t], a.slope) : -INFINITY;
             big = fmaxf(big, e[t]);
         }
-        const float f = exp2_rel(m, big), ref = big == -INFINITY ? 0.f : big;
+        const float f = exp_rel(m, big), ref = big == -INFINITY ? 0.f : big;
         m = big;
         den *= f; c *= f; b1 *= f; b2 *= f;
 #pragma unroll
         for (int t = 0; t < U; ++t) {
-            const float w = exp2_hw(e[t] - ref), wg = z[t] > 0.f ? w : w * a.slope, d = g.dot(x[t]);
+            const float w = exp_below(e[t], ref), wg = z[t] > 0.f ? w : w * a.slope, d = g.dot(x[t]);
             den += w;
             b2 += wg;
             c = fmaf(w, d, c);
@@ -301,7 +301,7 @@ struct GatDstPass {
         }
     }
     __device__ __forceinline__ void merge(float m2, float den2, float c2, float b12, float b22) {
-        const float big = fmaxf(m, m2), f = exp2_rel(m, big), f2 = exp2_rel(m2, big);
+        const float big = fmaxf(m, m2), f = exp_rel(m, big), f2 = exp_rel(m2, big);
         den = den * f + den2 * f2; c = c * f + c2 * f2; b1 = b1 * f + b12 * f2; b2 = b2 * f + b22 * f2;
         m = big;
     }
@@ -405,10 +405,10 @@ struct GatSrcPass {
     const float* dz;
     const float4* stats;
     int head, col;
-    float su, k_neg, ds, dc;            // ds: sum alpha g' <dz_v, p_u> over this lane's columns; dc: sum alpha g' c_v
+    float su, ds, dc;            // ds: sum alpha g' <dz_v, p_u> over this lane's columns; dc: sum alpha g' c_v
     Cols<W> px, acc;
     __device__ __forceinline__ GatSrcPass(const GatBwdArgs& a_, const GatLanes<LPG, W>& L)
-        : a(a_), dz(a_.dz + L.col), stats(a_.stats + L.head), head(L.head), col(L.col), k_neg(a_.slope * kLog2E) {}
+        : a(a_), dz(a_.dz + L.col), stats(a_.stats + L.head), head(L.head), col(L.col) {}
     __device__ __forceinline__ void begin(int64_t u) {
         su = __ldg(a.s + u * a.heads + head);
         px.load(a.p + u * a.ldp + col);
@@ -432,7 +432,7 @@ struct GatSrcPass {
 #pragma unroll
         for (int t = 0; t < U; ++t) {
             const float z = su + st[t].w;
-            const float alpha = st[t].y != 0.f ? exp2_hw(leaky2(z, kLog2E, k_neg) - st[t].x) * st[t].y : 0.f;
+            const float alpha = st[t].y != 0.f ? exp_below(leaky(z, a.slope), st[t].x) * st[t].y : 0.f;
             const float ag = z > 0.f ? alpha : alpha * a.slope;
             ds = fmaf(ag, px.dot(g[t]), ds);
             dc = fmaf(ag, st[t].z, dc);

@@ -133,19 +133,19 @@ struct Cols {
     }
 };
 
-// LeakyReLU(z) / ln 2 with k_pos = 1 / ln 2, k_neg = slope / ln 2: the lane kernels take their exponentials in base 2, so that
-// e^(x - m) is one subtraction and one hardware exponential (its error is two units in the last place, as the library
-// function's; the weights it gives are divided by their own sum).  z itself stays s_u + t_v: its sign decides which slope
-// an entry's gradient takes.
+__device__ __forceinline__ float leaky(float z, float slope) { return z * (z > 0.f ? 1.f : slope); }
+// e^(x - ref) for x <= ref (0 for x = -inf, ref finite), by the hardware's base-2 exponential.  The subtraction comes first and the
+// change of base second, so the error depends on how far x is below the row's maximum and not on how large scores are: at a
+// gap g, two units in the last place of the exponential and g / 2 of the product, where the weight itself is e^-g.  (The product
+// first, one operation less, put half a unit in the last place of 1.44 |x| on the exponent: 4e-5 of a weight at |x| = 1000.)
 constexpr float kLog2E = 1.4426950408889634f;
-__device__ __forceinline__ float leaky2(float z, float k_pos, float k_neg) { return z * (z > 0.f ? k_pos : k_neg); }
-__device__ __forceinline__ float exp2_hw(float x) {
+__device__ __forceinline__ float exp_below(float x, float ref) {
     float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"((x - ref) * kLog2E));
     return y;
 }
-// 2^(x - ref) for x <= ref, 0 for x = -inf whatever ref is
-__device__ __forceinline__ float exp2_rel(float x, float ref) { return x == -INFINITY ? 0.f : exp2_hw(x - ref); }
+// The same where ref may be -inf too (a state without entries yet): 0 for x = -inf whatever ref is.
+__device__ __forceinline__ float exp_rel(float x, float ref) { return x == -INFINITY ? 0.f : exp_below(x, ref); }
 
 // Hands the entries of a CSR row to pass.batch<U>(u, ok), U neighbours per lane at a time; entry `deg`, if any, is the row's
 // own node `self`.  Where ok is false u is an entry of the row all the same (or `self`), so a pass may load its data

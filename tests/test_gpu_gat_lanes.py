@@ -43,3 +43,38 @@ def test_gat_forward_and_backward(heads, dh, pad):
     assert np.all(err <= 2e-5 * np.linalg.norm(ref_dp, axis=1) + 1e-5 * np.abs(ref_dp).max()), float(err.max())
     for got, ref in ((da_src, ref_as), (da_dst, ref_ad)):      # sums over the n nodes, as in the other backward tests
         np.testing.assert_allclose(got.cpu().numpy(), ref, rtol=0, atol=2e-6 * max(1.0, np.abs(ref).max()) * np.sqrt(n))
+
+
+@pytest.mark.parametrize("heads,dh,pad", [(4, 16, 0), (8, 4, 0), (1, 64, 0), (4, 16, 4), (2, 6, 0)])
+@pytest.mark.parametrize("level", [4000.0, -4000.0])
+def test_weights_of_large_scores(heads, dh, pad, level):
+    """Scores of +-4000 with gaps of order 1, all exact in fp32 (multiples of 1 / 64, slope 1 / 4): what is left is the error of the
+    weights, which may depend on the gap to the row's maximum but not on the scores' size."""
+    from paper_2302_13053_b200 import binding as B
+    n, rowptr, colidx, _ = wl.degree_ladder_graph([0, 1, 2, 3, 7, 31, 33, 63, 65, 129, 300], seed=heads)
+    rng = np.random.default_rng(dh)
+    d = heads * dh
+    buf = rng.standard_normal((n, d + pad)).astype(np.float32)
+    rows = buf[:, :d].reshape(n, heads, dh).copy()
+    rows[..., 0] = np.round(rows[..., 0] * 64) / 64       # s_u
+    rows[..., 1] = 1.0                                    # t_v = level
+    buf[:, :d] = rows.reshape(n, d)
+    p = np.ascontiguousarray(buf[:, :d])
+    dz = rng.standard_normal((n, d)).astype(np.float32)
+    gat = dict(heads=heads, head_dim=dh, negative_slope=0.25, add_self_loop=1, a_src=np.zeros((heads, dh), np.float32),
+               a_dst=np.zeros((heads, dh), np.float32))
+    gat["a_src"][:, 0] = 1.0
+    gat["a_dst"][:, 1] = level
+    g = dict(gat, a_src=torch.from_numpy(gat["a_src"]), a_dst=torch.from_numpy(gat["a_dst"]))
+    rp, ci = dev(rowptr.astype(np.int64)), dev(colidx.astype(np.int32))
+    dzb = torch.zeros((n, d + pad), device="cuda")
+    dzb[:, :d] = dev(dz)
+    out, _ = B.retexo_aggregate(B.GAT, rp, ci, dev(buf)[:, :d], gat=g)
+    # a weight: 2^-22 of the exponential and as much of the product at gaps up to 8 (2.4e-7 each); rows of up to 300 terms that cancel to
+    # a tenth of their size.  Half a unit in the last place of the scores on the exponent instead would be 1.7e-4.
+    assert_rows_close(out.cpu().numpy(), oracle.aggregate(oracle.GAT, rowptr, colidx, p, gat=gat), rel=6e-6)
+    dp, _, _, _ = B.retexo_gat_backward(rp, ci, dev(buf)[:, :d], g, dzb[:, :d])
+    ref = oracle.gat_backward(rowptr, colidx, p, gat, dz.astype(np.float64))[0]
+    # columns that neither attention vector reaches: sums of weighted gradients alone
+    free = np.delete(np.arange(d).reshape(heads, dh), [0, 1], axis=1).ravel()
+    assert_rows_close(dp.cpu().numpy()[:, free], ref[:, free], rel=6e-6)
