@@ -34,12 +34,14 @@ struct GatArgs {
 // Running soft-max state and weighted sum of one lane over the entries its group takes.
 template <int W>
 struct GatState {
-    float m, l;
+    float m, l, lost;            // lost: what rounding has added to l beyond its terms
     Cols<W> acc;
-    __device__ __forceinline__ void clear() { m = -INFINITY; l = 0.f; acc.zero(); }
+    __device__ __forceinline__ void clear() { m = -INFINITY; l = lost = 0.f; acc.zero(); }
     // Adds the states of the warp's groups in a fixed tree; every lane ends up with the total of its columns.
     template <int LPG>
     __device__ __forceinline__ void merge_groups() {
+        l -= lost;
+        lost = 0.f;
 #pragma unroll
         for (int o = LPG; o < kWarp; o <<= 1) {
             const float big = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -88,13 +90,16 @@ struct GatForwardPass {
         const float ref = big == -INFINITY ? 0.f : big;         // (a group without entries yet)
         st.m = big;
         st.l *= f;
+        st.lost *= f;
         st.acc.scale(f);
+        float more = -st.lost;
 #pragma unroll
         for (int t = 0; t < U; ++t) {
             const float w = exp_below(e[t], ref);
-            st.l += w;
+            more += w;
             st.acc.fma(w, x[t]);
         }
+        add_compensated(st.l, st.lost, more);
     }
 };
 
@@ -125,7 +130,7 @@ __global__ void __launch_bounds__(kGatThreads, kGatBlocksPerSm) gat_lane_rows_ke
     auto store_row = [&](int64_t v, int32_t total) {
         if (!L.on) return;
         if (total == 0) pass.st.acc.zero();                     // an empty row leaves zeros
-        store_cols(v, L.col, pass.st.acc, total > 0 ? pass.st.l : 1.f);
+        store_cols(v, L.col, pass.st.acc, total > 0 ? pass.st.l - pass.st.lost : 1.f);
     };
     if ((int)blockIdx.x >= hub_blocks) {
         const int64_t v0 = ((int64_t)(blockIdx.x - hub_blocks) * kGatWarps + warp) * G;

@@ -250,7 +250,8 @@ __global__ void __launch_bounds__(256) gat_bwd_reduce_kernel(const float* partia
 // Destinations: for row v, with its own gradient dz_v in registers, the soft-max statistics and the sums
 //   c_v = sum alpha dalpha,   dt_v = sum alpha g' dalpha - c_v sum alpha g'      (g' = 1 or the slope)
 // in one pass over the entries with a running maximum.  dalpha = <dz_v, p_u> over the head's columns enters linearly, so a lane
-// keeps the share of its own columns and the head's lanes are added once per row.
+// keeps the share of its own columns and the head's lanes are added once per row.  All four sums are compensated: c_v and dt_v are
+// what is left of sums that cancel.
 template <int LPG, int W>
 struct GatDstPass {
     const GatBwdArgs& a;
@@ -258,14 +259,14 @@ struct GatDstPass {
     const float* s;
     int head, col;
     bool on;
-    float tv, m, den, c, b1, b2;
+    float tv, m, den, c, b1, b2, den_lost, c_lost, b1_lost, b2_lost;
     Cols<W> g;
     __device__ __forceinline__ GatDstPass(const GatBwdArgs& a_, const GatLanes<LPG, W>& L)
         : a(a_), p(a_.p + L.col), s(a_.s + L.head), head(L.head), col(L.col), on(L.on) {}
     // Returns whether this lane's part of the gradient has a non-zero entry.
     __device__ __forceinline__ bool begin(int64_t v) {
         tv = __ldg(a.t + v * a.heads + head);
-        m = -INFINITY; den = c = b1 = b2 = 0.f;
+        m = -INFINITY; den = c = b1 = b2 = den_lost = c_lost = b1_lost = b2_lost = 0.f;
         g.load(a.dz + v * a.lddz + col);
         bool any = false;
 #pragma unroll
@@ -291,14 +292,20 @@ struct GatDstPass {
         const float f = exp_rel(m, big), ref = big == -INFINITY ? 0.f : big;
         m = big;
         den *= f; c *= f; b1 *= f; b2 *= f;
+        den_lost *= f; c_lost *= f; b1_lost *= f; b2_lost *= f;
+        float den_more = -den_lost, c_more = -c_lost, b1_more = -b1_lost, b2_more = -b2_lost;
 #pragma unroll
         for (int t = 0; t < U; ++t) {
             const float w = exp_below(e[t], ref), wg = z[t] > 0.f ? w : w * a.slope, d = g.dot(x[t]);
-            den += w;
-            b2 += wg;
-            c = fmaf(w, d, c);
-            b1 = fmaf(wg, d, b1);
+            den_more += w;
+            b2_more += wg;
+            c_more = fmaf(w, d, c_more);
+            b1_more = fmaf(wg, d, b1_more);
         }
+        add_compensated(den, den_lost, den_more);
+        add_compensated(c, c_lost, c_more);
+        add_compensated(b1, b1_lost, b1_more);
+        add_compensated(b2, b2_lost, b2_more);
     }
     __device__ __forceinline__ void merge(float m2, float den2, float c2, float b12, float b22) {
         const float big = fmaxf(m, m2), f = exp_rel(m, big), f2 = exp_rel(m2, big);
@@ -404,15 +411,15 @@ struct GatSrcPass {
     const GatBwdArgs& a;
     const float* dz;
     const float4* stats;
-    int head, col;
-    float su, ds, dc;            // ds: sum alpha g' <dz_v, p_u> over this lane's columns; dc: sum alpha g' c_v
+    int head, col, hw;
+    float su, ds, ds_lost;            // (the same in all lanes of a head)
     Cols<W> px, acc;
     __device__ __forceinline__ GatSrcPass(const GatBwdArgs& a_, const GatLanes<LPG, W>& L)
-        : a(a_), dz(a_.dz + L.col), stats(a_.stats + L.head), head(L.head), col(L.col) {}
+        : a(a_), dz(a_.dz + L.col), stats(a_.stats + L.head), head(L.head), col(L.col), hw(a_.head_dim / W) {}
     __device__ __forceinline__ void begin(int64_t u) {
         su = __ldg(a.s + u * a.heads + head);
         px.load(a.p + u * a.ldp + col);
-        ds = dc = 0.f;
+        ds = ds_lost = 0.f;
         acc.zero();
     }
     template <int U>
@@ -429,34 +436,38 @@ struct GatSrcPass {
             g[t].zero();
             if (st[t].y != 0.f) g[t].load(dz + (int64_t)v[t] * a.lddz);
         }
+        float more = -ds_lost;
 #pragma unroll
         for (int t = 0; t < U; ++t) {
             const float z = su + st[t].w;
             const float alpha = st[t].y != 0.f ? exp_below(leaky(z, a.slope), st[t].x) * st[t].y : 0.f;
             const float ag = z > 0.f ? alpha : alpha * a.slope;
-            ds = fmaf(ag, px.dot(g[t]), ds);
-            dc = fmaf(ag, st[t].z, dc);
+            float d = px.dot(g[t]);           // of the whole head: what d and c_v have in common goes before anything is added up
+            for (int o = 1; o < hw; o <<= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+            more = fmaf(ag, d - st[t].z, more);
             acc.fma(alpha, g[t]);
         }
+        add_compensated(ds, ds_lost, more);
     }
     __device__ __forceinline__ void merge_groups() {
 #pragma unroll
         for (int o = LPG; o < kWarp; o <<= 1) {
             ds += __shfl_xor_sync(0xffffffffu, ds, o);
-            dc += __shfl_xor_sync(0xffffffffu, dc, o);
             acc.add_xor(o);
         }
     }
-    // Warp-uniform call; as, ad: this lane's columns of the attention vectors.
-    __device__ __forceinline__ void finish(int64_t u, bool write, int hw, const Cols<W>& as, const Cols<W>& ad, bool vec, bool vec16) {
-        for (int o = 1; o < hw; o <<= 1) ds += __shfl_xor_sync(0xffffffffu, ds, o);
+    // (the attention vectors are read here: held through the walk, their 16 registers a lane were spilled)
+    __device__ __forceinline__ void finish(int64_t u, bool write, bool vec, bool vec16) {
         if (!write) return;
-        const float d = ds - dc, dt = __ldg(a.dt + u * a.heads + head);
-        acc.fma(d, as);
-        acc.fma(dt, ad);
+        const float dt = __ldg(a.dt + u * a.heads + head);
+        Cols<W> att;
+        att.load_unaligned(a.a_src + col);
+        acc.fma(ds, att);
+        att.load_unaligned(a.a_dst + col);
+        acc.fma(dt, att);
         if (a.dp) acc.store(a.dp + u * a.lddp + col, vec);
         if (a.dp16) acc.store(a.dp16 + u * a.lddp16 + col, vec16);
-        if (col % a.head_dim == 0) a.ds[u * a.heads + head] = d;
+        if (col % a.head_dim == 0) a.ds[u * a.heads + head] = ds;
     }
 };
 
@@ -466,14 +477,10 @@ __global__ void __launch_bounds__(kGatThreads, kGatBlocksPerSm) gat_lane_src_ker
                                                                                     int vec, int vec16) {
     constexpr int G = GatLanes<LPG, W>::G;
     __shared__ Cols<W> sm_acc[2][kGatWarps][LPG];
-    __shared__ float2 sm_ds[2][kGatWarps][LPG];
+    __shared__ float sm_ds[2][kGatWarps][LPG];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const GatLanes<LPG, W> L(lane, a.dim, a.head_dim);
     GatSrcPass<LPG, W> pass(a, L);
-    const int hw = a.head_dim / W;
-    Cols<W> as, ad;
-    as.zero(); ad.zero();
-    if (L.on) { as.load_unaligned(a.a_src + L.col); ad.load_unaligned(a.a_dst + L.col); }
     if ((int)blockIdx.x >= hub_blocks) {
         const int64_t u0 = ((int64_t)(blockIdx.x - hub_blocks) * kGatWarps + warp) * G;
         if (u0 >= a.n) return;
@@ -484,7 +491,7 @@ __global__ void __launch_bounds__(kGatThreads, kGatBlocksPerSm) gat_lane_src_ker
         const bool mine = total <= kGatGroupEntries;
         pass.begin(u);
         gat_walk_by_group<LPG, W>(pass, L, a.colidx, (int32_t)u, beg, deg, mine ? total : 0, __reduce_max_sync(0xffffffffu, mine ? total : 0));
-        pass.finish(u, mine && L.on, hw, as, ad, vec != 0, vec16 != 0);
+        pass.finish(u, mine && L.on, vec != 0, vec16 != 0);
         unsigned longer = __ballot_sync(0xffffffffu, L.li == 0 && !mine && total < hub_entries);
         while (longer) {
             const int src = __ffs(longer) - 1;
@@ -494,7 +501,7 @@ __global__ void __launch_bounds__(kGatThreads, kGatBlocksPerSm) gat_lane_src_ker
             pass.begin(w);
             gat_walk_by_warp<LPG, W>(pass, L, a.colidx, (int32_t)w, w_beg, w_deg, w_deg + a.self_loop, 0, kWarp, lane);
             pass.merge_groups();
-            pass.finish(w, L.g == 0 && L.on, hw, as, ad, vec != 0, vec16 != 0);
+            pass.finish(w, L.g == 0 && L.on, vec != 0, vec16 != 0);
         }
         return;
     }
@@ -509,16 +516,15 @@ __global__ void __launch_bounds__(kGatThreads, kGatBlocksPerSm) gat_lane_src_ker
         pass.merge_groups();
         if (L.g == 0) {
             sm_acc[turn][warp][L.li] = pass.acc;
-            sm_ds[turn][warp][L.li] = make_float2(pass.ds, pass.dc);
+            sm_ds[turn][warp][L.li] = pass.ds;
         }
         __syncthreads();
         if (warp == 0) {      // the warps' sums in warp order
             for (int w = 1; w < kGatWarps; ++w) {
                 pass.acc.fma(1.f, sm_acc[turn][w][L.li]);
-                pass.ds += sm_ds[turn][w][L.li].x;
-                pass.dc += sm_ds[turn][w][L.li].y;
+                pass.ds += sm_ds[turn][w][L.li];
             }
-            pass.finish(u, L.g == 0 && L.on, hw, as, ad, vec != 0, vec16 != 0);
+            pass.finish(u, L.g == 0 && L.on, vec != 0, vec16 != 0);
         }
     }
 }

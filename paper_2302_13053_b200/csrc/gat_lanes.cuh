@@ -147,6 +147,14 @@ __device__ __forceinline__ float exp_below(float x, float ref) {
 // The same where ref may be -inf too (a state without entries yet): 0 for x = -inf whatever ref is.
 __device__ __forceinline__ float exp_rel(float x, float ref) { return x == -INFINITY ? 0.f : exp_below(x, ref); }
 
+// sum += more, with what rounding adds beyond that in `lost`; the next `more` starts from -lost (Kahan's compensated sum: a row's
+// sums run entry after entry in one lane, and without it lose up to a third more than a tree over the entries).
+__device__ __forceinline__ void add_compensated(float& sum, float& lost, float more) {
+    const float s = __fadd_rn(sum, more);
+    lost = __fsub_rn(__fsub_rn(s, sum), more);
+    sum = s;
+}
+
 // Hands the entries of a CSR row to pass.batch<U>(u, ok), U neighbours per lane at a time; entry `deg`, if any, is the row's
 // own node `self`.  Where ok is false u is an entry of the row all the same (or `self`), so a pass may load its data
 // without a predicate and give it weight zero.

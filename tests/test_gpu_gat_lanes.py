@@ -78,3 +78,26 @@ def test_weights_of_large_scores(heads, dh, pad, level):
     # columns that neither attention vector reaches: sums of weighted gradients alone
     free = np.delete(np.arange(d).reshape(heads, dh), [0, 1], axis=1).ravel()
     assert_rows_close(dp.cpu().numpy()[:, free], ref[:, free], rel=6e-6)
+
+
+@pytest.mark.parametrize("heads,dh", [(1, 8), (4, 16), (8, 4), (8, 32)])
+def test_gradients_of_rows_with_a_common_part(heads, dh):
+    """Rows around 20 and gradients around 1: <dz_v, p_u> and its mean over the row agree to one part in a hundred, and their difference is
+    what reaches ds and dt.  Its error may be a few units in the last place of <dz_v, p_u> for every unit of attention a node
+    receives (about ten for the node of 300 rows), not that of sums of the products themselves."""
+    from paper_2302_13053_b200 import binding as B
+    n, rowptr, colidx, _ = wl.degree_ladder_graph([1, 2, 3, 7, 15, 31, 32, 33, 63, 129, 300], seed=heads)
+    rng = np.random.default_rng(dh)
+    d = heads * dh
+    p = (20 + rng.standard_normal((n, d))).astype(np.float32)
+    dz = (1 + 0.1 * rng.standard_normal((n, d))).astype(np.float32)
+
+    def vector():      # (mean zero: scores of order 1 although the rows are not)
+        a = rng.standard_normal((heads, dh)) / np.sqrt(dh)
+        return (a - a.mean(axis=1, keepdims=True)).astype(np.float32)
+    gat = dict(heads=heads, head_dim=dh, negative_slope=0.2, add_self_loop=1, a_src=vector(), a_dst=vector())
+    g = dict(gat, a_src=torch.from_numpy(gat["a_src"]), a_dst=torch.from_numpy(gat["a_dst"]))
+    dp, _, _, _ = B.retexo_gat_backward(dev(rowptr.astype(np.int64)), dev(colidx.astype(np.int32)), dev(p), g, dev(dz))
+    ref = oracle.gat_backward(rowptr, colidx, p, gat, dz.astype(np.float64))[0]
+    size = 20.0 * dh                                        # of <dz_v, p_u>
+    assert np.abs(dp.cpu().numpy() - ref).max() <= 20 * 2.0 ** -24 * size
