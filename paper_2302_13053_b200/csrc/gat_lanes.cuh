@@ -1,7 +1,7 @@
 // Lane layout of the GAT kernels for head widths 4, 8, 16, ... 256 on aligned rows.  A lane owns W contiguous columns of one
-// head (8, or 4 where the heads are 4 wide) and LPG lanes (a power of two) one CSR entry, so a warp reads G = 32 / LPG whole
-// neighbour rows per load instruction and every lane scores its entry for its own head.  Nothing is exchanged between lanes
-// until a row is done: sums over a head's columns are linear, so they are reduced once per row, not once per entry.
+// head (8, or 4 where the heads are 4 wide or rows come in 16-byte pieces only) and LPG lanes (a power of two) one CSR entry, so
+// a warp reads G = 32 / LPG whole neighbour rows per load instruction and every lane scores its entry for its own head.  Sums
+// over a head's columns are linear, so they are reduced once per row, not once per entry, wherever they are not a difference.
 #pragma once
 #include "common.cuh"
 
@@ -36,11 +36,17 @@ struct GatLanes {
     }
 };
 
-// Whether the lane layout covers a shape (p and, where given, q hold its rows), and with how many lanes / columns per lane.
+// Whether the lane layout covers a shape (p and, where given, q hold its rows), and with how many lanes / columns per lane: 8 columns
+// where rows come in whole 32-byte pieces, else 4 where they come in 16-byte pieces and are no wider than 64 columns.  (A gradient of
+// 100 k nodes, 2 M entries, 4 x 16 at a stride of 68 floats: 296 us, on the general kernels 7380; at a stride of 64 220.)
 inline bool gat_lanes_cover(int32_t dim, int32_t head_dim, const float* p, int64_t ldp, const float* q, int64_t ldq, int* lpg, int* w) {
     if (head_dim < 4 || (head_dim & (head_dim - 1)) != 0 || dim > 256) return false;
-    *w = head_dim == 4 ? 4 : 8;
-    if (ldp % *w != 0 || !aligned_to(p, 4 * *w) || (q && (ldq % *w != 0 || !aligned_to(q, 4 * *w)))) return false;
+    auto pieces_of = [&](int columns) {
+        return ldp % columns == 0 && aligned_to(p, 4 * columns) && (!q || (ldq % columns == 0 && aligned_to(q, 4 * columns)));
+    };
+    if (head_dim >= 8 && pieces_of(8)) *w = 8;
+    else if (dim <= 64 && pieces_of(4)) *w = 4;
+    else return false;
     *lpg = 1;
     while (*lpg * *w < dim) *lpg <<= 1;
     return true;
@@ -51,6 +57,7 @@ template <typename F>
 inline int gat_lanes_dispatch(int lpg, int w, F&& go) {
     if (w == 4) {
         switch (lpg) {
+            case 16: return go.template operator()<16, 4>();
             case 8: return go.template operator()<8, 4>();
             case 4: return go.template operator()<4, 4>();
             case 2: return go.template operator()<2, 4>();

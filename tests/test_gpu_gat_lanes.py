@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("heads,dh,pad", [(1, 4, 0), (3, 4, 0), (8, 4, 0), (1, 8, 0), (3, 16, 0), (7, 8, 0), (1, 256, 0), (2, 128, 0), (5, 32, 8),
                                           (4, 16, 4)])
 def test_gat_forward_and_backward(heads, dh, pad):
-    """pad > 0: the rows have a stride of heads * dh + pad floats (4: not in 32-byte pieces, the general kernels)."""
+    """pad > 0: the rows have a stride of heads * dh + pad floats (4: in 16-byte pieces only, four columns a lane)."""
     from paper_2302_13053_b200 import binding as B
     n, rowptr, colidx, _ = wl.degree_ladder_graph([0, 1, 2, 3, 7, 8, 9, 30, 31, 32, 33, 61, 62, 63, 64, 65, 127, 129, 300], seed=heads)
     rng = np.random.default_rng(dh)
@@ -101,3 +101,59 @@ def test_gradients_of_rows_with_a_common_part(heads, dh):
     ref = oracle.gat_backward(rowptr, colidx, p, gat, dz.astype(np.float64))[0]
     size = 20.0 * dh                                        # of <dz_v, p_u>
     assert np.abs(dp.cpu().numpy() - ref).max() <= 20 * 2.0 ** -24 * size
+
+
+def _time(fn, repeats=5):
+    fn()
+    best = float("inf")
+    for _ in range(repeats):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        fn()
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b))
+    return best
+
+
+@pytest.mark.parametrize("heads,dh,ld,offset", [(1, 8, 12, 0), (4, 16, 68, 0), (4, 16, 64, 4), (2, 32, 68, 0), (1, 64, 68, 0), (8, 8, 76, 4),
+                                                (8, 4, 36, 0), (3, 16, 52, 4)])
+def test_rows_in_16_byte_pieces(heads, dh, ld, offset):
+    """Rows of up to 64 columns that start on 16-byte but not on 32-byte boundaries: the same results, and no more than a few times
+    the time of rows that do (the general kernels take ten to thirty times as long)."""
+    from paper_2302_13053_b200 import binding as B
+    n, rowptr, colidx, _ = wl.degree_ladder_graph([1, 5, 31, 33, 64, 200, 400], seed=heads)
+    rng = np.random.default_rng(dh + ld)
+    d = heads * dh
+    scale = 1.0 / np.sqrt(dh)
+    gat = dict(heads=heads, head_dim=dh, negative_slope=0.2, add_self_loop=1,
+               a_src=(rng.standard_normal((heads, dh)) * scale).astype(np.float32),
+               a_dst=(rng.standard_normal((heads, dh)) * scale).astype(np.float32))
+    g = dict(gat, a_src=torch.from_numpy(gat["a_src"]), a_dst=torch.from_numpy(gat["a_dst"]))
+    rp, ci = dev(rowptr.astype(np.int64)), dev(colidx.astype(np.int32))
+
+    def laid_out(a):
+        rows = torch.full((offset + n * ld,), float("nan"), device="cuda")[offset:].view(n, ld)
+        rows[:, :d] = dev(a)
+        return rows[:, :d]
+    p, dz = rng.standard_normal((n, d)).astype(np.float32), rng.standard_normal((n, d)).astype(np.float32)
+    dz[rng.random(n) < 0.4] = 0.0
+    q, gz = laid_out(p), laid_out(dz)
+    out, _ = B.retexo_aggregate(B.GAT, rp, ci, q, gat=g)
+    assert_rows_close(out.cpu().numpy(), oracle.aggregate(oracle.GAT, rowptr, colidx, p, gat=gat), what="%d x %d" % (heads, dh))
+    dp, _, da_src, da_dst = B.retexo_gat_backward(rp, ci, q, g, gz)
+    ref_dp, ref_as, ref_ad = oracle.gat_backward(rowptr, colidx, p, gat, dz.astype(np.float64))
+    err = np.abs(dp.cpu().numpy() - ref_dp).max(axis=1)      # as for aligned rows above
+    assert np.all(err <= 2e-5 * np.linalg.norm(ref_dp, axis=1) + 1e-5 * np.abs(ref_dp).max()), float(err.max())
+    for got, ref in ((da_src, ref_as), (da_dst, ref_ad)):
+        np.testing.assert_allclose(got.cpu().numpy(), ref, rtol=0, atol=2e-6 * max(1.0, np.abs(ref).max()) * np.sqrt(n))
+    if dh >= 8:
+        m = 20000                                            # a graph large enough to be bound by its entries: 200 a row
+        step = torch.arange(1, 201, device="cuda", dtype=torch.int64) * 37
+        cols = ((torch.arange(m, device="cuda")[:, None] + step) % m).sort(1).values
+        rp2, ci2 = torch.arange(m + 1, device="cuda") * 200, cols.to(torch.int32).flatten().contiguous()
+        base = torch.randn(m * 80 + 64, device="cuda")
+        odd, even = base[offset:offset + m * ld].view(m, ld)[:, :d], base[:m * d].view(m, d)
+        slow = _time(lambda: B.retexo_gat_backward(rp2, ci2, odd, g, odd))
+        fast = _time(lambda: B.retexo_gat_backward(rp2, ci2, even, g, even))
+        assert slow < 4 * fast, (slow, fast)
