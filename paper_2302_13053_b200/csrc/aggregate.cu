@@ -137,7 +137,7 @@ __device__ __forceinline__ void load_vec(const float* p, float (&v)[E]) {
     }
 }
 // ---------------------------------------------------------------- rows to lanes
-// A slab of LPG x E x NV columns is aggregated at a time.  LPG lanes (a power of two) take one CSR entry: lane `li` of group
+// A slab of up to LPG x E x NV columns is aggregated at a time.  LPG lanes (a power of two) take one CSR entry: lane `li` of group
 // `g` owns the NV vectors of E columns at E (li + LPG k) of the slab, so a warp reads G = 32 / LPG neighbour rows per load
 // instruction in whole runs.  A row of up to kGroupEntries entries is summed by one group in CSR order (a warp works on G rows
 // at once), a longer one by the whole warp: group g adds the entries g, g + G, ... and the groups' sums are added in a fixed tree.
@@ -146,21 +146,33 @@ constexpr int kGroupEntries = 32;
 template <int LPG, int E, int NV, int OP>
 struct AggLanes {
     static constexpr int G = kWarp / LPG, kCols = LPG * E * NV;
-    static constexpr int U = E >= 4 ? 4 : 8;      // entries in flight per lane
+    static constexpr bool kGcn = OP == kOpGcn;
+    static constexpr int U = E >= 4 || E * NV > 2 ? 4 : 8;      // entries in flight per lane
+    static constexpr int kBlocks = E < 4 && E * NV > 4 ? 8 : E == 4 && LPG == 32 ? 12 : kAggBlocksPerSm;      // (64, 40 and 56 registers)
     const AggArgs& a;
-    int g, li;
-    bool on[NV];                        // the vector exists; if not, vector 0 of the slab is read and dropped
-    int off[NV];
+    int g, li, c0;                      // c0: the lane's first column; vector k starts at c0 + E LPG k
+    bool on[NV];                        // the vector exists
     float acc[NV][E], self[NV][E];
 
-    __device__ __forceinline__ AggLanes(const AggArgs& a_, int lane, int slab) : a(a_) {
+    __device__ __forceinline__ AggLanes(const AggArgs& a_, int lane, int col0) : a(a_) {
         g = lane / LPG;
         li = lane % LPG;
+        c0 = col0 + E * li;
+#pragma unroll
+        for (int k = 0; k < NV; ++k) on[k] = c0 + E * LPG * k < a.dim;
+        if (NV == 1 && !on[0]) c0 = col0;      // (reads the group's first vector and drops it: no predicate on the load)
+    }
+    // This lane's vectors of row u.
+    __device__ __forceinline__ void load_row(int64_t u, float (&x)[NV][E]) {
+        const float* p = a.q + u * a.ldq + c0;
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
-            const int c = slab * kCols + E * (li + LPG * k);
-            on[k] = c < a.dim;
-            off[k] = on[k] ? c : slab * kCols;
+            if (NV == 1 || on[k]) {
+                load_vec<E>(p + E * LPG * k, x[k]);
+            } else {
+#pragma unroll
+                for (int i = 0; i < E; ++i) x[k][i] = 0.f;
+            }
         }
     }
     __device__ __forceinline__ void clear() {
@@ -169,12 +181,10 @@ struct AggLanes {
 #pragma unroll
             for (int i = 0; i < E; ++i) acc[k][i] = OP == kOpMax ? -INFINITY : 0.f;
     }
-    // Asks for what the end of row v needs, ahead of time.
-    __device__ __forceinline__ void begin(int64_t v) {
-        clear();
-        if (OP == kOpGcn || a.concat_self) {
-#pragma unroll
-            for (int k = 0; k < NV; ++k) load_vec<E>(a.q + v * a.ldq + off[k], self[k]);
+    // What the end of row v needs.
+    __device__ __forceinline__ void load_self(int64_t v) {
+        if (kGcn || a.concat_self) {
+            load_row(v, self);
         }
     }
     // Adds the rows u[t] where ok[t]; where it is not, u[t] is some node whose row is loaded and dropped.
@@ -183,8 +193,7 @@ struct AggLanes {
         float x[N][NV][E];
 #pragma unroll
         for (int t = 0; t < N; ++t)
-#pragma unroll
-            for (int k = 0; k < NV; ++k) load_vec<E>(a.q + (int64_t)u[t] * a.ldq + off[k], x[t][k]);
+            load_row(u[t], x[t]);
 #pragma unroll
         for (int t = 0; t < N; ++t) {
             if (!ok[t]) continue;
@@ -278,7 +287,7 @@ struct AggLanes {
     }
     // GCN adds the (scaled) self row and scales, SAGE divides by the degree and (optionally) copies the self row.
     __device__ __forceinline__ void finish(int64_t v, int64_t deg) {
-        const float cv = OP == kOpGcn ? gcn_coef(deg) : 0.f;
+        const float cv = kGcn ? gcn_coef(deg) : 0.f;
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
             if (!on[k]) continue;
@@ -287,39 +296,30 @@ struct AggLanes {
                 if (OP == kOpGcn) acc[k][i] = cv * (self[k][i] + acc[k][i]);
                 else acc[k][i] = deg <= 0 ? 0.f : OP == kOpMax ? acc[k][i] : acc[k][i] / (float)deg;
             }
-            const bool concat = OP != kOpGcn && a.concat_self;
-            const int n_cols = a.dim - off[k];
+            const bool concat = !kGcn && a.concat_self;
+            const int col = c0 + E * LPG * k, n_cols = a.dim - col;
             if (E == 1 || n_cols >= E) {
-                if (concat) store(v, off[k], self[k]);
-                store(v, off[k] + (concat ? a.dim : 0), acc[k]);
+                if (concat) store(v, col, self[k]);
+                store(v, col + (concat ? a.dim : 0), acc[k]);
             } else {                    // the ragged last vector
 #pragma unroll
                 for (int i = 0; i < E; ++i) {
                     if (i >= n_cols) break;
-                    if (concat) store_elem(a, v, off[k] + i, self[k][i]);
-                    store_elem(a, v, off[k] + (concat ? a.dim : 0) + i, acc[k][i]);
+                    if (concat) store_elem(a, v, col + i, self[k][i]);
+                    store_elem(a, v, col + (concat ? a.dim : 0) + i, acc[k][i]);
                 }
             }
         }
     }
 };
 
-// Blocks are ordered slab by slab, so that at any time the whole grid gathers from the same few columns of the matrix: a slab of
-// 64 columns stays in L2 where the whole matrix does not.  A slab's first seg_blocks blocks take the segments of the heavy rows
-// (their raw sums go to scratch), the others a fixed set of rows each, G per warp.
-// Bound by the L2 -> SM path (64 bytes a cycle and SM) on dense graphs, by row pointer -> column -> row latencies on sparse ones;
-// measured against a persistent kernel that drew its rows from one counter, a warp each (SAGE, bf16 out, with concatenation):
-//   233 k nodes, 115 M entries, 256 columns: 6.95 -> 6.4 ms (18.4 TB/s of neighbour rows); GCN 9.5 -> 7.8 ms
-//   58 k nodes, 7 M entries, 256 columns: 820 -> 467 us (15.8 TB/s); GCN 1036 -> 520 us
-//   600 k nodes, 30 M entries, 256 columns: 4.05 -> 3.4 ms;  20 k nodes, 88 k entries, 500 columns: 142 -> 66 us
-// Slabs of 32 or 128 columns instead of 64 take 1.4 and 1.2 times as long on the first of these; 4 entries in flight, since
-// with 56 registers 36 warps fit an SM (64: 32 warps, level; 48: spills, 5 % slower; 80 and more: 1.4 times as long).
+// One block's share of a slab: the first seg_blocks blocks take the segments of the heavy rows (their raw sums go to scratch), the
+// others a fixed set of rows each, rows_per_warp (up to G) per warp.
 template <int LPG, int E, int NV, int OP>
-__global__ void __launch_bounds__(kAggThreads, kAggBlocksPerSm) agg_lanes_kernel(AggArgs a, unsigned blocks_per_slab, unsigned seg_blocks) {
-    const unsigned slab = blockIdx.x / blocks_per_slab, b = blockIdx.x % blocks_per_slab;
+__device__ __forceinline__ void agg_block(const AggArgs& a, int col0, unsigned b, unsigned seg_blocks, int rows_per_warp) {
     constexpr int G = kWarp / LPG;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    AggLanes<LPG, E, NV, OP> L(a, lane, (int)slab);
+    AggLanes<LPG, E, NV, OP> L(a, lane, col0);
     const int32_t seg_entries = a.heavy.seg_entries;
     if (b < seg_blocks) {
         const int n_seg = a.heavy.counters[1];
@@ -334,21 +334,26 @@ __global__ void __launch_bounds__(kAggThreads, kAggBlocksPerSm) agg_lanes_kernel
 #pragma unroll
                 for (int k = 0; k < NV; ++k)
 #pragma unroll
-                    for (int i = 0; i < E; ++i) if (L.on[k] && L.off[k] + i < a.dim) dst[L.off[k] + i] = L.acc[k][i];
+                    for (int i = 0; i < E; ++i) {
+                        const int col = L.c0 + E * LPG * k + i;
+                        if (L.on[k] && col < a.dim) dst[col] = L.acc[k][i];
+                    }
             }
         }
         return;
     }
-    const int64_t v0 = ((int64_t)(b - seg_blocks) * kAggWarps + warp) * G;
+    const int64_t v0 = ((int64_t)(b - seg_blocks) * kAggWarps + warp) * rows_per_warp;
     if (v0 >= a.n) return;
     const int64_t v = min(v0 + L.g, a.n - 1);
     const int64_t beg = __ldg(a.rowptr + v);
-    const int32_t total = v0 + L.g < a.n ? (int32_t)(__ldg(a.rowptr + v + 1) - beg) : INT32_MAX;      // (beyond the last row: nobody's)
+    const bool some = L.g < rows_per_warp && v0 + L.g < a.n;
+    const int32_t total = some ? (int32_t)(__ldg(a.rowptr + v + 1) - beg) : INT32_MAX;      // (nobody's row)
     const bool mine = G > 1 && total <= kGroupEntries;
     if constexpr (G > 1) {
         if (__any_sync(0xffffffffu, mine)) {
             const int longest = __reduce_max_sync(0xffffffffu, mine ? total : 0);
-            L.begin(v);
+            L.clear();
+            L.load_self(v);                 // (ahead of time: short rows are bound by latencies)
             L.walk_by_group(beg, mine ? total : 0, longest, (int32_t)v);
             if (mine) L.finish(v, total);
         }
@@ -359,9 +364,37 @@ __global__ void __launch_bounds__(kAggThreads, kAggBlocksPerSm) agg_lanes_kernel
         longer &= longer - 1;
         const int64_t w = __shfl_sync(0xffffffffu, v, src), w_beg = __shfl_sync(0xffffffffu, beg, src);
         const int32_t w_total = __shfl_sync(0xffffffffu, total, src);
-        L.begin(w);
+        L.clear();
         L.walk_by_warp(w_beg, w_beg + w_total, lane);
+        L.load_self(w);
         if (L.g == 0) L.finish(w, w_total);
+    }
+}
+
+struct AggGrid {
+    unsigned slabs, blocks_per_slab, seg_blocks;      // whole slabs first, then the columns that are left
+    int rows_per_warp, tail_rows_per_warp;
+};
+
+// Blocks are ordered slab by slab, so that at any time the whole grid gathers from the same few columns of the matrix: a slab of
+// 64 columns stays in L2 where the whole matrix does not.  The columns left over are taken by groups of TLPG lanes, as many as they
+// need: a second slab for 8 columns of 72 with the lanes of a whole one costs as much as the first.
+// Bound by the L2 -> SM path (64 bytes a cycle and SM) on dense graphs, by row pointer -> column -> row latencies on sparse ones;
+// measured against a persistent kernel that drew its rows from one counter, a warp each (SAGE, bf16 out, with concatenation):
+//   233 k nodes, 115 M entries, 256 columns: 6.95 -> 6.4 ms (18.4 TB/s of neighbour rows); GCN 9.5 -> 7.8 ms
+//   58 k nodes, 7 M entries, 256 columns: 820 -> 467 us (15.8 TB/s); GCN 1036 -> 520 us
+//   600 k nodes, 30 M entries, 256 columns: 4.05 -> 3.4 ms;  20 k nodes, 88 k entries, 500 columns: 142 -> 66 us
+// Slabs of 32 or 128 columns instead of 64 take 1.4 and 1.2 times as long on the first of these; 4 entries in flight, since
+// with 56 registers 36 warps fit an SM (64: 32 warps, level; 48: spills, 5 % slower; 80 and more: 1.4 times as long).
+template <int LPG, int E, int NV, int TLPG, int TNV, int OP>
+__global__ void __launch_bounds__(kAggThreads, AggLanes<LPG, E, NV, OP>::kBlocks) agg_lanes_kernel(AggArgs a, AggGrid grid) {
+    constexpr int kCols = LPG * E * NV;
+    const unsigned whole = grid.slabs * grid.blocks_per_slab;
+    if ((LPG == TLPG && NV == TNV) || blockIdx.x < whole) {
+        const unsigned slab = blockIdx.x / grid.blocks_per_slab;
+        agg_block<LPG, E, NV, OP>(a, (int)slab * kCols, blockIdx.x - slab * grid.blocks_per_slab, grid.seg_blocks, grid.rows_per_warp);
+    } else {
+        agg_block<TLPG, E, TNV, OP>(a, (int)grid.slabs * kCols, blockIdx.x - whole, grid.seg_blocks, grid.tail_rows_per_warp);
     }
 }
 
@@ -403,29 +436,109 @@ static int launch_combine(int op, const AggArgs& a, int64_t n_edges, int self_sc
     return launch_status();
 }
 
-template <int LPG, int E, int NV>
+// Rows a warp takes side by side: as many as it has groups where rows are short.  Rows above kGroupEntries entries it takes one after
+// the other, so there should be few enough of them a warp to keep every SM busy (2 k nodes, 200 k entries, 8 columns: 65 us with
+// 32 rows a warp, 16 blocks in all).
+static int rows_per_warp(int groups, int64_t n, int64_t n_edges, int n_sm) {
+    int rows = groups;
+    if (n_edges > n * kGroupEntries)
+        while (rows > 1 && n < (int64_t)rows * kAggWarps * n_sm * kAggBlocksPerSm) rows /= 2;
+    return rows;
+}
+
+template <int LPG, int E, int NV, int TLPG, int TNV>
 static int launch_lanes(int op, const AggArgs& a, int64_t n_edges, int n_sm, cudaStream_t st) {
-    constexpr int64_t kRows = (int64_t)kAggWarps * (kWarp / LPG);
-    const int64_t n_slabs = (a.dim + LPG * E * NV - 1) / (LPG * E * NV);
-    const int64_t segs = n_edges >= heavy_degree(n_edges) ? (max_segments(n_edges) + kAggWarps - 1) / kAggWarps : 0;
-    const unsigned seg_blocks = (unsigned)(segs < 4ll * n_sm ? segs : 4ll * n_sm);
-    const int64_t per_slab = (a.n + kRows - 1) / kRows + seg_blocks;
-    if (per_slab * n_slabs > INT32_MAX) return RETEXO_ERR_UNSUPPORTED;
-    const unsigned grid = (unsigned)(per_slab * n_slabs);
-    if constexpr (E == 8) {
-        if (op == kOpGcn) agg_lanes_kernel<LPG, E, NV, kOpGcn><<<grid, kAggThreads, 0, st>>>(a, (unsigned)per_slab, seg_blocks);
+    constexpr int kCols = LPG * E * NV;
+    AggGrid g;
+    g.slabs = (unsigned)(a.dim / kCols);
+    int left = a.dim % kCols;
+    if (left && LPG == TLPG && NV == TNV) {      // the last slab is like the others
+        g.slabs += 1;
+        left = 0;
     }
-    if (op == kOpMax) agg_lanes_kernel<LPG, E, NV, kOpMax><<<grid, kAggThreads, 0, st>>>(a, (unsigned)per_slab, seg_blocks);
-    else if (op == kOpSum) agg_lanes_kernel<LPG, E, NV, kOpSum><<<grid, kAggThreads, 0, st>>>(a, (unsigned)per_slab, seg_blocks);
+    g.rows_per_warp = rows_per_warp(kWarp / LPG, a.n, n_edges, n_sm);
+    g.tail_rows_per_warp = rows_per_warp(kWarp / TLPG, a.n, n_edges, n_sm);
+    const int64_t segs = n_edges >= heavy_degree(n_edges) ? (max_segments(n_edges) + kAggWarps - 1) / kAggWarps : 0;
+    g.seg_blocks = (unsigned)(segs < 4ll * n_sm ? segs : 4ll * n_sm);
+    auto blocks = [&](int64_t rows) { return (a.n + kAggWarps * rows - 1) / (kAggWarps * rows) + g.seg_blocks; };
+    const int64_t total = g.slabs * blocks(g.rows_per_warp) + (left ? blocks(g.tail_rows_per_warp) : 0);
+    if (total > INT32_MAX) return RETEXO_ERR_UNSUPPORTED;
+    g.blocks_per_slab = (unsigned)blocks(g.rows_per_warp);
+    const unsigned grid = (unsigned)total;
+    if constexpr (E == 8) {
+        if (op == kOpGcn) agg_lanes_kernel<LPG, E, NV, TLPG, TNV, kOpGcn><<<grid, kAggThreads, 0, st>>>(a, g);
+    }
+    if (op == kOpMax) agg_lanes_kernel<LPG, E, NV, TLPG, TNV, kOpMax><<<grid, kAggThreads, 0, st>>>(a, g);
+    else if (op == kOpSum) agg_lanes_kernel<LPG, E, NV, TLPG, TNV, kOpSum><<<grid, kAggThreads, 0, st>>>(a, g);
     return launch_combine(op, a, n_edges, 1, n_sm, st);
 }
 
-// Rows in whole 32-byte pieces: as few lanes as a narrow matrix needs, 64 columns of a wide one.
+constexpr size_t kSlabBytes = (size_t)64 << 20;      // a slab of all rows may take this much of L2
+// The matrix does not fit L2, and its rows are read often enough for a slab that does to pay.
+static bool beyond_l2(int64_t n, int64_t n_edges, int32_t dim) { return (size_t)n * dim * 4 > ((size_t)100 << 20) && n_edges >= 16 * n; }
+
+// Rows in whole 32-byte pieces.
 static int launch_lanes8(int op, const AggArgs& a, int64_t n_edges, int n_sm, cudaStream_t st) {
-    if (a.dim <= 8) return launch_lanes<1, 8, 1>(op, a, n_edges, n_sm, st);
-    if (a.dim <= 16) return launch_lanes<2, 8, 1>(op, a, n_edges, n_sm, st);
-    if (a.dim <= 32) return launch_lanes<4, 8, 1>(op, a, n_edges, n_sm, st);
-    return launch_lanes<8, 8, 1>(op, a, n_edges, n_sm, st);
+    if (a.dim <= 8) return launch_lanes<1, 8, 1, 1, 1>(op, a, n_edges, n_sm, st);
+    if (a.dim <= 16) return launch_lanes<2, 8, 1, 2, 1>(op, a, n_edges, n_sm, st);
+    if (a.dim <= 32) return launch_lanes<4, 8, 1, 4, 1>(op, a, n_edges, n_sm, st);
+    if (a.dim > 96 && a.dim < 128 && (size_t)a.n * a.dim * 4 <= kSlabBytes) return launch_lanes<16, 8, 1, 16, 1>(op, a, n_edges, n_sm, st);
+    const int left = a.dim % 64;
+    if (left == 0 || left > 32 || a.dim > 320) return launch_lanes<8, 8, 1, 8, 1>(op, a, n_edges, n_sm, st);
+    if (left <= 8) return launch_lanes<8, 8, 1, 1, 1>(op, a, n_edges, n_sm, st);
+    if (left <= 16) return launch_lanes<8, 8, 1, 2, 1>(op, a, n_edges, n_sm, st);
+    return launch_lanes<8, 8, 1, 4, 1>(op, a, n_edges, n_sm, st);
+}
+// ... in 16-byte pieces.
+static int launch_lanes4(int op, const AggArgs& a, int64_t n_edges, int n_sm, cudaStream_t st) {
+    if (a.dim <= 8) return launch_lanes<2, 4, 1, 2, 1>(op, a, n_edges, n_sm, st);
+    if (a.dim <= 16) return launch_lanes<4, 4, 1, 4, 1>(op, a, n_edges, n_sm, st);
+    if (a.dim <= 32) return launch_lanes<8, 4, 1, 8, 1>(op, a, n_edges, n_sm, st);
+    if (a.dim <= 64) return launch_lanes<16, 4, 1, 16, 1>(op, a, n_edges, n_sm, st);
+    if (a.dim > 256 && beyond_l2(a.n, n_edges, a.dim) && (size_t)a.n * 256 <= kSlabBytes) return launch_lanes<16, 4, 1, 16, 1>(op, a, n_edges, n_sm, st);
+    const int left = a.dim % 128;
+    if (left == 0 || left > 64) return launch_lanes<32, 4, 1, 32, 1>(op, a, n_edges, n_sm, st);
+    if (left <= 16) return launch_lanes<32, 4, 1, 4, 1>(op, a, n_edges, n_sm, st);
+    if (left <= 32) return launch_lanes<32, 4, 1, 8, 1>(op, a, n_edges, n_sm, st);
+    return launch_lanes<32, 4, 1, 16, 1>(op, a, n_edges, n_sm, st);
+}
+// How many vectors of 32 lanes a slab of rows in narrow pieces takes, at most `most`: all of them where that is one pass, else about
+// equal slabs, of 64 MB where the matrix is beyond L2, such slabs fit it and rows are read often enough to come back to them.  (An
+// entry costs a warp as much in shuffles and addresses as in loads, so a second pass for a few columns costs almost what the first
+// does: 20 k nodes, 2 M entries, 96 / 97 columns in slabs of 96: 90 / 162 us, in one pass 77 / 79.)
+static int slab_vectors(int64_t n, int64_t n_edges, int32_t dim, int cols, int most) {
+    const int vecs = (dim + cols - 1) / cols;
+    if (beyond_l2(n, n_edges, dim)) {
+        const int64_t fit = (int64_t)kSlabBytes / (n * cols * 4);
+        if (fit * cols >= 64 && fit < most) most = (int)fit;
+    }
+    const int slabs = (vecs + most - 1) / most;
+    return (vecs + slabs - 1) / slabs;
+}
+// ... in 8-byte pieces.
+static int launch_lanes2(int op, const AggArgs& a, int64_t n_edges, int n_sm, cudaStream_t st) {
+    if (a.dim <= 8) return launch_lanes<4, 2, 1, 4, 1>(op, a, n_edges, n_sm, st);
+    if (a.dim <= 16) return launch_lanes<8, 2, 1, 8, 1>(op, a, n_edges, n_sm, st);
+    if (a.dim <= 32) return launch_lanes<16, 2, 1, 16, 1>(op, a, n_edges, n_sm, st);
+    switch (slab_vectors(a.n, n_edges, a.dim, 64, 3)) {
+        case 1: return launch_lanes<32, 2, 1, 32, 1>(op, a, n_edges, n_sm, st);
+        case 2: return launch_lanes<32, 2, 2, 32, 2>(op, a, n_edges, n_sm, st);
+        default: return launch_lanes<32, 2, 3, 32, 3>(op, a, n_edges, n_sm, st);
+    }
+}
+// ... float by float.
+static int launch_lanes1(int op, const AggArgs& a, int64_t n_edges, int n_sm, cudaStream_t st) {
+    if (a.dim <= 4) return launch_lanes<4, 1, 1, 4, 1>(op, a, n_edges, n_sm, st);
+    if (a.dim <= 8) return launch_lanes<8, 1, 1, 8, 1>(op, a, n_edges, n_sm, st);
+    if (a.dim <= 16) return launch_lanes<16, 1, 1, 16, 1>(op, a, n_edges, n_sm, st);
+    switch (slab_vectors(a.n, n_edges, a.dim, 32, 6)) {
+        case 1: return launch_lanes<32, 1, 1, 32, 1>(op, a, n_edges, n_sm, st);
+        case 2: return launch_lanes<32, 1, 2, 32, 2>(op, a, n_edges, n_sm, st);
+        case 3: return launch_lanes<32, 1, 3, 32, 3>(op, a, n_edges, n_sm, st);
+        case 4: return launch_lanes<32, 1, 4, 32, 4>(op, a, n_edges, n_sm, st);
+        case 5: return launch_lanes<32, 1, 5, 32, 5>(op, a, n_edges, n_sm, st);
+        default: return launch_lanes<32, 1, 6, 32, 6>(op, a, n_edges, n_sm, st);
+    }
 }
 
 // ---------------------------------------------------------------- GCN on matrices far larger than L2
@@ -699,8 +812,7 @@ int retexo::aggregate_rows(const retexo_csr* g, int32_t type, const float* q, in
     // (a last vector of 8 that holds 4 columns or fewer could reach beyond the last row's memory: 16-byte pieces then)
     if (aligned_to(q, 32) && ldq % 8 == 0 && ldq >= (dim + 7) / 8 * 8 && (whole_rows || (dim + 7) / 8 * 8 - dim <= 3))
         return launch_lanes8(op, a, e, n_sm, st);
-    if (v4) return dim <= 32 ? launch_lanes<8, 4, 1>(op, a, e, n_sm, st) : launch_lanes<16, 4, 1>(op, a, e, n_sm, st);
-    if (aligned_to(q, 8) && ldq % 2 == 0 && ldq >= (dim + 1) / 2 * 2) return launch_lanes<32, 2, 1>(op, a, e, n_sm, st);
-    if (dim <= 32) return launch_lanes<32, 1, 1>(op, a, e, n_sm, st);
-    return dim <= 64 ? launch_lanes<32, 1, 2>(op, a, e, n_sm, st) : launch_lanes<32, 1, 3>(op, a, e, n_sm, st);
+    if (v4) return launch_lanes4(op, a, e, n_sm, st);
+    if (aligned_to(q, 8) && ldq % 2 == 0 && ldq >= (dim + 1) / 2 * 2) return launch_lanes2(op, a, e, n_sm, st);
+    return launch_lanes1(op, a, e, n_sm, st);
 }

@@ -34,3 +34,44 @@ def test_layouts(aggr, dim, ld):
         np.testing.assert_array_equal(got, ref.astype(np.float32))
     else:
         assert_rows_close(got, ref, what="%d columns, stride %d" % (dim, ld))
+
+
+@pytest.mark.parametrize("aggr", [oracle.GCN, oracle.SAGE_MEAN, oracle.SAGE_MAX])
+@pytest.mark.parametrize("dim,ld", [(95, 96), (97, 97), (97, 97 + 7), (129, 129), (130, 130), (193, 193), (194, 194), (196, 196), (196, 200),
+                                    (257, 264), (260, 260), (500, 500), (602, 602), (603, 603), (769, 776), (1030, 1030)])
+def test_leftover_columns(aggr, dim, ld):
+    """Whole slabs of columns and the layouts that take what is left, with every load width; all hubs, so that a wide row has many pieces."""
+    test_layouts(aggr, dim, ld)
+
+
+def _time(fn, repeats=7):
+    """Device time of 8 calls: as a graph, so that small calls are not timed by their launches."""
+    fn()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for _ in range(8):
+            fn()
+    best = float("inf")
+    for _ in range(repeats):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        graph.replay()
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b))
+    return best
+
+
+@pytest.mark.parametrize("n,degree,dim,other,factor", [(20000, 100, 97, 95, 1.45), (2000, 100, 8, 64, 1.45)])
+def test_cost_of_leftover_columns_and_of_small_dense_graphs(n, degree, dim, other, factor):
+    """Two columns more cost no second pass over lanes that have none (1.8 times the time before they had their own layout); a narrow
+    row takes no longer than a wide one (2.1 times when a warp walked as many rows as on a graph that fills the device)."""
+    from paper_2302_13053_b200 import binding as B
+    rng = np.random.default_rng(n)
+    rp, ci = dev(np.arange(n + 1, dtype=np.int64) * degree), dev(rng.integers(0, n, size=n * degree).astype(np.int32))
+    times = []
+    for d in (dim, other):
+        q = torch.randn((n, d), device="cuda")
+        out = torch.empty((n, d), device="cuda")
+        times.append(_time(lambda: B.retexo_aggregate(oracle.SAGE_MEAN, rp, ci, q, concat_self=False, out=out)))
+    assert times[0] <= factor * times[1], times
