@@ -61,18 +61,22 @@ __global__ void prep_rows_kernel(int64_t n, const int64_t* __restrict__ rowptr, 
     list_if_heavy(h, v, deg);
 }
 
-// The same for a GCN round whose rows are scaled ahead: qs[u] = n_u q[u] in rows of ld_qs = round_up(dim, 8) floats, so that the
-// gather needs no coefficient per entry (one more random access each, a quarter of the gather's time) and always finds
-// rows in whole 32-byte pieces.  1 << lanes_log2 lanes a row, 8 columns each; a stream over q.
-__global__ void __launch_bounds__(256) gcn_scale_rows_kernel(int64_t n, const int64_t* __restrict__ rowptr, HeavyRows h,
-                                                             const float* __restrict__ q, int64_t ldq, int32_t dim, int vec4,
-                                                             float* __restrict__ qs, int64_t ld_qs, int lanes_log2) {
+// The same for a GCN round whose rows are laid out ahead in rows of ld_qs floats (a multiple of 8): scaled, qs[u] = n_u q[u], so that the
+// gather needs no coefficient per entry, or as they are (coef != nullptr: the coefficients go there).  1 << lanes_log2 lanes a row,
+// 8 columns each; a stream over q.
+__global__ void __launch_bounds__(256) gcn_lay_out_rows_kernel(int64_t n, const int64_t* __restrict__ rowptr, HeavyRows h,
+                                                               const float* __restrict__ q, int64_t ldq, int32_t dim, int vec4,
+                                                               float* __restrict__ qs, int64_t ld_qs, int lanes_log2, float* __restrict__ coef) {
     const int64_t t = blockIdx.x * 256ll + threadIdx.x, v = t >> lanes_log2;
     if (v >= n) return;
     const int lanes = 1 << lanes_log2, lane = (int)t & (lanes - 1);
     const int64_t deg = rowptr[v + 1] - rowptr[v];
     if (lane == 0) list_if_heavy(h, v, deg);
-    const float c = gcn_coef(deg);
+    float c = gcn_coef(deg);
+    if (coef) {
+        if (lane == 0) coef[v] = c;
+        c = 1.f;
+    }
     const float* src = q + v * ldq;
     float* dst = qs + v * ld_qs;
     for (int col = 8 * lane; col < ld_qs; col += 8 * lanes) {
@@ -89,9 +93,9 @@ __global__ void __launch_bounds__(256) gcn_scale_rows_kernel(int64_t n, const in
     }
 }
 
-// What a row's accumulator does with a neighbour row: plain sum (SAGE mean; GCN: of rows scaled ahead, or weighted by coef[u]
-// as they come), or element-wise maximum (SAGE max-pooling).
-constexpr int kOpSum = 0, kOpGcn = 1, kOpMax = 2;
+// What a row's accumulator does with a neighbour row: plain sum (SAGE mean; GCN of rows scaled ahead), element-wise maximum (SAGE
+// max-pooling), sum weighted by coef[u] (GCN of rows as they are), or compensated sum (GCN of narrow rows scaled ahead).
+constexpr int kOpSum = 0, kOpGcn = 1, kOpMax = 2, kOpGcnWeighted = 3, kOpGcnNarrow = 4;
 
 struct AggArgs {
     int64_t n;
@@ -100,7 +104,7 @@ struct AggArgs {
     const float* q;         // the rows that are gathered (GCN through agg_lanes_kernel: scaled by n_u)
     int64_t ldq;
     int32_t dim;
-    const float* coef;      // agg_rows_kernel only
+    const float* coef;      // GCN weighted
     float* out;             // may be null
     int64_t ldout;
     __nv_bfloat16* out16;   // may be null
@@ -146,13 +150,14 @@ constexpr int kGroupEntries = 32;
 template <int LPG, int E, int NV, int OP>
 struct AggLanes {
     static constexpr int G = kWarp / LPG, kCols = LPG * E * NV;
-    static constexpr bool kGcn = OP == kOpGcn;
-    static constexpr int U = E >= 4 || E * NV > 2 ? 4 : 8;      // entries in flight per lane
+    static constexpr bool kGcn = OP == kOpGcn || OP == kOpGcnWeighted || OP == kOpGcnNarrow, kCompensated = OP == kOpGcnNarrow;
+    static constexpr int U = kCompensated ? 2 : E >= 4 || E * NV > 2 ? 4 : 8;      // entries in flight per lane
     static constexpr int kBlocks = E < 4 && E * NV > 4 ? 8 : E == 4 && LPG == 32 ? 12 : kAggBlocksPerSm;      // (64, 40 and 56 registers)
     const AggArgs& a;
     int g, li, c0;                      // c0: the lane's first column; vector k starts at c0 + E LPG k
     bool on[NV];                        // the vector exists
     float acc[NV][E], self[NV][E];
+    float lost[NV][kCompensated ? E : 1];      // what rounding has added to acc beyond its terms
 
     __device__ __forceinline__ AggLanes(const AggArgs& a_, int lane, int col0) : a(a_) {
         g = lane / LPG;
@@ -179,7 +184,10 @@ struct AggLanes {
 #pragma unroll
         for (int k = 0; k < NV; ++k)
 #pragma unroll
-            for (int i = 0; i < E; ++i) acc[k][i] = OP == kOpMax ? -INFINITY : 0.f;
+            for (int i = 0; i < E; ++i) {
+                acc[k][i] = OP == kOpMax ? -INFINITY : 0.f;
+                if constexpr (kCompensated) lost[k][i] = 0.f;
+            }
     }
     // What the end of row v needs.
     __device__ __forceinline__ void load_self(int64_t v) {
@@ -187,9 +195,9 @@ struct AggLanes {
             load_row(v, self);
         }
     }
-    // Adds the rows u[t] where ok[t]; where it is not, u[t] is some node whose row is loaded and dropped.
+    // Adds the rows u[t] (GCN weighted: times w[t]) where ok[t]; where it is not, u[t] is some node whose row is loaded and dropped.
     template <int N>
-    __device__ __forceinline__ void batch(const int32_t (&u)[N], const bool (&ok)[N]) {
+    __device__ __forceinline__ void batch(const int32_t (&u)[N], const bool (&ok)[N], const float (&w)[N]) {
         float x[N][NV][E];
 #pragma unroll
         for (int t = 0; t < N; ++t)
@@ -200,9 +208,19 @@ struct AggLanes {
 #pragma unroll
             for (int k = 0; k < NV; ++k)
 #pragma unroll
-                for (int i = 0; i < E; ++i) acc[k][i] = OP == kOpMax ? fmaxf(acc[k][i], x[t][k][i]) : acc[k][i] + x[t][k][i];
+                for (int i = 0; i < E; ++i) {
+                    if constexpr (kCompensated) {
+                        const float more = __fsub_rn(x[t][k][i], lost[k][i]), sum = __fadd_rn(acc[k][i], more);
+                        lost[k][i] = __fsub_rn(__fsub_rn(sum, acc[k][i]), more);
+                        acc[k][i] = sum;
+                    } else {
+                        acc[k][i] = OP == kOpMax ? fmaxf(acc[k][i], x[t][k][i])
+                                  : OP == kOpGcnWeighted ? fmaf(w[t], x[t][k][i], acc[k][i]) : acc[k][i] + x[t][k][i];
+                    }
+                }
         }
     }
+    __device__ __forceinline__ float weight(int32_t u) const { return OP == kOpGcnWeighted ? __ldg(a.coef + u) : 1.f; }
     // Entries [first, last) of the CSR by the whole warp, 32 columns at a time, fetched two trips ahead.
     __device__ __forceinline__ void walk_by_warp(int64_t first, int64_t last, int lane) {
         auto column = [&](int64_t e0) -> int32_t { return __ldcs(a.colidx + (e0 + lane < last ? e0 + lane : first)); };
@@ -213,18 +231,21 @@ struct AggLanes {
             const int32_t my_u = next_u;
             next_u = after_u;
             if (e0 + 2 * kWarp < last) after_u = column(e0 + 2 * kWarp);
+            const float my_w = weight(my_u);
             constexpr int N = G * U > kWarp ? kWarp / G : U;
 #pragma unroll 1
             for (int j = 0; j < cnt; j += G * N) {
                 int32_t u[N];
                 bool ok[N];
+                float w[N];
 #pragma unroll
                 for (int t = 0; t < N; ++t) {
                     const int at = j + t * G + g;
                     u[t] = __shfl_sync(0xffffffffu, my_u, at & 31);
+                    w[t] = OP == kOpGcnWeighted ? __shfl_sync(0xffffffffu, my_w, at & 31) : 1.f;
                     ok[t] = at < cnt;
                 }
-                batch<N>(u, ok);
+                batch<N>(u, ok, w);
             }
         }
 #pragma unroll
@@ -247,16 +268,19 @@ struct AggLanes {
             const int32_t my_u = next_u;
             if (e0 + LPG < longest) next_u = column(e0 + LPG + li);
             const int cnt = min(LPG, longest - e0);
+            const float my_w = weight(my_u);
 #pragma unroll 1
             for (int j = 0; j < cnt; j += N) {
                 int32_t u[N];
                 bool ok[N];
+                float w[N];
 #pragma unroll
                 for (int t = 0; t < N; ++t) {
                     u[t] = __shfl_sync(0xffffffffu, my_u, g * LPG + j + t);
+                    w[t] = OP == kOpGcnWeighted ? __shfl_sync(0xffffffffu, my_w, g * LPG + j + t) : 1.f;
                     ok[t] = e0 + j + t < total;
                 }
-                batch<N>(u, ok);
+                batch<N>(u, ok, w);
             }
         }
     }
@@ -294,6 +318,8 @@ struct AggLanes {
 #pragma unroll
             for (int i = 0; i < E; ++i) {
                 if (OP == kOpGcn) acc[k][i] = cv * (self[k][i] + acc[k][i]);
+                else if constexpr (kCompensated) acc[k][i] = cv * __fadd_rn(acc[k][i], __fsub_rn(self[k][i], lost[k][i]));
+                else if (OP == kOpGcnWeighted) acc[k][i] = cv * fmaf(cv, self[k][i], acc[k][i]);
                 else acc[k][i] = deg <= 0 ? 0.f : OP == kOpMax ? acc[k][i] : acc[k][i] / (float)deg;
             }
             const bool concat = !kGcn && a.concat_self;
@@ -468,9 +494,16 @@ static int launch_lanes(int op, const AggArgs& a, int64_t n_edges, int n_sm, cud
     if constexpr (E == 8) {
         if (op == kOpGcn) agg_lanes_kernel<LPG, E, NV, TLPG, TNV, kOpGcn><<<grid, kAggThreads, 0, st>>>(a, g);
     }
+    if constexpr (E == 8 && kCols <= 16) {
+        if (op == kOpGcnNarrow) agg_lanes_kernel<LPG, E, NV, TLPG, TNV, kOpGcnNarrow><<<grid, kAggThreads, 0, st>>>(a, g);
+    }
+    if constexpr (E >= 4) {
+        if (op == kOpGcnWeighted) agg_lanes_kernel<LPG, E, NV, TLPG, TNV, kOpGcnWeighted><<<grid, kAggThreads, 0, st>>>(a, g);
+    }
     if (op == kOpMax) agg_lanes_kernel<LPG, E, NV, TLPG, TNV, kOpMax><<<grid, kAggThreads, 0, st>>>(a, g);
     else if (op == kOpSum) agg_lanes_kernel<LPG, E, NV, TLPG, TNV, kOpSum><<<grid, kAggThreads, 0, st>>>(a, g);
-    return launch_combine(op, a, n_edges, 1, n_sm, st);
+    const bool gcn = op == kOpGcn || op == kOpGcnWeighted || op == kOpGcnNarrow;
+    return launch_combine(gcn ? kOpGcn : op, a, n_edges, op != kOpGcnWeighted, n_sm, st);
 }
 
 constexpr size_t kSlabBytes = (size_t)64 << 20;      // a slab of all rows may take this much of L2
@@ -576,7 +609,7 @@ __device__ __forceinline__ void accumulate_range(const AggArgs& a, int64_t beg, 
                                                  float4 (&acc)[CH]) {
     const int64_t ldv = a.ldq / 4;
     const float4* __restrict__ qv = reinterpret_cast<const float4*>(a.q);
-    const bool hinting = a.hub_coef > 0.f;
+    const bool hinting = a.hub_coef > 0.f;      // (always here; the test keeps the loads' registers apart: 256 columns 16.1 ms, without it 17.3)
     uint64_t keep = 0, pass = 0;
     if (hinting) { keep = l2_policy_evict_last(); pass = l2_policy_evict_first(); }
     for (int64_t e0 = beg; e0 < end; e0 += kWarp) {
@@ -690,10 +723,31 @@ static int launch_rows(const AggArgs& a, int64_t n_edges, int n_sm, cudaStream_t
     return launch_combine(kOpGcn, a, n_edges, 0, n_sm, st);
 }
 
+// ---------------------------------------------------------------- which way a GCN round goes (by its sizes alone)
+// Dense: rows of 32 entries or more on average.
+static bool gcn_dense(int64_t n, int64_t n_edges) { return n_edges >= 32 * n; }
+
 // From here on the gather is bound by HBM, not by L2, and the priorities pay: 2.45 M nodes, 124 M entries, agg_rows_kernel
 // against agg_lanes_kernel: 64 columns (627 MB) 5.3-6.9 against 4.4 ms, 100 columns (980 MB) 7.9 against 10.3 ms, 256 columns
 // 15.8 against 17.5 ms.
 constexpr size_t kHbmBoundBytes = (size_t)768 << 20;
+
+// Stride of the copy of a GCN matrix: whole 32-byte pieces; whole 128-byte lines where a row is read often enough to pay for
+// writing them.
+static int64_t gcn_copy_stride(int32_t dim, int64_t n, int64_t n_edges) {
+    const int64_t unit = dim > 64 && gcn_dense(n, n_edges) ? 32 : 8;
+    return (dim + unit - 1) / unit * unit;
+}
+
+// What a GCN round adds up.  Scaling the rows ahead saves a gathered coefficient per entry but rounds every row once more: on dense
+// graphs the longer rows' sums, in several parts, more than make up for it, on others the error against 64 bits would be 4 to 9 % up
+// (uniform graphs of 2, 8, 16, 24 entries a row: 4.75, 8.1, 9.7, 10.9e-8, weighted 4.38, 7.5, 9.1, 10.3, 32 entries: 10.6 / 10.1 / 11.7
+// before rows were scaled).  There the rows are weighted as they come, or, where a coefficient is as much to gather as a row, scaled and
+// added with compensation (4.5, 6.5, 6.6, 6.8e-8; 1 M nodes, 8 M entries, 8 columns 84 us, weighted 128; 32 columns 268 / 211).
+enum class GcnWay { kScaled, kNarrow, kWeighted };
+static GcnWay gcn_way(int64_t n, int64_t n_edges, int32_t dim) {
+    return gcn_dense(n, n_edges) ? GcnWay::kScaled : dim <= 16 ? GcnWay::kNarrow : GcnWay::kWeighted;
+}
 
 }  // namespace retexo
 
@@ -713,7 +767,7 @@ extern "C" size_t retexo_aggregate_workspace_size(int64_t n_nodes, int64_t n_edg
         s.take<float>((size_t)max_segments(n_edges) * (size_t)((dim + 3) / 4 * 4));   // segment sums
         if (type == RETEXO_GCN) {
             s.take<float>((size_t)n_nodes);                               // coef
-            s.take<float>((size_t)n_nodes * (size_t)((dim + 7) / 8 * 8)); // scaled rows
+            s.take<float>((size_t)n_nodes * (size_t)gcn_copy_stride(dim, n_nodes, n_edges));      // rows scaled ahead or laid out
         }
     }
     return s.off + kAlign;
@@ -781,10 +835,16 @@ int retexo::aggregate_rows(const retexo_csr* g, int32_t type, const float* q, in
     a.vec_out16 = out_bf16 && aligned_to(out_bf16, 8) && ldout_bf16 % 4 == 0 && cols4;
     RETEXO_CUDA_TRY(cudaMemsetAsync(a.heavy.counters, 0, 64 * sizeof(int32_t), st));
 
+    // the widest pieces the rows come in (a last piece of 8 that holds 4 columns or fewer could reach beyond the last row's memory)
+    const bool v8 = aligned_to(q, 32) && ldq % 8 == 0 && ldq >= (dim + 7) / 8 * 8 && (whole_rows || (dim + 7) / 8 * 8 - dim <= 3);
     const bool v4 = aligned_to(q, 16) && ldq % 4 == 0 && ldq >= (dim + 3) / 4 * 4;
+    const bool v2 = aligned_to(q, 8) && ldq % 2 == 0 && ldq >= (dim + 1) / 2 * 2;
+    auto lanes = [&](int op) {
+        return v8 ? launch_lanes8(op, a, e, n_sm, st) : v4 ? launch_lanes4(op, a, e, n_sm, st)
+             : v2 ? launch_lanes2(op, a, e, n_sm, st) : launch_lanes1(op, a, e, n_sm, st);
+    };
     const unsigned prep_blocks = (unsigned)((n + 255) / 256);
     if (type == RETEXO_GCN) {
-        const int64_t ld_qs = ((int64_t)dim + 7) / 8 * 8;
         float* coef = ws.take<float>((size_t)n);
         if (v4 && (size_t)n * (size_t)dim * 4 >= kHbmBoundBytes) {
             prep_rows_kernel<<<prep_blocks, 256, 0, st>>>(n, g->rowptr, a.heavy, coef);
@@ -798,21 +858,24 @@ int retexo::aggregate_rows(const retexo_csr* g, int32_t type, const float* q, in
             if (chunks <= 5) return launch_rows<5>(a, e, n_sm, st);
             return launch_rows<6>(a, e, n_sm, st);
         }
+        const GcnWay way = gcn_way(n, e, dim);
+        if (way == GcnWay::kWeighted && v4) {
+            prep_rows_kernel<<<prep_blocks, 256, 0, st>>>(n, g->rowptr, a.heavy, coef);
+            a.coef = coef;
+            return lanes(kOpGcnWeighted);
+        }
+        const int64_t ld_qs = gcn_copy_stride(dim, n, e);
         float* qs = ws.take<float>((size_t)n * (size_t)ld_qs);
         int lanes_log2 = 0;
         while (lanes_log2 < 5 && (8 << lanes_log2) < ld_qs) ++lanes_log2;
-        gcn_scale_rows_kernel<<<(unsigned)(((n << lanes_log2) + 255) / 256), 256, 0, st>>>(n, g->rowptr, a.heavy, q, ldq, dim, v4 ? 1 : 0,
-                                                                                           qs, ld_qs, lanes_log2);
+        const bool weighted = way == GcnWay::kWeighted;
+        gcn_lay_out_rows_kernel<<<(unsigned)(((n << lanes_log2) + 255) / 256), 256, 0, st>>>(n, g->rowptr, a.heavy, q, ldq, dim, v4 ? 1 : 0,
+                                                                                             qs, ld_qs, lanes_log2, weighted ? coef : nullptr);
         a.q = qs;
         a.ldq = ld_qs;
-        return launch_lanes8(kOpGcn, a, e, n_sm, st);
+        a.coef = coef;
+        return launch_lanes8(weighted ? kOpGcnWeighted : way == GcnWay::kNarrow ? kOpGcnNarrow : kOpGcn, a, e, n_sm, st);
     }
     if (e >= heavy_degree(e)) prep_rows_kernel<<<prep_blocks, 256, 0, st>>>(n, g->rowptr, a.heavy, nullptr);
-    const int op = type == RETEXO_SAGE_MAX ? kOpMax : kOpSum;
-    // (a last vector of 8 that holds 4 columns or fewer could reach beyond the last row's memory: 16-byte pieces then)
-    if (aligned_to(q, 32) && ldq % 8 == 0 && ldq >= (dim + 7) / 8 * 8 && (whole_rows || (dim + 7) / 8 * 8 - dim <= 3))
-        return launch_lanes8(op, a, e, n_sm, st);
-    if (v4) return launch_lanes4(op, a, e, n_sm, st);
-    if (aligned_to(q, 8) && ldq % 2 == 0 && ldq >= (dim + 1) / 2 * 2) return launch_lanes2(op, a, e, n_sm, st);
-    return launch_lanes1(op, a, e, n_sm, st);
+    return lanes(type == RETEXO_SAGE_MAX ? kOpMax : kOpSum);
 }
