@@ -1,7 +1,6 @@
 // Full-graph neighbour aggregation of one message-passing round (Eq. 1) over a CSR graph:
 // GCN symmetric-normalised sum, GraphSAGE mean and max (+ self concat); the GAT pass is in gat.cu.
 //
-//
 // The work is a gather-reduce bound by the memory system, not a dense contraction: neighbour rows are streamed with the
 // widest aligned vector loads, several rows in flight per lane, sums kept in registers.  Rows go to lanes by a fixed
 // rule (no work counter: a draw per row from one address is 2 ns each, more than a row of ten entries takes the chip),
@@ -497,10 +496,8 @@ static int launch_lanes(int op, const AggArgs& a, int64_t n_edges, int n_sm, cud
     if constexpr (E == 8 && kCols <= 16) {
         if (op == kOpGcnNarrow) agg_lanes_kernel<LPG, E, NV, TLPG, TNV, kOpGcnNarrow><<<grid, kAggThreads, 0, st>>>(a, g);
     }
-    if constexpr (E >= 4) {
-        if (op == kOpGcnWeighted) agg_lanes_kernel<LPG, E, NV, TLPG, TNV, kOpGcnWeighted><<<grid, kAggThreads, 0, st>>>(a, g);
-    }
-    if (op == kOpMax) agg_lanes_kernel<LPG, E, NV, TLPG, TNV, kOpMax><<<grid, kAggThreads, 0, st>>>(a, g);
+    if (op == kOpGcnWeighted) agg_lanes_kernel<LPG, E, NV, TLPG, TNV, kOpGcnWeighted><<<grid, kAggThreads, 0, st>>>(a, g);
+    else if (op == kOpMax) agg_lanes_kernel<LPG, E, NV, TLPG, TNV, kOpMax><<<grid, kAggThreads, 0, st>>>(a, g);
     else if (op == kOpSum) agg_lanes_kernel<LPG, E, NV, TLPG, TNV, kOpSum><<<grid, kAggThreads, 0, st>>>(a, g);
     const bool gcn = op == kOpGcn || op == kOpGcnWeighted || op == kOpGcnNarrow;
     return launch_combine(gcn ? kOpGcn : op, a, n_edges, op != kOpGcnWeighted, n_sm, st);
@@ -574,7 +571,7 @@ static int launch_lanes1(int op, const AggArgs& a, int64_t n_edges, int n_sm, cu
     }
 }
 
-// ---------------------------------------------------------------- GCN on matrices far larger than L2
+// ---------------------------------------------------------------- GCN on dense graphs far larger than L2
 // Bound by HBM, so what counts is which rows stay in L2: a power-law graph reads its hubs' rows again and again, every other
 // row a few times, and left to itself the cache keeps neither.  Rows of hubs (coef <= hub_coef) are loaded "evict last",
 // all others "evict first"; the coefficient, gathered per entry anyway, tells which.  (2.45 M x 256 floats, 124 M entries:
@@ -712,25 +709,159 @@ __global__ void __launch_bounds__(kRowThreads) agg_rows_kernel(AggArgs a) {
     }
 }
 
-template <int CH>
-static int launch_rows(const AggArgs& a, int64_t n_edges, int n_sm, cudaStream_t st) {
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, agg_rows_kernel<CH>, kRowThreads, 0) != cudaSuccess || per_sm < 1) {
-        (void)cudaGetLastError();
-        per_sm = 1;
+// The same for rows in 8- or 4-byte pieces, without priorities.
+// Adds the weighted rows of CSR entries [beg, end), in order, for the pieces vec0 + 32 c + lane of this lane.
+template <int E, int CH>
+__device__ __forceinline__ void accumulate_pieces(const AggArgs& a, int64_t beg, int64_t end, int lane, int vec0, int nvec,
+                                                 float (&acc)[CH][E]) {
+    for (int64_t e0 = beg; e0 < end; e0 += kWarp) {
+        const int cnt = (int)min((int64_t)kWarp, end - e0);
+        int my_u = 0;
+        float my_w = 0.f;
+        if (lane < cnt) {
+            my_u = __ldg(a.colidx + e0 + lane);
+            my_w = __ldg(a.coef + my_u);
+        }
+        int j = 0;
+        for (; j + kUnroll <= cnt; j += kUnroll) {
+            float x[kUnroll][CH][E], w[kUnroll];
+#pragma unroll
+            for (int t = 0; t < kUnroll; ++t) {
+                const int u = __shfl_sync(0xffffffffu, my_u, j + t);
+                w[t] = __shfl_sync(0xffffffffu, my_w, j + t);
+                const float* row = a.q + (int64_t)u * a.ldq;
+#pragma unroll
+                for (int c = 0; c < CH; ++c) {
+                    const int vi = vec0 + c * kWarp + lane;
+#pragma unroll
+                    for (int i = 0; i < E; ++i) x[t][c][i] = 0.f;
+                    if (vi < nvec) load_vec<E>(row + E * vi, x[t][c]);
+                }
+            }
+#pragma unroll
+            for (int t = 0; t < kUnroll; ++t)
+#pragma unroll
+                for (int c = 0; c < CH; ++c)
+#pragma unroll
+                    for (int i = 0; i < E; ++i) acc[c][i] = fmaf(w[t], x[t][c][i], acc[c][i]);
+        }
+        for (; j < cnt; ++j) {
+            const int u = __shfl_sync(0xffffffffu, my_u, j);
+            const float w = __shfl_sync(0xffffffffu, my_w, j);
+            const float* row = a.q + (int64_t)u * a.ldq;
+#pragma unroll
+            for (int c = 0; c < CH; ++c) {
+                const int vi = vec0 + c * kWarp + lane;
+                if (vi >= nvec) continue;
+                float x[E];
+                load_vec<E>(row + E * vi, x);
+#pragma unroll
+                for (int i = 0; i < E; ++i) acc[c][i] = fmaf(w, x[i], acc[c][i]);
+            }
+        }
     }
-    agg_rows_kernel<CH><<<n_sm * per_sm, kRowThreads, 0, st>>>(a);
+}
+
+// Persistent: items [0, n_seg) are segments of heavy rows, [n_seg, n_seg + n) whole rows (heavy ones are skipped).
+template <int E, int CH>
+__global__ void __launch_bounds__(kRowThreads) agg_pieces_kernel(AggArgs a) {
+    const int lane = threadIdx.x & 31;
+    const int nvec = (a.dim + E - 1) / E;
+    const int64_t n_seg = a.heavy.counters[1];
+    const int64_t total = n_seg + a.n;
+    for (;;) {
+        int64_t item = 0;
+        if (lane == 0) item = atomicAdd(reinterpret_cast<unsigned int*>(a.next_item), 1u);
+        item = __shfl_sync(0xffffffffu, item, 0);
+        if (item >= total) break;
+        if (item < n_seg) {
+            const int32_t slot = a.heavy.seg_slot[item];
+            const int64_t v = a.heavy.list[slot];
+            const int64_t beg = a.rowptr[v] + (item - a.heavy.seg_base[slot]) * a.heavy.seg_entries;
+            const int64_t end = min(a.rowptr[v + 1], beg + a.heavy.seg_entries);
+            for (int vec0 = 0; vec0 < nvec; vec0 += CH * kWarp) {
+                float acc[CH][E];
+#pragma unroll
+                for (int c = 0; c < CH; ++c)
+#pragma unroll
+                    for (int i = 0; i < E; ++i) acc[c][i] = 0.f;
+                accumulate_pieces<E, CH>(a, beg, end, lane, vec0, nvec, acc);
+#pragma unroll
+                for (int c = 0; c < CH; ++c) {
+                    const int vi = vec0 + c * kWarp + lane;
+                    if (vi >= nvec) continue;
+#pragma unroll
+                    for (int i = 0; i < E; ++i) if (E * vi + i < a.dim) a.seg_partial[item * a.ld_partial + E * vi + i] = acc[c][i];
+                }
+            }
+            continue;
+        }
+        const int64_t v = item - n_seg;
+        const int64_t beg = a.rowptr[v], end = a.rowptr[v + 1];
+        if (end - beg >= 2 * a.heavy.seg_entries) continue;
+        for (int vec0 = 0; vec0 < nvec; vec0 += CH * kWarp) {
+            float acc[CH][E];
+#pragma unroll
+            for (int c = 0; c < CH; ++c)
+#pragma unroll
+                for (int i = 0; i < E; ++i) acc[c][i] = 0.f;
+            accumulate_pieces<E, CH>(a, beg, end, lane, vec0, nvec, acc);
+            const float cv = a.coef[v];
+#pragma unroll
+            for (int c = 0; c < CH; ++c) {
+                const int vi = vec0 + c * kWarp + lane;
+                if (vi >= nvec) continue;
+                float self[E];
+                load_vec<E>(a.q + v * a.ldq + E * vi, self);
+#pragma unroll
+                for (int i = 0; i < E; ++i)
+                    if (E * vi + i < a.dim) store_elem(a, v, E * vi + i, cv * fmaf(cv, self[i], acc[c][i]));
+            }
+        }
+    }
+}
+
+template <int E, int CH>
+static int launch_rows(const AggArgs& a, int64_t n_edges, int n_sm, cudaStream_t st) {
+    auto go = [&](auto kernel) {
+        int per_sm = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kRowThreads, 0) != cudaSuccess || per_sm < 1) {
+            (void)cudaGetLastError();
+            per_sm = 1;
+        }
+        kernel<<<n_sm * per_sm, kRowThreads, 0, st>>>(a);
+    };
+    if constexpr (E == 4) go(agg_rows_kernel<CH>);
+    else go(agg_pieces_kernel<E, CH>);
     return launch_combine(kOpGcn, a, n_edges, 0, n_sm, st);
+}
+
+// Rows in pieces of E floats, as many chunks of 32 pieces as they need in one pass, up to 6.
+template <int E>
+static int launch_rows(const AggArgs& a, int64_t n_edges, int n_sm, cudaStream_t st) {
+    const int chunks = (a.dim + 32 * E - 1) / (32 * E);
+    if (chunks <= 1) return launch_rows<E, 1>(a, n_edges, n_sm, st);
+    if (chunks <= 2) return launch_rows<E, 2>(a, n_edges, n_sm, st);
+    if (chunks <= 3) return launch_rows<E, 3>(a, n_edges, n_sm, st);
+    if (chunks <= 4) return launch_rows<E, 4>(a, n_edges, n_sm, st);
+    if (chunks <= 5) return launch_rows<E, 5>(a, n_edges, n_sm, st);
+    return launch_rows<E, 6>(a, n_edges, n_sm, st);
 }
 
 // ---------------------------------------------------------------- which way a GCN round goes (by its sizes alone)
 // Dense: rows of 32 entries or more on average.
 static bool gcn_dense(int64_t n, int64_t n_edges) { return n_edges >= 32 * n; }
 
-// From here on the gather is bound by HBM, not by L2, and the priorities pay: 2.45 M nodes, 124 M entries, agg_rows_kernel
-// against agg_lanes_kernel: 64 columns (627 MB) 5.3-6.9 against 4.4 ms, 100 columns (980 MB) 7.9 against 10.3 ms, 256 columns
-// 15.8 against 17.5 ms.
-constexpr size_t kHbmBoundBytes = (size_t)768 << 20;
+// agg_rows_kernel pays where the gather is bound by HBM whatever is done about locality: slabs of 64 columns far beyond L2, and rows
+// read often enough for L2 to keep the hubs'.  Milliseconds, agg_rows_kernel / agg_lanes_kernel, graphs without hubs / with the
+// largest degree 60 / 6000 times the mean: 2.45 M nodes, 50 entries a row, 100 columns 10.0 / 7.9 / 7.8 against 11.2 / 10.6 / 10.1,
+// 256 columns 18.6 / 16.6 / 16.0 against 18.1 / 17.6 / 17.2; 25 entries a row, 100 columns 8.0 / 7.8 / 7.9 against 6.3 / 5.9 / 5.8,
+// 256 columns 10.1 / 9.9 / 8.9 against 10.8 / 10.5 / 10.5; 1 M nodes, 50 entries, 256 columns 7.3 / 6.4 / 6.3 against 6.2 / 6.1 / 6.0;
+// 200 k nodes, 40 entries, 1024 columns 6.6 against 3.3.
+static bool gcn_hbm_bound(int64_t n, int64_t n_edges, int32_t dim) {
+    return n_edges >= (dim >= 192 ? 16 : 32) * n && (size_t)n * (size_t)dim * 4 >= ((size_t)768 << 20) &&
+           (size_t)n * 256 >= ((size_t)512 << 20);
+}
 
 // Stride of the copy of a GCN matrix: whole 32-byte pieces; whole 128-byte lines where a row is read often enough to pay for
 // writing them.
@@ -744,17 +875,28 @@ static int64_t gcn_copy_stride(int32_t dim, int64_t n, int64_t n_edges) {
 // (uniform graphs of 2, 8, 16, 24 entries a row: 4.75, 8.1, 9.7, 10.9e-8, weighted 4.38, 7.5, 9.1, 10.3, 32 entries: 10.6 / 10.1 / 11.7
 // before rows were scaled).  There the rows are weighted as they come, or, where a coefficient is as much to gather as a row, scaled and
 // added with compensation (4.5, 6.5, 6.6, 6.8e-8; 1 M nodes, 8 M entries, 8 columns 84 us, weighted 128; 32 columns 268 / 211).
-enum class GcnWay { kScaled, kNarrow, kWeighted };
+enum class GcnWay { kHbm, kScaled, kNarrow, kWeighted };
 static GcnWay gcn_way(int64_t n, int64_t n_edges, int32_t dim) {
+    if (gcn_hbm_bound(n, n_edges, dim)) return GcnWay::kHbm;
+    if (n * gcn_copy_stride(dim, n, n_edges) > ((int64_t)2 << 30) / 4) return GcnWay::kWeighted;
     return gcn_dense(n, n_edges) ? GcnWay::kScaled : dim <= 16 ? GcnWay::kNarrow : GcnWay::kWeighted;
+}
+
+// Floats of the copy, 0 where there is none: scaled rows, and rows to be weighted that do not come in 16-byte pieces, up to 2 GB (beyond
+// that a round gathers the caller's rows as they are, a few per cent slower when dense, up to half when narrow pieces are all there
+// is; the largest graphs are where memory is short).
+static int64_t gcn_copy_floats(int64_t n, int64_t n_edges, int32_t dim, bool pieces16) {
+    const GcnWay way = gcn_way(n, n_edges, dim);
+    if (way == GcnWay::kHbm || (way == GcnWay::kWeighted && pieces16)) return 0;
+    const int64_t floats = n * gcn_copy_stride(dim, n, n_edges);
+    return floats <= ((int64_t)2 << 30) / 4 ? floats : 0;
 }
 
 }  // namespace retexo
 
 using namespace retexo;
 
-extern "C" size_t retexo_aggregate_workspace_size(int64_t n_nodes, int64_t n_edges, int32_t type,
-                                                  int32_t dim, int32_t heads) {
+size_t retexo::aggregate_rows_workspace_size(int64_t n_nodes, int64_t n_edges, int32_t type, int32_t dim, int32_t heads, bool pieces16) {
     Sizer s;
     if (n_nodes < 0) return 0;
     if (type == RETEXO_GAT) {
@@ -767,23 +909,20 @@ extern "C" size_t retexo_aggregate_workspace_size(int64_t n_nodes, int64_t n_edg
         s.take<float>((size_t)max_segments(n_edges) * (size_t)((dim + 3) / 4 * 4));   // segment sums
         if (type == RETEXO_GCN) {
             s.take<float>((size_t)n_nodes);                               // coef
-            s.take<float>((size_t)n_nodes * (size_t)gcn_copy_stride(dim, n_nodes, n_edges));      // rows scaled ahead or laid out
+            s.take<float>((size_t)gcn_copy_floats(n_nodes, n_edges, dim, pieces16));
         }
     }
     return s.off + kAlign;
 }
 
-extern "C" int retexo_aggregate(const retexo_csr* g, int32_t type, const float* q, int64_t ldq, int32_t dim,
-                                const retexo_gat_params* gat, float* out, int64_t ldout,
-                                int32_t concat_self, void* out_bf16, int64_t ldout_bf16,
-                                void* workspace, size_t workspace_bytes, void* stream) {
-    return aggregate_rows(g, type, q, ldq, dim, false, gat, out, ldout, concat_self, out_bf16, ldout_bf16, workspace, workspace_bytes,
-                          stream);
+// (the caller's alignment is not known here)
+extern "C" size_t retexo_aggregate_workspace_size(int64_t n_nodes, int64_t n_edges, int32_t type, int32_t dim, int32_t heads) {
+    return aggregate_rows_workspace_size(n_nodes, n_edges, type, dim, heads, false);
 }
 
-int retexo::aggregate_rows(const retexo_csr* g, int32_t type, const float* q, int64_t ldq, int32_t dim, bool whole_rows,
-                           const retexo_gat_params* gat, float* out, int64_t ldout, int32_t concat_self, void* out_bf16,
-                           int64_t ldout_bf16, void* workspace, size_t workspace_bytes, void* stream) {
+static int aggregate(const retexo_csr* g, int32_t type, const float* q, int64_t ldq, int32_t dim, bool whole_rows, bool pieces16,
+                     const retexo_gat_params* gat, float* out, int64_t ldout, int32_t concat_self, void* out_bf16,
+                     int64_t ldout_bf16, void* workspace, size_t workspace_bytes, void* stream) {
     if (!g || g->n_nodes < 0 || g->n_edges < 0 || g->n_nodes > INT32_MAX) return RETEXO_ERR_INVALID_ARG;
     if (type != RETEXO_GCN && type != RETEXO_SAGE_MEAN && type != RETEXO_GAT && type != RETEXO_SAGE_MAX)
         return RETEXO_ERR_INVALID_ARG;
@@ -801,7 +940,7 @@ int retexo::aggregate_rows(const retexo_csr* g, int32_t type, const float* q, in
         if ((int64_t)gat->heads * gat->head_dim != dim) return RETEXO_ERR_INVALID_ARG;
         if (gat->heads > kGatMaxHeads || dim > 256) return RETEXO_ERR_UNSUPPORTED;
     }
-    const size_t need = retexo_aggregate_workspace_size(g->n_nodes, g->n_edges, type, dim, gat ? gat->heads : 0);
+    const size_t need = aggregate_rows_workspace_size(g->n_nodes, g->n_edges, type, dim, gat ? gat->heads : 0, pieces16);
     if (!workspace || !aligned_to(workspace, kAlign) || workspace_bytes < need) return RETEXO_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int n_sm = sm_count();
@@ -839,6 +978,7 @@ int retexo::aggregate_rows(const retexo_csr* g, int32_t type, const float* q, in
     const bool v8 = aligned_to(q, 32) && ldq % 8 == 0 && ldq >= (dim + 7) / 8 * 8 && (whole_rows || (dim + 7) / 8 * 8 - dim <= 3);
     const bool v4 = aligned_to(q, 16) && ldq % 4 == 0 && ldq >= (dim + 3) / 4 * 4;
     const bool v2 = aligned_to(q, 8) && ldq % 2 == 0 && ldq >= (dim + 1) / 2 * 2;
+    if (pieces16 && !v4) return RETEXO_ERR_ALIGNMENT;
     auto lanes = [&](int op) {
         return v8 ? launch_lanes8(op, a, e, n_sm, st) : v4 ? launch_lanes4(op, a, e, n_sm, st)
              : v2 ? launch_lanes2(op, a, e, n_sm, st) : launch_lanes1(op, a, e, n_sm, st);
@@ -846,26 +986,17 @@ int retexo::aggregate_rows(const retexo_csr* g, int32_t type, const float* q, in
     const unsigned prep_blocks = (unsigned)((n + 255) / 256);
     if (type == RETEXO_GCN) {
         float* coef = ws.take<float>((size_t)n);
-        if (v4 && (size_t)n * (size_t)dim * 4 >= kHbmBoundBytes) {
-            prep_rows_kernel<<<prep_blocks, 256, 0, st>>>(n, g->rowptr, a.heavy, coef);
-            a.coef = coef;
-            a.hub_coef = (float)(1.0 / sqrt(4.0 * (double)e / (double)n + 1.0));      // hubs: at least four times the mean degree
-            const int chunks = (dim + 127) / 128;      // of 32 float4 vectors; more than 6: several passes
-            if (chunks <= 1) return launch_rows<1>(a, e, n_sm, st);
-            if (chunks <= 2) return launch_rows<2>(a, e, n_sm, st);
-            if (chunks <= 3) return launch_rows<3>(a, e, n_sm, st);
-            if (chunks <= 4) return launch_rows<4>(a, e, n_sm, st);
-            if (chunks <= 5) return launch_rows<5>(a, e, n_sm, st);
-            return launch_rows<6>(a, e, n_sm, st);
-        }
         const GcnWay way = gcn_way(n, e, dim);
-        if (way == GcnWay::kWeighted && v4) {
+        const int64_t copy = gcn_copy_floats(n, e, dim, v4);
+        if (copy == 0) {
             prep_rows_kernel<<<prep_blocks, 256, 0, st>>>(n, g->rowptr, a.heavy, coef);
             a.coef = coef;
-            return lanes(kOpGcnWeighted);
+            if (way != GcnWay::kHbm) return lanes(kOpGcnWeighted);
+            a.hub_coef = (float)(1.0 / sqrt(4.0 * (double)e / (double)n + 1.0));      // hubs: at least four times the mean degree
+            return v4 ? launch_rows<4>(a, e, n_sm, st) : v2 ? launch_rows<2>(a, e, n_sm, st) : launch_rows<1>(a, e, n_sm, st);
         }
+        float* qs = ws.take<float>((size_t)copy);
         const int64_t ld_qs = gcn_copy_stride(dim, n, e);
-        float* qs = ws.take<float>((size_t)n * (size_t)ld_qs);
         int lanes_log2 = 0;
         while (lanes_log2 < 5 && (8 << lanes_log2) < ld_qs) ++lanes_log2;
         const bool weighted = way == GcnWay::kWeighted;
@@ -878,4 +1009,19 @@ int retexo::aggregate_rows(const retexo_csr* g, int32_t type, const float* q, in
     }
     if (e >= heavy_degree(e)) prep_rows_kernel<<<prep_blocks, 256, 0, st>>>(n, g->rowptr, a.heavy, nullptr);
     return lanes(type == RETEXO_SAGE_MAX ? kOpMax : kOpSum);
+}
+
+extern "C" int retexo_aggregate(const retexo_csr* g, int32_t type, const float* q, int64_t ldq, int32_t dim,
+                                const retexo_gat_params* gat, float* out, int64_t ldout,
+                                int32_t concat_self, void* out_bf16, int64_t ldout_bf16,
+                                void* workspace, size_t workspace_bytes, void* stream) {
+    return aggregate(g, type, q, ldq, dim, false, false, gat, out, ldout, concat_self, out_bf16, ldout_bf16, workspace, workspace_bytes,
+                     stream);
+}
+
+int retexo::aggregate_rows(const retexo_csr* g, int32_t type, const float* q, int64_t ldq, int32_t dim, bool whole_rows, float* out,
+                           int64_t ldout, int32_t concat_self, void* out_bf16, int64_t ldout_bf16, void* workspace,
+                           size_t workspace_bytes, void* stream) {
+    return aggregate(g, type, q, ldq, dim, whole_rows, true, nullptr, out, ldout, concat_self, out_bf16, ldout_bf16, workspace,
+                     workspace_bytes, stream);
 }

@@ -233,7 +233,7 @@ static void lmp_layout(const retexo_lmp_config& c, int64_t n, int64_t e, int64_t
         if (s > step_b) step_b = s;
         s = retexo_embed_workspace_size_norm(r.d_in, r.hidden, c.n_classes, n, c.norm);
         if (s > embed_b) embed_b = s;
-        s = retexo_aggregate_workspace_size(n, e, c.aggr, r.agg_dim, c.gat_heads);
+        s = aggregate_rows_workspace_size(n, e, c.aggr, r.agg_dim, c.gat_heads, true);
         if (s > agg_b) agg_b = s;
     }
     const int64_t ld16 = round_up(max_din, 64);      // bf16 rows start on 128-byte lines
@@ -479,7 +479,7 @@ extern "C" int retexo_lmp_train(const retexo_lmp_config* cfg, const retexo_lmp_i
             }
         } else {
             // (the caller's own features need not hold the last row's padding)
-            RETEXO_TRY(aggregate_rows(&g, c.aggr, q, ldq, r.agg_dim, q != in->features, nullptr, nullptr, 0, 1, b.x16, ld16, b.ws_agg,
+            RETEXO_TRY(aggregate_rows(&g, c.aggr, q, ldq, r.agg_dim, q != in->features, nullptr, 0, 1, b.x16, ld16, b.ws_agg,
                                       b.ws_agg_bytes, st));
         }
 

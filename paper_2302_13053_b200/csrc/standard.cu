@@ -230,7 +230,7 @@ static void std_layout(const retexo_standard_config& c, int64_t n, int64_t e, in
     b.ws_step = t.template take<uint8_t>(b.ws_step_bytes);
     size_t agg = 0;
     for (int m = 0; m < c.K; ++m) {
-        const size_t s = retexo_aggregate_workspace_size(n, e, c.aggr, b.L[m].rep, 0);
+        const size_t s = aggregate_rows_workspace_size(n, e, c.aggr, b.L[m].rep, 0, true);
         if (s > agg) agg = s;
     }
     b.ws_agg_bytes = agg;
@@ -310,7 +310,7 @@ extern "C" int retexo_standard_train(const retexo_standard_config* cfg, const re
         feat = b.feat;
         ld_feat = b.ld_feat;
     }
-    RETEXO_TRY(aggregate_rows(&g, c.aggr, feat, ld_feat, c.d0, relaid, nullptr, nullptr, 0, sage ? 1 : 0, b.L[0].x, b.L[0].ldx, b.ws_agg,
+    RETEXO_TRY(aggregate_rows(&g, c.aggr, feat, ld_feat, c.d0, relaid, nullptr, 0, sage ? 1 : 0, b.L[0].x, b.L[0].ldx, b.ws_agg,
                               b.ws_agg_bytes, st));
 
     const MlpPlan plan = make_plan(last.d, 0, c.n_classes, n_tr, n_val);
@@ -334,7 +334,7 @@ extern "C" int retexo_standard_train(const retexo_standard_config* cfg, const re
             f.relu_bits = l.bits; f.ld_bits = l.ld_bits; f.status = sb.status;
             RETEXO_TRY(tc_gemm_launch(f, st));
             StdLayer& nx = b.L[m + 1];
-            RETEXO_TRY(aggregate_rows(&g, c.aggr, l.h, l.ld_h32, c.hidden, true, nullptr, nullptr, 0, sage ? 1 : 0, nx.x, nx.ldx,
+            RETEXO_TRY(aggregate_rows(&g, c.aggr, l.h, l.ld_h32, c.hidden, true, nullptr, 0, sage ? 1 : 0, nx.x, nx.ldx,
                                         b.ws_agg, b.ws_agg_bytes, st));
         }
         return RETEXO_OK;
@@ -375,11 +375,11 @@ extern "C" int retexo_standard_train(const retexo_standard_config* cfg, const re
             const unsigned eb = std_row_blocks(n), et = 32 * kStdRowWarps;
             if (sage) {
                 if (m < K - 2) std_prescale_kernel<<<eb, et, 0, st>>>(b.g, b.ld_g, H, H, g.rowptr, n, b.s, b.ld_a);
-                RETEXO_TRY(aggregate_rows(&g, RETEXO_SAGE_MEAN, b.s, b.ld_a, H, true, nullptr, b.a, b.ld_a, 0, nullptr, 0, b.ws_agg,
+                RETEXO_TRY(aggregate_rows(&g, RETEXO_SAGE_MEAN, b.s, b.ld_a, H, true, b.a, b.ld_a, 0, nullptr, 0, b.ws_agg,
                                             b.ws_agg_bytes, st));
                 std_gate_kernel<<<eb, et, 0, st>>>(b.a, b.ld_a, b.g, b.ld_g, g.rowptr, l.bits, l.ld_bits, n, H, b.dz, b.ld_dz);
             } else {
-                RETEXO_TRY(retexo_aggregate(&g, RETEXO_GCN, b.g, b.ld_g, H, nullptr, b.a, b.ld_a, 0, nullptr, 0, b.ws_agg,
+                RETEXO_TRY(aggregate_rows(&g, RETEXO_GCN, b.g, b.ld_g, H, true, b.a, b.ld_a, 0, nullptr, 0, b.ws_agg,
                                             b.ws_agg_bytes, st));
                 std_gate_kernel<<<eb, et, 0, st>>>(b.a, b.ld_a, nullptr, 0, g.rowptr, l.bits, l.ld_bits, n, H, b.dz, b.ld_dz);
             }

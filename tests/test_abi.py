@@ -49,6 +49,20 @@ def test_status_strings_and_sizes(lib):
     assert 0 < small < big
 
 
+def test_aggregation_workspace_holds_a_copy_of_the_rows_only_where_one_is_made(lib):
+    lib.retexo_aggregate_workspace_size.restype = C.c_size_t
+
+    def size(n, e, dim, type=0):
+        return lib.retexo_aggregate_workspace_size(C.c_int64(n), C.c_int64(e), C.c_int32(type), C.c_int32(dim), C.c_int32(0))
+
+    partial = size(2449029, 123718280, 100, type=1)                     # mean: segment sums alone
+    assert partial < 250 << 20
+    # the rows stay where they are: bound by memory, or copies beyond 2 GB
+    for n, e, dim in ((2449029, 123718280, 100), (2449029, 123718280, 256), (4000000, 4000000, 512)):
+        assert size(n, e, dim) - size(n, e, dim, type=1) < 4 * n + 1024
+    assert 4 * 100000 * 100 <= size(100000, 4000000, 100) - size(100000, 4000000, 100, type=1) <= 4 * 100000 * 132   # scaled rows
+
+
 def test_bad_arguments_are_rejected_on_the_host(lib):
     from paper_2302_13053_b200.binding import _Csr, _Mlp
     INVALID, WORKSPACE = 1, 4

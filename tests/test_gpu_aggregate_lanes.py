@@ -109,3 +109,34 @@ def test_gcn_precision_of_short_rows(n, degree, dim, ld):
     err, bound = (np.linalg.norm(x - ref) for x in (out.cpu().numpy(), chain))
     print(degree, dim, ld, err / bound)
     assert err <= 1.02 * bound, err / bound                   # 1.02: the noise of 1e5 to 2e6 rounding errors is below 1 %
+
+
+@pytest.mark.parametrize("degree,dim,ld", [(16, 340, 340), (16, 450, 452), (16, 602, 604),
+                                         (16, 768, 768), (16, 800, 800), (32, 97, 100),
+                                         (16, 250, 250), (16, 450, 450), (16, 193, 193)])
+def test_rows_bound_by_memory(degree, dim, ld):
+    """GCN on graphs whose slabs of 64 columns are far beyond the cache: every number of column chunks in one pass, two passes, rows in
+    8- and 4-byte pieces; rows of every length against 64 bits."""
+    from paper_2302_13053_b200 import binding as B
+    n = 2097152
+    g = torch.Generator(device="cuda").manual_seed(dim)
+    ladder = torch.tensor([0, 1, 2, 3, 31, 32, 33, 127, 129, 4000, 100000], device="cuda")
+    deg = torch.full((n,), degree, device="cuda")
+    rows = torch.randperm(n, generator=g, device="cuda")[:len(ladder)]
+    deg[rows] = ladder
+    rows = torch.cat([rows, torch.randint(0, n, (100,), generator=g, device="cuda"), torch.tensor([0, n - 1], device="cuda")])
+    rp = torch.zeros((n + 1,), dtype=torch.int64, device="cuda")
+    rp[1:] = torch.cumsum(deg, 0)
+    ci = torch.randint(0, n, (int(rp[-1]),), generator=g, device="cuda", dtype=torch.int32)
+    assert ci.numel() >= degree * n
+    q = torch.rand((n, ld), generator=g, device="cuda") + 0.1
+    q[:, dim:] = float("nan")
+    out, out16 = B.retexo_aggregate(oracle.GCN, rp, ci, q, dim=dim, want_bf16=True)
+    c = 1.0 / torch.sqrt(deg.double() + 1)
+    for v in rows.tolist():
+        u = ci[rp[v]:rp[v + 1]].long()
+        want = c[v] * ((q[u, :dim].double() * c[u][:, None]).sum(0) + c[v] * q[v, :dim].double())
+        assert (out[v].double() - want).norm() <= 1e-5 * want.norm(), (v, int(deg[v]))
+        assert torch.equal(out16[v, :dim], out[v].to(torch.bfloat16))
+    again, _ = B.retexo_aggregate(oracle.GCN, rp, ci, q, dim=dim)
+    assert torch.equal(out, again)
