@@ -119,6 +119,12 @@ __global__ void __launch_bounds__(256) relay_rows_kernel(const float* __restrict
         d[p] = make_float4(v[0], v[1], v[2], v[3]);
     }
 }
+// Rows of features that arrive in dense host rows at a time: 64 MB of them.  (A copy of that size runs at the link's rate, and the
+// re-lay of one chunk, 25 us, is small beside its copy, 1.2 ms.)
+static int64_t staged_rows(int64_t n, int32_t d0) {
+    const int64_t rows = ((int64_t)64 << 20) / (4 * (int64_t)d0);
+    return rows < 1 ? 1 : rows < n ? rows : n;
+}
 __global__ void fill_u64_kernel(unsigned long long* p, int64_t n, unsigned long long v) {
     const int64_t i = blockIdx.x * 256ll + threadIdx.x;
     if (i < n) p[i] = v;
@@ -239,8 +245,8 @@ static void lmp_layout(const retexo_lmp_config& c, int64_t n, int64_t e, int64_t
     const int64_t ld16 = round_up(max_din, 64);      // bf16 rows start on 128-byte lines
     l.features = t.template take<float>((size_t)n * round_up(c.d0, 32));   // 128-byte-row copy of the features
     if (host) {
-        // rows as the caller packs them, where they have to be re-laid on the device
-        l.features_in = t.template take<float>(c.d0 % 4 != 0 ? (size_t)n * c.d0 : 1);
+        // some rows as the caller packs them, where they have to be re-laid on the device
+        l.features_in = t.template take<float>(c.d0 % 4 != 0 ? (size_t)staged_rows(n, c.d0) * c.d0 : 1);
         l.rowptr = t.template take<int64_t>((size_t)n + 1);
         l.colidx = t.template take<int32_t>((size_t)e);
         l.labels = t.template take<int32_t>((size_t)n);
@@ -390,9 +396,15 @@ extern "C" int retexo_lmp_train(const retexo_lmp_config* cfg, const retexo_lmp_i
         const bool dense = ld_feat == c.d0, keep = dense && c.d0 % 4 == 0;
         const int64_t ldp = keep ? c.d0 : round_up(c.d0, 32);
         if (dense) {
-            float* to = keep ? b.features : b.features_in;
-            RETEXO_CUDA_TRY(cudaMemcpyAsync(to, feat, sizeof(float) * (size_t)n * c.d0, in_kind, st));
-            if (!keep) relay_rows_kernel<<<(unsigned)((n + 7) / 8), 256, 0, st>>>(to, c.d0, c.d0, n, b.features, ldp);
+            const int64_t step = keep ? n : staged_rows(n, c.d0);
+            for (int64_t r = 0; r < n; r += step) {
+                const int64_t rows = step < n - r ? step : n - r;
+                RETEXO_CUDA_TRY(cudaMemcpyAsync(keep ? b.features : b.features_in, feat + r * c.d0,
+                                                sizeof(float) * (size_t)rows * c.d0, in_kind, st));
+                if (!keep)
+                    relay_rows_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(b.features_in, c.d0, c.d0, rows,
+                                                                                  b.features + r * ldp, ldp);
+            }
         } else {
             if (ldp != c.d0) RETEXO_CUDA_TRY(cudaMemsetAsync(b.features, 0, sizeof(float) * (size_t)n * ldp, st));
             RETEXO_CUDA_TRY(cudaMemcpy2DAsync(b.features, sizeof(float) * ldp, feat, sizeof(float) * ld_feat,

@@ -63,6 +63,21 @@ def test_aggregation_workspace_holds_a_copy_of_the_rows_only_where_one_is_made(l
     assert 4 * 100000 * 100 <= size(100000, 4000000, 100) - size(100000, 4000000, 100, type=1) <= 4 * 100000 * 132   # scaled rows
 
 
+def test_host_features_need_no_second_matrix_on_the_device(lib):
+    from paper_2302_13053_b200.binding import _LmpConfig
+    lib.retexo_lmp_workspace_size.restype = C.c_size_t
+    n, e = 2449029, 123718280
+
+    def size(d0, host):
+        cfg = _LmpConfig(0, 2, 10, d0, 64, 47, 0, 0.01, 0.9, 0.999, 1e-8, 1, 0, 0, 0.2, host, 0.0, 0, 0, 0, 1e-5, 0.1)
+        return lib.retexo_lmp_workspace_size(C.byref(cfg), C.c_int64(n), C.c_int64(e), C.c_int64(200000), C.c_int64(40000),
+                                             C.c_int64(2000000), C.c_int32(0))
+
+    # rows of 99 columns are re-laid on the device from pieces of 64 MB; rows of 100 stay as they come
+    assert size(100, 0) > 0
+    assert 0 < size(99, 1) - size(100, 1) <= (64 << 20)
+
+
 def test_bad_arguments_are_rejected_on_the_host(lib):
     from paper_2302_13053_b200.binding import _Csr, _Mlp
     INVALID, WORKSPACE = 1, 4

@@ -206,6 +206,27 @@ def test_host_buffer_run_gives_the_same_bits_as_the_device_run():
     assert res[0]["counts"]["boundary_pairs"] == res[1]["counts"]["boundary_pairs"]
 
 
+def test_host_features_that_arrive_in_several_pieces():
+    """Dense host rows that don't start on 16-byte boundaries come over 64 MB at a time: three pieces, the last one short."""
+    from paper_2302_13053_b200 import binding as B
+    rng = np.random.default_rng(5)
+    n, d0, classes = 20000, 2049, 5
+    rowptr, colidx = wl.csr_from_edge_list(n, rng.integers(0, n, size=(2 * n, 2)))
+    features = rng.standard_normal((n, d0), dtype=np.float32)
+    labels = rng.integers(0, classes, size=n).astype(np.int32)
+    perm = rng.permutation(n).astype(np.int32)
+    ws = [dict(w1=rng.standard_normal((d0, classes)).astype(np.float32) / 45, b1=np.zeros(classes, np.float32))]
+    res = []
+    for host in (False, True):
+        prob = B.LmpProblem(wl.GCN, 1, 3, 0, classes, 0.01, rowptr, colidx, features, labels, perm[:10000], perm[10000:12000],
+                            perm[12000:], ws, host=host)
+        B.retexo_lmp_train(prob)
+        torch.cuda.synchronize()
+        res.append(prob.results())
+    np.testing.assert_array_equal(res[0]["loss_history"], res[1]["loss_history"])
+    np.testing.assert_array_equal(res[0]["final_logits"], res[1]["final_logits"])
+
+
 def test_eval_every_skips_validation_and_marks_the_gaps():
     w = wl.make_config(1, scale=0.3)
     ref, got = run_both(w, 10, eval_every=4)
