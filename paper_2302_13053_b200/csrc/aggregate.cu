@@ -848,6 +848,26 @@ static int launch_rows(const AggArgs& a, int64_t n_edges, int n_sm, cudaStream_t
     return launch_rows<E, 6>(a, n_edges, n_sm, st);
 }
 
+// ---------------------------------------------------------------- rows laid out for wide loads
+// dst[i] = [src[i] | zeros], rows of ld_dst (a multiple of 4) floats from densely packed or strided rows of dim floats: the re-lay
+// of features whose rows do not start on 16-byte boundaries.  A warp a row, whole 16-byte stores; a stream (561 MB in, 566 MB
+// out: 193 us; a pitched device-to-device copy and the clearing of its padding took 420 us).
+__global__ void __launch_bounds__(256) relay_rows_kernel(const float* __restrict__ src, int64_t ld_src, int32_t dim, int64_t n,
+                                                         float* __restrict__ dst, int64_t ld_dst) {
+    const int lane = threadIdx.x & 31;
+    const int64_t i = blockIdx.x * 8ll + (threadIdx.x >> 5);
+    if (i >= n) return;
+    const float* s = src + i * ld_src;
+    float4* d = reinterpret_cast<float4*>(dst + i * ld_dst);
+#pragma unroll 4
+    for (int p = lane; p < (int)(ld_dst >> 2); p += 32) {
+        float v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = 4 * p + k < dim ? __ldcs(s + 4 * p + k) : 0.f;
+        d[p] = make_float4(v[0], v[1], v[2], v[3]);
+    }
+}
+
 // ---------------------------------------------------------------- which way a GCN round goes (by its sizes alone)
 // Dense: rows of 32 entries or more on average.
 static bool gcn_dense(int64_t n, int64_t n_edges) { return n_edges >= 32 * n; }
@@ -882,12 +902,12 @@ static GcnWay gcn_way(int64_t n, int64_t n_edges, int32_t dim) {
     return gcn_dense(n, n_edges) ? GcnWay::kScaled : dim <= 16 ? GcnWay::kNarrow : GcnWay::kWeighted;
 }
 
-// Floats of the copy, 0 where there is none: scaled rows, and rows to be weighted that do not come in 16-byte pieces, up to 2 GB (beyond
-// that a round gathers the caller's rows as they are, a few per cent slower when dense, up to half when narrow pieces are all there
-// is; the largest graphs are where memory is short).
-static int64_t gcn_copy_floats(int64_t n, int64_t n_edges, int32_t dim, bool pieces16) {
+// Floats of the copy, 0 where there is none: scaled rows, and (lay_out) rows to be weighted that do not come in 16-byte pieces, up to
+// 2 GB (beyond that a round gathers the caller's rows as they are, a few per cent slower when dense, up to half when narrow pieces are
+// all there is; the largest graphs are where memory is short).
+static int64_t gcn_copy_floats(int64_t n, int64_t n_edges, int32_t dim, bool lay_out) {
     const GcnWay way = gcn_way(n, n_edges, dim);
-    if (way == GcnWay::kHbm || (way == GcnWay::kWeighted && pieces16)) return 0;
+    if (way == GcnWay::kHbm || (way == GcnWay::kWeighted && !lay_out)) return 0;
     const int64_t floats = n * gcn_copy_stride(dim, n, n_edges);
     return floats <= ((int64_t)2 << 30) / 4 ? floats : 0;
 }
@@ -896,7 +916,7 @@ static int64_t gcn_copy_floats(int64_t n, int64_t n_edges, int32_t dim, bool pie
 
 using namespace retexo;
 
-size_t retexo::aggregate_rows_workspace_size(int64_t n_nodes, int64_t n_edges, int32_t type, int32_t dim, int32_t heads, bool pieces16) {
+size_t retexo::aggregate_rows_workspace_size(int64_t n_nodes, int64_t n_edges, int32_t type, int32_t dim, int32_t heads, bool lay_out) {
     Sizer s;
     if (n_nodes < 0) return 0;
     if (type == RETEXO_GAT) {
@@ -909,7 +929,7 @@ size_t retexo::aggregate_rows_workspace_size(int64_t n_nodes, int64_t n_edges, i
         s.take<float>((size_t)max_segments(n_edges) * (size_t)((dim + 3) / 4 * 4));   // segment sums
         if (type == RETEXO_GCN) {
             s.take<float>((size_t)n_nodes);                               // coef
-            s.take<float>((size_t)gcn_copy_floats(n_nodes, n_edges, dim, pieces16));
+            s.take<float>((size_t)gcn_copy_floats(n_nodes, n_edges, dim, lay_out));
         }
     }
     return s.off + kAlign;
@@ -917,10 +937,10 @@ size_t retexo::aggregate_rows_workspace_size(int64_t n_nodes, int64_t n_edges, i
 
 // (the caller's alignment is not known here)
 extern "C" size_t retexo_aggregate_workspace_size(int64_t n_nodes, int64_t n_edges, int32_t type, int32_t dim, int32_t heads) {
-    return aggregate_rows_workspace_size(n_nodes, n_edges, type, dim, heads, false);
+    return aggregate_rows_workspace_size(n_nodes, n_edges, type, dim, heads, true);
 }
 
-static int aggregate(const retexo_csr* g, int32_t type, const float* q, int64_t ldq, int32_t dim, bool whole_rows, bool pieces16,
+static int aggregate(const retexo_csr* g, int32_t type, const float* q, int64_t ldq, int32_t dim, bool whole_rows, bool lay_out,
                      const retexo_gat_params* gat, float* out, int64_t ldout, int32_t concat_self, void* out_bf16,
                      int64_t ldout_bf16, void* workspace, size_t workspace_bytes, void* stream) {
     if (!g || g->n_nodes < 0 || g->n_edges < 0 || g->n_nodes > INT32_MAX) return RETEXO_ERR_INVALID_ARG;
@@ -940,7 +960,7 @@ static int aggregate(const retexo_csr* g, int32_t type, const float* q, int64_t 
         if ((int64_t)gat->heads * gat->head_dim != dim) return RETEXO_ERR_INVALID_ARG;
         if (gat->heads > kGatMaxHeads || dim > 256) return RETEXO_ERR_UNSUPPORTED;
     }
-    const size_t need = aggregate_rows_workspace_size(g->n_nodes, g->n_edges, type, dim, gat ? gat->heads : 0, pieces16);
+    const size_t need = aggregate_rows_workspace_size(g->n_nodes, g->n_edges, type, dim, gat ? gat->heads : 0, lay_out);
     if (!workspace || !aligned_to(workspace, kAlign) || workspace_bytes < need) return RETEXO_ERR_WORKSPACE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int n_sm = sm_count();
@@ -978,7 +998,6 @@ static int aggregate(const retexo_csr* g, int32_t type, const float* q, int64_t 
     const bool v8 = aligned_to(q, 32) && ldq % 8 == 0 && ldq >= (dim + 7) / 8 * 8 && (whole_rows || (dim + 7) / 8 * 8 - dim <= 3);
     const bool v4 = aligned_to(q, 16) && ldq % 4 == 0 && ldq >= (dim + 3) / 4 * 4;
     const bool v2 = aligned_to(q, 8) && ldq % 2 == 0 && ldq >= (dim + 1) / 2 * 2;
-    if (pieces16 && !v4) return RETEXO_ERR_ALIGNMENT;
     auto lanes = [&](int op) {
         return v8 ? launch_lanes8(op, a, e, n_sm, st) : v4 ? launch_lanes4(op, a, e, n_sm, st)
              : v2 ? launch_lanes2(op, a, e, n_sm, st) : launch_lanes1(op, a, e, n_sm, st);
@@ -987,7 +1006,7 @@ static int aggregate(const retexo_csr* g, int32_t type, const float* q, int64_t 
     if (type == RETEXO_GCN) {
         float* coef = ws.take<float>((size_t)n);
         const GcnWay way = gcn_way(n, e, dim);
-        const int64_t copy = gcn_copy_floats(n, e, dim, v4);
+        const int64_t copy = gcn_copy_floats(n, e, dim, lay_out && !v4);
         if (copy == 0) {
             prep_rows_kernel<<<prep_blocks, 256, 0, st>>>(n, g->rowptr, a.heavy, coef);
             a.coef = coef;
@@ -1011,17 +1030,26 @@ static int aggregate(const retexo_csr* g, int32_t type, const float* q, int64_t 
     return lanes(type == RETEXO_SAGE_MAX ? kOpMax : kOpSum);
 }
 
+bool retexo::aggregate_copies_rows(int64_t n_nodes, int64_t n_edges, int32_t type, int32_t dim) {
+    return type == RETEXO_GCN && gcn_copy_floats(n_nodes, n_edges, dim, false) > 0;
+}
+
+int retexo::relay_rows_launch(const float* src, int64_t ld_src, int32_t dim, int64_t n, float* dst, int64_t ld_dst, cudaStream_t st) {
+    relay_rows_kernel<<<(unsigned)((n + 7) / 8), 256, 0, st>>>(src, ld_src, dim, n, dst, ld_dst);
+    return launch_status();
+}
+
 extern "C" int retexo_aggregate(const retexo_csr* g, int32_t type, const float* q, int64_t ldq, int32_t dim,
                                 const retexo_gat_params* gat, float* out, int64_t ldout,
                                 int32_t concat_self, void* out_bf16, int64_t ldout_bf16,
                                 void* workspace, size_t workspace_bytes, void* stream) {
-    return aggregate(g, type, q, ldq, dim, false, false, gat, out, ldout, concat_self, out_bf16, ldout_bf16, workspace, workspace_bytes,
+    return aggregate(g, type, q, ldq, dim, false, true, gat, out, ldout, concat_self, out_bf16, ldout_bf16, workspace, workspace_bytes,
                      stream);
 }
 
 int retexo::aggregate_rows(const retexo_csr* g, int32_t type, const float* q, int64_t ldq, int32_t dim, bool whole_rows, float* out,
                            int64_t ldout, int32_t concat_self, void* out_bf16, int64_t ldout_bf16, void* workspace,
                            size_t workspace_bytes, void* stream) {
-    return aggregate(g, type, q, ldq, dim, whole_rows, true, nullptr, out, ldout, concat_self, out_bf16, ldout_bf16, workspace,
+    return aggregate(g, type, q, ldq, dim, whole_rows, false, nullptr, out, ldout, concat_self, out_bf16, ldout_bf16, workspace,
                      workspace_bytes, stream);
 }

@@ -101,24 +101,6 @@ __global__ void merge_status_kernel(int32_t* run, const int32_t* a, const int32_
     if (*run == 0 && a && *a != 0) *run = *a;
     if (*run == 0 && b && *b != 0) *run = *b;
 }
-// dst[i] = [src[i] | zeros], rows of ld_dst (a multiple of 4) floats from densely packed or strided rows of dim floats: the re-lay
-// of features whose rows do not start on 16-byte boundaries.  A warp a row, whole 16-byte stores; a stream (561 MB in, 566 MB
-// out: 193 us; a pitched device-to-device copy and the clearing of its padding took 420 us).
-__global__ void __launch_bounds__(256) relay_rows_kernel(const float* __restrict__ src, int64_t ld_src, int32_t dim, int64_t n,
-                                                         float* __restrict__ dst, int64_t ld_dst) {
-    const int lane = threadIdx.x & 31;
-    const int64_t i = blockIdx.x * 8ll + (threadIdx.x >> 5);
-    if (i >= n) return;
-    const float* s = src + i * ld_src;
-    float4* d = reinterpret_cast<float4*>(dst + i * ld_dst);
-#pragma unroll 4
-    for (int p = lane; p < (int)(ld_dst >> 2); p += 32) {
-        float v[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) v[k] = 4 * p + k < dim ? __ldcs(s + 4 * p + k) : 0.f;
-        d[p] = make_float4(v[0], v[1], v[2], v[3]);
-    }
-}
 // Rows of features that arrive in dense host rows at a time: 64 MB of them.  (A copy of that size runs at the link's rate, and the
 // re-lay of one chunk, 25 us, is small beside its copy, 1.2 ms.)
 static int64_t staged_rows(int64_t n, int32_t d0) {
@@ -239,7 +221,7 @@ static void lmp_layout(const retexo_lmp_config& c, int64_t n, int64_t e, int64_t
         if (s > step_b) step_b = s;
         s = retexo_embed_workspace_size_norm(r.d_in, r.hidden, c.n_classes, n, c.norm);
         if (s > embed_b) embed_b = s;
-        s = aggregate_rows_workspace_size(n, e, c.aggr, r.agg_dim, c.gat_heads, true);
+        s = aggregate_rows_workspace_size(n, e, c.aggr, r.agg_dim, c.gat_heads, false);
         if (s > agg_b) agg_b = s;
     }
     const int64_t ld16 = round_up(max_din, 64);      // bf16 rows start on 128-byte lines
@@ -401,9 +383,7 @@ extern "C" int retexo_lmp_train(const retexo_lmp_config* cfg, const retexo_lmp_i
                 const int64_t rows = step < n - r ? step : n - r;
                 RETEXO_CUDA_TRY(cudaMemcpyAsync(keep ? b.features : b.features_in, feat + r * c.d0,
                                                 sizeof(float) * (size_t)rows * c.d0, in_kind, st));
-                if (!keep)
-                    relay_rows_kernel<<<(unsigned)((rows + 7) / 8), 256, 0, st>>>(b.features_in, c.d0, c.d0, rows,
-                                                                                  b.features + r * ldp, ldp);
+                if (!keep) RETEXO_TRY(relay_rows_launch(b.features_in, c.d0, c.d0, rows, b.features + r * ldp, ldp, st));
             }
         } else {
             if (ldp != c.d0) RETEXO_CUDA_TRY(cudaMemsetAsync(b.features, 0, sizeof(float) * (size_t)n * ldp, st));
@@ -422,7 +402,7 @@ extern "C" int retexo_lmp_train(const retexo_lmp_config* cfg, const retexo_lmp_i
         // rows that do not start on 16-byte boundaries would force narrow loads on the dominant
         // gather of round 1: re-lay them once with rows of whole 128-byte lines
         const int64_t ldp = round_up(c.d0, 32);
-        relay_rows_kernel<<<(unsigned)((n + 7) / 8), 256, 0, st>>>(feat, ld_feat, c.d0, n, b.features, ldp);
+        RETEXO_TRY(relay_rows_launch(feat, ld_feat, c.d0, n, b.features, ldp, st));
         feat = b.features;
         ld_feat = ldp;
     }

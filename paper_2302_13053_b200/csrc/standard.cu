@@ -46,14 +46,6 @@ constexpr int kStdRowWarps = 8;
 __device__ __forceinline__ int64_t std_row() { return blockIdx.x * (int64_t)kStdRowWarps + (threadIdx.x >> 5); }
 static unsigned std_row_blocks(int64_t n) { return (unsigned)((n + kStdRowWarps - 1) / kStdRowWarps); }
 
-// dst[i] = [src[i][0 .. dim) | zeros]: features whose rows do not start on 16-byte boundaries, laid out for wide loads.
-static __global__ void __launch_bounds__(32 * kStdRowWarps) std_relay_kernel(const float* __restrict__ src, int64_t ld_src, int32_t dim, int64_t n,
-                                                                             float* __restrict__ dst, int64_t ld_dst) {
-    const int64_t v = std_row();
-    if (v >= n) return;
-#pragma unroll 8
-    for (int c = threadIdx.x & 31; c < ld_dst; c += 32) dst[v * ld_dst + c] = c < dim ? __ldcs(src + v * ld_src + c) : 0.f;
-}
 // The batch-ordered gradient dx[i][0 .. dim) goes to node order (the destinations are cleared before).  GCN (s == nullptr): all of
 // it to g.  SAGE: the self half to g, the mean half, divided by the degree for the transposed mean, to s.
 static __global__ void __launch_bounds__(32 * kStdRowWarps) std_scatter_rows_kernel(const float* __restrict__ dx, int64_t ld_dx,
@@ -140,7 +132,7 @@ struct StdLayer {
 
 struct StdBuffers {
     StdLayer L[kStdMaxLayers];
-    float* feat; int64_t ld_feat;   // features in rows of whole 128-byte lines (copied only if the caller's rows are not 16-byte aligned)
+    float* later; int64_t n_later;  // every H^m, then g, a and s
     float* g; int64_t ld_g;     // gradient at an aggregated matrix X^m, node order [n x ld_g]
     float* a; int64_t ld_a;     // result of a transposed aggregation [n x ld_a]
     float* s;                   // SAGE: scaled mean half [n x ld_a]
@@ -193,7 +185,6 @@ static void std_layout(const retexo_standard_config& c, int64_t n, int64_t e, in
         if (m < c.K - 1) {
             l.ld_h32 = std_round_up(c.hidden, 32);
             l.ld_bits = 2 * (((int64_t)c.hidden + 63) / 64);
-            l.h = t.template take<float>((size_t)n * l.ld_h32);
             l.bits = t.template take<uint32_t>((size_t)n * l.ld_bits);
             l.wt16 = t.template take<bf16>((size_t)l.out * l.ld_k);
             l.wr16 = t.template take<bf16>((size_t)l.d * l.ld_o1);
@@ -204,14 +195,20 @@ static void std_layout(const retexo_standard_config& c, int64_t n, int64_t e, in
         if (l.rep > max_rep && m > 0) max_rep = l.rep;
     }
     const StdLayer& last = b.L[c.K - 1];
-    b.ld_feat = std_round_up(c.d0, 32);
-    b.feat = t.template take<float>((size_t)n * b.ld_feat);
     b.ld_g = std_round_up(max_d, 32);
     b.ld_a = std_round_up(c.K > 1 ? c.hidden : 1, 32);
     b.ld_dz = std_round_up(c.K > 1 ? c.hidden : 1, 64);
-    b.g = t.template take<float>(c.K > 1 ? (size_t)n * b.ld_g : 1);
-    b.a = t.template take<float>(c.K > 1 ? (size_t)n * b.ld_a : 1);
-    b.s = t.template take<float>((c.K > 1 && c.aggr == RETEXO_SAGE_MEAN) ? (size_t)n * b.ld_a : 1);
+    // the matrices that are not in use before X^1 is: together, since the features may be laid out anew in their place
+    const int64_t per_h = std_round_up(n * b.ld_a, 64), per_g = std_round_up(n * b.ld_g, 64);
+    b.n_later = c.K > 1 ? (c.K - 1) * per_h + per_g + (c.aggr == RETEXO_SAGE_MEAN ? 2 : 1) * per_h : 0;
+    b.later = t.template take<float>(b.n_later > 0 ? (size_t)b.n_later : 1);
+    if (c.K > 1 && b.later) {
+        float* p = b.later;
+        for (int m = 0; m < c.K - 1; ++m, p += per_h) b.L[m].h = p;
+        b.g = p;
+        b.a = p + per_g;
+        if (c.aggr == RETEXO_SAGE_MEAN) b.s = b.a + per_h;
+    }
     b.dz = t.template take<bf16>(c.K > 1 ? (size_t)n * b.ld_dz : 1);
     const int64_t n_batch = n_tr + n_val > n_te ? n_tr + n_val : n_te;
     b.ld_xb = last.ldx;
@@ -230,7 +227,7 @@ static void std_layout(const retexo_standard_config& c, int64_t n, int64_t e, in
     b.ws_step = t.template take<uint8_t>(b.ws_step_bytes);
     size_t agg = 0;
     for (int m = 0; m < c.K; ++m) {
-        const size_t s = aggregate_rows_workspace_size(n, e, c.aggr, b.L[m].rep, 0, true);
+        const size_t s = aggregate_rows_workspace_size(n, e, c.aggr, b.L[m].rep, 0, false);
         if (s > agg) agg = s;
     }
     b.ws_agg_bytes = agg;
@@ -304,11 +301,15 @@ extern "C" int retexo_standard_train(const retexo_standard_config* cfg, const re
     RETEXO_TRY(launch_status());
     const float* feat = in->features;
     int64_t ld_feat = in->ld_features;
-    const bool relaid = ld_feat % 4 != 0 || !aligned_to(feat, 16);
+    // Rows that do not start on 16-byte boundaries would be gathered in narrower loads: they are laid out anew, once, where the room for
+    // it is there and the aggregation would not do so itself (230 k nodes, 57 M entries, SAGE mean of 602 columns: 17.7 ms and
+    // 0.2 to lay them out, 26.2 as they come).
+    const bool relaid = (ld_feat % 4 != 0 || !aligned_to(feat, 16)) && n * std_round_up(c.d0, 32) <= b.n_later &&
+                        !aggregate_copies_rows(n, e, c.aggr, c.d0);
     if (relaid) {
-        std_relay_kernel<<<std_row_blocks(n), 32 * kStdRowWarps, 0, st>>>(feat, ld_feat, c.d0, n, b.feat, b.ld_feat);
-        feat = b.feat;
-        ld_feat = b.ld_feat;
+        ld_feat = std_round_up(c.d0, 32);
+        RETEXO_TRY(relay_rows_launch(feat, in->ld_features, c.d0, n, b.later, ld_feat, st));
+        feat = b.later;
     }
     RETEXO_TRY(aggregate_rows(&g, c.aggr, feat, ld_feat, c.d0, relaid, nullptr, 0, sage ? 1 : 0, b.L[0].x, b.L[0].ldx, b.ws_agg,
                               b.ws_agg_bytes, st));

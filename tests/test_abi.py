@@ -78,6 +78,20 @@ def test_host_features_need_no_second_matrix_on_the_device(lib):
     assert 0 < size(99, 1) - size(100, 1) <= (64 << 20)
 
 
+def test_standard_training_holds_no_copy_of_the_features(lib):
+    from paper_2302_13053_b200.binding import _StandardConfig
+    lib.retexo_standard_workspace_size.restype = C.c_size_t
+    n = 232965
+
+    def size(d0):
+        cfg = _StandardConfig(1, 2, 10, d0, 256, 41, 0, 0.01, 0.9, 0.999, 1e-8)
+        return lib.retexo_standard_workspace_size(C.byref(cfg), C.c_int64(n), C.c_int64(1000000), C.c_int64(100000), C.c_int64(10000),
+                                                  C.c_int64(20000))
+
+    # [X^1 | 1] has 1216 columns of 2 bytes either way; rows of 608 columns instead of 576 are 30 MB of a copy (parameters: 5 MB)
+    assert 0 < size(576) <= size(607) < size(576) + (16 << 20)
+
+
 def test_bad_arguments_are_rejected_on_the_host(lib):
     from paper_2302_13053_b200.binding import _Csr, _Mlp
     INVALID, WORKSPACE = 1, 4

@@ -111,3 +111,37 @@ def test_a_second_run_gives_the_same_bits_and_other_aggregators_are_refused():
     with pytest.raises(B().RetexoError):
         B().StandardProblem(B().GAT, 1, w.hidden, w.n_classes, w.lr, w.rowptr, w.colidx, w.features, w.labels,
                             w.train_idx, w.val_idx, w.test_idx, ws)
+
+
+@pytest.mark.parametrize("aggr,hidden,d0,entries", [(1, 8, 77, 8), (1, 8, 203, 8), (0, 64, 77, 8), (0, 8, 203, 8), (0, 8, 77, 70), (0, 64, 77, 70)])
+def test_features_of_any_stride(aggr, hidden, d0, entries):
+    """Packed rows of an odd width, laid out anew in memory that is free at first, gathered as they come where that is too small, or
+    copied by the aggregation itself, against rows of 16-byte pieces: fp32 sums in another order."""
+    from paper_2302_13053_b200 import workloads as wl
+    rng = np.random.default_rng(d0)
+    n, classes = 3000, 7
+    rowptr, colidx = wl.csr_from_edge_list(n, rng.integers(0, n, size=(entries * n // 2, 2)))
+    x = rng.standard_normal((n, d0), dtype=np.float32)
+    mult = 2 if aggr == 1 else 1
+    dims = [(d0 * mult, hidden), (hidden * mult, classes)]
+    ws = [dict(w1=(rng.standard_normal(d) / np.sqrt(d[0])).astype(np.float32), b1=np.zeros(d[1], np.float32)) for d in dims]
+    perm = rng.permutation(n).astype(np.int32)
+    labels = rng.integers(0, classes, size=n).astype(np.int32)
+    got = []
+    for ld in (d0, (d0 + 7) // 8 * 8):
+        prob = B().StandardProblem(aggr, 1, hidden, classes, 0.01, rowptr, colidx, x, labels,
+                                   perm[:1000], perm[1000:1500], perm[1500:], ws, want_grad=True)
+        if ld != d0:
+            prob.features = torch.full((n, ld), float("nan"), device="cuda")
+            prob.features[:, :d0] = torch.from_numpy(x).cuda()
+            prob.inputs.features = prob.features.data_ptr()
+            prob.inputs.ld_features = ld
+        B().retexo_standard_train(prob)
+        torch.cuda.synchronize()
+        got.append(prob.results())
+        assert got[-1]["status"] == 0
+    a, b = got
+    assert abs(a["loss_history"][0] - b["loss_history"][0]) <= 2e-4 * max(1.0, abs(b["loss_history"][0]))
+    for ga, gb in zip(a["grad_last"], b["grad_last"]):
+        # (single units may pass the ReLU on one side only, as above)
+        assert np.median(np.abs(ga - gb)) <= 4e-5 * np.abs(gb).max()
