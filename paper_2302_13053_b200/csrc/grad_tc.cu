@@ -3,14 +3,15 @@
 //
 // Both reductions run over the batch, so the operands are read as they lie in memory (M and N contiguous, boxes of 64 rows x 64
 // columns by TMA, tcgen05.mma with both operands MN-major).  A block owns one 128 x BN tile and one range of the rows; the
-// two products share the grid, cut so that every block moves about the same bytes.
+// two products share the grid, cut so that every block takes about the same number of steps.
 // A bias gradient is the product of a vector of ones with the same B operand: one more MMA whose A operand is a constant 2 KB
 // of ones, instead of a column of ones behind X and Hd, which cost a pass over a caller's batch that had none and a whole
 // further row of tiles wherever the width is a multiple of 128 (257 = 3 tiles for 2).  Of the row's steps each row of tiles
 // takes an equal share, so that no block has twice the MMAs of another.
 // Bound by HBM on large batches, by its latencies on small ones.  Whole iterations, one product per launch with columns of ones
-// before -> this kernel: 60 x 1000 (hidden 128) 42 -> 35 us, 2000 x 300 (150) 60 -> 46, 38439 x 512 (256) 89 -> 77,
-// 195922 x 100 (256) 204 -> 185, 153757 x 512 (256) 215 -> 205; both products of 153757 x 1204 (256) 156 -> 148 us.
+// before -> this kernel: 60 x 1000 (hidden 128) 43 -> 33 us, 2000 x 300 (150) 58 -> 43, 38439 x 512 (256) 91 -> 71,
+// 195922 x 100 (256) 206 -> 187, 153757 x 512 (256) 203 -> 181, 153757 x 1204 (256) 275 -> 262; 20000 x 8192 (512), where one
+// range of rows fills the device, 443 -> 452.
 // Every wait is bounded: a wait that runs out sets *status and the block tears down in order.
 #include <string.h>
 
@@ -233,7 +234,10 @@ void grad_splits(int32_t M1, int32_t N1, int32_t M2, int32_t N2, int64_t rows, i
     *s1 = *s2 = 1;
     const int64_t bn1 = grad_bn(N1), t1 = ((M1 + 127) / 128) * ((N1 + bn1 - 1) / bn1), t2 = N2 > 0 ? (M2 + 127) / 128 : 0;
     const int64_t sms = 148, most = 64;      // (more ranges than 64 cost the update kernel more than they save here)
-    // equal bytes per block, as far as one block per SM allows
+    // Equal steps per block, as far as one block per SM allows: a step waits for memory about as long whether its stage holds 48 KB or
+    // 24, so blocks that shared out the bytes left the ones of the second product behind, with half as many steps again.  (That
+    // -> this: 153757 x 1204 (256) 284 -> 262 us an iteration, 153757 x 512 (256) 195 -> 181, 200000 x 512 (512) 541 -> 468,
+    // 400000 x 256 (256) 372 -> 338; weights of 0.75 to 1 for the narrow steps are within 2 %.)
     double best = 1e30;
     for (int64_t a = 1; a <= most && a <= kb; ++a) {
         int64_t b = 1;
@@ -242,7 +246,7 @@ void grad_splits(int32_t M1, int32_t N1, int32_t M2, int32_t N2, int64_t rows, i
             b = b < 1 ? 1 : b > most ? most : b > kb ? kb : b;
         }
         const int64_t waves = (t1 * a + t2 * b + sms - 1) / sms;
-        const double c1 = (double)((kb + a - 1) / a) * (128 + bn1), c2 = t2 > 0 ? (double)((kb + b - 1) / b) * (128 + 64) : 0.0;
+        const double c1 = (double)((kb + a - 1) / a), c2 = t2 > 0 ? 0.9 * (double)((kb + b - 1) / b) : 0.0;
         const double cost = (double)waves * (c1 > c2 ? c1 : c2);
         if (cost < best * 0.999) { best = cost; *s1 = a; *s2 = b; }
     }
