@@ -2,6 +2,7 @@
 partitions), rows around the 128-entry trip and the 1024-entry limit above which a block shares a row, rows without entries."""
 import numpy as np
 import pytest
+import torch
 
 from paper_2302_13053_b200 import workloads as wl
 from test_gpu_counts import compare
@@ -16,3 +17,30 @@ def test_row_lengths_around_the_limits(n_parts):
         n, rowptr, colidx, _ = wl.degree_ladder_graph(degrees, seed=n_parts)
         compare(rowptr, colidx, rng.integers(0, n_parts, n).astype(np.int32), n_parts)
         compare(rowptr, colidx, np.full(n, n_parts - 1, dtype=np.int32), n_parts)
+
+
+def _time(fn, repeats=7):
+    fn()
+    best = float("inf")
+    for _ in range(repeats):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        fn()
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b))
+    return best
+
+
+@pytest.mark.parametrize("n_parts", [8192])
+def test_cost_of_the_number_of_parts(n_parts):
+    """Messages per partition of short rows: a bitmap eight times as wide (1.84 times the time of 1000 partitions when each row read it whole)."""
+    from paper_2302_13053_b200 import binding as B
+    n, degree = 2000000, 24
+    rp = torch.arange(n + 1, device="cuda") * degree
+    ci = torch.randint(0, n, (n * degree,), device="cuda", dtype=torch.int32)
+    times = []
+    for parts in (n_parts, 1000):
+        part = torch.randint(0, parts, (n,), device="cuda", dtype=torch.int32)
+        times.append(_time(lambda: B.retexo_cross_partition_bytes(rp, ci, part, parts, [64])))
+    assert times[0] <= 1.5 * times[1], times
