@@ -10,7 +10,7 @@ from test_gpu_counts import compare
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n_parts", [1024, 1025, 2049, 4096, 4097])
+@pytest.mark.parametrize("n_parts", [1, 2, 255, 256, 257, 1024, 1025, 2049, 4096, 4097])
 def test_row_lengths_around_the_limits(n_parts):
     rng = np.random.default_rng(n_parts)
     for degrees in ([1], [0, 1, 31, 127, 128, 129, 1023], [1024, 1025, 2047, 2048, 5000] + [1100] * 20):
@@ -32,9 +32,10 @@ def _time(fn, repeats=7):
     return best
 
 
-@pytest.mark.parametrize("n_parts", [8192])
+@pytest.mark.parametrize("n_parts", [8192, 10])
 def test_cost_of_the_number_of_parts(n_parts):
-    """Messages per partition of short rows: a bitmap eight times as wide (1.84 times the time of 1000 partitions when each row read it whole)."""
+    """Messages per partition of short rows: a bitmap eight times as wide (1.84 times the time of 1000 partitions when each row read it whole), and
+    ten partitions, whose counts all rows add to (2.4 times when each row did so in global memory)."""
     from paper_2302_13053_b200 import binding as B
     n, degree = 2000000, 24
     rp = torch.arange(n + 1, device="cuda") * degree
