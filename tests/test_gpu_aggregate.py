@@ -201,9 +201,9 @@ def ladder_in_a_large_graph(n, seed):
 @pytest.mark.parametrize("aggr,n,dim", [(oracle.SAGE_MEAN, 120000, 850), (oracle.GCN, 170000, 602),
                                         (oracle.SAGE_MEAN, 300000, 340), (oracle.GCN, 300000, 342),
                                         (oracle.SAGE_MAX, 170000, 600)])
-def test_matrices_beyond_the_cache_take_the_column_slab_variant(aggr, n, dim):
-    """A feature matrix of 200 MB or more is aggregated slab of columns by slab of columns (32, 16
-    or 8 vectors per slab, by the number of rows): same tolerance, every degree bin, ragged last slab."""
+def test_matrices_beyond_the_cache(aggr, n, dim):
+    """Feature matrices of 400 MB, slab of 64 columns by slab and a ragged last one: same tolerance, every degree bin.  (Rows bound by
+    memory, gathered whole, are in test_gpu_aggregate_lanes.py.)"""
     rowptr, colidx = ladder_in_a_large_graph(n, seed=dim)
     rng = np.random.default_rng(dim)
     q = rng.standard_normal((n, dim)).astype(np.float32)

@@ -138,9 +138,32 @@ def test_embed_matches_checker_and_stated_tolerance(d_in, hidden, n_classes, n):
     # row gather
     idx = rng.integers(0, n, 77).astype(np.int32)
     sub = B().retexo_embed(gpu, x16, row_idx=dev(idx), want_logits=True)
-    # (gathered rows take the CUDA-core product, dense ones the tensor cores: same values up to
-    # summation order and the bf16 rounding of the hidden layer that follows it)
+    # (packed into a dense batch first; another tile shape may add in another order, and the hidden layer is rounded after it)
     assert_logits_close(sub["logits"].cpu().numpy(), lg[idx], rel=5e-3, what="row gather")
+
+
+@pytest.mark.parametrize("norm", [{}, dict(layer_norm=True), dict(batch_norm=True)])
+@pytest.mark.parametrize("n_rows", [75776, 75777, 160001])
+def test_embed_of_more_picked_rows_than_are_packed_at_a_time(n_rows, norm):
+    """Picked rows are packed 75776 at a time: exactly that many, one more, and three passes, against the dense rows."""
+    d_in, hidden, n_classes, n = 40, 72, 5, 3000
+    rng = np.random.default_rng(n_rows)
+    w = [rng.standard_normal(s).astype(np.float32) * 0.2 for s in ((d_in, hidden), (hidden,), (hidden, n_classes), (n_classes,))]
+    gpu = B().Mlp(d_in, hidden, n_classes, *w, **norm)
+    x16, _ = B().retexo_pack_rows(dev(rng.standard_normal((n, d_in)).astype(np.float32)))
+    y = rng.integers(0, n_classes, n).astype(np.int32)
+    idx = rng.integers(0, n, n_rows).astype(np.int32)
+    dense = B().retexo_embed(gpu, x16, want_hidden=True, want_logits=True)
+    got = B().retexo_embed(gpu, x16, row_idx=dev(idx), y=dev(y[idx]), want_hidden=True, want_hidden_bf16=True, want_logits=True, want_pred=True)
+    pick = dev(idx).long()
+    for name in ("hidden", "logits"):
+        want, have = dense[name][pick], got[name]
+        scale = want.abs().amax(dim=1, keepdim=True) + 1e-6
+        assert ((have - want).abs() <= 5e-3 * scale).all(), name
+    assert torch.equal(got["hidden_bf16"][:, :hidden], got["hidden"].to(torch.bfloat16))
+    pred = got["logits"].argmax(1)
+    assert torch.equal(got["pred"].long(), pred)
+    assert got["correct"] == int((pred.cpu().numpy() == y[idx]).sum())
 
 
 def test_argmax_tie_rule_lowest_index():
