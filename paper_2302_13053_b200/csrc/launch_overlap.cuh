@@ -1,10 +1,13 @@
-// Programmatic dependent launch for the kernels of one training iteration.  A kernel launched
-// through OverlapLaunch may be made resident while its predecessor in the stream is still
-// draining; it sets up what depends on no other kernel (barriers, tensor memory, descriptor
-// prefetch), then calls grid_dependency_wait(), which returns once the predecessor has finished
-// and its writes are visible.  Every such kernel calls the wait in every thread before its first
-// access to global memory, and releases its own successor only after that wait, so a kernel's
-// set-up never overlaps anything older than its direct predecessor.
+// Programmatic dependent launch for the kernels of one training iteration.  A kernel launched through OverlapLaunch may be made
+// resident while its predecessor in the stream is still draining; it sets up what depends on no other kernel (barriers, tensor memory,
+// descriptor prefetch), then calls grid_dependency_wait(), which returns once the predecessor has finished and its writes are visible.
+// Two rules:
+//  - Every such kernel calls the wait in every thread, and releases its own successor only after its wait.  So when a kernel starts,
+//    everything before its direct predecessor has finished: the predecessor's blocks have all seen that from their own wait.
+//  - Before the wait a kernel may read only what no direct predecessor writes, at any of its launch sites: between the kernel that wrote
+//    it and the one that reads it early at least one whole kernel lies in the stream.  It writes nothing before the wait.  Early reads
+//    are made by head_backward_kernel and reduce_update_kernel; their launches name the kernels in between, and whoever fuses or moves
+//    one of those has to look at these reads again.
 #pragma once
 #include <cuda_runtime.h>
 

@@ -393,6 +393,8 @@ int mlp_train_step_launch(const MlpPlan& p, const MlpBuffers& b, const retexo_ml
     const int64_t tiles = (((int64_t)d_in + 16) / 16) * ((out1 + 15) / 16) + (H > 0 ? (((int64_t)H + 16) / 16) * ((O + 15) / 16) : 0) +
                           ((ln || bn) ? ((int64_t)H + 15) / 16 : 0);      // (a normalisation's segment has 2 or 4 rows of hidden entries)
     u.status_out = model->status_out;
+    // (reads parameters, moments, iteration state and the validation count early: between the update, or the head's kernel that counted,
+    // and this lies the kernel of the weight gradients)
     OverlapLaunch ol(dim3((unsigned)tiles), dim3(256), 0, st);
     if (cudaLaunchKernelEx(&ol.cfg, p.split_w1 <= 16 ? reduce_update_kernel<16> : reduce_update_kernel<32>, u) != cudaSuccess) {
         (void)cudaGetLastError();
@@ -415,6 +417,7 @@ int linear_update_launch(int32_t d_in, int32_t out, float* theta, float* adam_m,
     u.w1t16 = wt16; u.ld_k = ld_k; u.w1r16 = wr16; u.ld_o1 = ld_o1;
     u.d_in = d_in; u.out1 = out; u.hidden = 0; u.n_classes = out;
     const int64_t tiles = (((int64_t)d_in + 16) / 16) * ((out + 15) / 16);
+    // (reads parameters and moments early: between two updates of a layer lie the next iteration's products)
     OverlapLaunch ol(dim3((unsigned)tiles), dim3(256), 0, st);
     if (cudaLaunchKernelEx(&ol.cfg, splits <= 16 ? reduce_update_kernel<16> : reduce_update_kernel<32>, u) != cudaSuccess) {
         (void)cudaGetLastError();

@@ -90,7 +90,7 @@ head_backward_kernel(const __grid_constant__ CUtensorMap map_hd, const __grid_co
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
-    // the weights are older than the kernel that this one overlaps (it wrote Hd): they need not wait for it
+    // W2 and b2 are older than the kernel that this one overlaps (it wrote Hd): they need not wait for it
     if (threadIdx.x == 0 && nt > 0) {
         mbar_expect_tx(bars + HB_W2_FULL, (uint32_t)np * kHbW2PanelBytes);
         for (int p = 0; p < np; ++p) tma_load_2d(w2_s + p * kHbW2PanelBytes, &map_w2, 64 * p, 0, bars + HB_W2_FULL);
@@ -427,6 +427,7 @@ int head_backward_launch(const HeadBackward& h, cudaStream_t st) {
     const int n_sm = sm_count();
     if (n_sm <= 0) return RETEXO_ERR_CUDA;
     const unsigned grid = (unsigned)(n_tiles < n_sm ? n_tiles : n_sm);
+    // (reads W2 and b2 early: between the update or the conversion that wrote them and this lies the product that writes Hd)
     OverlapLaunch ol(dim3(grid), dim3(kHbThreads), smem, st);
     if (cudaLaunchKernelEx(&ol.cfg, head_backward_kernel, m_hd, m_w2, m_dl, m_dhd, g) != cudaSuccess) {
         (void)cudaGetLastError();

@@ -12,8 +12,9 @@ typedef __nv_bfloat16 bf16;
 // dst[i][c] = bf16(src[idx ? idx[i] : i][c]); dst_t[c][i] likewise.  Padding
 // columns of both outputs are written as zero.  With ones, dst gets one more
 // column (index dim) and dst_t one more row (index dim) holding 1 for every
-// batch row: the all-ones vector that makes the bias gradient one more output
-// row of the weight-gradient product.
+// batch row, for callers whose bias gradient is one more output row of a
+// product over the batch (standard training's hidden layers; grad_kernel has
+// its own vector of ones and needs none).
 template <bool SRC_BF16>
 __global__ void __launch_bounds__(256) pack_rows_kernel(const void* __restrict__ src, int64_t ld_src, int32_t dim,
                                                         const int32_t* __restrict__ idx, int64_t n_rows,
