@@ -117,12 +117,20 @@ size_t retexo_aggregate_workspace_size(int64_t n_nodes, int64_t n_edges, int32_t
  *          row stride ldout_bf16 elements; NULL if not wanted.
  * Sums are taken in fp32 in an order that depends on the row's length and the
  * layout only (short rows in CSR order, longer ones in a few interleaved or
- * consecutive parts that are added in a fixed order); GCN may scale q by n_u
- * into the workspace first.  256-bit loads are used when q is 32-byte aligned,
- * ldq % 8 == 0 and ldq >= round_up(dim, 8), 128-bit loads when it is 16-byte
+ * consecutive parts that are added in a fixed order; GCN rows of up to 16
+ * columns on graphs of fewer than 32 entries a row with compensation).
+ * 256-bit loads are used when q is 32-byte aligned, ldq % 8 == 0,
+ * ldq >= round_up(dim, 8) and round_up(dim, 8) - dim <= 3 (a wider ragged end
+ * could reach beyond the last row's memory), 128-bit loads when it is 16-byte
  * aligned, ldq % 4 == 0 and ldq >= round_up(dim, 4), 64-bit loads under the
  * analogous rule, otherwise scalar loads.  Nothing is an error for being
  * unaligned.
+ * GCN and the workspace: on graphs of 32 entries a row and more, and for rows
+ * of up to 16 columns, q is scaled by n_u into the workspace first; on others
+ * it is gathered as it is where it comes in 16-byte pieces, else laid out in
+ * the workspace first.  The size query does not know the alignment and counts
+ * that copy, n_nodes x round_up(dim, 32) floats at most, up to 2 GB; larger
+ * matrices, and those of 768 MB and more that HBM bounds, are never copied.
  * dim <= 4096.  Errors: INVALID_ARG, WORKSPACE, UNSUPPORTED. */
 int retexo_aggregate(const retexo_csr* g, int32_t type,
                      const float* q, int64_t ldq, int32_t dim,
@@ -140,7 +148,8 @@ size_t retexo_gat_backward_workspace_size(int64_t n_nodes, int64_t n_edges, int3
  *   dp      fp32 [n x lddp] and / or bf16 [n x lddp_bf16] (either may be NULL, not both): dLoss / dp,
  *           through the weighted sum and through both score terms;
  *   da_src, da_dst  fp32 [heads x head_dim]: gradients of the attention vectors.
- * Scores, soft-max and every sum are fp32; sums run in CSR order per row, the parameter gradients are
+ * Scores, soft-max and every sum are fp32; a row's sums run in CSR order or, for head widths that are powers of
+ * two, in a few interleaved parts with compensation, each added in a fixed order; the parameter gradients are
  * summed per thread block and then in block order (deterministic).  The graph must be symmetric (the rows
  * that attend over u are read off u's own row).  heads <= 8, heads * head_dim <= 256.
  * Errors: INVALID_ARG, WORKSPACE, UNSUPPORTED. */
@@ -215,6 +224,8 @@ int64_t retexo_theta_size_norm(int32_t d_in, int32_t hidden, int32_t n_classes, 
  * (ld_dst > dim required) and dst_t has one more row (index dim) that holds 1
  * for every batch row; the form retexo_mlp_train_step takes with
  * x_has_ones = 1.  dst may be NULL if only the transpose is wanted.
+ * Rows on 16-byte boundaries are read in 16-byte pieces, the last one to its
+ * end, which never leaves the aligned 16 bytes that hold a row's last column.
  * Needs no workspace. */
 int retexo_pack_rows(const void* src, int32_t src_is_bf16, int64_t ld_src, int32_t dim,
                      const int32_t* idx, int64_t n_rows,
