@@ -54,21 +54,19 @@ def source_fingerprint(names) -> str:
 # have changed since, `traffic` is reported as null.
 AGG_SOURCES = ("aggregate.cu",)
 AGG_DRAM_TRAFFIC = {
-    "fingerprint": "b169e13d7982",      # profiles/agg_kernels_cfg4.txt, profiles/agg_rows_kernel_cfg5.txt
-    "bytes": {("cfg4_sage_reddit_like", 1): 14.68e9, ("cfg4_sage_reddit_like", 2): 6.24e9,
-              ("cfg4_sage_reddit_like", 3): 5.99e9, ("cfg5_gcn_products_like", 1): 46.68e9,
-              ("cfg5_gcn_products_like", 2): 102.92e9, ("cfg5_gcn_products_like", 3): 102.93e9}}
-# one stand-alone training iteration (its tensor-core launches and reduce_update_kernel): profiles/mlp_iteration_cfg4.txt
+    "fingerprint": "b169e13d7982",      # profiles/agg_rows_kernel_cfg5.txt
+    "bytes": {("cfg5_gcn_products_like", 1): 46.68e9, ("cfg5_gcn_products_like", 2): 102.92e9,
+              ("cfg5_gcn_products_like", 3): 102.93e9}}
+# one stand-alone training iteration (its tensor-core launches and reduce_update_kernel): profiles/kernel_counters.txt
 STEP_SOURCES = ("gemm_tc.cu", "grad_tc.cu", "mlp_fused.cu", "mlp.cu", "mlp_kernels.cuh", "tc_common.cuh", "launch_overlap.cuh")
 STEP_DRAM_TRAFFIC = {
-    "fingerprint": "16175fb90a45",
-    "bytes": {("cfg4_sage_reddit_like", 1): 1.241e9, ("cfg4_sage_reddit_like", 2): 0.823e9,
-              ("cfg4_sage_reddit_like", 3): 0.3415e9}}
+    "fingerprint": "2b5f4ad07051",
+    "bytes": {("cfg4_sage_reddit_like", 1): 1.147e9}}
 
 
-# Peak of the L2 -> SM path in GB/s, as the profiler normalises it: in the section capture of the slab gather
-# (profiles/agg_kernels_cfg4.txt) the kernel delivered 15.6 / 16.7 TB/s of neighbour rows, all of them out of L2
-# (L1 hit rate 2 %), at lts__throughput = 68.3 / 72.5 % of peak; both give 22.9 TB/s for 100 %.
+# Peak of the L2 -> SM path in GB/s, as the profiler normalises it: an earlier gather kernel delivered 15.6 / 16.7 TB/s of
+# neighbour rows, all of them out of L2 (L1 hit rate 2 %), at lts__throughput = 68.3 / 72.5 % of peak; both give 22.9 TB/s for
+# 100 %.  Today's (profiles/kernel_counters.txt): 18.7 TB/s at 80.9 %, 23.1.
 L2_PEAK_GBS = 22900.0
 
 
@@ -251,7 +249,7 @@ def measure_l2_gather_peak(rp, ci, n: int, e: int) -> float:
 
 def aggregation_phases(w, ws, peaks, rp, ci, l2_peak):
     """Times every round's aggregation alone, in the launch configuration of the K-round run, and says
-    which ceiling binds: the L2 -> SM path where the kernel gathers from L2-resident column slabs (its DRAM
+    which ceiling binds: the L2 -> SM path where the slab of columns that is gathered from stays in L2 (the kernel's DRAM
     traffic is a small fraction of the bytes it delivers), HBM otherwise."""
     import torch
     from paper_2302_13053_b200 import binding as B
@@ -288,9 +286,9 @@ def aggregation_phases(w, ws, peaks, rp, ci, l2_peak):
                   dram_frac=(traffic / mean_ms / 1e6 / peaks["hbm_gbs"]) if traffic else None, x16=x16)
         if traffic and traffic < 0.25 * alg:
             ph.update(bound="l2", achieved=alg_gbs, peak=L2_PEAK_GBS, unit="GB/s",
-                      ceiling="L2 -> SM path: neighbour rows gathered from L2-resident column slabs (DRAM traffic is %.2f "
+                      ceiling="L2 -> SM path: neighbour rows gathered a slab of columns at a time, out of L2 (DRAM traffic is %.2f "
                               "of the bytes delivered); peak = 100 %% of the profiler's lts__throughput, from the "
-                              "section capture of this kernel; the plain kernel on a 64-column matrix that fits L2 "
+                              "captures of such gathers; the same kernel on a 64-column matrix that fits L2 "
                               "whole delivers %.1f TB/s in this run" % (traffic / alg, (l2_peak or 0.0) / 1e3))
         elif traffic:
             ph.update(bound="hbm", achieved=traffic / mean_ms / 1e6, peak=peaks["hbm_gbs"], unit="GB/s",
@@ -730,7 +728,7 @@ def main():
                  edges_per_s=p["edges_per_s"], algorithmic_gbs=p["algorithmic_gbs"], dram_gbs=p["dram_gbs"],
                  dram_frac=p["dram_frac"], hbm_peak=peaks["hbm_gbs"], ceiling=p["ceiling"])
             for p in agg]
-        line["l2"] = dict(peak_gbs=L2_PEAK_GBS, peak_source="ncu lts__throughput, profiles/agg_kernels_cfg4.txt",
+        line["l2"] = dict(peak_gbs=L2_PEAK_GBS, peak_source="ncu lts__throughput, profiles/kernel_counters.txt",
                           plain_gather_on_l2_resident_matrix_gbs=l2_peak)
         line["phases"] = [dict(kernel=p["kernel"], round=p["round"], ms=round(p["ms"], 4), calls=p["calls_per_step"],
                                share=round(p["share_of_step"], 4), bound=p["bound"], achieved=round(p["achieved"], 2),

@@ -406,11 +406,12 @@ struct AggGrid {
 // need: a second slab for 8 columns of 72 with the lanes of a whole one costs as much as the first.
 // Bound by the L2 -> SM path (64 bytes a cycle and SM) on dense graphs, by row pointer -> column -> row latencies on sparse ones;
 // measured against a persistent kernel that drew its rows from one counter, a warp each (SAGE, bf16 out, with concatenation):
-//   233 k nodes, 115 M entries, 256 columns: 6.95 -> 6.4 ms (18.4 TB/s of neighbour rows); GCN 9.5 -> 7.8 ms
-//   58 k nodes, 7 M entries, 256 columns: 820 -> 467 us (15.8 TB/s); GCN 1036 -> 520 us
-//   600 k nodes, 30 M entries, 256 columns: 4.05 -> 3.4 ms;  20 k nodes, 88 k entries, 500 columns: 142 -> 66 us
+//   233 k nodes, 113 M entries, 256 columns: 6.95 -> 6.3 ms (18.5 TB/s of neighbour rows); GCN 9.5 -> 6.6 ms
+//   58 k nodes, 7 M entries, 256 columns: 820 -> 492 us (14.4 TB/s); GCN 1036 -> 498 us
+//   600 k nodes, 30 M entries, 256 columns: 4.05 -> 3.2 ms;  20 k nodes, 88 k entries, 500 columns: 142 -> 62 us
 // Slabs of 32 or 128 columns instead of 64 take 1.4 and 1.2 times as long on the first of these; 4 entries in flight, since
-// with 56 registers 36 warps fit an SM (64: 32 warps, level; 48: spills, 5 % slower; 80 and more: 1.4 times as long).
+// with 56 registers 36 warps fit an SM (64: 32 warps, level; 48: 5 % slower; 80 and more: 1.4 times as long).  At 8 columns a lane the compiler
+// spills 4 to 64 bytes a thread of these.
 template <int LPG, int E, int NV, int TLPG, int TNV, int OP>
 __global__ void __launch_bounds__(kAggThreads, AggLanes<LPG, E, NV, OP>::kBlocks) agg_lanes_kernel(AggArgs a, AggGrid grid) {
     constexpr int kCols = LPG * E * NV;

@@ -110,8 +110,9 @@ struct GatForwardPass {
 // Bound by the gather of the neighbour rows (4 dim + 4 heads bytes an entry, out of L2 where p fits it) and, below that, by
 // the chain row pointer -> column -> row and the instructions an entry takes: hence a row per group, 32-byte loads and no
 // shuffles per entry.  Measured with the score kernel (a warp per row, 4-byte loads, a soft-max reduction over the warp every
-// 32 entries before): 717 k nodes, 14 M entries, 4 x 16: 2667 -> 640 us; 60 k nodes, 12 M entries: 847 -> 248 us (12.4 TB/s of
-// neighbour rows); 100 k nodes, 3 M entries, 8 x 32: 1392 -> 304 us; 200 k nodes, 4 M entries, 1 x 8: 409 -> 86 us.
+// 32 entries before): 717 k nodes, 14 M entries, 4 x 16: 2667 -> 684 us (5.9 TB/s of neighbour rows, L2 hit rate 45 %); 60 k
+// nodes, 12 M entries: 847 -> 266 us (12.1 TB/s); 100 k nodes, 3 M entries, 8 x 32: 1392 -> 335 us; 200 k nodes, 4 M entries,
+// 1 x 8: 409 -> 84 us.
 template <int LPG, int W>
 __global__ void __launch_bounds__(kGatThreads, kGatBlocksPerSm) gat_lane_rows_kernel(GatArgs a, int hub_entries, int hub_blocks,
                                                                                      int vec_out, int vec_out16) {

@@ -337,8 +337,8 @@ struct GatDstPass {
 
 // Bound like the forward pass by the gather of p_u (4 dim + 4 heads bytes an entry); rows whose gradient is zero gather nothing.
 // Measured, whole backward pass (a lane per entry reading its own row in 16-byte pieces before; heads of other shapes a warp
-// per entry): 717 k nodes, 14 M entries, 4 x 16: 5319 -> 1950 us; 60 k nodes, 12 M entries: 2960 -> 684 us; 100 k nodes, 3 M
-// entries, 8 x 32: 26.6 -> 0.87 ms; 200 k nodes, 4 M entries, 1 x 8: 834 -> 163 us.
+// per entry): 717 k nodes, 14 M entries, 4 x 16: 5319 -> 1936 us; 60 k nodes, 12 M entries: 2960 -> 733 us; 100 k nodes, 3 M
+// entries, 8 x 32: 26.6 -> 0.92 ms; 200 k nodes, 4 M entries, 1 x 8: 834 -> 160 us.
 template <int LPG, int W>
 __global__ void __launch_bounds__(kGatThreads, kGatBlocksPerSm) gat_lane_dst_kernel(GatBwdArgs a, int hub_entries, int hub_blocks) {
     constexpr int G = GatLanes<LPG, W>::G;

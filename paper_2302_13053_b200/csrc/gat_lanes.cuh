@@ -8,7 +8,8 @@
 namespace retexo {
 
 constexpr int kGatThreads = 128, kGatWarps = kGatThreads / kWarp;      // (256: a block's slots idle until its longest row is done)
-constexpr int kGatBlocksPerSm = 9;      // 56 registers a thread: 36 warps an SM (10 blocks spill, 7 at 69 registers wait longer)
+constexpr int kGatBlocksPerSm = 9;      // 56 registers a thread: 36 warps an SM.  (At 8 columns a lane the backward kernels spill 4 to 20 bytes; 10 blocks spill
+                                        // more, 7 at 69 registers wait longer.)
 // A row of up to kGatGroupEntries entries is taken by one group of lanes (so a warp works on G rows at once), a longer one
 // by a whole warp, and one of `hub_entries` or more by a whole block.
 constexpr int kGatGroupEntries = 32;
