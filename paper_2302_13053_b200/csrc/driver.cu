@@ -5,6 +5,7 @@
 #include <vector>
 
 #include "aggregate.h"
+#include "gat_lanes.cuh"
 #include "common.cuh"
 #include "gemm_tc.h"
 #include "mlp_plan.h"
@@ -43,29 +44,11 @@ __global__ void record_validation_kernel(const unsigned long long* cur, unsigned
         *have_best = 1;
     }
 }
-// dz[idx[i]][0 .. dim) = dx[i][0 .. dim): the batch-ordered input gradient goes back to node order.
-// Blocks from scatter_blocks on: att_best = att if *decision is set (the trained aggregator's parameters follow theta into the
-// kept copy).  One launch for both: each is a few hundred kilobytes, so a launch of its own is what it costs (a run of 100 trained
-// iterations 15.18 ms with two, 15.00 with one).  vec: four columns a thread.
-__global__ void scatter_rows_kernel(const float* __restrict__ dx, int64_t ld_dx, const int32_t* __restrict__ idx,
-                                    int64_t n_rows, int32_t dim, int vec, float* __restrict__ dz, int64_t ld_dz, unsigned scatter_blocks,
-                                    const int32_t* __restrict__ decision, const float* __restrict__ att, float* __restrict__ att_best, int64_t n_att) {
-    if (blockIdx.x >= scatter_blocks) {
-        const int64_t p = (blockIdx.x - scatter_blocks) * 256ll + threadIdx.x;
-        if (p < n_att && *decision) att_best[p] = att[p];
-        return;
-    }
-    const int64_t t = blockIdx.x * 256ll + threadIdx.x;
-    const int32_t per_row = vec ? dim >> 2 : dim;
-    const int64_t i = t / per_row;
-    const int32_t c = (int32_t)(t % per_row);
-    if (i >= n_rows) return;
-    if (vec) reinterpret_cast<float4*>(dz + (int64_t)idx[i] * ld_dz)[c] = reinterpret_cast<const float4*>(dx + i * ld_dx)[c];
-    else dz[(int64_t)idx[i] * ld_dz + c] = dx[i * ld_dx + c];
-}
 // One optimiser update of the aggregator's parameters [W_att | a_src | a_dst]: the gradient of W_att is the
 // sum of split-K partials (added in index order), those of the attention vectors come ready-made.
-// `step` is the 1-based number of this update, read on the device.
+// `step` is the 1-based number of this update, read on the device.  First the kept copy follows theta's (*decision), and at the
+// end the bf16 copy W_att^T that the next projection reads is brought up to date: in launches of their own both cost what a launch
+// costs (a few hundred kilobytes).
 __device__ __forceinline__ double whole_power(double base, unsigned long long e) {      // base^e by repeated squaring
     double r = 1.0;
     for (; e; e >>= 1, base *= base) if (e & 1ull) r *= base;
@@ -77,23 +60,48 @@ struct AttUpdateArgs {
     const float* da; int64_t n_att;
     int optimizer; float lr, beta1, beta2, eps;
     const unsigned long long* step;
-    float* grad_out;      // optional
+    const int32_t* decision; float* att_best;
+    int32_t hd; bf16* wt16; int64_t ld_wt;      // W_att^T [hd x ld_wt]
 };
-__global__ void att_update_kernel(AttUpdateArgs a) {
-    const int64_t p = blockIdx.x * 256ll + threadIdx.x;
-    if (p >= a.n_att) return;
-    float g = 0.f;
-    if (p < a.n_w) for (int64_t z = 0; z < a.splits; ++z) g += a.partial[z * a.n_w + p];
-    else g = a.da[p - a.n_w];
-    if (a.grad_out) a.grad_out[p] = g;
-    if (a.optimizer == RETEXO_SGD) { a.att[p] -= a.lr * g; return; }
+__global__ void __launch_bounds__(128) att_update_kernel(AttUpdateArgs a) {
+    const int32_t p = (int32_t)(blockIdx.x * 128 + threadIdx.x), n_w = (int32_t)a.n_w;
+    if (p >= (int32_t)a.n_att) return;
+    // everything is asked for before anything is used or stored
+    const float old = a.att[p];
+    const int32_t decision = *a.decision;
     const unsigned long long t = *a.step;
-    const float c1 = (float)(1.0 - whole_power((double)a.beta1, t)), c2 = (float)(1.0 - whole_power((double)a.beta2, t));
-    const float m = a.beta1 * a.m[p] + (1.f - a.beta1) * g;
-    const float v = a.beta2 * a.v[p] + (1.f - a.beta2) * g * g;
-    a.m[p] = m;
-    a.v[p] = v;
-    a.att[p] -= a.lr * (m / c1) / (sqrtf(v / c2) + a.eps);
+    const bool adam = a.optimizer != RETEXO_SGD;
+    const float m0 = adam ? a.m[p] : 0.f, v0 = adam ? a.v[p] : 0.f;
+    float g = 0.f;
+    if (p < n_w) {
+        constexpr int kAhead = 16;      // partials in flight
+        const float* part = a.partial + p;
+        int z = 0;
+        for (; z + kAhead <= (int)a.splits; z += kAhead) {
+            float x[kAhead];
+#pragma unroll
+            for (int k = 0; k < kAhead; ++k) x[k] = __ldg(part + (int64_t)(z + k) * n_w);
+#pragma unroll
+            for (int k = 0; k < kAhead; ++k) g += x[k];
+        }
+        for (; z < (int)a.splits; ++z) g += __ldg(part + (int64_t)z * n_w);
+    } else {
+        g = a.da[p - n_w];
+    }
+    float now;
+    if (adam) {
+        const float c1 = (float)(1.0 - whole_power((double)a.beta1, t)), c2 = (float)(1.0 - whole_power((double)a.beta2, t));
+        const float m = a.beta1 * m0 + (1.f - a.beta1) * g;
+        const float v = a.beta2 * v0 + (1.f - a.beta2) * g * g;
+        a.m[p] = m;
+        a.v[p] = v;
+        now = old - a.lr * (m / c1) / (sqrtf(v / c2) + a.eps);
+    } else {
+        now = old - a.lr * g;
+    }
+    if (decision) a.att_best[p] = old;
+    a.att[p] = now;
+    if (p < n_w) a.wt16[(int64_t)(p % a.hd) * a.ld_wt + p / a.hd] = f32_to_bf16(now);
 }
 // Keeps the first non-zero status of the run.
 __global__ void merge_status_kernel(int32_t* run, const int32_t* a, const int32_t* b) {
@@ -187,8 +195,9 @@ struct LmpBuffers {
     // representations
     float* q[2];
     bf16* x16; bf16* q16; float* proj; bf16* watt_t16;
-    float *att, *att_m, *att_v, *att_best, *att_partial, *da, *dx, *dz; bf16* dp16; int32_t* decision; int32_t* status;
+    float *att, *att_m, *att_v, *att_best, *att_partial, *da, *dz; bf16* dp16; int32_t* decision; int32_t* status;
     int64_t att_splits; void* ws_gatbwd; size_t ws_gatbwd_bytes;
+    GatRow *rows_all, *rows_batch, *rows_train; int32_t *slots, *order_bins;      // row orders of a run that trains its aggregator
     bf16 *xtr16, *xval16;
     int32_t *y_tr, *y_val, *y_test;
     float *theta, *adam_m, *adam_v, *theta_best;
@@ -254,13 +263,17 @@ static void lmp_layout(const retexo_lmp_config& c, int64_t n, int64_t e, int64_t
         l.att_splits = gemm_split((int64_t)max_rep, hd, n);
         l.att_partial = t.template take<float>((size_t)l.att_splits * (size_t)max_rep * hd);
         l.da = t.template take<float>((size_t)2 * hd);
-        l.dx = t.template take<float>((size_t)n_tr * round_up(hd, 32));
         l.dz = t.template take<float>((size_t)n * round_up(hd, 32));
         l.dp16 = t.template take<bf16>((size_t)n * round_up(hd, 64));
         l.decision = t.template take<int32_t>(64);
         l.status = t.template take<int32_t>(64);
         l.ws_gatbwd_bytes = retexo_gat_backward_workspace_size(n, e, c.gat_heads, hd);
         l.ws_gatbwd = t.template take<char>(l.ws_gatbwd_bytes);
+        l.rows_all = t.template take<GatRow>((size_t)n);
+        l.rows_batch = t.template take<GatRow>((size_t)(n_tr + n_val));
+        l.rows_train = t.template take<GatRow>((size_t)n_tr);
+        l.slots = t.template take<int32_t>((size_t)(n_tr + n_val));
+        l.order_bins = t.template take<int32_t>(3 * kGatOrderInts);
     }
     // training rows, then validation rows; after the round's last iteration the test rows take their place
     l.xtr16 = t.template take<bf16>((size_t)(n_tr + n_val > n_te ? n_tr + n_val : n_te) * (size_t)ld16);
@@ -429,6 +442,25 @@ extern "C" int retexo_lmp_train(const retexo_lmp_config* cfg, const retexo_lmp_i
         for (int m = 1; m <= c.K; ++m) if (round_dims(c, m).d_in > max_din) max_din = round_dims(c, m).d_in;
         RETEXO_CUDA_TRY(cudaMemsetAsync(b.x16, 0, sizeof(bf16) * (size_t)n * (size_t)round_up(max_din, 64), st));
     }
+    // A run that trains its aggregator walks the same rows in every iteration: their orders are found once.  An iteration needs the
+    // aggregated rows of its batch only, and only training rows have a gradient.
+    const bool kept_orders = c.aggr == RETEXO_GAT && !c.gat_freeze_attention &&
+                             gat_lanes_usable(c.gat_heads, c.gat_head_dim, b.proj, round_up(c.gat_heads * c.gat_head_dim, 32), b.dz,
+                                              round_up(c.gat_heads * c.gat_head_dim, 32));
+    const int n_sm = sm_count();
+    if (n_sm <= 0) return RETEXO_ERR_CUDA;
+    GatRowOrder all_rows{}, batch_rows{}, train_rows{};
+    if (kept_orders) {
+        int32_t* bins = b.order_bins;
+        all_rows = {b.rows_all, bins + kGatOrderCounts, nullptr, n};
+        batch_rows = {b.rows_batch, bins + kGatOrderInts + kGatOrderCounts, b.slots, n_tr + n_val};
+        train_rows = {b.rows_train, bins + 2 * kGatOrderInts + kGatOrderCounts, nullptr, n_tr};
+        const int32_t* lists[3] = {nullptr, train_idx, val_idx};
+        const int64_t sizes[3] = {n, n_tr, n_val};
+        RETEXO_TRY(gat_order_launch(g, 1, lists, sizes, 1, b.rows_all, nullptr, bins, n_sm, st));
+        RETEXO_TRY(gat_order_launch(g, 1, lists + 1, sizes + 1, 2, b.rows_batch, b.slots, bins + kGatOrderInts, n_sm, st));
+        RETEXO_TRY(gat_order_launch(g, 1, lists + 1, sizes + 1, 1, b.rows_train, nullptr, bins + 2 * kGatOrderInts, n_sm, st));
+    }
     const float* q = feat;
     int64_t ldq = ld_feat;
     for (int m = 1; m <= c.K; ++m) {
@@ -443,9 +475,10 @@ extern "C" int retexo_lmp_train(const retexo_lmp_config* cfg, const retexo_lmp_i
         const int64_t ldq16 = round_up(r.rep_dim, 64), ldp = round_up(hd > 0 ? hd : 1, 32);
         const int64_t n_att = (int64_t)r.rep_dim * hd + 2 * (int64_t)hd;
         // GAT: P = Q W_att on the tensor cores (a bias-free product), then scores, soft-max and weighted sum in
-        // one pass, with the projection and attention vectors at `att` = [W_att | a_src | a_dst]
-        auto gat_forward = [&](const float* att) -> int {
-            RETEXO_TRY(retexo_pack_rows(att, 0, hd, hd, nullptr, r.rep_dim, nullptr, 0, b.watt_t16, ldq16, 0, st));
+        // one pass, with the projection and attention vectors at `att` = [W_att | a_src | a_dst].  batch: with kept orders the
+        // rows of the batch only, which go to their places in it; packed: W_att's bf16 copy is up to date.
+        auto gat_forward = [&](const float* att, bool batch = false, bool packed = false) -> int {
+            if (!packed) RETEXO_TRY(retexo_pack_rows(att, 0, hd, hd, nullptr, r.rep_dim, nullptr, 0, b.watt_t16, ldq16, 0, st));
             TcGemm pr{};
             pr.A = b.q16; pr.lda = ldq16; pr.B = b.watt_t16; pr.ldb = ldq16; pr.M = n; pr.N = hd; pr.K = r.rep_dim;
             pr.mode = TC_EPI_BIAS; pr.out_f32 = b.proj; pr.ld_f32 = ldp; pr.status = b.status;
@@ -453,8 +486,13 @@ extern "C" int retexo_lmp_train(const retexo_lmp_config* cfg, const retexo_lmp_i
             retexo_gat_params gp;
             gp.heads = c.gat_heads; gp.head_dim = c.gat_head_dim; gp.a_src = att + (int64_t)r.rep_dim * hd;
             gp.a_dst = gp.a_src + hd; gp.negative_slope = c.gat_negative_slope; gp.add_self_loop = 1;
-            return retexo_aggregate(&g, RETEXO_GAT, b.proj, ldp, hd, &gp, nullptr, 0, 0, b.x16, ld16, b.ws_agg,
-                                    b.ws_agg_bytes, st);
+            if (!kept_orders)
+                return retexo_aggregate(&g, RETEXO_GAT, b.proj, ldp, hd, &gp, nullptr, 0, 0, b.x16, ld16, b.ws_agg, b.ws_agg_bytes, st);
+            GatForward f{};
+            f.g = g; f.p = b.proj; f.ldp = ldp; f.gat = gp; f.out16 = batch ? b.xtr16 : b.x16; f.ldout16 = ld16;
+            f.order = batch ? batch_rows : all_rows;
+            Arena ws(b.ws_agg, b.ws_agg_bytes);
+            return gat_forward_launch(f, ws, n_sm, st);
         };
         if (gat) {
             RETEXO_CUDA_TRY(cudaMemcpyAsync(b.att, in->gat_w[m - 1], sizeof(float) * (size_t)n_att, cudaMemcpyDefault, st));
@@ -466,6 +504,11 @@ extern "C" int retexo_lmp_train(const retexo_lmp_config* cfg, const retexo_lmp_i
                 RETEXO_CUDA_TRY(cudaMemsetAsync(b.att_v, 0, sizeof(float) * (size_t)n_att, st));
                 RETEXO_CUDA_TRY(cudaMemsetAsync(b.dz, 0, sizeof(float) * (size_t)n * (size_t)ldp, st));
                 RETEXO_CUDA_TRY(cudaMemsetAsync(b.decision, 0, sizeof(int32_t), st));
+                if (kept_orders) {
+                    RETEXO_TRY(gat_backward_prepare(n, g.n_edges, c.gat_heads, c.gat_head_dim, b.ws_gatbwd, b.ws_gatbwd_bytes, st));
+                    // (the batch's padding columns, which its rows' own writes leave alone, stay defined)
+                    RETEXO_CUDA_TRY(cudaMemsetAsync(b.xtr16, 0, sizeof(bf16) * (size_t)(n_tr + n_val) * (size_t)ld16, st));
+                }
             } else {
                 RETEXO_TRY(gat_forward(b.att));
             }
@@ -526,21 +569,17 @@ extern "C" int retexo_lmp_train(const retexo_lmp_config* cfg, const retexo_lmp_i
         // launches with the same arguments: the second one is recorded as a graph, the rest replay it.
         const bool uniform = work.own && c.R > 3 && (n_val == 0 || c.eval_every == 1);
         tail.decision = gat_train ? b.decision : nullptr;
-        const int64_t ld_dx = ldp;
         // What a round that trains its aggregator adds to an iteration (Section 3.1: after the round's exchange
         // everything an iteration needs is local, so the aggregation is redone with the current parameters):
-        // before the step, projection + aggregation + batches; after it, the kept copy follows theta's, the
-        // input gradient goes back through the attention, and [W_att | a_src | a_dst] take their update.
+        // before the step, projection + aggregation into the batch; after it, the input gradient (which the step has put in node
+        // order) goes back through the attention, the kept copy follows theta's, and [W_att | a_src | a_dst] take their update.
         auto gat_backward_and_update = [&]() -> int {
-            const int vec = hd % 4 == 0 && ld_dx % 4 == 0 && ldp % 4 == 0;      // (the buffers start on 256-byte boundaries)
-            const unsigned scatter_blocks = (unsigned)((n_tr * (vec ? hd / 4 : hd) + 255) / 256);
-            scatter_rows_kernel<<<scatter_blocks + (unsigned)((n_att + 255) / 256), 256, 0, st>>>(
-                b.dx, ld_dx, train_idx, n_tr, hd, vec, b.dz, ldp, scatter_blocks, b.decision, b.att, b.att_best, n_att);
             retexo_gat_params gp;
             gp.heads = c.gat_heads; gp.head_dim = c.gat_head_dim; gp.a_src = b.att + (int64_t)r.rep_dim * hd;
             gp.a_dst = gp.a_src + hd; gp.negative_slope = c.gat_negative_slope; gp.add_self_loop = 1;
-            RETEXO_TRY(retexo_gat_backward(&g, b.proj, ldp, &gp, b.dz, ldp, nullptr, 0, b.dp16, round_up(hd, 64), b.da,
-                                           b.da + hd, b.ws_gatbwd, b.ws_gatbwd_bytes, st));
+            const GatBackwardKept kept{train_rows, all_rows, gat_forward_s(b.ws_agg), gat_forward_t(b.ws_agg, n, c.gat_heads)};
+            RETEXO_TRY(gat_backward(&g, b.proj, ldp, &gp, b.dz, ldp, nullptr, 0, b.dp16, round_up(hd, 64), b.da,
+                                    b.da + hd, b.ws_gatbwd, b.ws_gatbwd_bytes, kept_orders ? &kept : nullptr, st));
             TcGemm gw{};      // dW_att = Q^T dP, reduced over the nodes
             gw.A = b.q16; gw.lda = ldq16; gw.B = b.dp16; gw.ldb = round_up(hd, 64); gw.M = r.rep_dim; gw.N = hd; gw.K = n;
             gw.mode = TC_EPI_PARTIAL; gw.splits = (int)gemm_split(r.rep_dim, hd, n); gw.partial = b.att_partial;
@@ -550,7 +589,8 @@ extern "C" int retexo_lmp_train(const retexo_lmp_config* cfg, const retexo_lmp_i
             au.att = b.att; au.m = b.att_m; au.v = b.att_v; au.partial = b.att_partial; au.n_w = (int64_t)r.rep_dim * hd;
             au.splits = gw.splits; au.da = b.da; au.n_att = n_att; au.optimizer = c.optimizer; au.lr = c.lr;
             au.beta1 = c.beta1; au.beta2 = c.beta2; au.eps = c.eps; au.step = b.cur_correct + 2;      // (already advanced)
-            att_update_kernel<<<(unsigned)((n_att + 255) / 256), 256, 0, st>>>(au);
+            au.decision = b.decision; au.att_best = b.att_best; au.hd = hd; au.wt16 = b.watt_t16; au.ld_wt = ldq16;
+            att_update_kernel<<<(unsigned)((n_att + 127) / 128), 128, 0, st>>>(au);
             return launch_status();
         };
         iteration.reset();
@@ -573,11 +613,11 @@ extern "C" int retexo_lmp_train(const retexo_lmp_config* cfg, const retexo_lmp_i
                 if (!gat_train)
                     return mlp_train_step_launch(plan, sb, &model, b.xtr16, ld16, b.y_tr, loss_slot, nullptr,
                                                  shadows_ready, riding, st, &dev);
-                RETEXO_TRY(gat_forward(b.att));
-                RETEXO_TRY(pack_batches());
+                RETEXO_TRY(gat_forward(b.att, true, shadows_ready));
+                if (!kept_orders) RETEXO_TRY(pack_batches());
                 if (!riding) RETEXO_CUDA_TRY(cudaMemsetAsync(b.decision, 0, sizeof(int32_t), st));
                 RETEXO_TRY(mlp_train_step_launch(plan, sb, &model, b.xtr16, ld16, b.y_tr, loss_slot, nullptr,
-                                                 shadows_ready, riding, st, &dev, b.dx, ld_dx));
+                                                 shadows_ready, riding, st, &dev, b.dz, ldp, true, train_idx));
                 return gat_backward_and_update();
             };
             if (uniform && it >= 2) {
@@ -621,8 +661,8 @@ extern "C" int retexo_lmp_train(const retexo_lmp_config* cfg, const retexo_lmp_i
             pending_it = (want && it < c.R) ? it : 0;
             if (want && it == c.R) {      // the last iterate has no next iteration to ride on
                 if (gat_train) {
-                    RETEXO_TRY(gat_forward(b.att));
-                    RETEXO_TRY(pack_batches());
+                    RETEXO_TRY(gat_forward(b.att, true));
+                    if (!kept_orders) RETEXO_TRY(pack_batches());
                 }
                 RETEXO_TRY(mlp_count_hits_launch(plan, sb, &model, xval16, ld16, n_val, val_hd, b.y_val,
                                                  b.cur_correct, st, val_z));

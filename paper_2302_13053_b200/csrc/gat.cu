@@ -26,9 +26,77 @@ struct GatArgs {
     int64_t ldout;
     __nv_bfloat16* out16;
     int64_t ldout16;
-    int32_t* hub_list;      // rows a whole block takes, listed by gat_scores_kernel (order arbitrary; no result depends on it)
-    int32_t* hub_count;
+    int32_t* hub_list;      // general kernels: rows a whole block takes, listed by gat_scores_kernel (order arbitrary; no result
+    int32_t* hub_count;     // depends on it)
 };
+
+// ---------------------------------------------------------------- rows in order of their lengths (gat_lanes.cuh)
+__global__ void __launch_bounds__(256) gat_order_count_kernel(int64_t n, const int32_t* __restrict__ idx, const int64_t* __restrict__ rowptr,
+                                                              int32_t self_loop, int32_t hub_entries, int32_t* __restrict__ bins) {
+    __shared__ int32_t count[kGatBins];
+    if (threadIdx.x < kGatBins) count[threadIdx.x] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kGatOrderRows / 256; ++k) {
+        const int64_t i = (int64_t)blockIdx.x * kGatOrderRows + k * 256 + threadIdx.x;
+        if (i >= n) break;
+        const int64_t v = idx ? idx[i] : i;
+        atomicAdd(count + gat_bin((int32_t)(rowptr[v + 1] - rowptr[v]) + self_loop, hub_entries), 1);
+    }
+    __syncthreads();
+    if (threadIdx.x < kGatBins && count[threadIdx.x]) atomicAdd(bins + threadIdx.x, count[threadIdx.x]);
+}
+
+// A stream over the row pointers: a block finds its rows' ranks per class in shared memory and reserves a run of each class with one
+// addition (717 k rows: 8 us).
+__global__ void __launch_bounds__(256) gat_order_kernel(int64_t n, const int32_t* __restrict__ idx, const int64_t* __restrict__ rowptr,
+                                                        int32_t self_loop, int32_t hub_entries, int32_t* __restrict__ bins,
+                                                        GatRow* __restrict__ rows, int32_t* __restrict__ slots, int32_t slot0) {
+    constexpr int kRows = kGatOrderRows / 256;
+    __shared__ int32_t count[kGatBins], base[kGatBins], warp_total[kGatBins / kWarp];
+    const int t = threadIdx.x, lane = t & 31;
+    int32_t mine = 0, before = 0;      // rows of class t; of the classes up to it
+    if (t < kGatBins) {
+        count[t] = 0;
+        mine = before = bins[t];
+#pragma unroll
+        for (int o = 1; o < kWarp; o <<= 1) {
+            const int32_t y = __shfl_up_sync(0xffffffffu, before, o);
+            if (lane >= o) before += y;
+        }
+        if (lane == kWarp - 1) warp_total[t / kWarp] = before;
+    }
+    __syncthreads();
+    GatRow row[kRows];
+    int bin[kRows], rank[kRows];
+#pragma unroll
+    for (int k = 0; k < kRows; ++k) {
+        const int64_t i = (int64_t)blockIdx.x * kGatOrderRows + k * 256 + t;
+        bin[k] = -1;
+        if (i >= n) continue;
+        const int64_t v = idx ? idx[i] : i;
+        row[k].beg = rowptr[v];
+        row[k].deg = (int32_t)(rowptr[v + 1] - row[k].beg);
+        row[k].v = (int32_t)v;
+        bin[k] = gat_bin(row[k].deg + self_loop, hub_entries);
+        rank[k] = atomicAdd(count + bin[k], 1);
+    }
+    __syncthreads();
+    if (t < kGatBins) {
+        for (int w = 0; w < t / kWarp; ++w) before += warp_total[w];
+        if (blockIdx.x == 0 && t == 0) bins[kGatOrderCounts] = mine;
+        if (blockIdx.x == 0 && t == kGatLongBins - 1) bins[kGatOrderCounts + 1] = before;
+        base[t] = before - mine + (count[t] ? atomicAdd(bins + kGatBins + t, count[t]) : 0);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < kRows; ++k) {
+        if (bin[k] < 0) continue;
+        const int32_t at = base[bin[k]] + rank[k];
+        rows[at] = row[k];
+        if (slots) slots[at] = slot0 + (int32_t)((int64_t)blockIdx.x * kGatOrderRows + k * 256 + t);
+    }
+}
 
 // ---------------------------------------------------------------- lane layout
 // Running soft-max state and weighted sum of one lane over the entries its group takes.
@@ -99,53 +167,52 @@ struct GatForwardPass {
             more += w;
             st.acc.fma(w, x[t]);
         }
-        add_compensated(st.l, st.lost, more);
+        if (ok[0]) add_compensated(st.l, st.lost, more);      // (beyond the row's end nothing may change, not even what is lost)
     }
 };
 
-// Blocks [0, hub_blocks): one block per listed hub row at a time; warp w takes the trips w, w + 4, ... and the warps' states are
-// merged in warp order, so the result does not depend on scheduling.  They come first in launch order: the longest rows
-// start ahead of the short ones.  Blocks from hub_blocks on: G rows a warp, the short ones at once, a group each, the
-// longer ones one after the other.
+// Blocks [0, hub_blocks): one block per hub row at a time; warp w takes the trips w, w + 4, ... and the warps' states are
+// merged in warp order, so the result does not depend on scheduling.  Blocks from hub_blocks on: G rows a warp in the order of
+// lengths, the short ones at once, a group each, the longer ones one after the other.
 // Bound by the gather of the neighbour rows (4 dim + 4 heads bytes an entry, out of L2 where p fits it) and, below that, by
-// the chain row pointer -> column -> row and the instructions an entry takes: hence a row per group, 32-byte loads and no
+// the chain row -> column -> neighbour row and the instructions an entry takes: hence a row per group, 32-byte loads and no
 // shuffles per entry.  Measured with the score kernel (a warp per row, 4-byte loads, a soft-max reduction over the warp every
-// 32 entries before): 717 k nodes, 14 M entries, 4 x 16: 2667 -> 684 us (5.9 TB/s of neighbour rows, L2 hit rate 45 %); 60 k
+// 32 entries before): 717 k nodes, 14 M entries, 4 x 16: 2667 -> 684 us, in order of lengths 510 (8.2 TB/s of neighbour rows, 45 % of them out of L2); 60 k
 // nodes, 12 M entries: 847 -> 266 us (12.1 TB/s); 100 k nodes, 3 M entries, 8 x 32: 1392 -> 335 us; 200 k nodes, 4 M entries,
 // 1 x 8: 409 -> 84 us.
 template <int LPG, int W>
-__global__ void __launch_bounds__(kGatThreads, kGatBlocksPerSm) gat_lane_rows_kernel(GatArgs a, int hub_entries, int hub_blocks,
+__global__ void __launch_bounds__(kGatThreads, kGatBlocksPerSm) gat_lane_rows_kernel(GatArgs a, GatRowOrder order, GatGrid grid,
                                                                                      int vec_out, int vec_out16) {
-    constexpr int G = GatLanes<LPG, W>::G;
     __shared__ Cols<W> sm_acc[2][kGatWarps][LPG];      // (used in turn: one barrier a hub row)
     __shared__ float2 sm_ml[2][kGatWarps][LPG];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const GatLanes<LPG, W> L(lane, a.dim, a.head_dim);
     GatForwardPass<LPG, W> pass(a, L);
-    auto store_cols = [&](int64_t v, int col, Cols<W> z, float den) {
+    auto store_cols = [&](int64_t i, int64_t v, Cols<W> z, float den) {      // (entry i of the order)
 #pragma unroll
-        for (int i = 0; i < W; ++i) z.v[i] /= den;
-        if (a.out) z.store(a.out + v * a.ldout + col, vec_out != 0);
-        if (a.out16) z.store(a.out16 + v * a.ldout16 + col, vec_out16 != 0);
+        for (int k = 0; k < W; ++k) z.v[k] /= den;
+        if (a.out) z.store(a.out + v * a.ldout + L.col, vec_out != 0);
+        if (a.out16) z.store(a.out16 + (order.slots ? (int64_t)order.slots[i] : v) * a.ldout16 + L.col, vec_out16 != 0);
     };
-    auto store_row = [&](int64_t v, int32_t total) {
+    auto store_row = [&](int64_t i, int64_t v, int32_t total) {
         if (!L.on) return;
         if (total == 0) pass.st.acc.zero();                     // an empty row leaves zeros
-        store_cols(v, L.col, pass.st.acc, total > 0 ? pass.st.l - pass.st.lost : 1.f);
+        store_cols(i, v, pass.st.acc, total > 0 ? pass.st.l - pass.st.lost : 1.f);
     };
-    if ((int)blockIdx.x >= hub_blocks) {
-        const int64_t v0 = ((int64_t)(blockIdx.x - hub_blocks) * kGatWarps + warp) * G;
-        if (v0 >= a.n) return;
-        const int64_t v = min(v0 + L.g, a.n - 1);
-        const int64_t beg = __ldg(a.rowptr + v);
-        const int32_t deg = (int32_t)(__ldg(a.rowptr + v + 1) - beg);
-        const int32_t total = v0 + L.g < a.n ? deg + a.self_loop : INT32_MAX;      // (beyond the last row: nobody's)
+    if ((int)blockIdx.x >= grid.hub_blocks) {
+        int rows;
+        const int64_t i0 = gat_first_row<LPG>(order, grid, (int64_t)((int)blockIdx.x - grid.hub_blocks) * kGatWarps + warp, rows);
+        if (rows == 0) return;
+        const GatRow row = load_row_entry(order.rows + i0 + min(L.g, rows - 1));
+        const int64_t v = row.v, beg = row.beg;
+        const int32_t deg = row.deg;
+        const int32_t total = L.g < rows ? deg + a.self_loop : INT32_MAX;      // (beyond the last row: nobody's)
         const bool mine = total <= kGatGroupEntries;
         const int32_t longest = __reduce_max_sync(0xffffffffu, mine ? total : 0);
         pass.begin(v);
         gat_walk_by_group<LPG, W>(pass, L, a.colidx, (int32_t)v, beg, deg, mine ? total : 0, longest);
-        if (mine) store_row(v, total);
-        unsigned longer = __ballot_sync(0xffffffffu, L.li == 0 && !mine && total < hub_entries);
+        if (mine) store_row(i0 + L.g, v, total);
+        unsigned longer = __ballot_sync(0xffffffffu, L.li == 0 && !mine && L.g < rows);
         while (longer) {
             const int src = __ffs(longer) - 1;
             longer &= longer - 1;
@@ -154,16 +221,16 @@ __global__ void __launch_bounds__(kGatThreads, kGatBlocksPerSm) gat_lane_rows_ke
             pass.begin(w);
             gat_walk_by_warp<LPG, W>(pass, L, a.colidx, (int32_t)w, w_beg, w_deg, w_deg + a.self_loop, 0, kWarp, lane);
             pass.st.template merge_groups<LPG>();
-            if (L.g == 0) store_row(w, w_deg + a.self_loop);
+            if (L.g == 0) store_row(i0 + src / LPG, w, w_deg + a.self_loop);
         }
         return;
     }
-    const int n_hubs = *a.hub_count;
+    const int n_hubs = *order.counts;
     int turn = 0;
-    for (int hub = blockIdx.x; hub < n_hubs; hub += hub_blocks, turn ^= 1) {
-        const int64_t v = a.hub_list[hub];
-        const int64_t beg = a.rowptr[v];
-        const int32_t deg = (int32_t)(a.rowptr[v + 1] - beg);
+    for (int hub = blockIdx.x; hub < n_hubs; hub += grid.hub_blocks, turn ^= 1) {
+        const GatRow row = order.rows[hub];
+        const int64_t v = row.v, beg = row.beg;
+        const int32_t deg = row.deg;
         pass.begin(v);
         gat_walk_by_warp<LPG, W>(pass, L, a.colidx, (int32_t)v, beg, deg, deg + a.self_loop, warp * kWarp, kGatWarps * kWarp, lane);
         pass.st.template merge_groups<LPG>();
@@ -182,7 +249,7 @@ __global__ void __launch_bounds__(kGatThreads, kGatBlocksPerSm) gat_lane_rows_ke
                 den = fmaf(sm_ml[turn][w][L.li].y, f, den);
                 z.fma(f, sm_acc[turn][w][L.li]);
             }
-            store_cols(v, L.col, z, den);
+            store_cols(hub, v, z, den);
         }
     }
 }
@@ -398,8 +465,26 @@ __global__ void __launch_bounds__(kGatRowThreads) gat_rows_kernel(GatArgs a, int
 void gat_forward_workspace(int64_t n_nodes, int32_t heads, Sizer& s) {
     s.take<float>((size_t)n_nodes * (size_t)heads);                   // s
     s.take<float>((size_t)n_nodes * (size_t)heads);                   // t
-    s.take<int32_t>((size_t)n_nodes);                                 // hub rows
-    s.take<int32_t>(64);                                              // their count
+    s.take<GatRow>((size_t)n_nodes);                                  // rows in order (general kernels: hub rows)
+    s.take<int32_t>(kGatOrderInts);                                   // rows per class of lengths (general kernels: hub rows)
+}
+
+bool gat_lanes_usable(int32_t heads, int32_t head_dim, const float* p, int64_t ldp, const float* q, int64_t ldq) {
+    int lpg, w;
+    return heads > 0 && heads <= kGatMaxHeads && head_dim > 0 && gat_lanes_cover(heads * head_dim, head_dim, p, ldp, q, ldq, &lpg, &w);
+}
+
+int gat_order_launch(const retexo_csr& g, int32_t self_loop, const int32_t* const* idx, const int64_t* n_idx, int lists, GatRow* rows,
+                     int32_t* slots, int32_t* bins, int n_sm, cudaStream_t st) {
+    const int hub_entries = gat_hub_entries(g.n_edges, n_sm);
+    RETEXO_CUDA_TRY(cudaMemsetAsync(bins, 0, kGatOrderInts * sizeof(int32_t), st));
+    for (int i = 0; i < lists; ++i)
+        if (n_idx[i]) gat_order_count_kernel<<<gat_order_blocks(n_idx[i]), 256, 0, st>>>(n_idx[i], idx[i], g.rowptr, self_loop, hub_entries, bins);
+    int32_t slot0 = 0;
+    for (int i = 0; i < lists; slot0 += (int32_t)n_idx[i++])
+        if (n_idx[i])
+            gat_order_kernel<<<gat_order_blocks(n_idx[i]), 256, 0, st>>>(n_idx[i], idx[i], g.rowptr, self_loop, hub_entries, bins, rows, slots, slot0);
+    return launch_status();
 }
 
 int gat_forward_launch(const GatForward& f, Arena& ws, int n_sm, cudaStream_t st) {
@@ -411,24 +496,33 @@ int gat_forward_launch(const GatForward& f, Arena& ws, int n_sm, cudaStream_t st
     a.self_loop = f.gat.add_self_loop ? 1 : 0;
     a.s = ws.take<float>((size_t)n * a.heads);
     a.t = ws.take<float>((size_t)n * a.heads);
-    a.hub_list = ws.take<int32_t>((size_t)n);
-    a.hub_count = ws.take<int32_t>(64);
-    RETEXO_CUDA_TRY(cudaMemsetAsync(a.hub_count, 0, sizeof(int32_t), st));
+    GatRow* rows = ws.take<GatRow>((size_t)n);
+    int32_t* bins = ws.take<int32_t>(kGatOrderInts);
+    a.hub_list = reinterpret_cast<int32_t*>(rows);
+    a.hub_count = bins;
     a.out = f.out; a.ldout = f.ldout; a.out16 = f.out16; a.ldout16 = f.ldout16;
     int lpg, w;
     if (gat_lanes_cover(a.dim, a.head_dim, a.p, a.ldp, nullptr, 0, &lpg, &w)) {
         const int vec_out = f.out && f.ldout % 4 == 0 && aligned_to(f.out, 16);
         const int vec_out16 = f.out16 && f.ldout16 % 4 == 0 && aligned_to(f.out16, 8);
-        const int hub_entries = gat_hub_entries(f.g.n_edges, n_sm), hub_blocks = 6 * n_sm;      // those without a row leave at once
-        return gat_lanes_dispatch(lpg, w, [&]<int LPG, int W>() {
-            const int64_t rows = kGatWarps * GatLanes<LPG, W>::G;
+        const int hub_entries = gat_hub_entries(f.g.n_edges, n_sm);
+        const bool own = !f.order.rows;
+        const GatRowOrder order = own ? GatRowOrder{rows, bins + kGatOrderCounts, nullptr, n} : f.order;
+        if (own) RETEXO_CUDA_TRY(cudaMemsetAsync(bins, 0, kGatOrderInts * sizeof(int32_t), st));
+        const int rc = gat_lanes_dispatch(lpg, w, [&]<int LPG, int W>() {
             gat_lane_scores_kernel<LPG, W><<<gat_lane_scores_grid<LPG, W>(n, n_sm), 256, 0, st>>>(
-                n, a.rowptr, a.p, a.ldp, a.heads, a.head_dim, a.a_src, a.a_dst, a.self_loop, hub_entries, a.s, a.t, a.hub_list, a.hub_count);
-            gat_lane_rows_kernel<LPG, W><<<(unsigned)((n + rows - 1) / rows + hub_blocks), kGatThreads, 0, st>>>(
-                a, hub_entries, hub_blocks, vec_out, vec_out16);
+                n, a.rowptr, a.p, a.ldp, a.heads, a.head_dim, a.a_src, a.a_dst, a.self_loop, hub_entries, a.s, a.t, own ? bins : nullptr);
+            return launch_status();
+        });
+        RETEXO_TRY(rc);
+        if (own) gat_order_kernel<<<gat_order_blocks(n), 256, 0, st>>>(n, nullptr, a.rowptr, a.self_loop, hub_entries, bins, rows, nullptr, 0);
+        return gat_lanes_dispatch(lpg, w, [&]<int LPG, int W>() {
+            const GatGrid grid = gat_grid<LPG>(order.n, f.g.n_edges + n, n_sm);
+            gat_lane_rows_kernel<LPG, W><<<grid.blocks, kGatThreads, 0, st>>>(a, order, grid, vec_out, vec_out16);
             return launch_status();
         });
     }
+    RETEXO_CUDA_TRY(cudaMemsetAsync(a.hub_count, 0, sizeof(int32_t), st));
     const unsigned blocks = (unsigned)((n + kGatRowWarps - 1) / kGatRowWarps);
     const int hub_blocks = 3 * n_sm;       // as many as are resident at once; those without a row leave at once
     const unsigned grid = blocks + (unsigned)hub_blocks;

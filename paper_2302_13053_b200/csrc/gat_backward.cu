@@ -36,7 +36,7 @@ struct GatBwdArgs {
     float* partial;                  // [blocks x 2 x dim]: per-block sums of ds_u p_u and dt_u p_u
     // lane layout only
     float* ds; float* dt;                       // [n x heads]
-    int32_t* hub_count; int32_t* hub_list;      // rows a whole block takes: how many ([1]: blocks that are done), which
+    int32_t* done;                              // blocks of the parameters' kernel that are done
 };
 
 __global__ void __launch_bounds__(kGbThreads) gat_bwd_scores_kernel(GatBwdArgs a) {
@@ -302,6 +302,7 @@ struct GatDstPass {
             c_more = fmaf(w, d, c_more);
             b1_more = fmaf(wg, d, b1_more);
         }
+        if (!ok[0]) return;      // (beyond the row's end nothing may change, not even what is lost)
         add_compensated(den, den_lost, den_more);
         add_compensated(c, c_lost, c_more);
         add_compensated(b1, b1_lost, b1_more);
@@ -337,23 +338,23 @@ struct GatDstPass {
 
 // Bound like the forward pass by the gather of p_u (4 dim + 4 heads bytes an entry); rows whose gradient is zero gather nothing.
 // Measured, whole backward pass (a lane per entry reading its own row in 16-byte pieces before; heads of other shapes a warp
-// per entry): 717 k nodes, 14 M entries, 4 x 16: 5319 -> 1936 us; 60 k nodes, 12 M entries: 2960 -> 733 us; 100 k nodes, 3 M
+// per entry): 717 k nodes, 14 M entries, 4 x 16: 5319 -> 1936 us, in order of lengths 1350; 60 k nodes, 12 M entries: 2960 -> 733 us; 100 k nodes, 3 M
 // entries, 8 x 32: 26.6 -> 0.92 ms; 200 k nodes, 4 M entries, 1 x 8: 834 -> 160 us.
 template <int LPG, int W>
-__global__ void __launch_bounds__(kGatThreads, kGatBlocksPerSm) gat_lane_dst_kernel(GatBwdArgs a, int hub_entries, int hub_blocks) {
-    constexpr int G = GatLanes<LPG, W>::G;
+__global__ void __launch_bounds__(kGatThreads, kGatBlocksPerSm) gat_lane_dst_kernel(GatBwdArgs a, GatRowOrder order, GatGrid grid) {
     __shared__ float sm[2][kGatWarps][5][LPG];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const GatLanes<LPG, W> L(lane, a.dim, a.head_dim);
     GatDstPass<LPG, W> pass(a, L);
     const int hw = a.head_dim / W;
-    if ((int)blockIdx.x >= hub_blocks) {
-        const int64_t v0 = ((int64_t)(blockIdx.x - hub_blocks) * kGatWarps + warp) * G;
-        if (v0 >= a.n) return;
-        const int64_t v = min(v0 + L.g, a.n - 1);
-        const int64_t beg = __ldg(a.rowptr + v);
-        const int32_t deg = (int32_t)(__ldg(a.rowptr + v + 1) - beg);
-        const int32_t total = v0 + L.g < a.n ? deg + a.self_loop : INT32_MAX;
+    if ((int)blockIdx.x >= grid.hub_blocks) {
+        int rows;
+        const int64_t i0 = gat_first_row<LPG>(order, grid, (int64_t)((int)blockIdx.x - grid.hub_blocks) * kGatWarps + warp, rows);
+        if (rows == 0) return;
+        const GatRow row = load_row_entry(order.rows + i0 + min(L.g, rows - 1));
+        const int64_t v = row.v, beg = row.beg;
+        const int32_t deg = row.deg;
+        const int32_t total = L.g < rows ? deg + a.self_loop : INT32_MAX;
         const bool mine = total <= kGatGroupEntries;
         const unsigned lanes = __ballot_sync(0xffffffffu, pass.begin(v));
         const unsigned group = LPG == 32 ? 0xffffffffu : ((1u << (LPG & 31)) - 1u) << (L.g * LPG);
@@ -361,7 +362,7 @@ __global__ void __launch_bounds__(kGatThreads, kGatBlocksPerSm) gat_lane_dst_ker
         const int32_t take = mine && live ? total : 0;
         gat_walk_by_group<LPG, W>(pass, L, a.colidx, (int32_t)v, beg, deg, take, __reduce_max_sync(0xffffffffu, take));
         pass.finish(v, live, mine, hw);
-        unsigned longer = __ballot_sync(0xffffffffu, L.li == 0 && !mine && total < hub_entries);
+        unsigned longer = __ballot_sync(0xffffffffu, L.li == 0 && !mine && L.g < rows);
         while (longer) {
             const int src = __ffs(longer) - 1;
             longer &= longer - 1;
@@ -376,12 +377,12 @@ __global__ void __launch_bounds__(kGatThreads, kGatBlocksPerSm) gat_lane_dst_ker
         }
         return;
     }
-    const int n_hubs = *a.hub_count;
+    const int n_hubs = *order.counts;
     int turn = 0;      // (of the rows that meet a barrier)
-    for (int hub = blockIdx.x; hub < n_hubs; hub += hub_blocks) {
-        const int64_t v = a.hub_list[hub];
-        const int64_t beg = a.rowptr[v];
-        const int32_t deg = (int32_t)(a.rowptr[v + 1] - beg);
+    for (int hub = blockIdx.x; hub < n_hubs; hub += grid.hub_blocks) {
+        const GatRow row = order.rows[hub];
+        const int64_t v = row.v, beg = row.beg;
+        const int32_t deg = row.deg;
         const bool live = __any_sync(0xffffffffu, pass.begin(v));      // (the same in every warp)
         if (live) {
             gat_walk_by_warp<LPG, W>(pass, L, a.colidx, (int32_t)v, beg, deg, deg + a.self_loop, warp * kWarp, kGatWarps * kWarp, lane);
@@ -447,7 +448,7 @@ struct GatSrcPass {
             more = fmaf(ag, d - st[t].z, more);
             acc.fma(alpha, g[t]);
         }
-        add_compensated(ds, ds_lost, more);
+        if (ok[0]) add_compensated(ds, ds_lost, more);
     }
     __device__ __forceinline__ void merge_groups() {
 #pragma unroll
@@ -473,26 +474,26 @@ struct GatSrcPass {
 
 // Bound by the gather of dz_v and the statistics (4 dim + 16 heads bytes an entry).
 template <int LPG, int W>
-__global__ void __launch_bounds__(kGatThreads, kGatBlocksPerSm) gat_lane_src_kernel(GatBwdArgs a, int hub_entries, int hub_blocks,
+__global__ void __launch_bounds__(kGatThreads, kGatBlocksPerSm) gat_lane_src_kernel(GatBwdArgs a, GatRowOrder order, GatGrid grid,
                                                                                     int vec, int vec16) {
-    constexpr int G = GatLanes<LPG, W>::G;
     __shared__ Cols<W> sm_acc[2][kGatWarps][LPG];
     __shared__ float sm_ds[2][kGatWarps][LPG];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const GatLanes<LPG, W> L(lane, a.dim, a.head_dim);
     GatSrcPass<LPG, W> pass(a, L);
-    if ((int)blockIdx.x >= hub_blocks) {
-        const int64_t u0 = ((int64_t)(blockIdx.x - hub_blocks) * kGatWarps + warp) * G;
-        if (u0 >= a.n) return;
-        const int64_t u = min(u0 + L.g, a.n - 1);
-        const int64_t beg = __ldg(a.rowptr + u);
-        const int32_t deg = (int32_t)(__ldg(a.rowptr + u + 1) - beg);
-        const int32_t total = u0 + L.g < a.n ? deg + a.self_loop : INT32_MAX;
+    if ((int)blockIdx.x >= grid.hub_blocks) {
+        int rows;
+        const int64_t i0 = gat_first_row<LPG>(order, grid, (int64_t)((int)blockIdx.x - grid.hub_blocks) * kGatWarps + warp, rows);
+        if (rows == 0) return;
+        const GatRow row = load_row_entry(order.rows + i0 + min(L.g, rows - 1));
+        const int64_t u = row.v, beg = row.beg;
+        const int32_t deg = row.deg;
+        const int32_t total = L.g < rows ? deg + a.self_loop : INT32_MAX;
         const bool mine = total <= kGatGroupEntries;
         pass.begin(u);
         gat_walk_by_group<LPG, W>(pass, L, a.colidx, (int32_t)u, beg, deg, mine ? total : 0, __reduce_max_sync(0xffffffffu, mine ? total : 0));
         pass.finish(u, mine && L.on, vec != 0, vec16 != 0);
-        unsigned longer = __ballot_sync(0xffffffffu, L.li == 0 && !mine && total < hub_entries);
+        unsigned longer = __ballot_sync(0xffffffffu, L.li == 0 && !mine && L.g < rows);
         while (longer) {
             const int src = __ffs(longer) - 1;
             longer &= longer - 1;
@@ -505,12 +506,12 @@ __global__ void __launch_bounds__(kGatThreads, kGatBlocksPerSm) gat_lane_src_ker
         }
         return;
     }
-    const int n_hubs = *a.hub_count;
+    const int n_hubs = *order.counts;
     int turn = 0;
-    for (int hub = blockIdx.x; hub < n_hubs; hub += hub_blocks, turn ^= 1) {
-        const int64_t u = a.hub_list[hub];
-        const int64_t beg = a.rowptr[u];
-        const int32_t deg = (int32_t)(a.rowptr[u + 1] - beg);
+    for (int hub = blockIdx.x; hub < n_hubs; hub += grid.hub_blocks, turn ^= 1) {
+        const GatRow row = order.rows[hub];
+        const int64_t u = row.v, beg = row.beg;
+        const int32_t deg = row.deg;
         pass.begin(u);
         gat_walk_by_warp<LPG, W>(pass, L, a.colidx, (int32_t)u, beg, deg, deg + a.self_loop, warp * kWarp, kGatWarps * kWarp, lane);
         pass.merge_groups();
@@ -575,9 +576,10 @@ __global__ void __launch_bounds__(256) gat_lane_params_kernel(GatBwdArgs a, floa
     }
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(a.hub_count + 1, 1) == (int)gridDim.x - 1;
+    if (threadIdx.x == 0) last = atomicAdd(a.done, 1) == (int)gridDim.x - 1;
     __syncthreads();
     if (!last) return;
+    if (threadIdx.x == 0) *a.done = 0;      // for the next pass over this scratch
     __threadfence();
     // every column by 256 / (2 dim) threads (one where the columns are more), each its share of the blocks in order
     const int cols = 2 * a.dim, shares = cols < 256 ? 256 / cols : 1;
@@ -625,8 +627,8 @@ extern "C" size_t retexo_gat_backward_workspace_size(int64_t n_nodes, int64_t n_
     s.take<float>((size_t)std::max<int64_t>((n_nodes + kGbWarps - 1) / kGbWarps, kGatParamBlocks) * 2 * (size_t)dim);
     s.take<float>((size_t)n_nodes * heads);
     s.take<float>((size_t)n_nodes * heads);
-    s.take<int32_t>(64);
-    s.take<int32_t>((size_t)n_nodes);
+    s.take<int32_t>(kGatOrderInts + 64);
+    s.take<GatRow>((size_t)n_nodes);
     return s.off + kAlign;
 }
 
@@ -634,13 +636,45 @@ extern "C" int retexo_gat_backward(const retexo_csr* g, const float* p, int64_t 
                                    const float* dz, int64_t lddz, float* dp, int64_t lddp, void* dp_bf16,
                                    int64_t lddp_bf16, float* da_src, float* da_dst, void* workspace,
                                    size_t workspace_bytes, void* stream) {
+    return gat_backward(g, p, ldp, gat, dz, lddz, dp, lddp, dp_bf16, lddp_bf16, da_src, da_dst, workspace, workspace_bytes, nullptr,
+                        static_cast<cudaStream_t>(stream));
+}
+
+// Scratch, in the order retexo_gat_backward_workspace_size lists it.
+struct GatBwdScratch { float *s, *t; float4* stats; float* partial; float *ds, *dt; int32_t* bins; GatRow* rows; };
+static GatBwdScratch backward_scratch(int64_t n, int32_t heads, int32_t dim, void* workspace, size_t workspace_bytes) {
+    Arena ws(workspace, workspace_bytes);
+    GatBwdScratch b;
+    b.s = ws.take<float>((size_t)n * heads);
+    b.t = ws.take<float>((size_t)n * heads);
+    b.stats = ws.take<float4>((size_t)n * heads);
+    b.partial = ws.take<float>((size_t)std::max<int64_t>((n + kGbWarps - 1) / kGbWarps, kGatParamBlocks) * 2 * (size_t)dim);
+    b.ds = ws.take<float>((size_t)n * heads);
+    b.dt = ws.take<float>((size_t)n * heads);
+    b.bins = ws.take<int32_t>(kGatOrderInts + 64);
+    b.rows = ws.take<GatRow>((size_t)n);
+    return b;
+}
+
+int retexo::gat_backward_prepare(int64_t n_nodes, int64_t n_edges, int32_t heads, int32_t head_dim, void* workspace, size_t workspace_bytes,
+                                 cudaStream_t st) {
+    if (workspace_bytes < retexo_gat_backward_workspace_size(n_nodes, n_edges, heads, heads * head_dim)) return RETEXO_ERR_WORKSPACE;
+    const GatBwdScratch b = backward_scratch(n_nodes, heads, heads * head_dim, workspace, workspace_bytes);
+    RETEXO_CUDA_TRY(cudaMemsetAsync(b.stats, 0, sizeof(float4) * (size_t)n_nodes * heads, st));
+    RETEXO_CUDA_TRY(cudaMemsetAsync(b.dt, 0, sizeof(float) * (size_t)n_nodes * heads, st));
+    RETEXO_CUDA_TRY(cudaMemsetAsync(b.bins, 0, (kGatOrderInts + 64) * sizeof(int32_t), st));
+    return RETEXO_OK;
+}
+
+int retexo::gat_backward(const retexo_csr* g, const float* p, int64_t ldp, const retexo_gat_params* gat, const float* dz, int64_t lddz,
+                         float* dp, int64_t lddp, void* dp_bf16, int64_t lddp_bf16, float* da_src, float* da_dst, void* workspace,
+                         size_t workspace_bytes, const GatBackwardKept* kept, cudaStream_t st) {
     if (!g || g->n_nodes < 0 || g->n_edges < 0 || g->n_nodes > INT32_MAX) return RETEXO_ERR_INVALID_ARG;
     if (!gat || gat->heads <= 0 || gat->head_dim <= 0 || !gat->a_src || !gat->a_dst) return RETEXO_ERR_INVALID_ARG;
     const int32_t dim = gat->heads * gat->head_dim;
     if (gat->heads > kGbMaxHeads || dim > 256) return RETEXO_ERR_UNSUPPORTED;
     if (!da_src || !da_dst || (!dp && !dp_bf16)) return RETEXO_ERR_INVALID_ARG;
     if (ldp < dim || lddz < dim || (dp && lddp < dim) || (dp_bf16 && lddp_bf16 < dim)) return RETEXO_ERR_INVALID_ARG;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (g->n_nodes == 0) {
         RETEXO_CUDA_TRY(cudaMemsetAsync(da_src, 0, sizeof(float) * dim, st));
         RETEXO_CUDA_TRY(cudaMemsetAsync(da_dst, 0, sizeof(float) * dim, st));
@@ -650,36 +684,40 @@ extern "C" int retexo_gat_backward(const retexo_csr* g, const float* p, int64_t 
     const size_t need = retexo_gat_backward_workspace_size(g->n_nodes, g->n_edges, gat->heads, dim);
     if (!workspace || !aligned_to(workspace, kAlign) || workspace_bytes < need) return RETEXO_ERR_WORKSPACE;
     const int64_t n = g->n_nodes;
-    Arena ws(workspace, workspace_bytes);
+    const GatBwdScratch b = backward_scratch(n, gat->heads, dim, workspace, workspace_bytes);
     GatBwdArgs a;
     a.n = n; a.rowptr = g->rowptr; a.colidx = g->colidx; a.p = p; a.ldp = ldp;
     a.heads = gat->heads; a.head_dim = gat->head_dim; a.dim = dim;
     a.a_src = gat->a_src; a.a_dst = gat->a_dst; a.slope = gat->negative_slope; a.self_loop = gat->add_self_loop ? 1 : 0;
     a.dz = dz; a.lddz = lddz;
-    a.s = ws.take<float>((size_t)n * gat->heads);
-    a.t = ws.take<float>((size_t)n * gat->heads);
-    a.stats = ws.take<float4>((size_t)n * gat->heads);
+    a.s = b.s; a.t = b.t; a.stats = b.stats; a.partial = b.partial; a.ds = b.ds; a.dt = b.dt; a.done = b.bins + kGatOrderInts;
     const unsigned blocks = (unsigned)((n + kGbWarps - 1) / kGbWarps);
-    a.partial = ws.take<float>((size_t)std::max<int64_t>(blocks, kGatParamBlocks) * 2 * (size_t)dim);
     a.dp = dp; a.lddp = lddp; a.dp16 = static_cast<__nv_bfloat16*>(dp_bf16); a.lddp16 = lddp_bf16;
-    a.ds = ws.take<float>((size_t)n * gat->heads);
-    a.dt = ws.take<float>((size_t)n * gat->heads);
-    a.hub_count = ws.take<int32_t>(64);
-    a.hub_list = ws.take<int32_t>((size_t)n);
     int lpg, w;
     if (gat_lanes_cover(dim, gat->head_dim, p, ldp, dz, lddz, &lpg, &w)) {
         const int n_sm = sm_count();
         if (n_sm <= 0) return RETEXO_ERR_CUDA;
-        RETEXO_CUDA_TRY(cudaMemsetAsync(a.hub_count, 0, 2 * sizeof(int32_t), st));
         const int vec = dp && lddp % 4 == 0 && aligned_to(dp, 16), vec16 = dp_bf16 && lddp_bf16 % 4 == 0 && aligned_to(dp_bf16, 8);
-        const int hub_entries = gat_hub_entries(g->n_edges, n_sm), hub_blocks = 6 * n_sm;
+        const int hub_entries = gat_hub_entries(g->n_edges, n_sm);
+        if (kept) {
+            a.s = const_cast<float*>(kept->s); a.t = const_cast<float*>(kept->t);
+        } else {
+            RETEXO_CUDA_TRY(cudaMemsetAsync(b.bins, 0, (kGatOrderInts + 1) * sizeof(int32_t), st));
+            RETEXO_TRY((gat_lanes_dispatch(lpg, w, [&]<int LPG, int W>() {
+                gat_lane_scores_kernel<LPG, W><<<gat_lane_scores_grid<LPG, W>(n, n_sm), 256, 0, st>>>(
+                    n, a.rowptr, a.p, a.ldp, a.heads, a.head_dim, a.a_src, a.a_dst, a.self_loop, hub_entries, a.s, a.t, b.bins);
+                return launch_status();
+            })));
+            gat_order_kernel<<<gat_order_blocks(n), 256, 0, st>>>(n, nullptr, a.rowptr, a.self_loop, hub_entries, b.bins, b.rows, nullptr, 0);
+        }
+        const GatRowOrder all{b.rows, b.bins + kGatOrderCounts, nullptr, n}, dst = kept ? kept->dst : all, src = kept ? kept->src : all;
+        RETEXO_TRY((gat_lanes_dispatch(lpg, w, [&]<int LPG, int W>() {
+            const GatGrid dst_grid = gat_grid<LPG>(dst.n, g->n_edges + n, n_sm), src_grid = gat_grid<LPG>(src.n, g->n_edges + n, n_sm);
+            gat_lane_dst_kernel<LPG, W><<<dst_grid.blocks, kGatThreads, 0, st>>>(a, dst, dst_grid);
+            gat_lane_src_kernel<LPG, W><<<src_grid.blocks, kGatThreads, 0, st>>>(a, src, src_grid, vec, vec16);
+            return launch_status();
+        })));
         return gat_lanes_dispatch(lpg, w, [&]<int LPG, int W>() {
-            constexpr int64_t rows = kGatWarps * GatLanes<LPG, W>::G;
-            const unsigned grid = (unsigned)((n + rows - 1) / rows + hub_blocks);
-            gat_lane_scores_kernel<LPG, W><<<gat_lane_scores_grid<LPG, W>(n, n_sm), 256, 0, st>>>(
-                n, a.rowptr, a.p, a.ldp, a.heads, a.head_dim, a.a_src, a.a_dst, a.self_loop, hub_entries, a.s, a.t, a.hub_list, a.hub_count);
-            gat_lane_dst_kernel<LPG, W><<<grid, kGatThreads, 0, st>>>(a, hub_entries, hub_blocks);
-            gat_lane_src_kernel<LPG, W><<<grid, kGatThreads, 0, st>>>(a, hub_entries, hub_blocks, vec, vec16);
             const int64_t want = (n + 64 * GatLanes<LPG, W>::G - 1) / (64 * GatLanes<LPG, W>::G);      // 8 nodes per group
             gat_lane_params_kernel<LPG, W><<<(unsigned)std::min(want, kGatParamBlocks), 256, 0, st>>>(a, da_src, da_dst);
             return launch_status();

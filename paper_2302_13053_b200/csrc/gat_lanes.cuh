@@ -4,6 +4,7 @@
 // over a head's columns are linear, so they are reduced once per row, not once per entry, wherever they are not a difference.
 #pragma once
 #include "common.cuh"
+#include "gat.h"
 
 namespace retexo {
 
@@ -18,6 +19,77 @@ constexpr int kGatGroupEntries = 32;
 inline int gat_hub_entries(int64_t n_edges, int n_sm) {
     const int64_t share = n_edges / ((int64_t)n_sm * 128);
     return (int)(share < 64 ? 64 : share > 65536 ? 65536 : share);
+}
+
+// The rows a kernel takes, in order of falling length, so that the rows that share a warp (and the warps that share a block) take
+// about the same time and the longest start first: hubs (hub_entries or more), then the others.  On a power-law graph of 20 entries a row
+// the longest of four rows is 2.3 times the mean, and the lanes of the other three wait for it (717 k nodes, 14 M entries, 4 x 16, in node
+// order / in this order: forward 617 / 440 to 470 us, destinations 763 / 520 to 550, sources 988 / 690).  Order inside a class of lengths
+// is arbitrary; no result depends on it.  Slabs of 32 columns, which halve what L2 has to hold, take 1.5 times as long.
+struct __align__(16) GatRow { int64_t beg; int32_t deg, v; };      // first entry, entries, node
+__device__ __forceinline__ GatRow load_row_entry(const GatRow* p) {
+    const int4 x = __ldg(reinterpret_cast<const int4*>(p));
+    return GatRow{(int64_t)((uint64_t)(uint32_t)x.x | ((uint64_t)(uint32_t)x.y << 32)), x.z, x.w};
+}
+// Classes of lengths: hubs, eight per octave above kGatGroupEntries, one per length below.
+constexpr int kGatOctave = 5, kGatLongBins = 1 + 8 * (16 - kGatOctave);      // (hubs start at 65536 entries at the latest)
+constexpr int kGatBins = 128;
+static_assert(kGatGroupEntries == 1 << kGatOctave && kGatLongBins + kGatGroupEntries < kGatBins, "classes of lengths");
+__device__ __forceinline__ int gat_bin(int32_t total, int32_t hub_entries) {
+    if (total >= hub_entries) return 0;
+    if (total <= kGatGroupEntries) return kGatLongBins + kGatGroupEntries - total;
+    const int octave = 31 - __clz(total);
+    return kGatLongBins - 1 - ((octave - kGatOctave) * 8 + ((total >> (octave - 3)) & 7));
+}
+static_assert(kGatOrderCounts == 2 * kGatBins, "rows counted per class, rows placed so far (all cleared before the count)");
+
+// Counts the rows idx[0, n) (null: all rows 0 .. n - 1) per class; see gat_order_kernel.
+__global__ void __launch_bounds__(256) gat_order_count_kernel(int64_t n, const int32_t* __restrict__ idx, const int64_t* __restrict__ rowptr,
+                                                              int32_t self_loop, int32_t hub_entries, int32_t* __restrict__ bins);
+// Places them behind one another once all are counted; slots[i] (optional) receives slot0 + the row's position in the list.
+__global__ void __launch_bounds__(256) gat_order_kernel(int64_t n, const int32_t* __restrict__ idx, const int64_t* __restrict__ rowptr,
+                                                        int32_t self_loop, int32_t hub_entries, int32_t* __restrict__ bins,
+                                                        GatRow* __restrict__ rows, int32_t* __restrict__ slots, int32_t slot0);
+constexpr int kGatOrderRows = 1024;      // rows a block of either takes
+inline unsigned gat_order_blocks(int64_t n) { return (unsigned)((n + kGatOrderRows - 1) / kGatOrderRows); }
+
+// Blocks of a pass over an order: hub_blocks take the hubs, a block a row; then warps for the long rows, one each as far as the grid has
+// some (long_warps), the rest of the order G rows a warp.  (22 k nodes, 365 k entries, long rows G to a warp one after the other instead: forward 22.3
+// against 11.8 us, sources 26.0 against 19.7.  Groups taking rows of up to 64 entries: 14.4 and 24.5 us there, 2 % less on 717 k nodes;
+// of up to 16: 12.6 and 20.2, 6 % more.)  How many long rows there are only the device knows, so the grid has as many
+// warps for them as the entries allow, up to four times what is resident (a block without a row leaves at once).
+struct GatGrid {
+    int hub_blocks, long_warps;
+    unsigned blocks;
+};
+template <int LPG>
+inline GatGrid gat_grid(int64_t n, int64_t n_entries, int n_sm) {
+    constexpr int64_t G = kWarp / LPG;
+    GatGrid g;
+    g.hub_blocks = 6 * n_sm;
+    const int64_t most = (int64_t)n_sm * 4 * kGatBlocksPerSm * kGatWarps;
+    int64_t want = n_entries / (kGatGroupEntries + 1) + 1;
+    if (want > n) want = n;
+    if (want > most) want = most;
+    g.long_warps = G > 1 ? (int)((want + kGatWarps - 1) / kGatWarps * kGatWarps) : 0;
+    g.blocks = (unsigned)(g.hub_blocks + (g.long_warps + (n + G - 1) / G + kGatWarps - 1) / kGatWarps);
+    return g;
+}
+// The first entry of the order that warp w (counted behind the hubs' blocks) takes, and how many (0: none).
+template <int LPG>
+__device__ __forceinline__ int64_t gat_first_row(const GatRowOrder& order, const GatGrid& grid, int64_t w, int& count) {
+    constexpr int G = kWarp / LPG;
+    const int n_hubs = __ldg(order.counts), n_long = __ldg(order.counts + 1);
+    const int64_t single = G > 1 ? min(n_long - n_hubs, grid.long_warps) : 0;      // rows with a warp of their own
+    int64_t first;
+    if (w < grid.long_warps) {
+        count = w < single ? 1 : 0;
+        first = n_hubs + w;
+    } else {
+        first = n_hubs + single + (w - grid.long_warps) * G;
+        count = (int)max((int64_t)0, min((int64_t)G, order.n - first));
+    }
+    return first;
 }
 
 template <int LPG, int W>
@@ -251,17 +323,21 @@ __device__ __forceinline__ float head_dot(const Cols<W>& a, const Cols<W>& x, in
 template <int W>
 __device__ __forceinline__ int head_last_block(int hw) { return hw > 32 / W ? hw - 32 / W : 0; }
 
-// s_u = <a_src, p_u>, t_u = <a_dst, p_u> per head, and the list of the rows long enough for a whole block (its order varies from
-// run to run; no result depends on it).  A stream over p: LPG lanes a node, kNodes nodes in flight per group.
+// s_u = <a_src, p_u>, t_u = <a_dst, p_u> per head, and (bins != nullptr) how many rows there are of each class of lengths.
+// A stream over p: LPG lanes a node, kNodes nodes in flight per group.
 // (717 k nodes, 4 x 16: 39 us; a warp per node with 4-byte loads and two shuffle trees per head took 366 us.)
 template <int LPG, int W>
 __global__ void __launch_bounds__(256) gat_lane_scores_kernel(int64_t n, const int64_t* __restrict__ rowptr,
                                                               const float* __restrict__ p, int64_t ldp, int32_t heads,
                                                               int32_t head_dim, const float* __restrict__ a_src,
                                                               const float* __restrict__ a_dst, int32_t self_loop, int32_t hub_entries,
-                                                              float* __restrict__ s, float* __restrict__ t,
-                                                              int32_t* __restrict__ hub_list, int32_t* __restrict__ hub_count) {
+                                                              float* __restrict__ s, float* __restrict__ t, int32_t* __restrict__ bins) {
     constexpr int kNodes = 2, G = GatLanes<LPG, W>::G;
+    __shared__ int32_t count[kGatBins];
+    if (bins) {
+        if (threadIdx.x < kGatBins) count[threadIdx.x] = 0;
+        __syncthreads();
+    }
     const int lane = threadIdx.x & 31;
     const GatLanes<LPG, W> L(lane, heads * head_dim, head_dim);
     const int hw = head_dim / W;                  // lanes a head spans
@@ -275,8 +351,10 @@ __global__ void __launch_bounds__(256) gat_lane_scores_kernel(int64_t n, const i
         Cols<W> x[kNodes];
 #pragma unroll
         for (int i = 0; i < kNodes; ++i) x[i].load(p + min(u0 + i * G + L.g, n - 1) * ldp + L.col);
-        for (int64_t u = u0 + lane; u < min(n, u0 + G * kNodes); u += kWarp)
-            if (rowptr[u + 1] - rowptr[u] + self_loop >= hub_entries) hub_list[atomicAdd(hub_count, 1)] = (int32_t)u;
+        if (bins) {
+            for (int64_t u = u0 + lane; u < min(n, u0 + G * kNodes); u += kWarp)
+                atomicAdd(count + gat_bin((int32_t)(rowptr[u + 1] - rowptr[u]) + self_loop, hub_entries), 1);
+        }
 #pragma unroll
         for (int i = 0; i < kNodes; ++i) {
             const int64_t u = u0 + i * G + L.g;
@@ -286,6 +364,10 @@ __global__ void __launch_bounds__(256) gat_lane_scores_kernel(int64_t n, const i
                 t[u * heads + L.head] = tt;
             }
         }
+    }
+    if (bins) {
+        __syncthreads();
+        if (threadIdx.x < kGatBins && count[threadIdx.x]) atomicAdd(bins + threadIdx.x, count[threadIdx.x]);
     }
 }
 

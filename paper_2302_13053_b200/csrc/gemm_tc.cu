@@ -55,6 +55,7 @@ struct TcKernelArgs {
     int mode, relu;
     const float* bias;
     float* out_f32; int64_t ld_f32;
+    const int32_t* f32_rows;
     __nv_bfloat16* out_bf16; int64_t ld_bf16;
     uint32_t* relu_bits; int64_t ld_bits;
     const __nv_bfloat16* mask; int64_t ld_mask;
@@ -665,7 +666,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                             g.relu_bits[row * g.ld_bits + (col0 >> 5)] = word;
                         }
                         if (g.out_f32 && row < g.M) {
-                            float* dst = g.out_f32 + row * g.ld_f32 + col0;
+                            float* dst = g.out_f32 + (g.f32_rows ? (int64_t)__ldg(g.f32_rows + row) : row) * g.ld_f32 + col0;
                             if (col0 + 32 <= g.N && (g.ld_f32 & 3) == 0 && aligned16(g.out_f32)) {
 #pragma unroll
                                 for (int j = 0; j < 32; j += 4)
@@ -765,7 +766,7 @@ static int launch_tc_mode(const TcGemm& t, const CUtensorMap& ma, const CUtensor
     g.k_blocks_per_split = (g.k_blocks_total + splits - 1) / splits;
     g.splits = splits;
     g.mode = t.mode; g.relu = t.relu; g.bias = t.bias;
-    g.out_f32 = t.out_f32; g.ld_f32 = t.ld_f32; g.out_bf16 = t.out_bf16; g.ld_bf16 = t.ld_bf16;
+    g.out_f32 = t.out_f32; g.ld_f32 = t.ld_f32; g.f32_rows = t.f32_rows; g.out_bf16 = t.out_bf16; g.ld_bf16 = t.ld_bf16;
     g.relu_bits = t.relu_bits; g.ld_bits = t.ld_bits;
     g.mask = t.mask; g.ld_mask = t.ld_mask;
     g.gate_scale = t.gate_scale != 0.f ? t.gate_scale : 1.f;
@@ -816,7 +817,7 @@ static int launch_tc_pair(const TcGemm& t, cudaStream_t st) {
     g.k_blocks_per_split = g.k_blocks_total;
     g.splits = 1;
     g.mode = t.mode; g.relu = t.relu; g.bias = t.bias;
-    g.out_f32 = t.out_f32; g.ld_f32 = t.ld_f32; g.out_bf16 = t.out_bf16; g.ld_bf16 = t.ld_bf16;
+    g.out_f32 = t.out_f32; g.ld_f32 = t.ld_f32; g.f32_rows = t.f32_rows; g.out_bf16 = t.out_bf16; g.ld_bf16 = t.ld_bf16;
     g.relu_bits = t.relu_bits; g.ld_bits = t.ld_bits;
     g.drop_thresh = t.drop_thresh; g.drop_step = t.drop_step; g.drop_key0 = t.drop_key[0]; g.drop_key1 = t.drop_key[1];
     g.drop_scale = t.drop_scale; g.drop_rows = t.drop_rows; g.drop_step_dev = t.drop_step_dev;

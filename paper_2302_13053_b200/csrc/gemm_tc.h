@@ -37,6 +37,7 @@ struct TcGemm {
     int mode, relu, splits;
     const float* bias;
     float* out_f32; int64_t ld_f32;
+    const int32_t* f32_rows;      // TC_EPI_BIAS (optional): row m of the result goes to row f32_rows[m] of out_f32
     __nv_bfloat16* out_bf16; int64_t ld_bf16;
     // TC_EPI_BIAS / TC_EPI_BIAS_DROP (optional): one bit per output element, bit n & 31 of word [m][n / 32] = [out > 0]
     uint32_t* relu_bits; int64_t ld_bits;

@@ -246,7 +246,7 @@ namespace retexo {
 int mlp_train_step_launch(const MlpPlan& p, const MlpBuffers& b, const retexo_mlp* model,
                           const bf16* x, int64_t ldx, const int32_t* y,
                           float* loss_out, float* grad_out, bool shadows_ready, const EvalTail* tail,
-                          cudaStream_t st, const DeviceIter* dev, float* dx_out, int64_t ld_dx, bool keep_shadows) {
+                          cudaStream_t st, const DeviceIter* dev, float* dx_out, int64_t ld_dx, bool keep_shadows, const int32_t* dx_rows) {
     const int64_t n = p.n_rows;
     const int64_t n_all = n + (tail ? p.n_eval : 0);          // evaluation rows ride along in the forward pass
     const int32_t d_in = p.d_in, H = p.hidden, O = p.n_classes, out1 = p.out1;
@@ -348,7 +348,7 @@ int mlp_train_step_launch(const MlpPlan& p, const MlpBuffers& b, const retexo_ml
     // ---- dX = grad1 W1^T, for a caller that trains what produced X (an aggregator with parameters)
     if (dx_out) {
         TcGemm dxg = tc_base(grad1, ld_grad1, b.w1r16, p.ld_o1, n, d_in, out1, b.status);
-        dxg.out_f32 = dx_out; dxg.ld_f32 = ld_dx;
+        dxg.out_f32 = dx_out; dxg.ld_f32 = ld_dx; dxg.f32_rows = dx_rows;
         RETEXO_TRY(tc_gemm_launch(dxg, st));
     }
     // ---- [dW1 ; db1] = [X | 1]^T grad1,  [dW2 ; db2] = [Hd | 1]^T dL

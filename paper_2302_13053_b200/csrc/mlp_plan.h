@@ -106,8 +106,9 @@ void mlp_step_buffers(const MlpPlan& p, void* workspace, size_t bytes, MlpBuffer
 int mlp_train_step_launch(const MlpPlan& p, const MlpBuffers& b, const retexo_mlp* model,
                           const __nv_bfloat16* x, int64_t ldx, const int32_t* y, float* loss_out, float* grad_out, bool shadows_ready,
                           const EvalTail* tail, cudaStream_t st, const DeviceIter* dev = nullptr,
-                          float* dx_out = nullptr, int64_t ld_dx = 0,      // dx_out: fp32 [n_rows x ld_dx], dLoss / dX
-                          bool keep_shadows = true);
+                          float* dx_out = nullptr, int64_t ld_dx = 0,      // dx_out: fp32 rows of ld_dx, dLoss / dX
+                          bool keep_shadows = true,
+                          const int32_t* dx_rows = nullptr);               // (optional) the row of dx_out that row i's gradient goes to
 
 // Forward + arg-max + hit count over a dense batch with the weight copies in `b` (which must
 // hold model->theta): what validation needs after every iteration.  hd_ws: bf16 [n_rows x p.ld_h];

@@ -45,6 +45,29 @@ def test_gat_forward_and_backward(heads, dh, pad):
         np.testing.assert_allclose(got.cpu().numpy(), ref, rtol=0, atol=2e-6 * max(1.0, np.abs(ref).max()) * np.sqrt(n))
 
 
+@pytest.mark.parametrize("heads,dh", [(2, 8), (1, 32)])
+def test_more_long_rows_than_warps_for_them(heads, dh):
+    """24000 rows of 41 entries with the node itself, longer than a group takes: the grid has 21312 warps for such rows, the others share."""
+    from paper_2302_13053_b200 import binding as B
+    n, half, d = 24000, 20, heads * dh
+    steps = np.concatenate([np.arange(-half, 0), np.arange(1, half + 1)])
+    colidx = np.sort((np.arange(n)[:, None] + steps) % n, axis=1).astype(np.int32).ravel()
+    rowptr = np.arange(n + 1, dtype=np.int64) * (2 * half)
+    rng = np.random.default_rng(heads)
+    p, dz = (rng.standard_normal((n, d)).astype(np.float32) for _ in range(2))
+    dz[rng.random(n) < 0.4] = 0.0
+    gat = dict(heads=heads, head_dim=dh, negative_slope=0.2, add_self_loop=1,
+               a_src=(rng.standard_normal((heads, dh)) / np.sqrt(dh)).astype(np.float32),
+               a_dst=(rng.standard_normal((heads, dh)) / np.sqrt(dh)).astype(np.float32))
+    g = dict(gat, a_src=torch.from_numpy(gat["a_src"]), a_dst=torch.from_numpy(gat["a_dst"]))
+    out, _ = B.retexo_aggregate(B.GAT, dev(rowptr), dev(colidx), dev(p), gat=g)
+    assert_rows_close(out.cpu().numpy(), oracle.aggregate(oracle.GAT, rowptr, colidx, p, gat=gat))
+    dp, _, _, _ = B.retexo_gat_backward(dev(rowptr), dev(colidx), dev(p), g, dev(dz))
+    ref = oracle.gat_backward(rowptr, colidx, p, gat, dz.astype(np.float64))[0]
+    err = np.abs(dp.cpu().numpy() - ref).max(axis=1)      # (as above)
+    assert np.all(err <= 2e-5 * np.linalg.norm(ref, axis=1) + 1e-5 * np.abs(ref).max()), float(err.max())
+
+
 @pytest.mark.parametrize("heads,dh,pad", [(4, 16, 0), (8, 4, 0), (1, 64, 0), (4, 16, 4), (2, 6, 0)])
 @pytest.mark.parametrize("level", [4000.0, -4000.0])
 def test_weights_of_large_scores(heads, dh, pad, level):
