@@ -249,93 +249,97 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
     const uint32_t tmem_acc = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
-            int64_t it = 0;                       // k-blocks issued so far, over all tiles
-            bool ok = true;
-            for (int32_t t = tile_first; t < n_tiles && ok; t += tile_stride) {
-                const int32_t z = t / per_split, rem = t % per_split;
-                const int32_t m0 = (int32_t)((rem % n_m) * kTileRows + pair_rank * kTcBM), n0 = (int32_t)((rem / n_m) * BN);
-                const int32_t kb0 = z * g.k_blocks_per_split;
-                const int32_t kb1 = min(g.k_blocks_total, kb0 + g.k_blocks_per_split);
-                for (int32_t kb = kb0; kb < kb1; ++kb, ++it) {
-                    const int s = (int)(it % STAGES);
-                    const uint32_t ph = (uint32_t)(it / STAGES) & 1;
-                    if (!mbar_wait(empty + s, ph ^ 1, g.status, abort_flag)) { ok = false; break; }
-                    uint8_t* a_dst = tiles + s * kStageBytes;
-                    if constexpr (PAIR) {
-                        // the even block's barrier counts the bytes of both blocks' loads
-                        if (pair_rank == 0) mbar_expect_tx(full + s, 2 * kStageBytes);
-                        tma_load_2d_pair(a_dst, &map_a, kb * kTcBK, m0, full + s);
-                        tma_load_2d_pair(a_dst + kABytes, &map_b, kb * kTcBK, n0 + (int32_t)pair_rank * (BN / 2), full + s);
-                        continue;
-                    }
-                    mbar_expect_tx(full + s, kStageBytes);
-                    if constexpr (kMnMajor) {
-                        // operands stored [reduction index][M or N]: boxes of 64 reduction rows x 64 elements
+        const bool leader = elect_one();
+        RingPos r;
+        int issued = 0;                       // k-blocks issued so far, over all tiles
+        bool ok = true;
+        for (int32_t t = tile_first; t < n_tiles && ok; t += tile_stride) {
+            const int32_t z = t / per_split, rem = t % per_split;
+            const int32_t m0 = (int32_t)((rem % n_m) * kTileRows + pair_rank * kTcBM), n0 = (int32_t)((rem / n_m) * BN);
+            const int32_t kb0 = z * g.k_blocks_per_split;
+            const int32_t kb1 = min(g.k_blocks_total, kb0 + g.k_blocks_per_split);
+            for (int32_t kb = kb0; kb < kb1; ++kb, ++issued, r.next(STAGES)) {
+                uint64_t* bar = full + r.s;
+                if (!mbar_wait_warp(empty + r.s, r.ph ^ 1, g.status, abort_flag)) { ok = false; break; }
+                uint8_t* a_dst = tiles + r.s * kStageBytes;
+                if (!leader) continue;
+                if constexpr (PAIR) {
+                    // the even block's barrier counts the bytes of both blocks' loads
+                    if (pair_rank == 0) mbar_expect_tx(bar, 2 * kStageBytes);
+                    tma_load_2d_pair(a_dst, &map_a, kb * kTcBK, m0, bar);
+                    tma_load_2d_pair(a_dst + kABytes, &map_b, kb * kTcBK, n0 + (int32_t)pair_rank * (BN / 2), bar);
+                } else if constexpr (kMnMajor) {
+                    mbar_expect_tx(bar, kStageBytes);
+                    // operands stored [reduction index][M or N]: boxes of 64 reduction rows x 64 elements
 #pragma unroll
-                        for (int i = 0; i < kTcBM / 64; ++i)
-                            tma_load_2d(a_dst + i * kMnBoxBytes, &map_a, m0 + 64 * i, kb * kTcBK, full + s);
+                    for (int i = 0; i < kTcBM / 64; ++i)
+                        tma_load_2d(a_dst + i * kMnBoxBytes, &map_a, m0 + 64 * i, kb * kTcBK, bar);
 #pragma unroll
-                        for (int i = 0; i < BN / 64; ++i)
-                            tma_load_2d(a_dst + kABytes + i * kMnBoxBytes, &map_b, n0 + 64 * i, kb * kTcBK, full + s);
-                    } else {
-                        tma_load_2d(a_dst, &map_a, kb * kTcBK, m0, full + s);
-                        tma_load_2d(a_dst + kABytes, &map_b, kb * kTcBK, n0, full + s);
-                    }
-                }
-            }
-            if (*abort_flag && !(PAIR && pair_rank != 0)) {    // await (bounded) what was issued and not consumed, so nothing lands after exit
-                for (int64_t i = it > STAGES ? it - STAGES : 0; i < it; ++i) {
-                    const int s = (int)(i % STAGES);
-                    const uint32_t ph = (uint32_t)(i / STAGES) & 1;
-                    for (uint32_t w = 0; w < (1u << 20); ++w) if (mbar_try_wait(full + s, ph)) break;
+                    for (int i = 0; i < BN / 64; ++i)
+                        tma_load_2d(a_dst + kABytes + i * kMnBoxBytes, &map_b, n0 + 64 * i, kb * kTcBK, bar);
+                } else {
+                    mbar_expect_tx(bar, kStageBytes);
+                    tma_load_2d(a_dst, &map_a, kb * kTcBK, m0, bar);
+                    tma_load_2d(a_dst + kABytes, &map_b, kb * kTcBK, n0, bar);
                 }
             }
         }
+        if (*abort_flag && !(PAIR && pair_rank != 0)) {    // await (bounded) what was issued and not consumed, so nothing lands after exit
+            for (int i = issued > STAGES ? issued - STAGES : 0; i < issued; ++i)
+                for (uint32_t w = 0; w < (1u << 20); ++w) if (mbar_try_wait(full + i % STAGES, (uint32_t)(i / STAGES) & 1)) break;
+        }
     } else if (warp == 1) {
-        if (lane == 0 && pair_rank == 0) {        // (of a pair, the even block issues the MMAs for both)
+        if (pair_rank == 0) {        // (of a pair, the even block issues the MMAs for both)
+            const bool leader = elect_one();
             constexpr uint32_t idesc = make_idesc(BN, kMnMajor, kMnMajor, kTileRows);
-            int64_t it = 0, lt = 0;               // k-blocks consumed, tiles done by this block
-            bool ok = true;
+            const uint32_t tiles_addr = smem_u32(tiles);
+            RingPos r;
+            int lt = 0;               // tiles done by this block
+            bool ok = true, ready = false;      // ready: the stage at r has been seen full
             for (int32_t t = tile_first; t < n_tiles && ok; t += tile_stride, ++lt) {
                 const int32_t z = t / per_split;
                 const int32_t kb0 = z * g.k_blocks_per_split;
                 const int32_t kb1 = min(g.k_blocks_total, kb0 + g.k_blocks_per_split);
-                const int b = (int)(lt % NACC);
+                const int b = lt % NACC;
                 const uint32_t pb = (uint32_t)(lt / NACC) & 1;
-                ok = mbar_wait(acc_empty + b, pb ^ 1, g.status, abort_flag);      // drained by the epilogue
+                ok = mbar_wait_warp(acc_empty + b, pb ^ 1, g.status, abort_flag);      // drained by the epilogue
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t acc_addr = tmem_acc + (uint32_t)(b * BN);
-                for (int32_t kb = kb0; kb < kb1; ++kb, ++it) {
-                    const int s = (int)(it % STAGES);
-                    const uint32_t ph = (uint32_t)(it / STAGES) & 1;
-                    ok = mbar_wait(full + s, ph, g.status, abort_flag);
+                for (int32_t kb = kb0; kb < kb1; ++kb) {
+                    if (!ready) ok = mbar_wait_warp(full + r.s, r.ph, g.status, abort_flag);
                     if (!ok) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t a_addr = smem_u32(tiles + s * kStageBytes);
-                    if constexpr (kMnMajor) {
-                        const uint64_t adesc = make_smem_desc_mn(a_addr, kMnBoxBytes);
-                        const uint64_t bdesc = make_smem_desc_mn(a_addr + kABytes, kMnBoxBytes);
+                    const uint32_t a_addr = tiles_addr + (uint32_t)r.s * kStageBytes;
+                    uint64_t* const used = empty + r.s;
+                    r.next(STAGES);
+                    const bool next_ready = mbar_test(full + r.s, r.ph);
+                    if (leader) {
+                        if constexpr (kMnMajor) {
+                            const uint64_t adesc = make_smem_desc_mn(a_addr, kMnBoxBytes);
+                            const uint64_t bdesc = make_smem_desc_mn(a_addr + kABytes, kMnBoxBytes);
 #pragma unroll
-                        for (int k = 0; k < kTcBK / 16; ++k)      // 16 reduction rows = two 1024-byte atoms: +128 in 16-byte units
-                            umma_bf16(acc_addr, adesc + 128 * k, bdesc + 128 * k, idesc, (kb > kb0 || k > 0) ? 1u : 0u);
-                    } else if constexpr (PAIR) {
-                        // one MMA over both blocks' shared memory (same offsets in either) and tensor memory
-                        const uint64_t adesc = make_smem_desc(a_addr), bdesc = make_smem_desc(a_addr + kABytes);
+                            for (int k = 0; k < kTcBK / 16; ++k)      // 16 reduction rows = two 1024-byte atoms: +128 in 16-byte units
+                                umma_bf16(acc_addr, adesc + 128 * k, bdesc + 128 * k, idesc, (kb > kb0 || k > 0) ? 1u : 0u);
+                            umma_commit(used);              // frees the stage once these MMAs have read it
+                        } else if constexpr (PAIR) {
+                            // one MMA over both blocks' shared memory (same offsets in either) and tensor memory
+                            const uint64_t adesc = make_smem_desc(a_addr), bdesc = make_smem_desc(a_addr + kABytes);
 #pragma unroll
-                        for (int k = 0; k < kTcBK / 16; ++k)
-                            umma_bf16_pair(acc_addr, adesc + 2 * k, bdesc + 2 * k, idesc, (kb > kb0 || k > 0) ? 1u : 0u);
-                    } else {
-                        const uint64_t adesc = make_smem_desc(a_addr), bdesc = make_smem_desc(a_addr + kABytes);
+                            for (int k = 0; k < kTcBK / 16; ++k)
+                                umma_bf16_pair(acc_addr, adesc + 2 * k, bdesc + 2 * k, idesc, (kb > kb0 || k > 0) ? 1u : 0u);
+                            umma_commit_pair(used);         // frees the stage in both blocks
+                        } else {
+                            const uint64_t adesc = make_smem_desc(a_addr), bdesc = make_smem_desc(a_addr + kABytes);
 #pragma unroll
-                        for (int k = 0; k < kTcBK / 16; ++k)      // 16 bf16 = 32 bytes per MMA along K: +2 in 16-byte units
-                            umma_bf16(acc_addr, adesc + 2 * k, bdesc + 2 * k, idesc, (kb > kb0 || k > 0) ? 1u : 0u);
+                            for (int k = 0; k < kTcBK / 16; ++k)      // 16 bf16 = 32 bytes per MMA along K: +2 in 16-byte units
+                                umma_bf16(acc_addr, adesc + 2 * k, bdesc + 2 * k, idesc, (kb > kb0 || k > 0) ? 1u : 0u);
+                            umma_commit(used);
+                        }
                     }
-                    if constexpr (PAIR) umma_commit_pair(empty + s);      // frees the stage in both blocks
-                    else umma_commit(empty + s);              // frees the stage once these MMAs have read it
+                    ready = __all_sync(0xffffffffu, next_ready);
                 }
-                if (ok) {                                     // accumulator complete (at once for an empty K range)
+                if (ok && leader) {                                     // accumulator complete (at once for an empty K range)
                     if constexpr (PAIR) umma_commit_pair(acc_full + b);
                     else umma_commit(acc_full + b);
                 }

@@ -85,72 +85,79 @@ grad_kernel(const __grid_constant__ CUtensorMap map_a0, const __grid_constant__ 
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
-            int it = 0;
-            bool ok = true;
-            for (int t = blockIdx.x; t < g.n_tiles && ok; t += gridDim.x) {
-                const GradTile tile = grad_tile(g, t);
-                const GradDims& d = g.p[tile.which];
-                const CUtensorMap* ma = tile.which ? &map_a1 : &map_a0;
-                const CUtensorMap* mb = tile.which ? &map_b1 : &map_b0;
-                const int m0 = tile.m * 128, n0 = tile.n * d.bn;
-                const int na = d.M - m0 > 64 ? 2 : 1, nb = min(d.bn / 64, (d.N - n0 + 63) / 64);      // boxes that hold anything
-                const int kb0 = tile.z * d.kb_per_split, kb1 = min(g.kb_total, kb0 + d.kb_per_split);
-                const uint32_t bytes = (uint32_t)(na + nb) * kGradBoxBytes;
-                for (int kb = kb0; kb < kb1; ++kb, ++it) {
-                    const int s = it % STAGES;
-                    if (!mbar_wait(empty + s, ((uint32_t)(it / STAGES) & 1) ^ 1, g.status, abort_flag)) { ok = false; break; }
-                    uint8_t* dst = tiles + s * kStageBytes;
-                    mbar_expect_tx(full + s, bytes);
-                    tma_load_2d(dst, ma, m0, kb * kTcBK, full + s);
-                    if (na > 1) tma_load_2d(dst + kGradBoxBytes, ma, m0 + 64, kb * kTcBK, full + s);
+        const bool leader = elect_one();
+        RingPos r;
+        int issued = 0;
+        bool ok = true;
+        for (int t = blockIdx.x; t < g.n_tiles && ok; t += gridDim.x) {
+            const GradTile tile = grad_tile(g, t);
+            const GradDims& d = g.p[tile.which];
+            const CUtensorMap* ma = tile.which ? &map_a1 : &map_a0;
+            const CUtensorMap* mb = tile.which ? &map_b1 : &map_b0;
+            const int m0 = tile.m * 128, n0 = tile.n * d.bn;
+            const int na = d.M - m0 > 64 ? 2 : 1, nb = min(d.bn / 64, (d.N - n0 + 63) / 64);      // boxes that hold anything
+            const int kb0 = tile.z * d.kb_per_split, kb1 = min(g.kb_total, kb0 + d.kb_per_split);
+            const uint32_t bytes = (uint32_t)(na + nb) * kGradBoxBytes;
+            for (int kb = kb0; kb < kb1; ++kb, ++issued, r.next(STAGES)) {
+                uint64_t* bar = full + r.s;
+                if (!mbar_wait_warp(empty + r.s, r.ph ^ 1, g.status, abort_flag)) { ok = false; break; }
+                uint8_t* dst = tiles + r.s * kStageBytes;
+                if (!leader) continue;
+                mbar_expect_tx(bar, bytes);
+                tma_load_2d(dst, ma, m0, kb * kTcBK, bar);
+                if (na > 1) tma_load_2d(dst + kGradBoxBytes, ma, m0 + 64, kb * kTcBK, bar);
 #pragma unroll
-                    for (int i = 0; i < BN / 64; ++i)
-                        if (i < nb) tma_load_2d(dst + kABytes + i * kGradBoxBytes, mb, n0 + 64 * i, kb * kTcBK, full + s);
-                }
-            }
-            if (*abort_flag) {      // await (bounded) what was issued and not consumed, so that nothing lands after the block has left
-                for (int i = it > STAGES ? it - STAGES : 0; i < it; ++i)
-                    for (uint32_t w = 0; w < (1u << 20); ++w) if (mbar_try_wait(full + i % STAGES, (uint32_t)(i / STAGES) & 1)) break;
+                for (int i = 0; i < BN / 64; ++i)
+                    if (i < nb) tma_load_2d(dst + kABytes + i * kGradBoxBytes, mb, n0 + 64 * i, kb * kTcBK, bar);
             }
         }
+        if (*abort_flag) {      // await (bounded) what was issued and not consumed, so that nothing lands after the block has left
+            for (int i = issued > STAGES ? issued - STAGES : 0; i < issued; ++i)
+                for (uint32_t w = 0; w < (1u << 20); ++w) if (mbar_try_wait(full + i % STAGES, (uint32_t)(i / STAGES) & 1)) break;
+        }
     } else if (warp == 1) {
-        if (lane == 0) {
-            const uint64_t ones_desc = make_smem_desc_mn(smem_u32(ones), 0);      // (both halves of M read the same 64 ones)
-            int it = 0, lt = 0;
-            bool ok = true;
-            for (int t = blockIdx.x; t < g.n_tiles && ok; t += gridDim.x, ++lt) {
-                const GradTile tile = grad_tile(g, t);
-                const GradDims& d = g.p[tile.which];
-                const int kb0 = tile.z * d.kb_per_split, kb1 = min(g.kb_total, kb0 + d.kb_per_split);
-                const uint32_t idesc = make_idesc(d.bn, true, true);
-                ok = mbar_wait(acc_empty, ((uint32_t)lt & 1) ^ 1, g.status, abort_flag);
+        const bool leader = elect_one();
+        const uint64_t ones_desc = make_smem_desc_mn(smem_u32(ones), 0);      // (both halves of M read the same 64 ones)
+        const uint32_t tiles_addr = smem_u32(tiles);
+        RingPos r;
+        int lt = 0;
+        bool ok = true, ready = false;      // ready: the stage at r has been seen full
+        for (int t = blockIdx.x; t < g.n_tiles && ok; t += gridDim.x, ++lt) {
+            const GradTile tile = grad_tile(g, t);
+            const GradDims& d = g.p[tile.which];
+            const int kb0 = tile.z * d.kb_per_split, kb1 = min(g.kb_total, kb0 + d.kb_per_split);
+            const uint32_t idesc = make_idesc(d.bn, true, true);
+            ok = mbar_wait_warp(acc_empty, ((uint32_t)lt & 1) ^ 1, g.status, abort_flag);
+            if (!ok) break;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            bool bias_begun = false;
+            const int shares = d.bias_shares;
+            int next_share = kb0 + (tile.m - kb0 % shares + shares) % shares;
+            for (int kb = kb0; kb < kb1; ++kb) {
+                if (!ready) ok = mbar_wait_warp(full + r.s, r.ph, g.status, abort_flag);
                 if (!ok) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                bool bias_begun = false;
-                const int shares = d.bias_shares;
-                int next_share = kb0 + (tile.m - kb0 % shares + shares) % shares;
-                for (int kb = kb0; kb < kb1; ++kb, ++it) {
-                    const int s = it % STAGES;
-                    ok = mbar_wait(full + s, (uint32_t)(it / STAGES) & 1, g.status, abort_flag);
-                    if (!ok) break;
-                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                    const uint32_t a_addr = smem_u32(tiles + s * kStageBytes);
-                    const uint64_t adesc = make_smem_desc_mn(a_addr, kGradBoxBytes), bdesc = make_smem_desc_mn(a_addr + kABytes, kGradBoxBytes);
+                const uint32_t a_addr = tiles_addr + (uint32_t)r.s * kStageBytes;
+                const uint64_t adesc = make_smem_desc_mn(a_addr, kGradBoxBytes), bdesc = make_smem_desc_mn(a_addr + kABytes, kGradBoxBytes);
+                uint64_t* const used = empty + r.s;
+                r.next(STAGES);
+                const bool next_ready = mbar_test(full + r.s, r.ph);
+                const bool share = kb == next_share;      // (the first step this block takes clears its row)
+                if (leader) {
 #pragma unroll
                     for (int k = 0; k < kTcBK / 16; ++k)      // 16 reduction rows = two 1024-byte atoms: +128 in 16-byte units
                         umma_bf16(tmem, adesc + 128 * k, bdesc + 128 * k, idesc, (kb > kb0 || k > 0) ? 1u : 0u);
-                    if (kb == next_share) {      // (the first step this block takes clears its row)
-                        next_share += shares;
+                    if (share) {
 #pragma unroll
                         for (int k = 0; k < kTcBK / 16; ++k)
                             umma_bf16(tmem + BN, ones_desc, bdesc + 128 * k, idesc, (bias_begun || k > 0) ? 1u : 0u);
-                        bias_begun = true;
                     }
-                    umma_commit(empty + s);
+                    umma_commit(used);
                 }
-                if (ok) umma_commit(acc_full);
+                ready = __all_sync(0xffffffffu, next_ready);
+                if (share) { next_share += shares; bias_begun = true; }
             }
+            if (ok && leader) umma_commit(acc_full);
         }
     } else {
         const int q = warp & 3, ew = warp - 2, half = ew >> 2;

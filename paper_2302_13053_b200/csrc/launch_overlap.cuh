@@ -6,8 +6,8 @@
 //    everything before its direct predecessor has finished: the predecessor's blocks have all seen that from their own wait.
 //  - Before the wait a kernel may read only what no direct predecessor writes, at any of its launch sites: between the kernel that wrote
 //    it and the one that reads it early at least one whole kernel lies in the stream.  It writes nothing before the wait.  Early reads
-//    are made by head_backward_kernel and reduce_update_kernel; their launches name the kernels in between, and whoever fuses or moves
-//    one of those has to look at these reads again.
+//    are made by head_backward_kernel, reduce_update_kernel and the kernels of mlp_small.cu; their launches name the kernels in between, and
+//    whoever fuses or moves one of those has to look at these reads again.
 #pragma once
 #include <cuda_runtime.h>
 

@@ -17,6 +17,7 @@
 #include "batch_norm.h"
 #include "layer_norm.h"
 #include "mlp_kernels.cuh"
+#include "mlp_small.h"
 #include "mlp_plan.h"
 
 using namespace retexo;
@@ -270,7 +271,19 @@ int mlp_train_step_launch(const MlpPlan& p, const MlpBuffers& b, const retexo_ml
     const float* ln_gamma = theta + retexo_theta_size(d_in, H, O);      // (normalisation) [gamma | beta (| r_mean | r_var)] end theta
     const BnScratch bns{b.bn_partial, b.bn_batch, b.bn_sums};
     if (bn && n < 2) return RETEXO_ERR_INVALID_ARG;                     // (the unbiased variance of the running statistics)
-    if (H > 0) {
+    const bool small = !ln && !bn && !dropping && small_step_supported(d_in, H, O, n, n_all);      // two kernels do (mlp_small.cu)
+    if (small) {
+        SmallForward sf{};
+        sf.x = x; sf.ldx = ldx; sf.w1t = b.w1t16; sf.ld_w1t = p.ld_k; sf.b1 = b1; sf.w2t = b.w2t16; sf.ld_w2t = p.ld_h; sf.b2 = b2;
+        sf.d_in = d_in; sf.hidden = H; sf.n_classes = O; sf.n_train = n; sf.n_all = n_all;
+        sf.y = y; sf.y_eval = tail ? tail->y_eval : nullptr; sf.inv_rows = 1.0f / (float)n;
+        sf.hd = b.hd16; sf.ld_hd = p.ld_h; sf.dl = b.dl16; sf.ld_dl = p.ld_dl; sf.dhd = b.dhd16; sf.ld_dhd = p.ld_h;
+        sf.loss_partial = b.loss_partial; sf.correct = tail ? tail->correct : nullptr; sf.status = b.status;
+        sf.x_early = dx_out == nullptr;      // (who trains what produced X has just written it; else the kernel before is an update or a conversion)
+        RETEXO_TRY(small_forward_launch(sf, st));
+        n_loss = (n_all + 31) / 32;
+        if (H > 0) { grad1 = b.dhd16; ld_grad1 = p.ld_h; }
+    } else if (H > 0) {
         if (ln || bn) {
             // the product leaves z = X W1 + b1 in fp32; the normalisation's kernel applies the ReLU and
             // writes Hd and the gate bits as the plain forward epilogue would
@@ -354,7 +367,7 @@ int mlp_train_step_launch(const MlpPlan& p, const MlpBuffers& b, const retexo_ml
     // ---- [dW1 ; db1] = [X | 1]^T grad1,  [dW2 ; db2] = [Hd | 1]^T dL
     GradProduct prod[2] = {{x, ldx, grad1, ld_grad1, d_in, out1, (int32_t)p.split_w1, b.pw1, b.pb1},
                            {b.hd16, p.ld_h, b.dl16, p.ld_dl, H, O, (int32_t)p.split_w2, b.pw2, b.pb2}};
-    RETEXO_TRY(grad_launch(prod, H > 0 ? 2 : 1, n, b.status, st));
+    if (!small) RETEXO_TRY(grad_launch(prod, H > 0 ? 2 : 1, n, b.status, st));      // (of a small batch: with the update)
 
     // ---- reduce the partials and update
     UpdateArgs u{};
@@ -374,7 +387,7 @@ int mlp_train_step_launch(const MlpPlan& p, const MlpBuffers& b, const retexo_ml
     u.corr2 = (float)(1.0 - pow((double)model->beta2, t));
     u.loss_partial = b.loss_partial; u.n_loss = n_loss;      // the partials this launch's loss kernel wrote
     u.inv_rows = 1.0f / (float)n; u.loss_out = loss_out;
-    u.status = b.status;
+    u.status = b.status; u.status_word = b.status;
     u.ld_k = p.ld_k; u.ld_o1 = p.ld_o1; u.ld_h = p.ld_h; u.ld_dl = p.ld_dl;
     if (keep_shadows) {
         u.w1t16 = b.w1t16; u.w1r16 = w1_rows ? b.w1r16 : nullptr;
@@ -393,6 +406,10 @@ int mlp_train_step_launch(const MlpPlan& p, const MlpBuffers& b, const retexo_ml
     const int64_t tiles = (((int64_t)d_in + 16) / 16) * ((out1 + 15) / 16) + (H > 0 ? (((int64_t)H + 16) / 16) * ((O + 15) / 16) : 0) +
                           ((ln || bn) ? ((int64_t)H + 15) / 16 : 0);      // (a normalisation's segment has 2 or 4 rows of hidden entries)
     u.status_out = model->status_out;
+    if (small) {
+        const SmallGrad sg{x, ldx, grad1, ld_grad1, b.hd16, p.ld_h, b.dl16, p.ld_dl, n, true};
+        return small_update_launch(sg, u, st);
+    }
     // (reads parameters, moments, iteration state and the validation count early: between the update, or the head's kernel that counted,
     // and this lies the kernel of the weight gradients)
     OverlapLaunch ol(dim3((unsigned)tiles), dim3(256), 0, st);

@@ -16,6 +16,7 @@
 // Every wait is bounded: one that runs out sets *status and the block tears down in order.
 #include <string.h>
 
+#include "class_loss.cuh"
 #include "gemm_tc.h"
 #include "tc_common.cuh"
 
@@ -27,12 +28,6 @@ constexpr uint32_t kHbPanelBytes = 128 * 128;       // [128 rows x 64 bf16], 128
 constexpr uint32_t kHbW2PanelBytes = 64 * 128;      // [64 classes x 64 hidden units]
 constexpr uint32_t kHbSlabBytes = 32 * 128;         // one warp's 32 rows of a panel
 constexpr uint32_t kHbLogitCols = 64, kHbGradCol0 = 256;
-
-__device__ __forceinline__ float fast_exp2(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 
 struct HbArgs {
     int64_t n_all, n_train;
@@ -132,21 +127,23 @@ head_backward_kernel(const __grid_constant__ CUtensorMap map_hd, const __grid_co
             }
         }
     } else if (warp == 1) {
-        if (lane == 0 && nt > 0) {
+        if (nt > 0) {
+            const bool leader = elect_one();
             const uint32_t idesc_logits = make_idesc((int)kHbLogitCols);
             const uint32_t idesc_grad = make_idesc(64 * np, false, true);
             const uint32_t w2_addr = smem_u32(w2_s);
             const uint64_t w2_desc = make_smem_desc(w2_addr), w2_desc_mn = make_smem_desc_mn(w2_addr, kHbW2PanelBytes);
-            bool ok = mbar_wait(bars + HB_W2_FULL, 0, g.status, abort_flag);
+            bool ok = mbar_wait_warp(bars + HB_W2_FULL, 0, g.status, abort_flag);
             // logits of tile i: A = the Hd tile (K-major panels), B = W2^T (K-major panels), K = hidden units
             auto issue_logits = [&](int64_t i) -> bool {
                 const int b = (int)(i & 1);
                 const uint32_t u = (uint32_t)(i >> 1) & 1;
-                if (!mbar_wait(bars + HB_HD_FULL + b, u, g.status, abort_flag)) return false;
-                if (!mbar_wait(bars + HB_D1_EMPTY + b, u ^ 1, g.status, abort_flag)) return false;
+                if (!mbar_wait_warp(bars + HB_HD_FULL + b, u, g.status, abort_flag)) return false;
+                if (!mbar_wait_warp(bars + HB_D1_EMPTY + b, u ^ 1, g.status, abort_flag)) return false;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 // (descriptor arithmetic in 16-byte units: a panel further on, or 32 bytes = 16 hidden units along K)
                 const uint64_t adesc = make_smem_desc(smem_u32(hd_buf + b * hd_bytes));
+                if (!leader) return true;
 #pragma unroll
                 for (int p = 0; p < 4; ++p) {
                     if (p < np) {
@@ -165,36 +162,32 @@ head_backward_kernel(const __grid_constant__ CUtensorMap map_hd, const __grid_co
                 // The logits of tile i + 1 go first only if their Hd tile has already arrived: waiting for it
                 // here would hold the gradient product of tile i (whose inputs may be ready) behind a load.
                 bool next_issued = i + 1 >= nt;
-                if (!next_issued && mbar_try_wait(bars + HB_HD_FULL + ((i + 1) & 1), (uint32_t)((i + 1) >> 1) & 1) &&
-                    mbar_try_wait(bars + HB_D1_EMPTY + ((i + 1) & 1), ((uint32_t)((i + 1) >> 1) & 1) ^ 1)) {
+                if (!next_issued &&
+                    __all_sync(0xffffffffu, mbar_try_wait(bars + HB_HD_FULL + ((i + 1) & 1), (uint32_t)((i + 1) >> 1) & 1) &&
+                                                mbar_try_wait(bars + HB_D1_EMPTY + ((i + 1) & 1), ((uint32_t)((i + 1) >> 1) & 1) ^ 1))) {
                     ok = issue_logits(i + 1);
                     if (!ok) break;
                     next_issued = true;
                 }
-                if (!mbar_wait(bars + HB_DL_FULL, (uint32_t)(i & 1), g.status, abort_flag)) break;
-                if (!mbar_wait(bars + HB_D2_EMPTY, (uint32_t)(i & 1) ^ 1, g.status, abort_flag)) break;
+                if (!mbar_wait_warp(bars + HB_DL_FULL, (uint32_t)(i & 1), g.status, abort_flag)) break;
+                if (!mbar_wait_warp(bars + HB_D2_EMPTY, (uint32_t)(i & 1) ^ 1, g.status, abort_flag)) break;
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 // dHd of tile i: A = the dL tile (K-major, K = classes), B = the same W2^T panels read MN-major
                 const uint64_t dl_desc = make_smem_desc(smem_u32(dl_buf));
+                if (leader) {
 #pragma unroll
-                for (int j = 0; j < 4; ++j)      // 16 classes along K: 32 bytes of a dL line, two 1024-byte atoms of W2^T
-                    umma_bf16(tmem + kHbGradCol0, dl_desc + (uint64_t)(2 * j), w2_desc_mn + (uint64_t)(128 * j), idesc_grad, j ? 1u : 0u);
-                umma_commit(bars + HB_D2_FULL);
-                umma_commit(bars + HB_DL_EMPTY);
+                    for (int j = 0; j < 4; ++j)      // 16 classes along K: 32 bytes of a dL line, two 1024-byte atoms of W2^T
+                        umma_bf16(tmem + kHbGradCol0, dl_desc + (uint64_t)(2 * j), w2_desc_mn + (uint64_t)(128 * j), idesc_grad, j ? 1u : 0u);
+                    umma_commit(bars + HB_D2_FULL);
+                    umma_commit(bars + HB_DL_EMPTY);
+                }
                 if (!next_issued) ok = issue_logits(i + 1);
             }
         }
     } else if (warp < kHbGateWarp0) {
-        // ---- loss role: two threads share a row of logits, in two warps of the same tensor-memory lane quarter
-        // (warp w and w + 4): the classes are cut into groups of eight, the first half of the groups goes to
-        // the one, the rest to the other; row maximum, sum and the label's logit are exchanged through shared
-        // memory.  Every reduction is a tree, so that a warp finds independent instructions to issue.
+        // ---- loss role: two threads share a row of logits, in warps w and w + 4 (class_loss.cuh)
         const int q = warp & 3, part = (warp - kHbLossWarp0) >> 2;
-        const int ng = (g.O + 7) >> 3, g_split = (ng + 1) >> 1;
-        const int g_first = part ? g_split : 0, g_count = part ? ng - g_split : g_split;      // this thread's groups (<= 4)
-        const int pair_bar = 1 + q;                                                            // named barrier of the two warps
-        float* x_max = xch + (q * 2) * 32, *x_sum = xch + (8 + q * 2) * 32, *x_ly = xch + (16 + q * 2) * 32;
-        int* x_best = reinterpret_cast<int*>(xch + (24 + q * 2) * 32);
+        ClassLoss cl(g.O, part, q, lane, xch, 1 + q);
         for (int64_t i = 0; i < nt; ++i) {
             const int b = (int)(i & 1);
             const uint32_t u = (uint32_t)(i >> 1) & 1;
@@ -205,116 +198,25 @@ head_backward_kernel(const __grid_constant__ CUtensorMap map_hd, const __grid_co
             const int32_t label = train ? g.y[row] : (eval ? g.y_eval[row - g.n_train] : -1);
             if (!mbar_wait(bars + HB_D1_FULL + b, u, g.status, abort_flag)) break;
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            float v[32];
-            {
-                uint32_t r[32];
-                tmem_ld_issue(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)b * kHbLogitCols + (uint32_t)(8 * g_first), r);
-                tmem_ld_wait(r);
-#pragma unroll
-                for (int gi = 0; gi < 4; ++gi) {
-                    if (gi < g_count) {
-                        const int c0 = 8 * (g_first + gi);
-                        const float4 b0 = *reinterpret_cast<const float4*>(bias_s + c0);
-                        const float4 b1 = *reinterpret_cast<const float4*>(bias_s + c0 + 4);
-                        const float bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-#pragma unroll
-                        for (int k = 0; k < 8; ++k)
-                            v[8 * gi + k] = c0 + k < g.O ? __uint_as_float(r[8 * gi + k]) + bb[k] : -INFINITY;
-                    }
-                }
-            }
+            cl.load(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)b * kHbLogitCols, bias_s);
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
             if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bars + HB_D1_EMPTY + b)) : "memory");
-            float mx = -INFINITY;
-#pragma unroll
-            for (int gi = 0; gi < 4; ++gi) {
-                if (gi < g_count) {
-                    const float m01 = fmaxf(v[8 * gi], v[8 * gi + 1]), m23 = fmaxf(v[8 * gi + 2], v[8 * gi + 3]);
-                    const float m45 = fmaxf(v[8 * gi + 4], v[8 * gi + 5]), m67 = fmaxf(v[8 * gi + 6], v[8 * gi + 7]);
-                    mx = fmaxf(mx, fmaxf(fmaxf(m01, m23), fmaxf(m45, m67)));
-                }
-            }
-            const bool has_eval = g.correct && row0 + 32 > g.n_train;      // evaluated rows among this warp's
-            if (has_eval) {      // arg-max: the lowest index that reaches this thread's maximum
-                int best = 0;
-#pragma unroll
-                for (int gi = 3; gi >= 0; --gi) {
-                    if (gi < g_count) {
-#pragma unroll
-                        for (int k = 7; k >= 0; --k) best = v[8 * gi + k] == mx ? 8 * (g_first + gi) + k : best;
-                    }
-                }
-                x_best[part * 32 + lane] = best;
-            }
-            x_max[part * 32 + lane] = mx;
-            asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
-            const float m0 = x_max[lane], m1 = x_max[32 + lane];
-            mx = fmaxf(m0, m1);
-            if (has_eval && part == 0) {      // the lower classes win ties
-                const int arg = m1 > m0 ? x_best[32 + lane] : x_best[lane];
-                const unsigned hits = __ballot_sync(0xffffffffu, eval && arg == label);
-                if (lane == 0 && hits) atomicAdd(g.correct, (unsigned long long)__popc(hits));
-            }
-            // exp(v - mx) as one multiply-add and one exponential per column; the label's logit is picked up on the way
-            const float kLog2e = 1.4426950408889634f;
-            const float shift = -mx * kLog2e;
-            float den = 0.f, ly = 0.f;
-#pragma unroll
-            for (int gi = 0; gi < 4; ++gi) {
-                if (gi < g_count) {
-                    float e[8];
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        ly = 8 * (g_first + gi) + k == label ? v[8 * gi + k] : ly;
-                        e[k] = fast_exp2(fmaf(v[8 * gi + k], kLog2e, shift));      // columns beyond the last class hold -inf: 0
-                        v[8 * gi + k] = e[k];
-                    }
-                    den += ((e[0] + e[1]) + (e[2] + e[3])) + ((e[4] + e[5]) + (e[6] + e[7]));
-                }
-            }
-            x_sum[part * 32 + lane] = den;
-            x_ly[part * 32 + lane] = ly;
-            asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
-            den = x_sum[lane] + x_sum[32 + lane];
-            ly = x_ly[lane] + x_ly[32 + lane];
-            const float scale = train ? g.inv_rows / den : 0.f;
-            const float hot = train ? g.inv_rows : 0.f;
+            cl.reduce(label, eval, g.correct && row0 + 32 > g.n_train, g.correct);
             // the dL tile of the previous tile has been read by its MMA and by its store
             if (!mbar_wait(bars + HB_DL_EMPTY, (uint32_t)(i & 1) ^ 1, g.status, abort_flag)) break;
             if (part == 0 && lane == 0) bulk_wait_read_all();
-            asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
+            cl.pair_sync();
             uint8_t* slab = dl_buf + q * kHbSlabBytes;
-#pragma unroll
-            for (int gi = 0; gi < 4; ++gi) {      // one 16-byte piece of the row's line per group of eight classes
-                const int piece = part ? g_split + gi : gi;      // part 1 also clears the pieces beyond the last class
-                if (piece < 8 && (part || gi < g_split)) {
-                    uint32_t pk[4] = {0u, 0u, 0u, 0u};
-                    if (gi < g_count) {
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const int c = 8 * piece + 2 * k;
-                            const float lo = fmaf(v[8 * gi + 2 * k], scale, c == label ? -hot : 0.f);
-                            const float hi = fmaf(v[8 * gi + 2 * k + 1], scale, c + 1 == label ? -hot : 0.f);
-                            __nv_bfloat162 b2 = __floats2bfloat162_rn(lo, hi);
-                            pk[k] = *reinterpret_cast<uint32_t*>(&b2);
-                        }
-                    }
-                    *reinterpret_cast<uint4*>(slab + lane * 128 + ((piece ^ (lane & 7)) * 16)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-                }
-            }
-            if (part == 1) {      // pieces that neither thread's four groups reach (few classes): zeros
-                for (int piece = g_split + 4; piece < 8; ++piece)
-                    *reinterpret_cast<uint4*>(slab + lane * 128 + ((piece ^ (lane & 7)) * 16)) = make_uint4(0u, 0u, 0u, 0u);
-            }
+            cl.store_dl(label, train, g.inv_rows, slab + lane * 128);
             fence_proxy_async_smem();
-            asm volatile("bar.sync %0, 64;" ::"r"(pair_bar) : "memory");
+            cl.pair_sync();
             if (part == 0) {
                 if (lane == 0) {
                     if (row0 < g.n_train) { tma_store_2d(&map_dl, slab, 0, (int32_t)row0); bulk_commit(); }
                     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bars + HB_DL_FULL)) : "memory");
                 }
-                const float loss = warp_sum(train ? (mx + __logf(den)) - ly : 0.f);
+                const float loss = warp_sum(cl.loss(train));
                 if (lane == 0 && g.loss_partial) g.loss_partial[tile * 4 + q] = loss;
             }
         }

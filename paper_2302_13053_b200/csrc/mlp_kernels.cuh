@@ -153,6 +153,7 @@ struct UpdateArgs {
     const float* loss_partial; int64_t n_loss; float inv_rows; float* loss_out;
     const int32_t* status;     // non-zero: a kernel of this step gave up on a bounded wait -> loss = NaN
     int32_t* status_out;       // (optional) receives *status
+    int32_t* status_word;      // the same word, for a kernel that waits itself
     // bf16 copies of the updated weights in the orientations the next products read (optional)
     bf16* w1t16; int64_t ld_k;       // W1^T [out1 x ld_k]
     bf16* w1r16; int64_t ld_o1;      // W1   [d_in x ld_o1]

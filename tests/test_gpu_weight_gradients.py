@@ -12,7 +12,11 @@ pytestmark = pytest.mark.gpu
 
 @pytest.mark.parametrize("d_in,hidden,n_classes,n", [(1, 1, 1, 1), (128, 0, 64, 64), (129, 0, 64, 65), (300, 0, 3, 9000), (64, 65, 1, 63),
                                                      (127, 128, 64, 129), (65, 129, 33, 200), (257, 256, 47, 4500),
-                                                     (130, 257, 5, 700), (1030, 512, 41, 1500)])
+                                                     (130, 257, 5, 700), (1030, 512, 41, 1500),
+                                                     # two kernels an iteration up to 512 rows and 128 hidden units, and just beyond
+                                                     (1433, 64, 7, 140), (63, 128, 41, 512), (200, 33, 17, 33), (64, 63, 8, 31), (1000, 128, 3, 60),
+                                                     (2400, 100, 9, 300), (4400, 0, 40, 65), (64, 128, 9, 513), (128, 0, 64, 513), (129, 0, 64, 600),
+                                                     (65, 64, 1, 600), (127, 128, 64, 700), (4481, 128, 3, 60)])
 def test_gradients_at_the_edges(d_in, hidden, n_classes, n):
     from paper_2302_13053_b200 import binding as B
     rng = np.random.default_rng(1000 * d_in + hidden)
