@@ -10,6 +10,7 @@
 #include "common.cuh"
 #include "aggregate.h"
 #include "gat.h"
+#include "gat_lanes.cuh"
 
 namespace retexo {
 
@@ -113,6 +114,7 @@ struct AggArgs {
     HeavyRows heavy;
     float* seg_partial;              // [segments x round_up(dim, 4)] raw sums
     int64_t ld_partial;
+    GatRowOrder order;               // agg_lanes_kernel: rows by falling length (null: as they come)
     int32_t* next_item;              // agg_rows_kernel: work counter
     float hub_coef;                  // agg_rows_kernel: rows of nodes with coef <= hub_coef (hubs) are loaded "evict last", all
                                      // others "evict first"
@@ -341,7 +343,7 @@ struct AggLanes {
 // One block's share of a slab: the first seg_blocks blocks take the segments of the heavy rows (their raw sums go to scratch), the
 // others a fixed set of rows each, rows_per_warp (up to G) per warp.
 template <int LPG, int E, int NV, int OP>
-__device__ __forceinline__ void agg_block(const AggArgs& a, int col0, unsigned b, unsigned seg_blocks, int rows_per_warp) {
+__device__ __forceinline__ void agg_block(const AggArgs& a, int col0, unsigned b, unsigned seg_blocks, int rows_per_warp, const GatGrid& by_length) {
     constexpr int G = kWarp / LPG;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     AggLanes<LPG, E, NV, OP> L(a, lane, col0);
@@ -367,12 +369,24 @@ __device__ __forceinline__ void agg_block(const AggArgs& a, int col0, unsigned b
         }
         return;
     }
-    const int64_t v0 = ((int64_t)(b - seg_blocks) * kAggWarps + warp) * rows_per_warp;
-    if (v0 >= a.n) return;
-    const int64_t v = min(v0 + L.g, a.n - 1);
-    const int64_t beg = __ldg(a.rowptr + v);
-    const bool some = L.g < rows_per_warp && v0 + L.g < a.n;
-    const int32_t total = some ? (int32_t)(__ldg(a.rowptr + v + 1) - beg) : INT32_MAX;      // (nobody's row)
+    int64_t v, beg;
+    int32_t total;
+    if (a.order.rows) {
+        int rows;
+        const int64_t i0 = gat_first_row<LPG>(a.order, by_length, (int64_t)(b - seg_blocks) * kAggWarps + warp, rows);
+        if (rows == 0) return;
+        const GatRow row = load_row_entry(a.order.rows + i0 + min(L.g, rows - 1));
+        v = row.v;
+        beg = row.beg;
+        total = L.g < rows ? row.deg : INT32_MAX;      // (nobody's row)
+    } else {
+        const int64_t v0 = ((int64_t)(b - seg_blocks) * kAggWarps + warp) * rows_per_warp;
+        if (v0 >= a.n) return;
+        v = min(v0 + L.g, a.n - 1);
+        beg = __ldg(a.rowptr + v);
+        const bool some = L.g < rows_per_warp && v0 + L.g < a.n;
+        total = some ? (int32_t)(__ldg(a.rowptr + v + 1) - beg) : INT32_MAX;
+    }
     const bool mine = G > 1 && total <= kGroupEntries;
     if constexpr (G > 1) {
         if (__any_sync(0xffffffffu, mine)) {
@@ -399,6 +413,7 @@ __device__ __forceinline__ void agg_block(const AggArgs& a, int col0, unsigned b
 struct AggGrid {
     unsigned slabs, blocks_per_slab, seg_blocks;      // whole slabs first, then the columns that are left
     int rows_per_warp, tail_rows_per_warp;
+    GatGrid by_length, tail_by_length;                // (rows by length)
 };
 
 // Blocks are ordered slab by slab, so that at any time the whole grid gathers from the same few columns of the matrix: a slab of
@@ -418,9 +433,11 @@ __global__ void __launch_bounds__(kAggThreads, AggLanes<LPG, E, NV, OP>::kBlocks
     const unsigned whole = grid.slabs * grid.blocks_per_slab;
     if ((LPG == TLPG && NV == TNV) || blockIdx.x < whole) {
         const unsigned slab = blockIdx.x / grid.blocks_per_slab;
-        agg_block<LPG, E, NV, OP>(a, (int)slab * kCols, blockIdx.x - slab * grid.blocks_per_slab, grid.seg_blocks, grid.rows_per_warp);
+        agg_block<LPG, E, NV, OP>(a, (int)slab * kCols, blockIdx.x - slab * grid.blocks_per_slab, grid.seg_blocks, grid.rows_per_warp,
+                                   grid.by_length);
     } else {
-        agg_block<TLPG, E, TNV, OP>(a, (int)grid.slabs * kCols, blockIdx.x - whole, grid.seg_blocks, grid.tail_rows_per_warp);
+        agg_block<TLPG, E, TNV, OP>(a, (int)grid.slabs * kCols, blockIdx.x - whole, grid.seg_blocks, grid.tail_rows_per_warp,
+                                     grid.tail_by_length);
     }
 }
 
@@ -486,10 +503,15 @@ static int launch_lanes(int op, const AggArgs& a, int64_t n_edges, int n_sm, cud
     g.tail_rows_per_warp = rows_per_warp(kWarp / TLPG, a.n, n_edges, n_sm);
     const int64_t segs = n_edges >= heavy_degree(n_edges) ? (max_segments(n_edges) + kAggWarps - 1) / kAggWarps : 0;
     g.seg_blocks = (unsigned)(segs < 4ll * n_sm ? segs : 4ll * n_sm);
-    auto blocks = [&](int64_t rows) { return (a.n + kAggWarps * rows - 1) / (kAggWarps * rows) + g.seg_blocks; };
-    const int64_t total = g.slabs * blocks(g.rows_per_warp) + (left ? blocks(g.tail_rows_per_warp) : 0);
+    static_assert(kAggWarps == kGatWarps && kGroupEntries == kGatGroupEntries, "one order serves both");
+    g.by_length = gat_grid<LPG>(a.n, n_edges, n_sm, 0);
+    g.tail_by_length = gat_grid<TLPG>(a.n, n_edges, n_sm, 0);
+    auto blocks = [&](int64_t rows, const GatGrid& by_length) {
+        return (a.order.rows ? (int64_t)by_length.blocks : (a.n + kAggWarps * rows - 1) / (kAggWarps * rows)) + g.seg_blocks;
+    };
+    const int64_t total = g.slabs * blocks(g.rows_per_warp, g.by_length) + (left ? blocks(g.tail_rows_per_warp, g.tail_by_length) : 0);
     if (total > INT32_MAX) return RETEXO_ERR_UNSUPPORTED;
-    g.blocks_per_slab = (unsigned)blocks(g.rows_per_warp);
+    g.blocks_per_slab = (unsigned)blocks(g.rows_per_warp, g.by_length);
     const unsigned grid = (unsigned)total;
     if constexpr (E == 8) {
         if (op == kOpGcn) agg_lanes_kernel<LPG, E, NV, TLPG, TNV, kOpGcn><<<grid, kAggThreads, 0, st>>>(a, g);
@@ -913,6 +935,15 @@ static int64_t gcn_copy_floats(int64_t n, int64_t n_edges, int32_t dim, bool lay
     return floats <= ((int64_t)2 << 30) / 4 ? floats : 0;
 }
 
+// Rows that share warps are taken by falling length (gat_lanes.cuh) on sparse graphs: on a power-law graph the longest of four rows is twice
+// the mean, and the lanes of the others wait for it.  The order takes two passes over the row pointers, about 10 us, and rows of a few
+// entries gain nothing.  In node order / by length: 1 M nodes, 20 M entries, 128 columns, concatenated bf16 1612 / 1187 us; 2 M nodes, 80 M
+// entries, 100 columns, GCN 6.2 / 5.2 ms; 1 M nodes, 16 M entries, 64 columns, GCN 711 / 590 us; 2 M nodes, 16 M entries, 8 columns 281 / 250.
+// (In node order stay: a warp per row, 89 k nodes, 0.9 M entries of 77 floats 102 / 107 us; uniform rows of 6 entries, 35 columns 609 / 678.)
+static bool rows_by_length(int64_t n, int64_t n_edges, int32_t dim) {
+    return n_edges >= 8 * n && n_edges <= 48 * n && n_edges * dim >= ((int64_t)32 << 20);
+}
+
 }  // namespace retexo
 
 using namespace retexo;
@@ -931,6 +962,10 @@ size_t retexo::aggregate_rows_workspace_size(int64_t n_nodes, int64_t n_edges, i
         if (type == RETEXO_GCN) {
             s.take<float>((size_t)n_nodes);                               // coef
             s.take<float>((size_t)gcn_copy_floats(n_nodes, n_edges, dim, lay_out));
+        }
+        if (rows_by_length(n_nodes, n_edges, dim)) {
+            s.take<GatRow>((size_t)n_nodes);
+            s.take<int32_t>(kGatOrderInts);
         }
     }
     return s.off + kAlign;
@@ -999,23 +1034,31 @@ static int aggregate(const retexo_csr* g, int32_t type, const float* q, int64_t 
     const bool v8 = aligned_to(q, 32) && ldq % 8 == 0 && ldq >= (dim + 7) / 8 * 8 && (whole_rows || (dim + 7) / 8 * 8 - dim <= 3);
     const bool v4 = aligned_to(q, 16) && ldq % 4 == 0 && ldq >= (dim + 3) / 4 * 4;
     const bool v2 = aligned_to(q, 8) && ldq % 2 == 0 && ldq >= (dim + 1) / 2 * 2;
+    const unsigned prep_blocks = (unsigned)((n + 255) / 256);
+    float* coef = type == RETEXO_GCN ? ws.take<float>((size_t)n) : nullptr;
+    const GcnWay way = gcn_way(n, e, dim);      // (GCN)
+    const int64_t copy = type == RETEXO_GCN ? gcn_copy_floats(n, e, dim, lay_out) : 0;
+    float* qs = ws.take<float>((size_t)copy);
+    const bool copies = copy > 0 && (way != GcnWay::kWeighted || !v4);      // (rows that come in whole pieces are weighted as they are)
+    if (rows_by_length(n, e, dim) && (v8 || copies) && !(type == RETEXO_GCN && way == GcnWay::kHbm)) {      // (heavy rows are the order's hubs)
+        GatRow* rows = ws.take<GatRow>((size_t)n);
+        int32_t* bins = ws.take<int32_t>(kGatOrderInts);
+        const int32_t* all = nullptr;
+        RETEXO_TRY(gat_order_launch(*g, 0, &all, &n, 1, rows, nullptr, bins, 2 * a.heavy.seg_entries, st));
+        a.order = {rows, bins + kGatOrderCounts, nullptr, n};
+    }
     auto lanes = [&](int op) {
         return v8 ? launch_lanes8(op, a, e, n_sm, st) : v4 ? launch_lanes4(op, a, e, n_sm, st)
              : v2 ? launch_lanes2(op, a, e, n_sm, st) : launch_lanes1(op, a, e, n_sm, st);
     };
-    const unsigned prep_blocks = (unsigned)((n + 255) / 256);
     if (type == RETEXO_GCN) {
-        float* coef = ws.take<float>((size_t)n);
-        const GcnWay way = gcn_way(n, e, dim);
-        const int64_t copy = gcn_copy_floats(n, e, dim, lay_out && !v4);
-        if (copy == 0) {
+        if (!copies) {
             prep_rows_kernel<<<prep_blocks, 256, 0, st>>>(n, g->rowptr, a.heavy, coef);
             a.coef = coef;
             if (way != GcnWay::kHbm) return lanes(kOpGcnWeighted);
             a.hub_coef = (float)(1.0 / sqrt(4.0 * (double)e / (double)n + 1.0));      // hubs: at least four times the mean degree
             return v4 ? launch_rows<4>(a, e, n_sm, st) : v2 ? launch_rows<2>(a, e, n_sm, st) : launch_rows<1>(a, e, n_sm, st);
         }
-        float* qs = ws.take<float>((size_t)copy);
         const int64_t ld_qs = gcn_copy_stride(dim, n, e);
         int lanes_log2 = 0;
         while (lanes_log2 < 5 && (8 << lanes_log2) < ld_qs) ++lanes_log2;

@@ -455,11 +455,12 @@ extern "C" int retexo_lmp_train(const retexo_lmp_config* cfg, const retexo_lmp_i
         all_rows = {b.rows_all, bins + kGatOrderCounts, nullptr, n};
         batch_rows = {b.rows_batch, bins + kGatOrderInts + kGatOrderCounts, b.slots, n_tr + n_val};
         train_rows = {b.rows_train, bins + 2 * kGatOrderInts + kGatOrderCounts, nullptr, n_tr};
+        const int hub_entries = gat_hub_entries(g.n_edges, n_sm);
         const int32_t* lists[3] = {nullptr, train_idx, val_idx};
         const int64_t sizes[3] = {n, n_tr, n_val};
-        RETEXO_TRY(gat_order_launch(g, 1, lists, sizes, 1, b.rows_all, nullptr, bins, n_sm, st));
-        RETEXO_TRY(gat_order_launch(g, 1, lists + 1, sizes + 1, 2, b.rows_batch, b.slots, bins + kGatOrderInts, n_sm, st));
-        RETEXO_TRY(gat_order_launch(g, 1, lists + 1, sizes + 1, 1, b.rows_train, nullptr, bins + 2 * kGatOrderInts, n_sm, st));
+        RETEXO_TRY(gat_order_launch(g, 1, lists, sizes, 1, b.rows_all, nullptr, bins, hub_entries, st));
+        RETEXO_TRY(gat_order_launch(g, 1, lists + 1, sizes + 1, 2, b.rows_batch, b.slots, bins + kGatOrderInts, hub_entries, st));
+        RETEXO_TRY(gat_order_launch(g, 1, lists + 1, sizes + 1, 1, b.rows_train, nullptr, bins + 2 * kGatOrderInts, hub_entries, st));
     }
     const float* q = feat;
     int64_t ldq = ld_feat;

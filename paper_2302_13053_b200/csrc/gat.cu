@@ -475,8 +475,7 @@ bool gat_lanes_usable(int32_t heads, int32_t head_dim, const float* p, int64_t l
 }
 
 int gat_order_launch(const retexo_csr& g, int32_t self_loop, const int32_t* const* idx, const int64_t* n_idx, int lists, GatRow* rows,
-                     int32_t* slots, int32_t* bins, int n_sm, cudaStream_t st) {
-    const int hub_entries = gat_hub_entries(g.n_edges, n_sm);
+                     int32_t* slots, int32_t* bins, int hub_entries, cudaStream_t st) {
     RETEXO_CUDA_TRY(cudaMemsetAsync(bins, 0, kGatOrderInts * sizeof(int32_t), st));
     for (int i = 0; i < lists; ++i)
         if (n_idx[i]) gat_order_count_kernel<<<gat_order_blocks(n_idx[i]), 256, 0, st>>>(n_idx[i], idx[i], g.rowptr, self_loop, hub_entries, bins);
@@ -517,7 +516,7 @@ int gat_forward_launch(const GatForward& f, Arena& ws, int n_sm, cudaStream_t st
         RETEXO_TRY(rc);
         if (own) gat_order_kernel<<<gat_order_blocks(n), 256, 0, st>>>(n, nullptr, a.rowptr, a.self_loop, hub_entries, bins, rows, nullptr, 0);
         return gat_lanes_dispatch(lpg, w, [&]<int LPG, int W>() {
-            const GatGrid grid = gat_grid<LPG>(order.n, f.g.n_edges + n, n_sm);
+            const GatGrid grid = gat_grid<LPG>(order.n, f.g.n_edges + n, n_sm, 6 * n_sm);
             gat_lane_rows_kernel<LPG, W><<<grid.blocks, kGatThreads, 0, st>>>(a, order, grid, vec_out, vec_out16);
             return launch_status();
         });

@@ -28,9 +28,10 @@ void gat_forward_workspace(int64_t n_nodes, int32_t heads, Sizer& s);
 bool gat_lanes_usable(int32_t heads, int32_t head_dim, const float* p, int64_t ldp, const float* q, int64_t ldq);
 constexpr int kGatOrderCounts = 256, kGatOrderInts = kGatOrderCounts + 64;      // rows per class of lengths, rows placed so far, GatRowOrder::counts
 // Builds the order of the rows of some index lists (a null list: all rows); its counts are at bins + kGatOrderCounts.  rows, slots (optional:
-// slots count on through the lists): one entry per row listed; bins: kGatOrderInts words.
+// slots count on through the lists): one entry per row listed; bins: kGatOrderInts words; rows of hub_entries
+// or more are hubs.
 int gat_order_launch(const retexo_csr& g, int32_t self_loop, const int32_t* const* idx, const int64_t* n_idx, int lists, GatRow* rows,
-                     int32_t* slots, int32_t* bins, int n_sm, cudaStream_t st);
+                     int32_t* slots, int32_t* bins, int hub_entries, cudaStream_t st);
 // Arguments as checked by retexo_aggregate; scratch is taken from ws in the order gat_forward_workspace lists.
 int gat_forward_launch(const GatForward& f, Arena& ws, int n_sm, cudaStream_t st);
 

@@ -63,10 +63,10 @@ struct GatGrid {
     unsigned blocks;
 };
 template <int LPG>
-inline GatGrid gat_grid(int64_t n, int64_t n_entries, int n_sm) {
+inline GatGrid gat_grid(int64_t n, int64_t n_entries, int n_sm, int hub_blocks) {
     constexpr int64_t G = kWarp / LPG;
     GatGrid g;
-    g.hub_blocks = 6 * n_sm;
+    g.hub_blocks = hub_blocks;
     const int64_t most = (int64_t)n_sm * 4 * kGatBlocksPerSm * kGatWarps;
     int64_t want = n_entries / (kGatGroupEntries + 1) + 1;
     if (want > n) want = n;

@@ -140,3 +140,24 @@ def test_rows_bound_by_memory(degree, dim, ld):
         assert torch.equal(out16[v, :dim], out[v].to(torch.bfloat16))
     again, _ = B.retexo_aggregate(oracle.GCN, rp, ci, q, dim=dim)
     assert torch.equal(out, again)
+
+
+@pytest.mark.parametrize("dim", [128, 200, 301])
+@pytest.mark.parametrize("aggr", [oracle.GCN, oracle.SAGE_MEAN, oracle.SAGE_MAX])
+def test_rows_by_length(aggr, dim):
+    """A graph sparse and large enough for the rows to be taken in order of their lengths: empty rows, rows around what a group of lanes and a
+    segment take, and more rows above a group's length than there are warps for them."""
+    from paper_2302_13053_b200 import binding as B
+    rng = np.random.default_rng(dim)
+    deg = np.concatenate([np.full(22500, 33), np.repeat([0, 1, 2, 31, 32, 34, 127, 128, 129, 400], 10), rng.integers(0, 12, 60000)])
+    deg = deg[rng.permutation(deg.size)]
+    n, e = deg.size, int(deg.sum())
+    rowptr = np.concatenate([[0], np.cumsum(deg)]).astype(np.int64)
+    assert 8 * n <= e <= 48 * n and e * dim >= 32 << 20
+    colidx = rng.integers(0, n, e).astype(np.int32)
+    q = rng.standard_normal((n, dim)).astype(np.float32)
+    out, out16 = B.retexo_aggregate(aggr, dev(rowptr), dev(colidx), dev(q), want_bf16=True)
+    assert_rows_close(out.cpu().numpy(), oracle.aggregate(aggr, rowptr, colidx, q), what="aggr %d" % aggr)
+    assert torch.equal(out16[:, :out.shape[1]], out.to(torch.bfloat16))
+    again, _ = B.retexo_aggregate(aggr, dev(rowptr), dev(colidx), dev(q))
+    assert torch.equal(out, again)
