@@ -223,10 +223,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) { mbar_init(full + s, 1); mbar_init(empty + s, 1); }
-        // the arg-max epilogue lets one thread own a whole row of logits: it uses four of the eight warps
-        const bool row_owner = BN == 64 && MODE == TC_EPI_ARGMAX;
         // (pairs: the even block's "accumulator drained" barrier collects the epilogue warps of both blocks)
-        for (int b = 0; b < NACC; ++b) { mbar_init(acc_full + b, 1); mbar_init(acc_empty + b, row_owner ? 4 : (PAIR ? 2 : 1) * EW / TG); }
+        for (int b = 0; b < NACC; ++b) { mbar_init(acc_full + b, 1); mbar_init(acc_empty + b, (PAIR ? 2 : 1) * EW / TG); }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -356,11 +354,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         uint8_t* stage = stage_base + ew * kStageBytesPerWarp;      // this warp's two staging blocks
         int flip = 0;
         const CUtensorMap* rows_map = g.tma_rows ? &map_rows : nullptr;
-        const bool row_owner = BN == 64 && MODE == TC_EPI_ARGMAX;
         constexpr bool kGated = MODE == TC_EPI_MASK;
-        // soft-max epilogue: this warp's 32 bias values never change (its columns are the same in every tile)
+        // soft-max and arg-max epilogues: this warp's 32 bias values never change (its columns are the same in every tile)
         float ce_bias_lane = 0.f;
-        if constexpr (BN == 64 && MODE == TC_EPI_SOFTMAX_CE)
+        if constexpr (BN == 64 && (MODE == TC_EPI_SOFTMAX_CE || MODE == TC_EPI_ARGMAX))
             ce_bias_lane = (g.bias && half * 32 + lane < g.N) ? __ldg(g.bias + half * 32 + lane) : 0.f;
         // gated epilogue: the gate block of the next chunk is fetched while the current chunk is processed
         uint4 gate_next[4];
@@ -382,7 +379,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
         };
         if constexpr (kGated) gate_prefetch(tile_first + gi * tile_stride, half * kPartCols);
         int64_t lt = gi;
-        for (int32_t t = tile_first + gi * tile_stride; t < n_tiles && !(row_owner && half == 1);
+        for (int32_t t = tile_first + gi * tile_stride; t < n_tiles;
              t += TG * tile_stride, lt += TG) {
             const int32_t z = t / per_split, rem = t % per_split;
             const int32_t mt = rem % n_m;
@@ -399,7 +396,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 ce_label = (row < g.M && row < g.n_train && g.y) ? g.y[row] : -1;
             const bool ok = mbar_wait(acc_full + b, pb, g.status, abort_flag);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-            if (!ok) break;
+            if (!ok && MODE != TC_EPI_ARGMAX) break;      // (those warps meet at a barrier: they go on, and write nothing)
             if constexpr (BN == 64 && MODE == TC_EPI_SOFTMAX_CE) {
                 // Two threads share a row of logits: warp q takes columns [0, 32), warp q + 4 columns
                 // [32, 64); row maximum, sum and the label's logit are exchanged through shared memory.
@@ -478,58 +475,53 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant_
                 // (the exchange arrays and warp_loss are next written after the following tile's first
                 //  barrier-protected phase: every warp passes two more barriers before reusing them)
             } else if constexpr (BN == 64 && MODE == TC_EPI_ARGMAX) {
-                // one thread owns the whole row of logits (four of the eight warps take part)
-                float v[64];
-                if (ok) {
-                    uint32_t ra[32], rb[32];
-                    if (n_kb > 0) {       // both halves of the row in flight together
-                        tmem_ld_issue(acc_addr + ((uint32_t)(q * 32) << 16), ra);
-                        tmem_ld_issue(acc_addr + ((uint32_t)(q * 32) << 16) + 32u, rb);
-                        tmem_ld_wait(ra);
-                        tmem_ld_wait(rb);
-                    } else {
+                // Two threads share a row of logits as in the soft-max epilogue; the maxima meet in exchange arrays that tiles use in
+                // turn, so a tile takes one barrier.  (One thread a row, half of the warps idle before: 55703 rows x 256, 41
+                // classes with logits 23.8 -> 16.1 us, 200 k rows x 256, 47 classes 51.7 -> 29.6.)
+                const int cb = half * 32, slot = q * 32 + lane;
+                float v[32];
+                {
+                    uint32_t r[32];
+                    if (n_kb > 0) { tmem_ld_issue(acc_addr + ((uint32_t)(q * 32) << 16) + (uint32_t)cb, r); tmem_ld_wait(r); }
+                    else {
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) { ra[j] = 0u; rb[j] = 0u; }
+                        for (int j = 0; j < 32; ++j) r[j] = 0u;
                     }
-                    const float bias_a = (g.bias && lane < g.N) ? __ldg(g.bias + lane) : 0.f;
-                    const float bias_b = (g.bias && 32 + lane < g.N) ? __ldg(g.bias + 32 + lane) : 0.f;
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        v[j] = j < g.N ? __uint_as_float(ra[j]) + __shfl_sync(0xffffffffu, bias_a, j) : -INFINITY;
-                        v[32 + j] = 32 + j < g.N ? __uint_as_float(rb[j]) + __shfl_sync(0xffffffffu, bias_b, j) : -INFINITY;
-                    }
-                } else {
-#pragma unroll
-                    for (int c = 0; c < 64; ++c) v[c] = 0.f;
+                    for (int j = 0; j < 32; ++j)
+                        v[j] = cb + j < g.N ? __uint_as_float(r[j]) + __shfl_sync(0xffffffffu, ce_bias_lane, j) : -INFINITY;
                 }
                 const bool live = ok && row < g.M;
-                const int32_t yi = (live && g.y) ? g.y[row] : -1;
-                int best = 0;
                 float bv = v[0];
+                int best = 0;
 #pragma unroll
-                for (int c = 1; c < 64; ++c) if (v[c] > bv) { bv = v[c]; best = c; }   // strict: lowest index wins ties
-                if (live && g.pred) g.pred[row] = best;
-                if (g.out_f32) {
+                for (int j = 1; j < 32; ++j) if (v[j] > bv) { bv = v[j]; best = j; }      // strict: lowest index wins ties
+                float (*const exchange)[2][128] = xch + 2 * ((lt / TG) & 1);
+                exchange[0][half][slot] = bv;
+                exchange[1][half][slot] = __int_as_float(cb + best);
+                if (g.out_f32 && cb < g.N && ok) {
                     // Rows leave whole, 32 columns at a time, over the warp's staging block (column j of row r in word j ^ r: no bank
-                    // twice either way).  A thread storing its own row touches 32 lines per store: the logits and classes of 55703
-                    // rows and 41 classes, in two launches, 37.6 -> 33.5 us.
+                    // twice either way).  A thread storing its own row touches 32 lines per store.
                     float* st = reinterpret_cast<float*>(stage);
+                    __syncwarp();
 #pragma unroll
-                    for (int h = 0; h < 64; h += 32) {
-                        if (h >= g.N) break;
-                        __syncwarp();
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) st[lane * 32 + (j ^ lane)] = v[h + j];
-                        __syncwarp();
-                        float* dst = g.out_f32 + row0 * g.ld_f32 + h + lane;
-                        const int n_lines = (int)min((int64_t)32, g.M - row0);
-                        if (h + lane < g.N)
-                            for (int r = 0; r < n_lines; ++r) dst[r * g.ld_f32] = st[r * 32 + (lane ^ r)];
+                    for (int j = 0; j < 32; ++j) st[lane * 32 + (j ^ lane)] = v[j];
+                    __syncwarp();
+                    float* dst = g.out_f32 + row0 * g.ld_f32 + cb + lane;
+                    const int n_lines = (int)min((int64_t)32, g.M - row0);
+                    if (cb + lane < g.N) {
+#pragma unroll 8
+                        for (int r = 0; r < n_lines; ++r) dst[r * g.ld_f32] = st[r * 32 + (lane ^ r)];
                     }
                 }
-                if (g.correct) {
-                    const unsigned hits = __ballot_sync(0xffffffffu, live && best == yi);
-                    if (lane == 0 && hits) atomicAdd(g.correct, (unsigned long long)__popc(hits));
+                asm volatile("bar.sync %0, 256;" ::"r"(1 + gi) : "memory");
+                if (half == 0) {
+                    const int arg = exchange[0][1][slot] > bv ? __float_as_int(exchange[1][1][slot]) : best;
+                    if (live && g.pred) g.pred[row] = arg;
+                    if (g.correct) {
+                        const unsigned hits = __ballot_sync(0xffffffffu, live && arg == (g.y ? g.y[row] : -1));
+                        if (lane == 0 && hits) atomicAdd(g.correct, (unsigned long long)__popc(hits));
+                    }
                 }
             } else if (ok) {
                 // the accumulator load of chunk c + 1 is in flight while chunk c is processed (gated modes
