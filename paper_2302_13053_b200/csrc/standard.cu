@@ -94,6 +94,90 @@ static __global__ void __launch_bounds__(32 * kStdRowWarps) std_gate_kernel(cons
         dz[v * ld_dz + j] = f32_to_bf16((__ldg(bits + v * ld_bits + k) >> lane) & 1u ? d : 0.f);
     }
 }
+// ---- the graph without entries that an iteration has no use for (SAGE, whose rows depend on their entries and nothing else)
+constexpr uint8_t kStdTrain = 1, kStdBatch = 2;      // marks of a node: a training row; a training or validation row
+static __global__ void std_mark_kernel(const int32_t* __restrict__ idx, int64_t n, uint8_t value, uint8_t* __restrict__ marks) {
+    const int64_t i = blockIdx.x * 256ll + threadIdx.x;
+    if (i < n) marks[idx[i]] = value;
+}
+// Entries of row v that are kept: all of a batch row's (columns == 0), or those whose column is a training row.
+__device__ __forceinline__ bool std_row_kept(const uint8_t* marks, int64_t v, int columns) { return columns || (marks[v] & kStdBatch); }
+// The rows' kept entries: a warp a row, 128 entries a trip.
+static __global__ void __launch_bounds__(32 * kStdRowWarps) std_count_kept_kernel(int64_t n, const int64_t* __restrict__ rowptr,
+                                                                                  const int32_t* __restrict__ colidx, const uint8_t* __restrict__ marks,
+                                                                                  int columns, int64_t* __restrict__ count) {
+    const int64_t v = std_row();
+    if (v >= n) return;
+    const int lane = threadIdx.x & 31;
+    const int64_t beg = rowptr[v], end = rowptr[v + 1];
+    int kept = 0;
+    if (columns) {
+#pragma unroll 4
+        for (int64_t e = beg + lane; e < end; e += 32) kept += __ldg(marks + __ldcs(colidx + e)) & kStdTrain;
+        kept = __reduce_add_sync(0xffffffffu, kept);
+    }
+    if (lane == 0) count[v] = columns ? (int64_t)kept : std_row_kept(marks, v, columns) ? end - beg : 0;
+}
+// count[v] = sum of count[0, v), in place, and the total behind them, in two launches: every block its own kStdScanRows rows and their total,
+// then every block what lies before it.
+constexpr int kStdScanPer = 8, kStdScanRows = 256 * kStdScanPer;
+static __global__ void __launch_bounds__(256) std_scan_kernel(int64_t n, int64_t* __restrict__ count, int64_t* __restrict__ totals) {
+    __shared__ int64_t warp_total[8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t i = (int64_t)blockIdx.x * kStdScanRows + threadIdx.x * kStdScanPer;
+    int64_t c[kStdScanPer], mine = 0;
+#pragma unroll
+    for (int k = 0; k < kStdScanPer; ++k) {
+        c[k] = i + k < n ? count[i + k] : 0;
+        mine += c[k];
+    }
+    int64_t at = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int64_t y = __shfl_up_sync(0xffffffffu, at, o);
+        if (lane >= o) at += y;
+    }
+    if (lane == 31) warp_total[warp] = at;
+    at -= mine;
+    __syncthreads();
+    for (int w = 0; w < warp; ++w) at += warp_total[w];
+#pragma unroll
+    for (int k = 0; k < kStdScanPer; ++k) {
+        if (i + k < n) count[i + k] = at;
+        at += c[k];
+    }
+    if (threadIdx.x == 255) totals[blockIdx.x] = at;
+}
+static __global__ void __launch_bounds__(256) std_scan_add_kernel(int64_t n, int64_t* __restrict__ count, const int64_t* __restrict__ totals) {
+    __shared__ unsigned long long before_s;
+    if (threadIdx.x == 0) before_s = 0ull;
+    __syncthreads();
+    unsigned long long part = 0;
+    for (unsigned b = threadIdx.x; b < blockIdx.x; b += 256) part += (unsigned long long)totals[b];
+    if (part) atomicAdd(&before_s, part);
+    __syncthreads();
+    const int64_t before = (int64_t)before_s;
+    for (int64_t i = (int64_t)blockIdx.x * kStdScanRows + threadIdx.x; i < n && i < ((int64_t)blockIdx.x + 1) * kStdScanRows; i += 256) count[i] += before;
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) count[n] = before + totals[blockIdx.x];
+}
+static __global__ void __launch_bounds__(32 * kStdRowWarps) std_copy_kept_kernel(int64_t n, const int64_t* __restrict__ rowptr,
+                                                                                 const int32_t* __restrict__ colidx, const uint8_t* __restrict__ marks,
+                                                                                 int columns, const int64_t* __restrict__ first,
+                                                                                 int32_t* __restrict__ kept) {
+    const int64_t v = std_row();
+    if (v >= n || !std_row_kept(marks, v, columns)) return;
+    const int lane = threadIdx.x & 31;
+    const int64_t beg = rowptr[v], end = rowptr[v + 1];
+    int32_t* dst = kept + first[v];
+    for (int64_t e0 = beg; e0 < end; e0 += 32) {
+        const int64_t e = e0 + lane;
+        const int32_t u = e < end ? __ldcs(colidx + e) : -1;
+        const bool keep = u >= 0 && (!columns || (__ldg(marks + u) & kStdTrain));
+        const unsigned all = __ballot_sync(0xffffffffu, keep);
+        if (keep) dst[__popc(all & ((1u << lane) - 1u))] = u;
+        dst += __popc(all);
+    }
+}
 static __global__ void std_copy_if_kernel(const int32_t* decision, const float* src, float* dst, int64_t n) {
     if (!*decision) return;
     const int64_t p = blockIdx.x * 256ll + threadIdx.x;
@@ -146,6 +230,8 @@ struct StdBuffers {
     void* ws_step; size_t ws_step_bytes;
     void* ws_agg; size_t ws_agg_bytes;
     void* ws_embed; size_t ws_embed_bytes;
+    // dense SAGE: node marks, and the graph's batch rows alone ([0]) and its columns that are training rows alone ([1])
+    uint8_t* marks; int64_t* kept_rowptr[2]; int32_t* kept_colidx[2]; int64_t* scan_totals;
 };
 
 static int std_check(const retexo_standard_config* c) {
@@ -168,6 +254,9 @@ static void std_dims(const retexo_standard_config& c, int m, StdLayer* l) {
     l->ld_o1 = std_round_up(l->out, 64);
     l->nt = ((int64_t)l->d + 1) * l->out;
 }
+
+// On dense graphs (two graphs take a pass over the entries each, 0.2 ms at 58 k nodes and 7.2 M entries; on sparse ones the layers cost more).
+static bool std_keeps(const retexo_standard_config& c, int64_t n, int64_t e) { return c.aggr == RETEXO_SAGE_MEAN && c.K > 1 && e >= 32 * n; }
 
 template <typename Taker>
 static void std_layout(const retexo_standard_config& c, int64_t n, int64_t e, int64_t n_tr, int64_t n_val, int64_t n_te,
@@ -234,6 +323,14 @@ static void std_layout(const retexo_standard_config& c, int64_t n, int64_t e, in
     b.ws_agg = t.template take<uint8_t>(agg);
     b.ws_embed_bytes = retexo_embed_workspace_size(last.d, 0, c.n_classes, n);
     b.ws_embed = t.template take<uint8_t>(b.ws_embed_bytes);
+    if (std_keeps(c, n, e)) {
+        b.scan_totals = t.template take<int64_t>((size_t)((n + kStdScanRows - 1) / kStdScanRows));
+        b.marks = t.template take<uint8_t>((size_t)n);
+        for (int i = 0; i < 2; ++i) {
+            b.kept_rowptr[i] = t.template take<int64_t>((size_t)n + 1);
+            b.kept_colidx[i] = t.template take<int32_t>((size_t)e);
+        }
+    }
     if (out) *out = b;
 }
 
@@ -325,8 +422,31 @@ extern "C" int retexo_standard_train(const retexo_standard_config* cfg, const re
     retexo_mlp best = model;
     best.theta = last.best;
 
-    // Forward of the hidden layers over all nodes with the weights as they stand; leaves X^K in last.x.
-    auto forward_hidden = [&]() -> int {
+    // An iteration reads X^K at the rows of its batch only, and the gradient there reaches no other rows than the training ones: with SAGE,
+    // whose aggregation looks at a row's entries alone, the last aggregation forward runs on the batch's rows, and the first one back gathers
+    // training rows only (58 k nodes, 7.2 M entries, 66 % trained on: an iteration 2.75 -> 2.60 ms; 0.2 ms once for the two graphs).  The entry counts are upper bounds.
+    const bool keeps = std_keeps(c, n, e);
+    retexo_csr batch_rows = g, train_cols = g;
+    if (keeps) {
+        RETEXO_CUDA_TRY(cudaMemsetAsync(b.marks, 0, (size_t)n, st));
+        if (n_val) std_mark_kernel<<<(unsigned)((n_val + 255) / 256), 256, 0, st>>>(in->val_idx, n_val, kStdBatch, b.marks);
+        std_mark_kernel<<<(unsigned)((n_tr + 255) / 256), 256, 0, st>>>(in->train_idx, n_tr, kStdBatch | kStdTrain, b.marks);
+        for (int i = 0; i < 2; ++i) {
+            const unsigned blocks = std_row_blocks(n), threads = 32 * kStdRowWarps;
+            std_count_kept_kernel<<<blocks, threads, 0, st>>>(n, g.rowptr, g.colidx, b.marks, i, b.kept_rowptr[i]);
+            const unsigned scan_blocks = (unsigned)((n + kStdScanRows - 1) / kStdScanRows);
+            std_scan_kernel<<<scan_blocks, 256, 0, st>>>(n, b.kept_rowptr[i], b.scan_totals);
+            std_scan_add_kernel<<<scan_blocks, 256, 0, st>>>(n, b.kept_rowptr[i], b.scan_totals);
+            std_copy_kept_kernel<<<blocks, threads, 0, st>>>(n, g.rowptr, g.colidx, b.marks, i, b.kept_rowptr[i], b.kept_colidx[i]);
+            retexo_csr& kept = i ? train_cols : batch_rows;
+            kept.rowptr = b.kept_rowptr[i];
+            kept.colidx = b.kept_colidx[i];
+        }
+    }
+
+    // Forward of the hidden layers over all nodes with the weights as they stand; leaves X^K in last.x, of all rows or (batch) of the
+    // batch's.
+    auto forward_hidden = [&](bool batch) -> int {
         for (int m = 0; m < K - 1; ++m) {
             StdLayer& l = b.L[m];
             TcGemm f{};
@@ -335,8 +455,8 @@ extern "C" int retexo_standard_train(const retexo_standard_config* cfg, const re
             f.relu_bits = l.bits; f.ld_bits = l.ld_bits; f.status = sb.status;
             RETEXO_TRY(tc_gemm_launch(f, st));
             StdLayer& nx = b.L[m + 1];
-            RETEXO_TRY(aggregate_rows(&g, c.aggr, l.h, l.ld_h32, c.hidden, true, nullptr, 0, sage ? 1 : 0, nx.x, nx.ldx,
-                                        b.ws_agg, b.ws_agg_bytes, st));
+            RETEXO_TRY(aggregate_rows(batch && m == K - 2 ? &batch_rows : &g, c.aggr, l.h, l.ld_h32, c.hidden, true, nullptr, 0, sage ? 1 : 0,
+                                        nx.x, nx.ldx, b.ws_agg, b.ws_agg_bytes, st));
         }
         return RETEXO_OK;
     };
@@ -347,7 +467,7 @@ extern "C" int retexo_standard_train(const retexo_standard_config* cfg, const re
 
     int pending_it = 0;       // iteration whose weights still await their validation count
     for (int it = 1; it <= c.R; ++it) {
-        RETEXO_TRY(forward_hidden());
+        RETEXO_TRY(forward_hidden(true));
         RETEXO_TRY(retexo_pack_rows(last.x, 1, last.ldx, last.d, b.batch_idx, n_tr + n_val, b.xb, b.ld_xb, nullptr, 0, 1, st));
         // last layer: loss, dX of the train rows, its own update; the validation rows ride along and count the hits of
         // the weights as they stand, i.e. of iteration it - 1, which the update kernel keeps if they are the best so far
@@ -361,9 +481,9 @@ extern "C" int retexo_standard_train(const retexo_standard_config* cfg, const re
                                          K > 1 ? b.dx : nullptr, b.ld_dx));
         model.step += 1;
         if (K > 1) {
-            // rows outside the batch have no gradient; the columns beyond the scattered ones are not read
+            // rows outside the batch have no gradient; the columns beyond the scattered ones are not read, nor (training columns alone) such rows of s
             RETEXO_CUDA_TRY(cudaMemset2DAsync(b.g, sizeof(float) * b.ld_g, 0, sizeof(float) * c.hidden, (size_t)n, st));
-            if (sage) RETEXO_CUDA_TRY(cudaMemsetAsync(b.s, 0, sizeof(float) * (size_t)n * b.ld_a, st));
+            if (sage && !keeps) RETEXO_CUDA_TRY(cudaMemsetAsync(b.s, 0, sizeof(float) * (size_t)n * b.ld_a, st));
             std_scatter_rows_kernel<<<std_row_blocks(n_tr), 32 * kStdRowWarps, 0, st>>>(b.dx, b.ld_dx, in->train_idx, n_tr, last.d, g.rowptr,
                                                                                         b.g, b.ld_g, sage ? b.s : nullptr, b.ld_a);
         }
@@ -376,9 +496,10 @@ extern "C" int retexo_standard_train(const retexo_standard_config* cfg, const re
             const unsigned eb = std_row_blocks(n), et = 32 * kStdRowWarps;
             if (sage) {
                 if (m < K - 2) std_prescale_kernel<<<eb, et, 0, st>>>(b.g, b.ld_g, H, H, g.rowptr, n, b.s, b.ld_a);
-                RETEXO_TRY(aggregate_rows(&g, RETEXO_SAGE_MEAN, b.s, b.ld_a, H, true, b.a, b.ld_a, 0, nullptr, 0, b.ws_agg,
+                const retexo_csr& from = m == K - 2 ? train_cols : g;      // (the gate undoes the division by this graph's degrees)
+                RETEXO_TRY(aggregate_rows(&from, RETEXO_SAGE_MEAN, b.s, b.ld_a, H, true, b.a, b.ld_a, 0, nullptr, 0, b.ws_agg,
                                             b.ws_agg_bytes, st));
-                std_gate_kernel<<<eb, et, 0, st>>>(b.a, b.ld_a, b.g, b.ld_g, g.rowptr, l.bits, l.ld_bits, n, H, b.dz, b.ld_dz);
+                std_gate_kernel<<<eb, et, 0, st>>>(b.a, b.ld_a, b.g, b.ld_g, from.rowptr, l.bits, l.ld_bits, n, H, b.dz, b.ld_dz);
             } else {
                 RETEXO_TRY(aggregate_rows(&g, RETEXO_GCN, b.g, b.ld_g, H, true, b.a, b.ld_a, 0, nullptr, 0, b.ws_agg,
                                             b.ws_agg_bytes, st));
@@ -402,7 +523,7 @@ extern "C" int retexo_standard_train(const retexo_standard_config* cfg, const re
         pending_it = (n_val && it < c.R) ? it : 0;
     }
     // ---- the last iterate has no next iteration to ride on: one more forward pass
-    RETEXO_TRY(forward_hidden());
+    RETEXO_TRY(forward_hidden(false));
     if (n_val) {
         RETEXO_TRY(retexo_pack_rows(last.x, 1, last.ldx, last.d, in->val_idx, n_val, b.xb, b.ld_xb, nullptr, 0, 0, st));
         RETEXO_TRY(mlp_count_hits_launch(plan, sb, &model, b.xb, b.ld_xb, n_val, nullptr, b.y_val, b.counters, st));
@@ -438,7 +559,7 @@ extern "C" int retexo_standard_train(const retexo_standard_config* cfg, const re
         RETEXO_CUDA_TRY(cudaMemcpyAsync(l.theta, l.best, sizeof(float) * (size_t)l.nt, cudaMemcpyDeviceToDevice, st));
         RETEXO_TRY(linear_shadows_launch(l.d, l.out, l.theta, l.wt16, l.ld_k, nullptr, 0, st));
     }
-    RETEXO_TRY(forward_hidden());
+    RETEXO_TRY(forward_hidden(false));
     if (out->test_correct) {
         if (n_te) {
             RETEXO_TRY(retexo_pack_rows(last.x, 1, last.ldx, last.d, in->test_idx, n_te, b.xb, b.ld_xb, nullptr, 0, 0, st));
