@@ -6,6 +6,7 @@
 
 #include "aggregate.h"
 #include "gat_lanes.cuh"
+#include "kept_graph.cuh"
 #include "common.cuh"
 #include "gemm_tc.h"
 #include "mlp_plan.h"
@@ -197,7 +198,8 @@ struct LmpBuffers {
     bf16* x16; bf16* q16; float* proj; bf16* watt_t16;
     float *att, *att_m, *att_v, *att_best, *att_partial, *da, *dz; bf16* dp16; int32_t* decision; int32_t* status;
     int64_t att_splits; void* ws_gatbwd; size_t ws_gatbwd_bytes;
-    GatRow *rows_all, *rows_batch, *rows_train; int32_t *slots, *order_bins;      // row orders of a run that trains its aggregator
+    GatRow *rows_all, *rows_batch, *rows_train, *rows_src; int32_t *slots, *order_bins;      // row orders of a run that trains its aggregator
+    uint8_t* marks; int64_t *src_rowptr, *scan_totals; int32_t* src_colidx;                  // ... and its training columns
     bf16 *xtr16, *xval16;
     int32_t *y_tr, *y_val, *y_test;
     float *theta, *adam_m, *adam_v, *theta_best;
@@ -273,7 +275,12 @@ static void lmp_layout(const retexo_lmp_config& c, int64_t n, int64_t e, int64_t
         l.rows_batch = t.template take<GatRow>((size_t)(n_tr + n_val));
         l.rows_train = t.template take<GatRow>((size_t)n_tr);
         l.slots = t.template take<int32_t>((size_t)(n_tr + n_val));
-        l.order_bins = t.template take<int32_t>(3 * kGatOrderInts);
+        l.rows_src = t.template take<GatRow>((size_t)n);
+        l.order_bins = t.template take<int32_t>(4 * kGatOrderInts);
+        l.marks = t.template take<uint8_t>((size_t)n);
+        l.src_rowptr = t.template take<int64_t>((size_t)n + 1);
+        l.src_colidx = t.template take<int32_t>((size_t)e);
+        l.scan_totals = t.template take<int64_t>((size_t)kept_scan_words(n));
     }
     // training rows, then validation rows; after the round's last iteration the test rows take their place
     l.xtr16 = t.template take<bf16>((size_t)(n_tr + n_val > n_te ? n_tr + n_val : n_te) * (size_t)ld16);
@@ -443,13 +450,13 @@ extern "C" int retexo_lmp_train(const retexo_lmp_config* cfg, const retexo_lmp_i
         RETEXO_CUDA_TRY(cudaMemsetAsync(b.x16, 0, sizeof(bf16) * (size_t)n * (size_t)round_up(max_din, 64), st));
     }
     // A run that trains its aggregator walks the same rows in every iteration: their orders are found once.  An iteration needs the
-    // aggregated rows of its batch only, and only training rows have a gradient.
+    // aggregated rows of its batch only, and only training rows have a gradient, so the way back meets no other columns.
     const bool kept_orders = c.aggr == RETEXO_GAT && !c.gat_freeze_attention &&
                              gat_lanes_usable(c.gat_heads, c.gat_head_dim, b.proj, round_up(c.gat_heads * c.gat_head_dim, 32), b.dz,
                                               round_up(c.gat_heads * c.gat_head_dim, 32));
     const int n_sm = sm_count();
     if (n_sm <= 0) return RETEXO_ERR_CUDA;
-    GatRowOrder all_rows{}, batch_rows{}, train_rows{};
+    GatRowOrder all_rows{}, batch_rows{}, train_rows{}, src_rows{};
     if (kept_orders) {
         int32_t* bins = b.order_bins;
         all_rows = {b.rows_all, bins + kGatOrderCounts, nullptr, n};
@@ -461,6 +468,13 @@ extern "C" int retexo_lmp_train(const retexo_lmp_config* cfg, const retexo_lmp_i
         RETEXO_TRY(gat_order_launch(g, 1, lists, sizes, 1, b.rows_all, nullptr, bins, hub_entries, st));
         RETEXO_TRY(gat_order_launch(g, 1, lists + 1, sizes + 1, 2, b.rows_batch, b.slots, bins + kGatOrderInts, hub_entries, st));
         RETEXO_TRY(gat_order_launch(g, 1, lists + 1, sizes + 1, 1, b.rows_train, nullptr, bins + 2 * kGatOrderInts, hub_entries, st));
+        src_rows = {b.rows_src, bins + 3 * kGatOrderInts + kGatOrderCounts, nullptr, n};
+        RETEXO_CUDA_TRY(cudaMemsetAsync(b.marks, 0, (size_t)n, st));
+        mark_nodes_kernel<<<(unsigned)((n_tr + 255) / 256), 256, 0, st>>>(train_idx, n_tr, kMarkTrain, b.marks);
+        RETEXO_TRY(keep_entries_launch(g, b.marks, 1, b.src_rowptr, b.src_colidx, b.scan_totals, st));
+        retexo_csr kept = g;
+        kept.rowptr = b.src_rowptr;
+        RETEXO_TRY(gat_order_launch(kept, 1, lists, sizes, 1, b.rows_src, nullptr, bins + 3 * kGatOrderInts, hub_entries, st));
     }
     const float* q = feat;
     int64_t ldq = ld_feat;
@@ -578,7 +592,7 @@ extern "C" int retexo_lmp_train(const retexo_lmp_config* cfg, const retexo_lmp_i
             retexo_gat_params gp;
             gp.heads = c.gat_heads; gp.head_dim = c.gat_head_dim; gp.a_src = b.att + (int64_t)r.rep_dim * hd;
             gp.a_dst = gp.a_src + hd; gp.negative_slope = c.gat_negative_slope; gp.add_self_loop = 1;
-            const GatBackwardKept kept{train_rows, all_rows, gat_forward_s(b.ws_agg), gat_forward_t(b.ws_agg, n, c.gat_heads)};
+            const GatBackwardKept kept{train_rows, src_rows, b.src_colidx, gat_forward_s(b.ws_agg), gat_forward_t(b.ws_agg, n, c.gat_heads)};
             RETEXO_TRY(gat_backward(&g, b.proj, ldp, &gp, b.dz, ldp, nullptr, 0, b.dp16, round_up(hd, 64), b.da,
                                     b.da + hd, b.ws_gatbwd, b.ws_gatbwd_bytes, kept_orders ? &kept : nullptr, st));
             TcGemm gw{};      // dW_att = Q^T dP, reduced over the nodes

@@ -43,7 +43,8 @@ inline const float* gat_forward_t(void* ws, int64_t n, int32_t heads) {
 
 // What a caller of retexo_gat_backward that makes many passes over one graph keeps between them (lane layout only).
 struct GatBackwardKept {
-    GatRowOrder dst, src;       // dst: rows whose gradient may be other than zero; src: all rows
+    GatRowOrder dst, src;       // dst: rows whose gradient may be other than zero; src: all rows, of the entries in src_colidx
+    const int32_t* src_colidx;  // the graph's entries whose column is in dst
     const float* s; const float* t;
 };
 // Before the first pass with `kept`: clears what the passes leave as it is for rows that dst does not list.

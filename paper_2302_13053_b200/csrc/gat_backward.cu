@@ -714,6 +714,7 @@ int retexo::gat_backward(const retexo_csr* g, const float* p, int64_t ldp, const
         RETEXO_TRY((gat_lanes_dispatch(lpg, w, [&]<int LPG, int W>() {
             const GatGrid dst_grid = gat_grid<LPG>(dst.n, g->n_edges + n, n_sm, 6 * n_sm), src_grid = gat_grid<LPG>(src.n, g->n_edges + n, n_sm, 6 * n_sm);
             gat_lane_dst_kernel<LPG, W><<<dst_grid.blocks, kGatThreads, 0, st>>>(a, dst, dst_grid);
+            if (kept) a.colidx = kept->src_colidx;
             gat_lane_src_kernel<LPG, W><<<src_grid.blocks, kGatThreads, 0, st>>>(a, src, src_grid, vec, vec16);
             return launch_status();
         })));

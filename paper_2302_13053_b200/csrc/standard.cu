@@ -18,6 +18,7 @@
 #include "aggregate.h"
 #include "common.cuh"
 #include "gemm_tc.h"
+#include "kept_graph.cuh"
 #include "mlp_plan.h"
 
 using namespace retexo;
@@ -92,90 +93,6 @@ static __global__ void __launch_bounds__(32 * kStdRowWarps) std_gate_kernel(cons
         float d = __ldcs(a + v * ld_a + j);
         if (self) d = __ldcs(self + v * ld_self + j) + deg * d;
         dz[v * ld_dz + j] = f32_to_bf16((__ldg(bits + v * ld_bits + k) >> lane) & 1u ? d : 0.f);
-    }
-}
-// ---- the graph without entries that an iteration has no use for (SAGE, whose rows depend on their entries and nothing else)
-constexpr uint8_t kStdTrain = 1, kStdBatch = 2;      // marks of a node: a training row; a training or validation row
-static __global__ void std_mark_kernel(const int32_t* __restrict__ idx, int64_t n, uint8_t value, uint8_t* __restrict__ marks) {
-    const int64_t i = blockIdx.x * 256ll + threadIdx.x;
-    if (i < n) marks[idx[i]] = value;
-}
-// Entries of row v that are kept: all of a batch row's (columns == 0), or those whose column is a training row.
-__device__ __forceinline__ bool std_row_kept(const uint8_t* marks, int64_t v, int columns) { return columns || (marks[v] & kStdBatch); }
-// The rows' kept entries: a warp a row, 128 entries a trip.
-static __global__ void __launch_bounds__(32 * kStdRowWarps) std_count_kept_kernel(int64_t n, const int64_t* __restrict__ rowptr,
-                                                                                  const int32_t* __restrict__ colidx, const uint8_t* __restrict__ marks,
-                                                                                  int columns, int64_t* __restrict__ count) {
-    const int64_t v = std_row();
-    if (v >= n) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t beg = rowptr[v], end = rowptr[v + 1];
-    int kept = 0;
-    if (columns) {
-#pragma unroll 4
-        for (int64_t e = beg + lane; e < end; e += 32) kept += __ldg(marks + __ldcs(colidx + e)) & kStdTrain;
-        kept = __reduce_add_sync(0xffffffffu, kept);
-    }
-    if (lane == 0) count[v] = columns ? (int64_t)kept : std_row_kept(marks, v, columns) ? end - beg : 0;
-}
-// count[v] = sum of count[0, v), in place, and the total behind them, in two launches: every block its own kStdScanRows rows and their total,
-// then every block what lies before it.
-constexpr int kStdScanPer = 8, kStdScanRows = 256 * kStdScanPer;
-static __global__ void __launch_bounds__(256) std_scan_kernel(int64_t n, int64_t* __restrict__ count, int64_t* __restrict__ totals) {
-    __shared__ int64_t warp_total[8];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t i = (int64_t)blockIdx.x * kStdScanRows + threadIdx.x * kStdScanPer;
-    int64_t c[kStdScanPer], mine = 0;
-#pragma unroll
-    for (int k = 0; k < kStdScanPer; ++k) {
-        c[k] = i + k < n ? count[i + k] : 0;
-        mine += c[k];
-    }
-    int64_t at = mine;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int64_t y = __shfl_up_sync(0xffffffffu, at, o);
-        if (lane >= o) at += y;
-    }
-    if (lane == 31) warp_total[warp] = at;
-    at -= mine;
-    __syncthreads();
-    for (int w = 0; w < warp; ++w) at += warp_total[w];
-#pragma unroll
-    for (int k = 0; k < kStdScanPer; ++k) {
-        if (i + k < n) count[i + k] = at;
-        at += c[k];
-    }
-    if (threadIdx.x == 255) totals[blockIdx.x] = at;
-}
-static __global__ void __launch_bounds__(256) std_scan_add_kernel(int64_t n, int64_t* __restrict__ count, const int64_t* __restrict__ totals) {
-    __shared__ unsigned long long before_s;
-    if (threadIdx.x == 0) before_s = 0ull;
-    __syncthreads();
-    unsigned long long part = 0;
-    for (unsigned b = threadIdx.x; b < blockIdx.x; b += 256) part += (unsigned long long)totals[b];
-    if (part) atomicAdd(&before_s, part);
-    __syncthreads();
-    const int64_t before = (int64_t)before_s;
-    for (int64_t i = (int64_t)blockIdx.x * kStdScanRows + threadIdx.x; i < n && i < ((int64_t)blockIdx.x + 1) * kStdScanRows; i += 256) count[i] += before;
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) count[n] = before + totals[blockIdx.x];
-}
-static __global__ void __launch_bounds__(32 * kStdRowWarps) std_copy_kept_kernel(int64_t n, const int64_t* __restrict__ rowptr,
-                                                                                 const int32_t* __restrict__ colidx, const uint8_t* __restrict__ marks,
-                                                                                 int columns, const int64_t* __restrict__ first,
-                                                                                 int32_t* __restrict__ kept) {
-    const int64_t v = std_row();
-    if (v >= n || !std_row_kept(marks, v, columns)) return;
-    const int lane = threadIdx.x & 31;
-    const int64_t beg = rowptr[v], end = rowptr[v + 1];
-    int32_t* dst = kept + first[v];
-    for (int64_t e0 = beg; e0 < end; e0 += 32) {
-        const int64_t e = e0 + lane;
-        const int32_t u = e < end ? __ldcs(colidx + e) : -1;
-        const bool keep = u >= 0 && (!columns || (__ldg(marks + u) & kStdTrain));
-        const unsigned all = __ballot_sync(0xffffffffu, keep);
-        if (keep) dst[__popc(all & ((1u << lane) - 1u))] = u;
-        dst += __popc(all);
     }
 }
 static __global__ void std_copy_if_kernel(const int32_t* decision, const float* src, float* dst, int64_t n) {
@@ -324,7 +241,7 @@ static void std_layout(const retexo_standard_config& c, int64_t n, int64_t e, in
     b.ws_embed_bytes = retexo_embed_workspace_size(last.d, 0, c.n_classes, n);
     b.ws_embed = t.template take<uint8_t>(b.ws_embed_bytes);
     if (std_keeps(c, n, e)) {
-        b.scan_totals = t.template take<int64_t>((size_t)((n + kStdScanRows - 1) / kStdScanRows));
+        b.scan_totals = t.template take<int64_t>((size_t)kept_scan_words(n));
         b.marks = t.template take<uint8_t>((size_t)n);
         for (int i = 0; i < 2; ++i) {
             b.kept_rowptr[i] = t.template take<int64_t>((size_t)n + 1);
@@ -429,15 +346,10 @@ extern "C" int retexo_standard_train(const retexo_standard_config* cfg, const re
     retexo_csr batch_rows = g, train_cols = g;
     if (keeps) {
         RETEXO_CUDA_TRY(cudaMemsetAsync(b.marks, 0, (size_t)n, st));
-        if (n_val) std_mark_kernel<<<(unsigned)((n_val + 255) / 256), 256, 0, st>>>(in->val_idx, n_val, kStdBatch, b.marks);
-        std_mark_kernel<<<(unsigned)((n_tr + 255) / 256), 256, 0, st>>>(in->train_idx, n_tr, kStdBatch | kStdTrain, b.marks);
+        if (n_val) mark_nodes_kernel<<<(unsigned)((n_val + 255) / 256), 256, 0, st>>>(in->val_idx, n_val, kMarkBatch, b.marks);
+        mark_nodes_kernel<<<(unsigned)((n_tr + 255) / 256), 256, 0, st>>>(in->train_idx, n_tr, kMarkBatch | kMarkTrain, b.marks);
         for (int i = 0; i < 2; ++i) {
-            const unsigned blocks = std_row_blocks(n), threads = 32 * kStdRowWarps;
-            std_count_kept_kernel<<<blocks, threads, 0, st>>>(n, g.rowptr, g.colidx, b.marks, i, b.kept_rowptr[i]);
-            const unsigned scan_blocks = (unsigned)((n + kStdScanRows - 1) / kStdScanRows);
-            std_scan_kernel<<<scan_blocks, 256, 0, st>>>(n, b.kept_rowptr[i], b.scan_totals);
-            std_scan_add_kernel<<<scan_blocks, 256, 0, st>>>(n, b.kept_rowptr[i], b.scan_totals);
-            std_copy_kept_kernel<<<blocks, threads, 0, st>>>(n, g.rowptr, g.colidx, b.marks, i, b.kept_rowptr[i], b.kept_colidx[i]);
+            RETEXO_TRY(keep_entries_launch(g, b.marks, i, b.kept_rowptr[i], b.kept_colidx[i], b.scan_totals, st));
             retexo_csr& kept = i ? train_cols : batch_rows;
             kept.rowptr = b.kept_rowptr[i];
             kept.colidx = b.kept_colidx[i];
