@@ -279,7 +279,9 @@ int mlp_train_step_launch(const MlpPlan& p, const MlpBuffers& b, const retexo_ml
         sf.y = y; sf.y_eval = tail ? tail->y_eval : nullptr; sf.inv_rows = 1.0f / (float)n;
         sf.hd = b.hd16; sf.ld_hd = p.ld_h; sf.dl = b.dl16; sf.ld_dl = p.ld_dl; sf.dhd = b.dhd16; sf.ld_dhd = p.ld_h;
         sf.loss_partial = b.loss_partial; sf.correct = tail ? tail->correct : nullptr; sf.status = b.status;
-        sf.x_early = dx_out == nullptr;      // (who trains what produced X has just written it; else the kernel before is an update or a conversion)
+        // the kernel before is the conversion of the weights or (a chain of iterations on one batch) the last update; it is not where X has
+        // just been packed or aggregated
+        sf.x_early = !shadows_ready || (dev && !dx_out);
         RETEXO_TRY(small_forward_launch(sf, st));
         n_loss = (n_all + 31) / 32;
         if (H > 0) { grad1 = b.dhd16; ld_grad1 = p.ld_h; }
