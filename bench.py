@@ -58,7 +58,7 @@ AGG_DRAM_TRAFFIC = {
     "bytes": {("cfg5_gcn_products_like", 1): 46.68e9, ("cfg5_gcn_products_like", 2): 102.92e9,
               ("cfg5_gcn_products_like", 3): 102.93e9}}
 # one stand-alone training iteration (its tensor-core launches and reduce_update_kernel): profiles/kernel_counters.txt
-STEP_SOURCES = ("gemm_tc.cu", "grad_tc.cu", "mlp_fused.cu", "mlp.cu", "mlp_kernels.cuh", "tc_common.cuh", "launch_overlap.cuh")
+STEP_SOURCES = ("gemm_tc.cu", "grad_tc.cu", "mlp_fused.cu", "class_loss.cuh", "mlp.cu", "mlp_kernels.cuh", "tc_common.cuh", "launch_overlap.cuh")
 STEP_DRAM_TRAFFIC = {
     "fingerprint": "2b5f4ad07051",
     "bytes": {("cfg4_sage_reddit_like", 1): 1.147e9}}
@@ -197,10 +197,11 @@ def launches_per_step(w, R: int) -> int:
             total += 3 + 2                           # prep, warp rows, block rows; train / val batches
         step = 5 if h > 0 else 3                     # products, fused middle, reduce + update (+ weight copies once)
         if trained_gat:
-            # the aggregator is trained with the model: per iteration projection + aggregation + batches before
-            # the step, input gradient inside it, kept copy + scatter + backward (4) + dW_att + update after it
-            step += gat_forward + 2 + 1 + 8
-            total += gat_forward + 2                 # the last iterate's own validation pass
+            # the aggregator is trained with the model: per iteration projection, scores and rows before the step, input
+            # gradient inside it, backward (3) + dW_att + update after it
+            step += 3 + 1 + 5
+            total += 11 if rd["round"] == 1 else 0   # the row orders and the graph of training columns, once
+            total += gat_forward                     # the last iterate's own validation pass
         total += R * step + 1 + (2 if h > 0 else 1)       # (the update kernel's last block books the validation count
                                                           #  that rides along; the last iterate's is booked by a kernel of its own)
         total += (2 if h > 0 else 1) + 1             # stand-alone validation of the last iterate + snapshot
@@ -209,13 +210,20 @@ def launches_per_step(w, R: int) -> int:
     return total
 
 
+def small_batches(w, rd) -> bool:
+    """Whether the round's iterations take the two kernels of a small batch."""
+    return rd["hidden"] <= 128 and rd["d_in"] <= 4480 and len(w.train_idx) <= 512 and len(w.train_idx) + len(w.val_idx) <= 4736
+
+
 def shared_launches(w, R: int) -> int:
-    """Of launches_per_step's kernels, those that share a launch: an iteration's two weight-gradient products, wherever the
-    weight copies are built both layers', and a trained aggregator's scatter and kept copy."""
-    from paper_2302_13053_b200 import workloads as wl
-    per_round = R + 1 + 2 + 1                        # iterations, the round's first copies, two test passes, the emission
-    total = per_round * sum(1 for rd in w.round_dims() if rd["hidden"] > 0)
-    return total + (R * w.K if w.aggr == wl.GAT and not FREEZE_ATTENTION else 0)
+    """Of launches_per_step's kernels, those that share a launch: an iteration's two weight-gradient products (of a small batch all
+    products but the weight gradients' and the update), and wherever the weight copies are built both layers'."""
+    total = 0
+    for rd in w.round_dims():
+        small, hidden = small_batches(w, rd), rd["hidden"] > 0
+        total += R * ((3 if hidden else 1) if small else (1 if hidden else 0))
+        total += 1 + 2 + 1 if hidden else 0          # the round's first copies, two test passes, the emission
+    return total
 
 
 def time_calls(fn, reps: int, warm: int = 3):
